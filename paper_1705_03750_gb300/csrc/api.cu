@@ -19,7 +19,7 @@ constexpr double kPi = 3.14159265358979323846;
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct Layout {
-  size_t fini, eta, f, tmp, map, slot1, rec_key, rec_site, holes_a, holes_b, ovf, gwin, seed, el, tay, tayf, M, a, da, d2a,
+  size_t fini, eta, f, tmp, map, slot1, rec_key, rec_site, holes_a, holes_b, ovf, gwin, seed, el, tay, tayf, tayx, M, a, da, d2a,
       thx, thv, thxf, thvf, rect, mpart, dpart, ds, total;
 };
 
@@ -80,6 +80,7 @@ Layout layout(const vm_config* c) {
   L.el = take(12 * ne * 8);
   L.tay = take(16 * ne * 8);
   L.tayf = take(32 * ne * 4);
+  L.tayx = take(sr == 8 ? ne * sizeof(vm::FxRec) : 0);
   L.M = take(c->nx * 8);
   L.a = take(c->nx * 8);
   L.da = take(c->nx * 8);
@@ -436,6 +437,22 @@ vm_status vm::solver_create(const vm_config* c, void* d_workspace, size_t bytes,
   g.inv_dvm = 1.0 / g.dvm;
   g.r_vx = g.dvm / g.dxm;
   g.r_xv = g.dxm / g.dvm;
+  g.dxm_f = (float)g.dxm;
+  g.dvm_f = (float)g.dvm;
+  g.r_vx_f = (float)g.r_vx;
+  g.r_xv_f = (float)g.r_xv;
+  g.inv_dxm_f = (float)g.inv_dxm;
+  g.inv_dvm_f = (float)g.inv_dvm;
+  g.fx_k[0] = -0.5 * g.dx;
+  g.fx_k[1] = -g.dv;
+  g.fx_k[2] = -0.5 * g.dv * g.r_vx;
+  g.fx_k[3] = -0.5 * g.dx * g.r_xv;
+  g.fx_k[4] = -g.dx;
+  g.fx_k[5] = -0.5 * g.dv;
+  // (strides and margins the fixed-point remap's formats hold)
+  const bool fx = g.s >= 2 && g.s <= 64 && c->beta <= 1.0;
+  g.fx_inv_s = fx ? (long long)((1ull << 63) / (unsigned)g.s) : 0;
+  g.fx_beta = fx ? (long long)(c->beta * (double)g.s * (double)(1ll << vm::FX_Q)) : 0;
   g.cx = 0.5 * (c->x_lo + c->x_hi);
   g.cv = 0.5 * (c->v_lo + c->v_hi);
   g.dxdv = g.dx * g.dv;
@@ -473,6 +490,7 @@ vm_status vm::solver_create(const vm_config* c, void* d_workspace, size_t bytes,
   s->el = (double*)(base + L.el);
   s->tay = (double*)(base + L.tay);
   s->tayf = (float*)(base + L.tayf);
+  s->tayx = s->fp32 ? nullptr : (vm::FxRec*)(base + L.tayx);
   s->M = (double*)(base + L.M);
   s->a = (double*)(base + L.a);
   s->da = (double*)(base + L.da);

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "../../include/vlamet.h"
+#include "fixed.cuh"
 
 namespace vm {
 
@@ -34,6 +35,9 @@ struct Grid {
   double alpha, beta;
   double dt, half_dt, A;  // A = 2 pi G
   double r_vx, r_xv;      // dv_m/dx_m and dx_m/dv_m
+  float dxm_f, dvm_f, r_vx_f, r_xv_f, inv_dxm_f, inv_dvm_f;  // rounded to FP32
+  double fx_k[6];         // second-order factors of the fixed-point records (cells per site^2), x axis then v
+  long long fx_inv_s, fx_beta;  // 2^63 / s; beta s in fixed-point cells (0: the remap in FP64)
   int32_t literal_fd;
   int32_t max_hole_rounds;
   // adaptive computing domain (Sec. 2.2.1, eq. constrf; Sec. 2.3): fth_on
@@ -182,6 +186,7 @@ struct vm_solver {
   double* el;               // 12 x ne
   double* tay;              // ne x 16
   float* tayf;              // ne x 32 (FP32 record, element units)
+  vm::FxRec* tayx;          // ne fixed-point records (FP64 solves; else NULL)
   double* M;                // pixel masses of the last step
   double* a;
   double* da;
@@ -306,6 +311,7 @@ struct SolveDesc {
   double* el;
   double* tay;
   float* tayf;
+  FxRec* tayx;
   double* M;
   double* a;
   double* da;

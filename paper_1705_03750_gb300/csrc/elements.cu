@@ -14,16 +14,27 @@
 namespace vm {
 namespace {
 
+// d rounded to the nearest FP32 value from its bits (ties away from zero):
+// the conversion instruction runs on the FP64 pipe, at 1/64 of the integer
+// rate.  Values below the normal FP32 range become 0.
+__device__ __forceinline__ float f32_of(double d) {
+  const int hi = __double2hiint(d), e = (hi >> 20) & 0x7ff;
+  const unsigned lo = (unsigned)__double2loint(d);
+  if (e > 1149) return (float)d;  // near or above the FP32 range, or not a number
+  const int b = (((hi & 0x7fffffff) - (896 << 20)) << 3) + (int)(lo >> 29) + (int)((lo >> 28) & 1u);
+  return __int_as_float((e > 896 ? b : 0) | (hi & (int)0x80000000));
+}
+
 // FP32 record of element m (see TF_* in common.cuh) from its FP64 terms,
 // in FP32 arithmetic (FP64 runs at 1/64 of the FP32 rate here): each
 // coefficient carries up to ten roundings, within the budget of the
 // certified decisions' bound constants; the bound coefficients are rounded
 // upwards at every operation, with a slack of 1e-5 over the FP32 values
 // that also covers their distance to the FP64 ones.
-__device__ __forceinline__ void taylor_f32(const Grid& g, const double* t, float* __restrict__ F) {
-  const float dxm = (float)g.dxm, dvm = (float)g.dvm;
-  const float ti00 = (float)t[TY_TI00], ti01 = (float)t[TY_TI01], ti10 = (float)t[TY_TI10], ti11 = (float)t[TY_TI11];
-  const float T00 = ti00, T01 = ti01 * (float)g.r_vx, T10 = ti10 * (float)g.r_xv, T11 = ti11;
+__device__ __forceinline__ void taylor_f32(const Grid& g, const double (&t)[TY_N], float (&F)[TF_N]) {
+  const float dxm = g.dxm_f, dvm = g.dvm_f;
+  const float ti00 = f32_of(t[TY_TI00]), ti01 = f32_of(t[TY_TI01]), ti10 = f32_of(t[TY_TI10]), ti11 = f32_of(t[TY_TI11]);
+  const float T00 = ti00, T01 = ti01 * g.r_vx_f, T10 = ti10 * g.r_xv_f, T11 = ti11;
   F[TF_T00] = T00;
   F[TF_T01] = T01;
   F[TF_T10] = T10;
@@ -31,13 +42,13 @@ __device__ __forceinline__ void taylor_f32(const Grid& g, const double* t, float
   float gs[2], G00[2], G01[2], G11[2];
 #pragma unroll
   for (int l = 0; l < 2; l++) {
-    G00[l] = (float)t[TY_GX00 + 3 * l] * (dxm * dxm);
-    G01[l] = (float)t[TY_GX01 + 3 * l] * (dxm * dvm);
-    G11[l] = (float)t[TY_GX11 + 3 * l] * (dvm * dvm);
+    G00[l] = f32_of(t[TY_GX00 + 3 * l]) * (dxm * dxm);
+    G01[l] = f32_of(t[TY_GX01 + 3 * l]) * (dxm * dvm);
+    G11[l] = f32_of(t[TY_GX11 + 3 * l]) * (dvm * dvm);
     gs[l] = __fadd_ru(__fadd_ru(fabsf(G00[l]), __fmul_ru(2.f, fabsf(G01[l]))), fabsf(G11[l]));
   }
-  const float K00 = ti00 * (float)g.inv_dxm, K01 = ti01 * (float)g.inv_dxm;
-  const float K10 = ti10 * (float)g.inv_dvm, K11 = ti11 * (float)g.inv_dvm;
+  const float K00 = ti00 * g.inv_dxm_f, K01 = ti01 * g.inv_dxm_f;
+  const float K10 = ti10 * g.inv_dvm_f, K11 = ti11 * g.inv_dvm_f;
   // -1/2 (K[a][0] s_x + K[a][1] s_v) = A_a p_x^2 + B_a p_x p_v + C_a p_v^2
   F[TF_AX] = -0.5f * (K00 * G00[0] + K01 * G00[1]);
   F[TF_BX] = -(K00 * G01[0] + K01 * G01[1]);
@@ -53,24 +64,79 @@ __device__ __forceinline__ void taylor_f32(const Grid& g, const double* t, float
   const double u = t[TY_U], w = t[TY_W];
   const double ui = floor(u), wi = floor(w);
   const bool ok = (u > -1e9 && u < 1e9 && w > -1e9 && w < 1e9);
-  F[TF_UF] = ok ? (float)(u - ui) : 0.f;
-  F[TF_WF] = ok ? (float)(w - wi) : 0.f;
-  reinterpret_cast<int*>(F)[TF_UI] = ok ? (int)ui : INT_MIN / 2;
-  reinterpret_cast<int*>(F)[TF_WI] = ok ? (int)wi : INT_MIN / 2;
-  reinterpret_cast<double2*>(F + TF_UD)[0] = make_double2(u, w);
+  F[TF_UF] = ok ? f32_of(u - ui) : 0.f;
+  F[TF_WF] = ok ? f32_of(w - wi) : 0.f;
+  F[TF_UI] = __int_as_float(ok ? (int)ui : INT_MIN / 2);
+  F[TF_WI] = __int_as_float(ok ? (int)wi : INT_MIN / 2);
+  F[TF_WI + 1] = F[TF_WI + 2] = 0.f;  // (unused words)
+  F[TF_UD] = __int_as_float(__double2loint(u));
+  F[TF_UD + 1] = __int_as_float(__double2hiint(u));
+  F[TF_UD + 2] = __int_as_float(__double2loint(w));
+  F[TF_UD + 3] = __int_as_float(__double2hiint(w));
 }
 
-__device__ __forceinline__ void taylor_one(const Grid& g, const double* __restrict__ el, int m,
-                                           double* __restrict__ tay, float* __restrict__ tayf) {
-  const int ne = g.ne;
-  double x = el[EL_X * ne + m], v = el[EL_V * ne + m];
-  double Txx = el[EL_TXX * ne + m], Txv = el[EL_TXV * ne + m];
-  double Tvx = el[EL_TVX * ne + m], Tvv = el[EL_TVV * ne + m];
+// Fixed-point record of element m (FxRec) from its FP64 terms t: the inverse
+// map in cells expanded about the start site (i0, l0) nearest to P_m.  With
+// delta the start site's offset from P_m, K the second-order coefficients of
+// the map and L its linear ones: c0 = half + L delta + K delta^2, c1 = L +
+// 2 K delta, c2 = K; the expansion in integers (one FP64 operation takes the
+// time of 64 of 32 bits here).  F: the element's FP32 record, whose bounds
+// C1, C2 of the uncombined terms set the largest site offset served, the one
+// up to which all terms together stay below FX_MAX cells.
+__device__ __forceinline__ void taylor_fixed(const Grid& g, const double (&t)[TY_N], double iu, double iw, int k,
+                                             int l, const float (&F)[TF_N], FxRec* __restrict__ X) {
+  const float C1 = F[TF_C1X] + F[TF_C1V], C2 = F[TF_C2X] + F[TF_C2V], sf = (float)g.s;
+  int lim = 0;
+#pragma unroll
+  for (int L = FX_LIM; L >= 2; L >>= 1) {
+    const float p = ((float)L + 0.51f) / sf;
+    if (lim == 0 && 0.51f + sf * (C1 * p + C2 * (p * p)) < (float)FX_MAX) lim = L;
+  }
+  if (!(fabs(iu) < 1e6 && fabs(iw) < 1e6)) lim = 0;
+  if (lim == 0) {
+    X->lim = 0;
+    return;
+  }
+  const int u2 = (g.nx - 1) + 2 * (k - g.Kx - 1) * g.s, w2 = (g.nv - 1) + 2 * (l - g.Kv - 1) * g.s;
+  const long long ex = fx_of(cells_from(t[TY_X], g.x_lo, g.dx, g.inv_dx, iu), 62);
+  const long long ev = fx_of(cells_from(t[TY_V], g.v_lo, g.dv, g.inv_dv, iw), 62);
+#pragma unroll
+  for (int a = 0; a < 2; a++) {
+    const double A = t[TY_TI00 + 2 * a], B = t[TY_TI01 + 2 * a];
+    const double s00 = fma(B, t[TY_GV00], A * t[TY_GX00]), s01 = fma(B, t[TY_GV01], A * t[TY_GX01]),
+                 s11 = fma(B, t[TY_GV11], A * t[TY_GX11]);
+    const long long L1 = fx_of(a == 0 ? A : A * g.r_xv, FX_Q), L2 = fx_of(a == 0 ? B * g.r_vx : B, FX_Q);
+    const long long K3 = fx_of(s00 * g.fx_k[3 * a], FX_Q), K4 = fx_of(s01 * g.fx_k[3 * a + 1], FX_Q),
+                    K5 = fx_of(s11 * g.fx_k[3 * a + 2], FX_Q);
+    const long long t1 = L1 + fx_mul62(K4, ev);
+    const long long half = (((a == 0 ? u2 : w2) & 1) ? 1ll : 0ll) << (FX_Q - 1);
+    const long long c0 = half + fx_mul62(t1 + fx_mul62(K3, ex), ex) + fx_mul62(L2 + fx_mul62(K5, ev), ev);
+    longlong2* c = reinterpret_cast<longlong2*>(X->c + 6 * a);
+    c[0] = make_longlong2(c0, t1 + fx_mul62(2 * K3, ex));
+    c[1] = make_longlong2(L2 + fx_mul62(K4, ex) + fx_mul62(2 * K5, ev), K3);
+    c[2] = make_longlong2(K4, K5);
+  }
+  *reinterpret_cast<int4*>(&X->i0) = make_int4((int)iu, (int)iw, u2 >> 1, w2 >> 1);
+  X->lim = lim;
+}
+
+__device__ __forceinline__ void load_element(const Grid& g, const double* __restrict__ el, int m, double (&e)[EL_N]) {
+#pragma unroll
+  for (int q = 0; q < EL_N; q++) e[q] = el[(size_t)q * g.ne + m];
+}
+
+__device__ __forceinline__ void taylor_one(const Grid& g, const double (&e)[EL_N], int m, double* __restrict__ tay,
+                                           float* __restrict__ tayf, FxRec* __restrict__ tayx) {
+  const double x = e[EL_X], v = e[EL_V];
+  const double Txx = e[EL_TXX], Txv = e[EL_TXV], Tvx = e[EL_TVX], Tvv = e[EL_TVV];
   // T^-1 = adj(T) (1/det T): one division (FP64 division is slow here)
   const double det = dsub(dmul(Txx, Tvv), dmul(Txv, Tvx));
   const double id = 1.0 / det;
   const double Ti00 = dmul(Tvv, id), Ti01 = dmul(-Txv, id), Ti10 = dmul(-Tvx, id), Ti11 = dmul(Txx, id);
-  double* t = tay + (size_t)m * TY_N;
+  // the records in registers, stored at the end in 16-byte words (read back
+  // from memory after each store they cost more than their arithmetic)
+  double t[TY_N];
+  float F[TF_N];
   t[TY_X] = x;
   t[TY_V] = v;
   t[TY_TI00] = Ti00;
@@ -79,9 +145,7 @@ __device__ __forceinline__ void taylor_one(const Grid& g, const double* __restri
   t[TY_TI11] = Ti11;
 #pragma unroll
   for (int l = 0; l < 2; l++) {
-    double h0 = el[(EL_HXXX + 3 * l) * ne + m];
-    double h1 = el[(EL_HXXV + 3 * l) * ne + m];
-    double h2 = el[(EL_HXVV + 3 * l) * ne + m];
+    const double h0 = e[EL_HXXX + 3 * l], h1 = e[EL_HXXV + 3 * l], h2 = e[EL_HXVV + 3 * l];
     // A = H_l T^-1, G_l = [T^-1]^T A
     double A00 = dadd(dmul(h0, Ti00), dmul(h1, Ti10));
     double A01 = dadd(dmul(h0, Ti01), dmul(h1, Ti11));
@@ -97,35 +161,52 @@ __device__ __forceinline__ void taylor_one(const Grid& g, const double* __restri
   // index position of P_m, as the start site of the percolation uses it
   t[TY_U] = dmul(dsub(x, g.x_lo), g.inv_dx);
   t[TY_W] = dmul(dsub(v, g.v_lo), g.inv_dv);
-  taylor_f32(g, t, tayf + (size_t)m * TF_N);
+  taylor_f32(g, t, F);
+  if (tayx) taylor_fixed(g, t, floor(t[TY_U] + 0.5), floor(t[TY_W] + 0.5), k, l, F, tayx + m);
+  double2* to = reinterpret_cast<double2*>(tay + (size_t)m * TY_N);
+#pragma unroll
+  for (int c = 0; c < TY_N / 2; c++) to[c] = make_double2(t[2 * c], t[2 * c + 1]);
+  float4* Fo = reinterpret_cast<float4*>(tayf + (size_t)m * TF_N);
+#pragma unroll
+  for (int c = 0; c < (TF_UD + 4) / 4; c++) Fo[c] = make_float4(F[4 * c], F[4 * c + 1], F[4 * c + 2], F[4 * c + 3]);
 }
 
 // Half drift (predictor or corrector of Sec. 2.4): x, T_x. and H_x.. move
 // with v, T_v. and H_v..; optionally followed by the Taylor terms.
 __device__ __forceinline__ void drift_body(const Grid& g, double* __restrict__ el, double* __restrict__ tay,
-                                           float* __restrict__ tayf, int taylor, int vb) {
+                                           float* __restrict__ tayf, FxRec* __restrict__ tayx, int taylor, int vb) {
   int m = vb * blockDim.x + threadIdx.x;
   if (m >= g.ne) return;
   const int ne = g.ne;
-  double h = g.half_dt;
-  el[EL_X * ne + m] = dadd(el[EL_X * ne + m], dmul(el[EL_V * ne + m], h));
-  el[EL_TXX * ne + m] = dadd(el[EL_TXX * ne + m], dmul(el[EL_TVX * ne + m], h));
-  el[EL_TXV * ne + m] = dadd(el[EL_TXV * ne + m], dmul(el[EL_TVV * ne + m], h));
+  const double h = g.half_dt;
+  double e[EL_N];
+  load_element(g, el, m, e);
+  e[EL_X] = dadd(e[EL_X], dmul(e[EL_V], h));
+  e[EL_TXX] = dadd(e[EL_TXX], dmul(e[EL_TVX], h));
+  e[EL_TXV] = dadd(e[EL_TXV], dmul(e[EL_TVV], h));
 #pragma unroll
-  for (int q = 0; q < 3; q++)
-    el[(EL_HXXX + q) * ne + m] = dadd(el[(EL_HXXX + q) * ne + m], dmul(el[(EL_HVXX + q) * ne + m], h));
-  if (taylor) taylor_one(g, el, m, tay, tayf);
+  for (int q = 0; q < 3; q++) e[EL_HXXX + q] = dadd(e[EL_HXXX + q], dmul(e[EL_HVXX + q], h));
+  el[EL_X * ne + m] = e[EL_X];
+  el[EL_TXX * ne + m] = e[EL_TXX];
+  el[EL_TXV * ne + m] = e[EL_TXV];
+#pragma unroll
+  for (int q = 0; q < 3; q++) el[(EL_HXXX + q) * ne + m] = e[EL_HXXX + q];
+  if (taylor) taylor_one(g, e, m, tay, tayf, tayx);
 }
 
 __global__ void k_drift(Grid g, double* __restrict__ el, double* __restrict__ tay, float* __restrict__ tayf,
-                        int taylor) {
-  drift_body(g, el, tay, tayf, taylor, blockIdx.x);
+                        FxRec* __restrict__ tayx, int taylor) {
+  drift_body(g, el, tay, tayf, tayx, taylor, blockIdx.x);
 }
 
-__global__ void k_taylor(Grid g, const double* __restrict__ el, double* __restrict__ tay, float* __restrict__ tayf) {
+__global__ void k_taylor(Grid g, const double* __restrict__ el, double* __restrict__ tay, float* __restrict__ tayf,
+                         FxRec* __restrict__ tayx) {
   if (gate_shut(g)) return;
   int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m < g.ne) taylor_one(g, el, m, tay, tayf);
+  if (m >= g.ne) return;
+  double e[EL_N];
+  load_element(g, el, m, e);
+  taylor_one(g, e, m, tay, tayf, tayx);
 }
 
 // Dual TSC interpolation (Sec. 2.5) at index coordinate u; beyond the grid
@@ -402,14 +483,18 @@ __global__ void k_force_diff(Grid g, const double* __restrict__ a, double* __res
 __global__ void k_drift_group(const SolveDesc* __restrict__ D, const int* __restrict__ off, int ns, int total,
                               int taylor) {
   GROUP_LOOP(off, ns, total)
-  drift_body(gsh, d.el, d.tay, d.tayf, taylor, vb);
+  drift_body(gsh, d.el, d.tay, d.tayf, d.tayx, taylor, vb);
   GROUP_END
 }
 
 __global__ void k_taylor_group(const SolveDesc* __restrict__ D, const int* __restrict__ off, int ns, int total) {
   GROUP_LOOP(off, ns, total)
   const int m = vb * blockDim.x + threadIdx.x;
-  if (m < gsh.ne) taylor_one(gsh, d.el, m, d.tay, d.tayf);
+  if (m < gsh.ne) {
+    double e[EL_N];
+    load_element(gsh, d.el, m, e);
+    taylor_one(gsh, e, m, d.tay, d.tayf, d.tayx);
+  }
   GROUP_END
 }
 
@@ -661,26 +746,27 @@ inline unsigned blocks_for(long long n, int t) { return (unsigned)((n + t - 1) /
 // Element kernels are FP64-bound (two FP64 lanes per SM per clock): small
 // blocks spread a small lattice over many SMs.
 constexpr int ET = 64;
+inline int elem_threads(int ne) { return ne <= 152 * 2 * ET ? 32 : ET; }
 
 }  // namespace
 
 void launch_drift(vm_solver* s, bool taylor) {
-  { const int ps_ = prof_begin(s, KID_DRIFT); k_drift<<<blocks_for(s->g.ne, ET), ET, 0, s->stream>>>(s->g, s->el, s->tay, s->tayf, taylor ? 1 : 0); prof_end(s, ps_); }
+  { const int ps_ = prof_begin(s, KID_DRIFT); k_drift<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el, s->tay, s->tayf, s->tayx, taylor ? 1 : 0); prof_end(s, ps_); }
   s->launches++;
 }
 
 void launch_taylor(vm_solver* s) {
-  { const int ps_ = prof_begin(s, KID_TAYLOR); k_taylor<<<blocks_for(s->g.ne, ET), ET, 0, s->stream>>>(s->g, s->el, s->tay, s->tayf); prof_end(s, ps_); }
+  { const int ps_ = prof_begin(s, KID_TAYLOR); k_taylor<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el, s->tay, s->tayf, s->tayx); prof_end(s, ps_); }
   s->launches++;
 }
 
 void launch_kick_drift(vm_solver* s) {
-  { const int ps_ = prof_begin(s, KID_KICK_DRIFT); k_kick_drift<<<blocks_for(s->g.ne, ET), ET, 0, s->stream>>>(s->g, s->el, s->a, s->da, s->d2a, s->ds); prof_end(s, ps_); }
+  { const int ps_ = prof_begin(s, KID_KICK_DRIFT); k_kick_drift<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el, s->a, s->da, s->d2a, s->ds); prof_end(s, ps_); }
   s->launches++;
 }
 
 void launch_reset_elements(vm_solver* s) {
-  { const int ps_ = prof_begin(s, KID_RESET); k_reset<<<blocks_for(s->g.ne, ET), ET, 0, s->stream>>>(s->g, s->el); prof_end(s, ps_); }
+  { const int ps_ = prof_begin(s, KID_RESET); k_reset<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el); prof_end(s, ps_); }
   s->launches++;
 }
 

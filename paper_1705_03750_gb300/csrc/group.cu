@@ -53,6 +53,7 @@ SolveDesc desc_of(const vm_solver* s, bool gated) {
   d.el = s->el;
   d.tay = s->tay;
   d.tayf = s->tayf;
+  d.tayx = s->tayx;
   d.M = s->M;
   d.a = s->a;
   d.da = s->da;

@@ -6,9 +6,9 @@
 // Q_r blended over the beta set of elements with the Monaghan kernel, then
 // the cubic B-spline of f_ini at Q_r.
 //
-// FP64 path: Q, the node choice and the interpolation in FP64, the decisions
-// taken in a fixed operation order (the remap's blend, continuous in its
-// inputs, in fused FP64 once the beta ranges are decided).  FP32-mixed path: Q from the element's FP32
+// FP64 path: offsets and sums in 64-bit fixed point (fixed.cuh), the node and
+// beta decisions those of the FP64 evaluation in a fixed operation order, which
+// also serves the sites the fixed-point records do not reach.  FP32-mixed path: Q from the element's FP32
 // record in element units, anchored on the exact lattice position of Q_m, so
 // that only the small offset carries FP32 rounding; the integer decisions
 // (nearest node, containing square, beta ranges) are taken from the FP32
@@ -93,54 +93,81 @@ __device__ __forceinline__ void zero_outside(const Grid& g, R* __restrict__ row,
   for (int j = j1 + 1 + threadIdx.x; j < g.nv; j += blockDim.x) row[j] = R(0);
 }
 
-// FP64 path.  The integer decisions (nearest node, containing cell) come
-// from the FP32 record's certified evaluation, which is the fixed-order FP64
-// evaluation's whenever its bound clears every decision boundary (as on the
-// FP32-mixed path); the offset Q - Q_m is then evaluated in FP64 with fused
-// operations, anchored on the exact lattice position of Q_m, and the
-// six-point value with fused operations (rounding changes only).  A site
-// whose decision the bound leaves open (the step after a remap puts every
-// Q on a node) is evaluated entirely in the fixed order.
-__device__ __forceinline__ bool recon64_fast(const Grid& g, const double* __restrict__ t, const float* __restrict__ F,
-                                             int m, int i, int j, double Px, double Pv,
-                                             const double* __restrict__ fini, float inv_Lv, double& val);
-
-__device__ __forceinline__ double qinterp64_fused(const double* __restrict__ F, const Grid& g, long long in,
-                                                  long long jn, long long ic, long long jc, double x, double y) {
-  const double hx = 0.5 * x, hy = 0.5 * y;
-  double f = F_at(F, g, in, jn) * fma(-y, y, fma(-x, x, 1.0));
-  f = fma(F_at(F, g, in + 1, jn), fma(hx, x, hx), f);
-  f = fma(F_at(F, g, in - 1, jn), fma(hx, x, -hx), f);
-  f = fma(F_at(F, g, in, jn + 1), fma(hy, y, hy), f);
-  f = fma(F_at(F, g, in, jn - 1), fma(hy, y, -hy), f);
-  const double cross = (F_at(F, g, ic + 1, jc + 1) + F_at(F, g, ic, jc)) - (F_at(F, g, ic + 1, jc) + F_at(F, g, ic, jc + 1));
-  return fma(cross, x * y, f);
+// FP64 path.  The offset Q - Q_m comes from the element's fixed-point record
+// (FxRec): an integer polynomial of the site's offset from the element's
+// start site, in units of 2^-52 cells, more exact than its FP64 evaluation
+// (whose index position of up to 2^13 cells keeps 39 bits of fraction).  The
+// nearest node is read from it when it clears the half-integer by FX_MARGIN,
+// and is then the fixed-order FP64 evaluation's; the containing cell is read
+// from its sign: f is continuous across the cell's edge (the cross term
+// vanishes there), so a cell taken on the other side of a rounding error
+// changes f by that rounding only.  The six node values are scaled to
+// integers of 60 bits by the largest one's exponent and the second-order
+// surface is evaluated on them exactly as in Sec. 2.2.1, regrouped by the
+// node's side of Q (s) and the opposite one (o):
+//   f = F0 + x [(Fxs - Fxo)/2 + x (Fxs + Fxo - 2 F0)/2 + y (F0 + Fd - Fxs - Fys)]
+//          + y [(Fys - Fyo)/2 + y (Fys + Fyo - 2 F0)/2],   x, y >= 0.
+// Returns false (nothing written) where the record, the margin, the grid's
+// edge or the values' range do not allow it.  At 4096^2: 0.361 ms per step,
+// bound by the integer pipes; the fused FP64 evaluation before it took
+// 1.857 ms, bound by the two FP64 lanes (some 69 operations a site).  Error
+// against 128-bit arithmetic (2-norm, 128^2 to 1023 x 640 evolved states):
+// 0.5 to 2.3e-16, before 0.9 to 2.3e-15.
+__device__ __forceinline__ bool recon64_fixed(const Grid& g, const FxRec* __restrict__ X, int i, int j,
+                                              const double* __restrict__ fini, double& val) {
+  long long ru, rw;
+  int4 o;
+  if (!fx_offset(X, i, j, ru, rw, o)) return false;
+  constexpr long long half = 1ll << (FX_Q - 1);
+  const long long nu = (ru + half) >> FX_Q, nw = (rw + half) >> FX_Q;
+  const long long xs = ru - (nu << FX_Q), ys = rw - (nw << FX_Q);
+  const long long xa = xs < 0 ? -xs : xs, ya = ys < 0 ? -ys : ys;
+  const int in = o.z + (int)nu, jn = o.w + (int)nw;
+  if (max(xa, ya) > half - FX_MARGIN || in < 1 || in > g.nx - 2 || jn < 1 || jn > g.nv - 2) return false;
+  const double* p = fini + (size_t)in * g.nv + jn;
+  const long long sx = xs < 0 ? -(long long)g.nv : (long long)g.nv;
+  const int sy = ys < 0 ? -1 : 1;
+  const double F0 = __ldg(p), Fxs = __ldg(p + sx), Fxo = __ldg(p - sx), Fys = __ldg(p + sy), Fyo = __ldg(p - sy),
+               Fd = __ldg(p + sx + sy);
+  const int em = max(max(max(fx_exp(F0), fx_exp(Fxs)), max(fx_exp(Fxo), fx_exp(Fys))), max(fx_exp(Fyo), fx_exp(Fd)));
+  if (em < 128 || em > 2040) {
+    val = 0.0;
+    return F0 == 0.0 && Fxs == 0.0 && Fxo == 0.0 && Fys == 0.0 && Fyo == 0.0 && Fd == 0.0;
+  }
+  const long long i0 = fx_int(F0, em), ixs = fx_int(Fxs, em), ixo = fx_int(Fxo, em), iys = fx_int(Fys, em),
+                  iyo = fx_int(Fyo, em), id = fx_int(Fd, em);
+  const long long x = xa << (64 - FX_Q), y = ya << (64 - FX_Q);  // Q64, below 1/2
+  const long long sumx = ixs + ixo - 2 * i0, sumy = iys + iyo - 2 * i0, cr = i0 + id - ixs - iys;
+  const long long gx = ((ixs - ixo + fx_mul(sumx, x)) >> 1) + fx_mul(cr, y);
+  const long long gy = (iys - iyo + fx_mul(sumy, y)) >> 1;
+  val = fx_double(i0 + fx_mul(gx, x) + fx_mul(gy, y), em);
+  return true;
 }
 
 __device__ __forceinline__ void k_recon64_body(const Grid& g, const uint32_t* __restrict__ map, const DevState* ds,
-                                                 const double* __restrict__ tay, const float* __restrict__ tayf,
+                                                 const double* __restrict__ tay, const FxRec* __restrict__ tayx,
                                                  const double* __restrict__ fini, double* __restrict__ f,
                                                  double* __restrict__ M, int vb) {
   using R = double;
   __shared__ double sh[32];
   const int i = vb;
-  const double Px = site_x(g, i);
   int js, je;
   row_span(g, ds, i, js, je);
   zero_outside(g, f + (size_t)i * g.nv, js, je);
-  const float inv_Lv = 1.0f / (float)g.Lv;
+  const uint32_t epoch = ds_epoch(ds);
   double acc = 0.0;
+  // the owner of the thread's next site is loaded one iteration ahead
+  int m = (js + (int)threadIdx.x <= je) ? owner(map, (size_t)i * g.nv + js + threadIdx.x, epoch, g.ne) : -1;
   for (int j = js + threadIdx.x; j <= je; j += blockDim.x) {
     const size_t p = (size_t)i * g.nv + j;
-    const int m = owner(map, p, ds_epoch(ds), g.ne);
+    const int mn = (j + (int)blockDim.x <= je) ? owner(map, p + blockDim.x, epoch, g.ne) : -1;
     double val = 0.0;
     if (m >= 0) {
-      const double* t = tay + (size_t)m * TY_N;
-      const double Pv = site_v(g, j);
-      if (!recon64_fast(g, t, tayf + (size_t)m * TF_N, m, i, j, Px, Pv, fini, inv_Lv, val)) {
-        // a decision the FP32 bound cannot settle: the fixed order
+      if (!recon64_fixed(g, tayx + m, i, j, fini, val)) {
+        // outside the fixed-point record's reach: the fixed order in FP64
+        const double* t = tay + (size_t)m * TY_N;
         double dqx, dqv;
-        qofp_exact(t, Px, Pv, dqx, dqv);
+        qofp_exact(t, site_x(g, i), site_v(g, j), dqx, dqv);
         const double u = dmul(dsub(dadd(t[TY_QX], dqx), g.x_lo), g.inv_dx);
         const double w = dmul(dsub(dadd(t[TY_QV], dqv), g.v_lo), g.inv_dv);
         val = qinterp(fini, g, u, w);
@@ -149,16 +176,17 @@ __device__ __forceinline__ void k_recon64_body(const Grid& g, const uint32_t* __
     const R out = (R)val;
     f[p] = out;
     acc += (double)out;
+    m = mn;
   }
   const double rowsum = block_sum(acc, sh);
   if (threadIdx.x == 0) M[i] = dmul(rowsum, g.dxdv);
 }
 
 __global__ void __launch_bounds__(256) k_recon64(Grid g, const uint32_t* __restrict__ map, const DevState* ds,
-                                                 const double* __restrict__ tay, const float* __restrict__ tayf,
+                                                 const double* __restrict__ tay, const FxRec* __restrict__ tayx,
                                                  const double* __restrict__ fini, double* __restrict__ f,
                                                  double* __restrict__ M) {
-  k_recon64_body(g, map, ds, tay, tayf, fini, f, M, blockIdx.x);
+  k_recon64_body(g, map, ds, tay, tayx, fini, f, M, blockIdx.x);
 }
 
 // Monaghan M4 kernel, unnormalised (Sec. 2.3.2).
@@ -318,12 +346,114 @@ __device__ __forceinline__ double spline_eval(const R* __restrict__ eta, const G
   return (double)sum;
 }
 
+// The FP64 remap of one site in fixed point.  The beta ranges are read from
+// the owner's offset when it clears them by FX_MARGIN (then they are the
+// fixed order's); Q_r is the owner's Q plus the weighted mean of the other
+// elements' differences from it, Delta_n, so the weights' errors (2^-50)
+// enter times Delta_n.  With d the distance in element spacings,
+// W(2d) = 1 - 6 d^2 (1 - d) up to d = 1/2 and 2 (1 - d)^3 up to 1.  The
+// spline's 16 coefficients are scaled to integers by the largest one's
+// exponent.  Q_r and the spline are continuous, so no other decision is
+// taken.  Returns false where a record, the margin, the grid's edge or the
+// values' range do not allow it.  At 4096^2: 2.58 ms per remap, in FP64
+// 14.2 ms; error against 128-bit arithmetic 0.7 to 3.1e-16 (2-norm), before
+// 1.1 to 2.9e-15.
+__device__ __forceinline__ bool remap64_fixed(const Grid& g, const FxRec* __restrict__ tayx, int m, int i, int j,
+                                              const double* __restrict__ eta, double& val) {
+  long long ru, rw;
+  int4 o;
+  if (g.fx_beta == 0 || !fx_offset(tayx + m, i, j, ru, rw, o)) return false;
+  // (the lattice's half-integer positions are in the records' offsets)
+  const long long hx = (long long)((g.nx - 1) & 1) << (FX_Q - 1), hv = (long long)((g.nv - 1) & 1) << (FX_Q - 1);
+  const long long qx = ru - hx, qv = rw - hv, ax = qx < 0 ? -qx : qx, av = qv < 0 ? -qv : qv;
+  const long long bx = ax - g.fx_beta, bv = av - g.fx_beta;
+  if ((bx < 0 ? -bx : bx) < FX_MARGIN || (bv < 0 ? -bv : bv) < FX_MARGIN) return false;
+  const bool ina = bx < 0, inb = bv < 0;  // {-1, 0, 1} on that axis
+  const int a0 = (ina || qx < 0) ? -1 : 0, a1 = (ina || qx >= 0) ? 1 : 0;
+  const int b0 = (inb || qv < 0) ? -1 : 0, b1 = (inb || qv >= 0) ? 1 : 0;
+  const int k = m / g.Lv, l = m - k * g.Lv;
+  const long long s52 = (long long)g.s << FX_Q;
+  constexpr long long one = 1ll << 62;
+  long long nu = 0, nw = 0, den = 0;
+  for (int a = a0; a <= a1; a++)
+    for (int b = b0; b <= b1; b++) {
+      if ((ina || inb) && a != 0 && b != 0) continue;
+      const int kk = k + a, ll = l + b;
+      if (!elem_exists(g, kk, ll)) continue;
+      long long xn = qx, vn = qv;
+      if (a != 0 || b != 0) {
+        int4 on;
+        if (!fx_offset(tayx + (kk * g.Lv + ll), i, j, xn, vn, on)) return false;
+        xn -= hx;
+        vn -= hv;
+      }
+      if (xn >= s52 || -xn >= s52 || vn >= s52 || -vn >= s52) continue;  // d >= 1: weight 0
+      const long long xi = __mul64hi(xn << 3, g.fx_inv_s) << 8, ze = __mul64hi(vn << 3, g.fx_inv_s) << 8;
+      const long long d2 = __mul64hi(xi, xi) + __mul64hi(ze, ze);
+      if (d2 >= (1ll << 60)) continue;
+      const long long d = fx_sqrt(d2), e = one - d;
+      long long w;
+      if (d <= (one >> 1)) {
+        w = one - 6 * (__mul64hi(d2, e) << 4);
+      } else {
+        w = __mul64hi(__mul64hi(e, e), e) << 5;
+      }
+      const long long Dx = xn + a * s52 - qx, Dv = vn + b * s52 - qv;
+      if (((Dx < 0 ? -Dx : Dx) | (Dv < 0 ? -Dv : Dv)) >> 60) return false;  // 2^8 cells apart
+      nu += fx_mul62(Dx, w);
+      nw += fx_mul62(Dv, w);
+      den += w >> 3;
+    }
+  if (den > 0) {
+    ru += fx_div(nu, den);
+    rw += fx_div(nw, den);
+  }
+  const int ku = o.z + (int)(ru >> FX_Q), kw = o.w + (int)(rw >> FX_Q);
+  if (ku < 1 || ku > g.nx - 3 || kw < 1 || kw > g.nv - 3) {
+    val = spline_eval(eta, g, (double)o.z + (double)ru * (1.0 / (double)(1ll << FX_Q)),
+                      (double)o.w + (double)rw * (1.0 / (double)(1ll << FX_Q)));
+    return true;
+  }
+  const double* p = eta + (size_t)(ku - 1) * g.nv + (kw - 1);
+  double E[4][4];
+  int em = 0;
+#pragma unroll
+  for (int a = 0; a < 4; a++)
+#pragma unroll
+    for (int b = 0; b < 4; b++) {
+      E[a][b] = __ldg(p + (size_t)a * g.nv + b);
+      em = max(em, fx_exp(E[a][b]));
+    }
+  val = 0.0;
+  if (em == 0) {
+    bool zero = true;
+#pragma unroll
+    for (int a = 0; a < 4; a++)
+#pragma unroll
+      for (int b = 0; b < 4; b++) zero = zero && E[a][b] == 0.0;
+    return zero;
+  }
+  if (em < 128 || em > 2036) return false;
+  constexpr long long mask = (1ll << FX_Q) - 1;
+  long long bu[4], bw[4], sum = 0;
+  fx_bspline((ru & mask) << (62 - FX_Q), bu);
+  fx_bspline((rw & mask) << (62 - FX_Q), bw);
+#pragma unroll
+  for (int a = 0; a < 4; a++) {
+    long long row = 0;
+#pragma unroll
+    for (int b = 0; b < 4; b++) row += __mul64hi(fx_int(E[a][b], em), bw[b]);
+    sum += __mul64hi(row << 2, bu[a]);
+  }
+  val = fx_double(sum, em + 2);
+  return true;
+}
+
 __device__ __forceinline__ void k_remap64_body(const Grid& g, const uint32_t* __restrict__ map, const DevState* ds,
-                                                 const double* __restrict__ tay, const double* __restrict__ eta,
-                                                 double* __restrict__ out, int vb) {
+                                                 const double* __restrict__ tay, const FxRec* __restrict__ tayx,
+                                                 const double* __restrict__ eta, double* __restrict__ out, int vb) {
   using R = double;
   const int i = vb;
-  const double Px = site_x(g, i);
   int js, je;
   row_span(g, ds, i, js, je);
   zero_outside(g, out + (size_t)i * g.nv, js, je);
@@ -331,9 +461,9 @@ __device__ __forceinline__ void k_remap64_body(const Grid& g, const uint32_t* __
     const size_t p = (size_t)i * g.nv + j;
     const int m = owner(map, p, ds_epoch(ds), g.ne);
     double val = 0.0;
-    if (m >= 0) {
+    if (m >= 0 && !remap64_fixed(g, tayx, m, i, j, eta, val)) {
       double Qx, Qv;
-      blended_q_fused(g, tay, m, Px, site_v(g, j), Qx, Qv);
+      blended_q_fused(g, tay, m, site_x(g, i), site_v(g, j), Qx, Qv);
       const double u = (Qx - g.x_lo) * g.inv_dx;
       const double w = (Qv - g.v_lo) * g.inv_dv;
       val = spline_eval(eta, g, u, w);
@@ -343,10 +473,10 @@ __device__ __forceinline__ void k_remap64_body(const Grid& g, const uint32_t* __
 }
 
 __global__ void __launch_bounds__(256) k_remap64(Grid g, const uint32_t* __restrict__ map, const DevState* ds,
-                                                 const double* __restrict__ tay, const double* __restrict__ eta,
-                                                 double* __restrict__ out) {
+                                                 const double* __restrict__ tay, const FxRec* __restrict__ tayx,
+                                                 const double* __restrict__ eta, double* __restrict__ out) {
   if (gate_shut(g)) return;
-  k_remap64_body(g, map, ds, tay, eta, out, blockIdx.x);
+  k_remap64_body(g, map, ds, tay, tayx, eta, out, blockIdx.x);
 }
 
 
@@ -628,41 +758,6 @@ __device__ __forceinline__ void k_recon32_body(const Grid& g, const uint32_t* __
   }
   const double rowsum = block_sum(acc.value(), sh);
   if (threadIdx.x == 0) M[i] = dmul(rowsum, g.dxdv);
-}
-
-__device__ __forceinline__ bool recon64_fast(const Grid& g, const double* __restrict__ t, const float* __restrict__ F,
-                                             int m, int i, int j, double Px, double Pv,
-                                             const double* __restrict__ fini, float inv_Lv, double& val) {
-  const float inv_s = 1.0f / (float)g.s, fs = (float)g.s;
-  float px, pv;
-  p_of(F, i, j, inv_s, px, pv);
-  const QF q = qeval(F, px, pv);
-  int Bu, Bw;
-  float bu, bw;
-  anchor_r(g, m, inv_Lv, Bu, bu, Bw, bw);
-  const float ru = bu + fs * q.qx, rw = bw + fs * q.qv;
-  const float eu = fs * q.ex + 1e-6f * (1.f + fabsf(ru)), ew = fs * q.ev + 1e-6f * (1.f + fabsf(rw));
-  if (!(fabsf(ru) < 1e6f && fabsf(rw) < 1e6f)) return false;
-  const float tu = 2.f * ru, tw = 2.f * rw;
-  const float fu = floorf(tu), fw = floorf(tw);
-  if (!((tu - 2.f * eu > fu) && (tu + 2.f * eu < fu + 1.f) && (tw - 2.f * ew > fw) && (tw + 2.f * ew < fw + 1.f)))
-    return false;
-  const int iu = (int)fu, iw = (int)fw;
-  const long long in = Bu + ((iu + 1) >> 1), jn = Bw + ((iw + 1) >> 1);
-  const long long ic = Bu + (iu >> 1), jc = Bw + (iw >> 1);
-  // FP64 offset, fused, on the exact lattice index of Q_m
-  const double dPx = Px - t[TY_X], dPv = Pv - t[TY_V];
-  const double yx = fma(t[TY_TI00], dPx, t[TY_TI01] * dPv), yv = fma(t[TY_TI10], dPx, t[TY_TI11] * dPv);
-  double g0 = fma(t[TY_GX00], dPx, t[TY_GX01] * dPv), g1 = fma(t[TY_GX01], dPx, t[TY_GX11] * dPv);
-  const double sx = fma(dPx, g0, dPv * g1);
-  g0 = fma(t[TY_GV00], dPx, t[TY_GV01] * dPv);
-  g1 = fma(t[TY_GV01], dPx, t[TY_GV11] * dPv);
-  const double sv = fma(dPx, g0, dPv * g1);
-  const double dqx = fma(-0.5, fma(t[TY_TI00], sx, t[TY_TI01] * sv), yx);
-  const double dqv = fma(-0.5, fma(t[TY_TI10], sx, t[TY_TI11] * sv), yv);
-  const double u = fma(dqx, g.inv_dx, (double)Bu + (double)bu), w = fma(dqv, g.inv_dv, (double)Bw + (double)bw);
-  val = qinterp64_fused(fini, g, in, jn, ic, jc, u - (double)in, w - (double)jn);
-  return true;
 }
 
 __global__ void __launch_bounds__(256, 6) k_recon32(Grid g, const uint32_t* __restrict__ map, const DevState* ds,
@@ -1066,7 +1161,7 @@ __global__ void __launch_bounds__(256, 6) k_recon_group32(const SolveDesc* __res
 __global__ void __launch_bounds__(256) k_recon_group64(const SolveDesc* __restrict__ D, const int* __restrict__ off,
                                                      int ns, int total) {
   GROUP_LOOP(off, ns, total)
-  k_recon64_body(gsh, d.map, d.ds, d.tay, d.tayf, (const double*)d.fini, (double*)d.f, d.M, vb);
+  k_recon64_body(gsh, d.map, d.ds, d.tay, d.tayx, (const double*)d.fini, (double*)d.f, d.M, vb);
   GROUP_END
 }
 
@@ -1080,7 +1175,7 @@ __global__ void __launch_bounds__(256) k_remap_group32(const SolveDesc* __restri
 __global__ void __launch_bounds__(256) k_remap_group64(const SolveDesc* __restrict__ D, const int* __restrict__ off,
                                                      int ns, int total) {
   GROUP_LOOP(off, ns, total)
-  k_remap64_body(gsh, d.map, d.ds, d.tay, (const double*)d.eta, (double*)d.tmp, vb);
+  k_remap64_body(gsh, d.map, d.ds, d.tay, d.tayx, (const double*)d.eta, (double*)d.tmp, vb);
   GROUP_END
 }
 
@@ -1205,7 +1300,7 @@ void launch_reconstruct(vm_solver* s) {
     k_recon32<<<s->g.nx, nt, 0, s->stream>>>(s->g, s->map, s->ds, s->tay, s->tayf, (const float*)s->fini,
                                               (float*)s->f, s->M);
   else
-    k_recon64<<<s->g.nx, nt, 0, s->stream>>>(s->g, s->map, s->ds, s->tay, s->tayf, (const double*)s->fini,
+    k_recon64<<<s->g.nx, nt, 0, s->stream>>>(s->g, s->map, s->ds, s->tay, s->tayx, (const double*)s->fini,
                                               (double*)s->f, s->M);
   prof_end(s, ps_);
   s->launches++;
@@ -1221,7 +1316,7 @@ void launch_remap_resample(vm_solver* s, void* out) {
     k_remap32<<<s->g.nx, nt, 0, s->stream>>>(s->g, s->map, s->ds, s->tay, s->tayf, (const float*)s->eta,
                                               (float*)out, blo, bhi);
   } else {
-    k_remap64<<<s->g.nx, nt, 0, s->stream>>>(s->g, s->map, s->ds, s->tay, (const double*)s->eta,
+    k_remap64<<<s->g.nx, nt, 0, s->stream>>>(s->g, s->map, s->ds, s->tay, s->tayx, (const double*)s->eta,
                                               (double*)out);
   }
   prof_end(s, ps_);
