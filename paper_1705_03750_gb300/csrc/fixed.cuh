@@ -92,19 +92,23 @@ __device__ __forceinline__ double fx_double(long long S, int emax) {
   return S ? __hiloint2double(__double2hiint(d) + ((emax - 1082) << 20), __double2loint(d)) : 0.0;
 }
 
-// Sum of products of values (|v| <= 2^60) with non-negative weights w (2^-60
-// units, their sum at most 1): v w / 2^63, three 32-bit products each, the
-// lowest one left out (below one unit in all); at most four terms.
+// Sum of at most four products of values (|v| <= 2^60) with non-negative
+// weights w (2^-60 units, their sum at most 1): four 32-bit products a term
+// accumulated in 64 bits each, to about two units.
 struct FxDot {
   long long hh = 0, hl = 0;
-  unsigned long long lh = 0;
+  unsigned long long lh = 0, ll = 0;
   __device__ __forceinline__ void add(long long v, int wh, int wl) {
     const int vh = (int)(v >> 32);
+    const unsigned vl = (unsigned)v;
     hh += (long long)vh * wh;
     hl += (long long)vh * wl;
-    lh += (unsigned long long)(unsigned)v * (unsigned)wh;
+    lh += (unsigned long long)vl * (unsigned)wh;
+    ll += (unsigned long long)(vl >> 2) * (unsigned)wl;
   }
-  __device__ __forceinline__ long long sum() const { return hh + (hl >> 31) + (long long)(lh >> 32); }
+  __device__ __forceinline__ long long sum() const {
+    return (hh << 3) + (hl >> 28) + (long long)(lh >> 29) + (long long)(ll >> 58);
+  }
 };
 // A weight in 2^-62 units as the two halves FxDot takes.
 __device__ __forceinline__ void fx_split(long long w, int& wh, int& wl) {
@@ -139,6 +143,15 @@ __device__ __forceinline__ long long fx_sqrt(long long d2) {
     D += (long long)((float)rem * r * 2147483648.f);  // rem / (2 d)
   }
   return D;
+}
+
+// The Monaghan kernel W(2d) (Sec. 2.3.2) from d^2 (2^-60 units, below 1), in
+// 2^-62 units: 1 - 6 d^2 (1 - d) up to d = 1/2, 2 (1 - d)^3 beyond.
+__device__ __forceinline__ long long fx_kernel(long long d2) {
+  constexpr long long one = 1ll << 62;
+  const long long e = one - fx_sqrt(d2);
+  if (e >= (one >> 1)) return one - 6 * (__mul64hi(d2, e) << 4);
+  return __mul64hi(__mul64hi(e << 1, e << 1) << 2, e << 1);
 }
 
 // num / den, den in 2^-59 units and positive, to about 2^-46 |num / den|

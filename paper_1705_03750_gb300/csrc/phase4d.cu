@@ -8,6 +8,7 @@
 //
 //   k4_drift        half drift of every element (one thread per element)
 //   k4_taylor       T^-1 = adj(T)/det T and G_l = [T^-1]^T H_l T^-1
+//   k4_records      the inverse map's FP32 and fixed-point records
 //   k4_percolate    one block per element: breadth-first flood fill of its
 //                   component in a shared-memory bit window around its start
 //                   site, frontier waves in shared memory, claims by a 128-bit
@@ -35,8 +36,8 @@
 // the method, or on FP32 values whose rigorous error bound shows the same
 // outcome; the map is therefore exactly the one that restatement gives for
 // the same elements.  Values that feed no such decision (the interpolated f,
-// the Q_r blend, the spline sums) use fused arithmetic and agree with it to
-// rounding; the spline solve divides by the same pivots in the same order;
+// the Q_r blend, the spline sums) use 64-bit fixed point (fixed.cuh) or fused
+// FP64 arithmetic and agree with it to rounding; the spline solve divides by the same pivots in the same order;
 // the pixel masses are block sums and the field is summed over blocks, so
 // element trajectories agree to rounding.
 
@@ -50,6 +51,7 @@
 #include <vector>
 
 #include "../../include/vlamet4d.h"
+#include "fixed.cuh"
 
 namespace {
 
@@ -71,6 +73,10 @@ struct G4 {
   int32_t E, We0, We1;  // field cache: nodes [-E, n0-1+E] x [-E, n1-1+E]
   int32_t R, W;         // flood window: side W = 2R+1 sites around the start site
   int32_t max_rounds;
+  // fixed-point remap: 2^63 / s, beta s and the axes' half-integer lattice
+  // positions in cells (fx_beta 0: the remap in FP64)
+  long long fx_inv_s, fx_beta, fx_half[4];
+  double rd[4][4];  // d[b] / d[a]
 };
 
 struct Dev4 {
@@ -266,8 +272,7 @@ __device__ void inverse4(const double* A, double* B) {
 // nB_a = sum_bc |B_a,bc|.  Layout: A[16], B[40], K[4], nA[4], nB[4], pad.
 constexpr int NF4 = 72;
 
-__global__ void __launch_bounds__(128) k4_taylor(G4 g, const double* __restrict__ el, double* __restrict__ tay,
-                                                 float* __restrict__ tay32) {
+__global__ void __launch_bounds__(128) k4_taylor(G4 g, const double* __restrict__ el, double* __restrict__ tay) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= g.ne) return;
   const double* e = el + (size_t)NE4 * m;
@@ -291,32 +296,160 @@ __global__ void __launch_bounds__(128) k4_taylor(G4 g, const double* __restrict_
   int k[4];
   elem_coords(g, m, k);
   for (int a = 0; a < 4; a++) t[60 + a] = A_(g.ctr[a], M_((double)(k[a] - g.K[a] - 1), g.dm[a]));
+}
+
+// Fixed-point record of an element's inverse map (fixed.cuh; 512 bytes): per
+// axis the 15 coefficients of the index position of Q at a site, relative to
+// the integer anchor B, as a polynomial of the site's offset j from the
+// element's start site i0: c0 + sum_b j_b (c_b + sum_{c>=b} j_c c_bc); the
+// sixteenth word packs i0 (low half) and B << 8 | lim, lim the largest |j|
+// served (0: none).
+struct Fx4 {
+  long long c[4][16];
+};
+constexpr int FX4_LIM = 32;
+// Fraction bits of the 4D offsets: the grids are coarser than the 2D path's
+// (positions below 2^8 cells keep 45 to 53 bits in FP64) and a neighbour's
+// second-order terms are multiplied by site offsets of 36 and more, so the
+// coefficients take five more bits, for a range of 2^6 cells.
+constexpr int FX4_Q = 57;
+constexpr double FX4_MAX = 60.0;
+constexpr long long FX4_MARGIN = 1ll << (FX4_Q - 26);
+
+// Records of the element's inverse map for the percolation (FP32) and for the
+// values (fixed point), four threads per element, one per axis of Q: the
+// second-order coefficients sum_l T^-1_al G_l,bc serve both.
+__global__ void __launch_bounds__(128) k4_records(G4 g, const double* __restrict__ tay, float* __restrict__ tay32,
+                                                  Fx4* __restrict__ tayx) {
+  const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int m = (int)(tid >> 2), a = (int)(tid & 3);
+  const unsigned quad = 0xFu << (threadIdx.x & 28);  // this element's lanes
+  if (m >= g.ne) return;
+  const double* t = tay + (size_t)NT4 * m;
   float* r = tay32 + (size_t)NF4 * m;
-  for (int a = 0; a < 4; a++) {
-    for (int b = 0; b < 4; b++) r[4 * a + b] = (float)(Ti[4 * a + b] * g.dm[b] * g.inv_dm[a]);
-    double kmax = 0.0;
-    for (int l = 0; l < 4; l++) {
-      double gm = 0.0;
-      for (int b = 0; b < 4; b++)
-        for (int c = b; c < 4; c++) gm = fmax(gm, fabs(t[20 + 10 * l + sym4(b, c)]) * g.dm[b] * g.dm[c]);
-      kmax += fabs(Ti[4 * a + l]) * gm;
+  const int lead = threadIdx.x & 28;
+  // |G_l,bc| dm_b dm_c at most, l = a on this thread
+  double gm = 0.0;
+  for (int b = 0; b < 4; b++)
+    for (int c = b; c < 4; c++) gm = fmax(gm, fabs(t[20 + 10 * a + sym4(b, c)]) * g.dm[b] * g.dm[c]);
+  double Ti[4], kmax = 0.0;
+#pragma unroll
+  for (int l = 0; l < 4; l++) {
+    Ti[l] = t[4 + 4 * a + l];
+    kmax += fabs(Ti[l]) * __shfl_sync(quad, gm, lead + l);
+  }
+  const float K = (float)(0.5 * kmax * g.inv_dm[a] * 1.0000001);
+  r[56 + a] = K;
+  float na = 0.f, nb = 0.f;
+  long long L[4], Q[10];
+#pragma unroll
+  for (int b = 0; b < 4; b++) {
+    const double A = Ti[b] * g.dm[b] * g.inv_dm[a];
+    const float Af = (float)A;
+    r[4 * a + b] = Af;
+    na += fabsf(Af);
+    L[b] = fabs(A) < FX4_MAX ? vm::fx_of(Ti[b] * g.rd[b][a], FX4_Q) : 0;
+  }
+  const double inv_s = 1.0 / (double)g.s;
+#pragma unroll
+  for (int b = 0; b < 4; b++)
+#pragma unroll
+    for (int c = b; c < 4; c++) {
+      double v = 0.0;
+#pragma unroll
+      for (int l = 0; l < 4; l++) v += Ti[l] * t[20 + 10 * l + sym4(b, c)];
+      const double B = -0.5 * (b == c ? 1.0 : 2.0) * v * g.dm[b] * g.dm[c] * g.inv_dm[a];
+      const float Bf = (float)B;
+      r[16 + 10 * a + sym4(b, c)] = Bf;
+      nb += fabsf(Bf);
+      Q[sym4(b, c)] = fabs(B) < FX4_MAX ? vm::fx_of(B * inv_s, FX4_Q) : 0;
     }
-    r[56 + a] = (float)(0.5 * kmax * g.inv_dm[a] * 1.0000001);
-    for (int b = 0; b < 4; b++)
-      for (int c = b; c < 4; c++) {
-        double v = 0.0;
-        for (int l = 0; l < 4; l++) v += Ti[4 * a + l] * t[20 + 10 * l + sym4(b, c)];
-        r[16 + 10 * a + sym4(b, c)] = (float)(-0.5 * (b == c ? 1.0 : 2.0) * v * g.dm[b] * g.dm[c] * g.inv_dm[a]);
-      }
+  na *= 1.000001f;
+  nb *= 1.000001f;
+  r[60 + a] = na;
+  r[64 + a] = nb;
+  r[68 + a] = 0.f;
+  // the largest offset up to which the terms on every axis together stay
+  // below FX4_MAX cells (the FP64 evaluation's uncombined ones, bounded by
+  // 16 K p^2, below 10^5: its error then stays far inside FX4_MARGIN)
+  float n1 = na, n2 = nb, n3 = K;
+  const bool fin = n1 < 1e30f && n2 < 1e30f && n3 < 1e30f;
+  for (int o = 1; o < 4; o <<= 1) {
+    n1 = fmaxf(n1, __shfl_xor_sync(quad, n1, o));
+    n2 = fmaxf(n2, __shfl_xor_sync(quad, n2, o));
+    n3 = fmaxf(n3, __shfl_xor_sync(quad, n3, o));
   }
+  int lim = 0;
+#pragma unroll
+  for (int Lm = FX4_LIM; Lm >= 2; Lm -= 2) {
+    const float p = ((float)Lm + 0.51f) / (float)g.s;
+    const float sf = (float)g.s;
+    if (lim == 0 && 0.51f + sf * (n1 * p + n2 * (p * p)) < (float)FX4_MAX && sf * n3 * (p * p) < 6e3f) lim = Lm;
+  }
+  // start site along this axis and its distance from P_m
+  const double u = (t[a] - g.lo[a]) * g.inv_d[a];
+  const bool near = u > -1e6 && u < 1e6;
+  const double i0 = near ? floor(u + 0.5) : 0.0;
+  if (__any_sync(quad, !near || !fin)) lim = 0;
+  const long long de = near ? vm::fx_of(vm::cells_from(t[a], g.lo[a], g.d[a], g.inv_d[a], i0), 62) : 0;
+  long long E[4];
+#pragma unroll
+  for (int b = 0; b < 4; b++) E[b] = __shfl_sync(quad, de, lead + b);
+  int k[4];
+  elem_coords(g, m, k);
+  int u2 = 0;
+#pragma unroll
+  for (int b = 0; b < 4; b++)
+    if (b == a) u2 = (g.n[b] - 1) + 2 * (k[b] - g.K[b] - 1) * g.s;
+  long long c0 = (long long)(u2 & 1) << (FX4_Q - 1), c1[4];
+#pragma unroll
+  for (int b = 0; b < 4; b++) {
+    long long tb = L[b];
+#pragma unroll
+    for (int c = b; c < 4; c++) tb += vm::fx_mul62(Q[sym4(b, c)], E[c]);
+    c0 += vm::fx_mul62(tb, E[b]);
+    c1[b] = tb;
+  }
+#pragma unroll
+  for (int b = 0; b < 4; b++)
+#pragma unroll
+    for (int c = 0; c <= b; c++) c1[b] += vm::fx_mul62(Q[sym4(c, b)], E[c]);
+  longlong2* o = reinterpret_cast<longlong2*>(tayx[m].c[a]);
+  o[0] = make_longlong2(c0, c1[0]);
+  o[1] = make_longlong2(c1[1], c1[2]);
+  o[2] = make_longlong2(c1[3], Q[0]);
+#pragma unroll
+  for (int q = 0; q < 4; q++) o[3 + q] = make_longlong2(Q[1 + 2 * q], Q[2 + 2 * q]);
+  const long long pack = ((long long)(((u2 >> 1) << 8) | lim) << 32) | (unsigned)(int)i0;
+  o[7] = make_longlong2(Q[9], pack);
+}
+
+// Offset of Q from the record's anchor along axis a at a site j from the
+// start site (FX_Q fraction bits), and the axis's packed word.
+__device__ __forceinline__ long long fx4_axis(const long long (&c)[16], const int* j) {
+  const longlong2* q = reinterpret_cast<const longlong2*>(c);
+  const longlong2 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3), q4 = __ldg(q + 4),
+                  q5 = __ldg(q + 5), q6 = __ldg(q + 6), q7 = __ldg(q + 7);
+  const long long j0 = j[0], j1 = j[1], j2 = j[2], j3 = j[3];
+  return q0.x + j0 * (q0.y + j0 * q2.y + j1 * q3.x + j2 * q3.y + j3 * q4.x) +
+         j1 * (q1.x + j1 * q4.y + j2 * q5.x + j3 * q5.y) + j2 * (q1.y + j2 * q6.x + j3 * q6.y) +
+         j3 * (q2.x + j3 * q7.x);
+}
+
+// The site's offsets j from the element's start site and the anchors B; false
+// when the record does not reach the site.
+__device__ __forceinline__ bool fx4_start(const Fx4* __restrict__ X, const int* site, int* j, int* B) {
+  int lim = 0, far = 0;
+#pragma unroll
   for (int a = 0; a < 4; a++) {
-    float na = 0.f, nb = 0.f;
-    for (int b = 0; b < 4; b++) na += fabsf(r[4 * a + b]);
-    for (int q = 0; q < 10; q++) nb += fabsf(r[16 + 10 * a + q]);
-    r[60 + a] = na * 1.000001f;
-    r[64 + a] = nb * 1.000001f;
+    const long long w = __ldg(&X->c[a][15]);
+    const int hi = (int)(w >> 32);
+    j[a] = site[a] - (int)w;
+    B[a] = hi >> 8;
+    lim = hi & 255;
+    far = max(far, abs(j[a]));
   }
-  for (int q = 68; q < NF4; q++) r[q] = 0.f;
+  return far <= lim;
 }
 
 // FP32 offsets xi of an element at a site with rigorous bounds e_a >=
@@ -1015,15 +1148,118 @@ __device__ double qinterp4_f(const G4& g, const double* __restrict__ F, const do
   return f;
 }
 
+// f at one site of an owner through FP64 (fixed_value's fallback): fused
+// evaluation, the nearest node (the one decision the interpolant is not
+// continuous across) re-taken in the exact order when a coordinate lies
+// within 1e-9 of a half-integer.
+__device__ __noinline__ double recon4_fp64(const G4& g, const double* __restrict__ t, const double* __restrict__ F,
+                                           const int* site) {
+  double P[4], dQ[4], u[4];
+  for (int a = 0; a < 4; a++) P[a] = site_coord(g, a, site[a]);
+  qofp4_f(t, P, dQ);
+  bool tie = false;
+  for (int a = 0; a < 4; a++) {
+    u[a] = ((__ldg(t + 60 + a) + dQ[a]) - g.lo[a]) * g.inv_d[a];
+    tie |= fabs((u[a] - floor(u[a])) - 0.5) < 1e-9;
+  }
+  if (tie) {
+    qofp4(t, P, dQ);
+    for (int a = 0; a < 4; a++) u[a] = M_(S_(A_(__ldg(t + 60 + a), dQ[a]), g.lo[a]), g.inv_d[a]);
+  }
+  return qinterp4_f(g, F, u);
+}
+
+// The same in fixed point (the 2D path's reconstruction in four dimensions,
+// recon.cu): offsets from the record's integer polynomials, the nearest node
+// where they clear the half-integer, the 15 node values as 58-bit integers
+// scaled by the largest one's exponent (0 outside the grid), and, with s the
+// side of the node that holds Q along an axis and o the other,
+//   f = F0 + sum_a x_a [(Fs_a - Fo_a)/2 + x_a (Fs_a + Fo_a - 2 F0)/2
+//                       + sum_{b > a} x_b (F0 + Fd_ab - Fs_a - Fs_b)],  x >= 0.
+// At 64^4: 0.93 ms per step, bound by the integer pipes and the record's 512
+// bytes a site through L1; in fused FP64 7.46 ms.  Error against 128-bit
+// arithmetic (20 x 18 x 22 x 16 and 24^4): 1.4e-16, before 7.6e-16 (2-norm).
+__device__ __forceinline__ bool recon4_fixed(const G4& g, const Fx4* __restrict__ X, const double* __restrict__ F,
+                                             const int* site, double& val) {
+  int j[4], B[4];
+  if (!fx4_start(X, site, j, B)) return false;
+  constexpr long long half = 1ll << (FX4_Q - 1);
+  long long x[4], off = 0, ds[4];
+  bool oc[4], os[4], oo[4], sure = true;
+#pragma unroll
+  for (int a = 0; a < 4; a++) {
+    const long long r = fx4_axis(X->c[a], j);
+    const long long nq = (r + half) >> FX4_Q, xs = r - (nq << FX4_Q), xa = xs < 0 ? -xs : xs;
+    sure = sure && xa <= half - FX4_MARGIN;
+    const int node = B[a] + (int)nq, sd = xs < 0 ? -1 : 1;
+    x[a] = xa << (64 - FX4_Q);
+    off += node * g.st[a];
+    ds[a] = sd * g.st[a];
+    oc[a] = (unsigned)node < (unsigned)g.n[a];
+    os[a] = (unsigned)(node + sd) < (unsigned)g.n[a];
+    oo[a] = (unsigned)(node - sd) < (unsigned)g.n[a];
+  }
+  if (!sure) return false;
+  const double* p = F + off;
+  const bool c01 = oc[0] && oc[1], c23 = oc[2] && oc[3], all = c01 && c23;
+  double F0 = all ? __ldg(p) : 0.0, Fs[4], Fo[4], Fd[6];
+#pragma unroll
+  for (int a = 0; a < 4; a++) {
+    const bool rest = a == 0 ? oc[1] && c23 : (a == 1 ? oc[0] && c23 : (a == 2 ? c01 && oc[3] : c01 && oc[2]));
+    Fs[a] = rest && os[a] ? __ldg(p + ds[a]) : 0.0;
+    Fo[a] = rest && oo[a] ? __ldg(p - ds[a]) : 0.0;
+  }
+#pragma unroll
+  for (int a = 0, q = 0; a < 4; a++)
+#pragma unroll
+    for (int b = a + 1; b < 4; b++, q++) {
+      bool ok = os[a] && os[b];
+#pragma unroll
+      for (int c = 0; c < 4; c++)
+        if (c != a && c != b) ok = ok && oc[c];
+      Fd[q] = ok ? __ldg(p + ds[a] + ds[b]) : 0.0;
+    }
+  int em = vm::fx_exp(F0);
+#pragma unroll
+  for (int a = 0; a < 4; a++) em = max(em, max(vm::fx_exp(Fs[a]), vm::fx_exp(Fo[a])));
+#pragma unroll
+  for (int q = 0; q < 6; q++) em = max(em, vm::fx_exp(Fd[q]));
+  if (em < 128 || em > 2036) {
+    bool zero = F0 == 0.0;
+#pragma unroll
+    for (int a = 0; a < 4; a++) zero = zero && Fs[a] == 0.0 && Fo[a] == 0.0;
+#pragma unroll
+    for (int q = 0; q < 6; q++) zero = zero && Fd[q] == 0.0;
+    val = 0.0;
+    return zero;
+  }
+  const long long i0 = vm::fx_int<5>(F0, em);
+  long long is[4], S = i0, gx[4];
+#pragma unroll
+  for (int a = 0; a < 4; a++) {
+    is[a] = vm::fx_int<5>(Fs[a], em);
+    const long long io = vm::fx_int<5>(Fo[a], em);
+    gx[a] = (is[a] - io + vm::fx_mul(is[a] + io - 2 * i0, x[a])) >> 1;
+  }
+#pragma unroll
+  for (int a = 0, q = 0; a < 4; a++) {
+#pragma unroll
+    for (int b = a + 1; b < 4; b++, q++)
+      gx[a] += vm::fx_mul(i0 + vm::fx_int<5>(Fd[q], em) - is[a] - is[b], x[b]);
+    S += vm::fx_mul(gx[a], x[a]);
+  }
+  val = vm::fx_double(S, em + 2);  // units of 2^(em - 1080)
+  return true;
+}
+
 // One block per (x, y) pixel: f(P) = f_ini(Q(P)) at every (vx, vy) site of
 // the pixel through the owner's inverse map, and the pixel mass
 // M = (sum f) dx dy dvx dvy.
-__global__ void __launch_bounds__(256) k4_recon(G4 g, const double* __restrict__ tay, const int32_t* __restrict__ map,
-                                                const double* __restrict__ fini, double* __restrict__ f,
-                                                double* __restrict__ Mpix, Dev4* ds) {
+__global__ void __launch_bounds__(256) k4_recon(G4 g, const double* __restrict__ tay, const Fx4* __restrict__ tayx,
+                                                const int32_t* __restrict__ map, const double* __restrict__ fini,
+                                                double* __restrict__ f, double* __restrict__ Mpix, Dev4* ds) {
   __shared__ double red[32];
   const int pix = blockIdx.x;
-  const long long i0 = pix / g.n[1], i1 = pix % g.n[1];
   const int nvel = g.n[2] * g.n[3];
   const long long base = (long long)pix * nvel;
   double sum = 0.0;
@@ -1032,26 +1268,8 @@ __global__ void __launch_bounds__(256) k4_recon(G4 g, const double* __restrict__
     const int m = map[p];
     double fv = 0.0;
     if (m >= 0 && m < g.ne) {
-      const double* t = tay + (size_t)NT4 * m;
-      double P[4], dQ[4], u[4];
-      P[0] = site_coord(g, 0, i0);
-      P[1] = site_coord(g, 1, i1);
-      P[2] = site_coord(g, 2, q / g.n[3]);
-      P[3] = site_coord(g, 3, q % g.n[3]);
-      // fused evaluation; the nearest node (the one decision the
-      // interpolant is not continuous across) is re-taken in the exact order
-      // when a coordinate lies within 1e-9 of a half-integer
-      qofp4_f(t, P, dQ);
-      bool tie = false;
-      for (int a = 0; a < 4; a++) {
-        u[a] = ((__ldg(t + 60 + a) + dQ[a]) - g.lo[a]) * g.inv_d[a];
-        tie |= fabs((u[a] - floor(u[a])) - 0.5) < 1e-9;
-      }
-      if (tie) {
-        qofp4(t, P, dQ);
-        for (int a = 0; a < 4; a++) u[a] = M_(S_(A_(__ldg(t + 60 + a), dQ[a]), g.lo[a]), g.inv_d[a]);
-      }
-      fv = qinterp4_f(g, fini, u);
+      const int site[4] = {pix / g.n[1], pix % g.n[1], q / g.n[3], q % g.n[3]};
+      if (!recon4_fixed(g, tayx + m, fini, site, fv)) fv = recon4_fp64(g, tay + (size_t)NT4 * m, fini, site);
     } else if (m >= g.ne) {
       bad(ds, 43);
     }
@@ -1298,91 +1516,207 @@ __device__ double spline_eval4_f(const G4& g, const double* __restrict__ eta, co
 // f_new(P) = spline[f_ini](Q_r(P)), Q_r = sum W(2 d_m') Q(P, m') / sum W(2 d_m')
 // over the beta set of the owner (per axis below -beta {-1,0}, below beta
 // {-1,0,1}, else {0,1}; an offset with two or more non-zero components is
-// dropped when one of them lies on a {-1,0,1} axis).  The beta ranges are
-// decided on the owner's offsets in the exact order; the blend and the spline
-// sum, continuous in their inputs, use fused arithmetic; an element whose
-// FP32 distance is certainly at least one element spacing (weight 0) is
-// skipped.
-__global__ void __launch_bounds__(128) k4_resample(G4 g, const double* __restrict__ tay,
-                                                  const float* __restrict__ tay32, const int32_t* __restrict__ map,
-                                                  const double* __restrict__ eta, double* __restrict__ fnew, Dev4* ds) {
+// dropped when one of them lies on a {-1,0,1} axis).
+
+// The blend through FP64 (resample4_fixed's fallback), as index coordinates:
+// the beta ranges decided on the owner's offsets in the exact order, the rest,
+// continuous in its inputs, in fused arithmetic.
+__device__ __noinline__ double resample4_fp64(const G4& g, const double* __restrict__ tay,
+                                              const double* __restrict__ eta, const int* site, int m) {
+  double P[4], x[4];
+  for (int a = 0; a < 4; a++) P[a] = site_coord(g, a, site[a]);
+  const double* tm = tay + (size_t)NT4 * m;
+  dist2_4(g, tm, P, x);
+  int lo[4], hi[4], full[4];
+  for (int a = 0; a < 4; a++) {
+    lo[a] = (x[a] < -g.beta) ? -1 : ((x[a] < g.beta) ? -1 : 0);
+    hi[a] = (x[a] < -g.beta) ? 0 : 1;
+    full[a] = (lo[a] == -1 && hi[a] == 1);
+  }
+  int k[4];
+  elem_coords(g, m, k);
+  double num[4] = {0.0, 0.0, 0.0, 0.0}, den = 0.0;
+  for (int o0 = lo[0]; o0 <= hi[0]; o0++)
+    for (int o1 = lo[1]; o1 <= hi[1]; o1++)
+      for (int o2 = lo[2]; o2 <= hi[2]; o2++)
+        for (int o3 = lo[3]; o3 <= hi[3]; o3++) {
+          const int o[4] = {o0, o1, o2, o3};
+          int nz = 0, onfull = 0;
+          for (int a = 0; a < 4; a++)
+            if (o[a] != 0) {
+              nz++;
+              onfull |= full[a];
+            }
+          if (nz >= 2 && onfull) continue;
+          int kk[4], ok = 1;
+          for (int a = 0; a < 4; a++) {
+            kk[a] = k[a] + o[a];
+            ok &= (kk[a] >= 0 && kk[a] < g.L[a]);
+          }
+          if (!ok) continue;
+          const int mm = ((kk[0] * g.L[1] + kk[1]) * g.L[2] + kk[2]) * g.L[3] + kk[3];
+          const double* t = tay + (size_t)NT4 * mm;
+          double dQ[4], dd = 0.0;
+          qofp4_f(t, P, dQ);
+          for (int a = 0; a < 4; a++) {
+            const double xa = dQ[a] * g.inv_dm[a];
+            dd = fma(xa, xa, dd);
+          }
+          const double w = W4f(2.0 * sqrt(dd));
+          for (int a = 0; a < 4; a++) num[a] = fma(w, __ldg(t + 60 + a) + dQ[a], num[a]);
+          den += w;
+        }
+  double Qr[4];
+  if (den > 0.0) {
+    const double id = 1.0 / den;
+    for (int a = 0; a < 4; a++) Qr[a] = num[a] * id;
+  } else {
+    double dQ[4];
+    qofp4_f(tm, P, dQ);
+    for (int a = 0; a < 4; a++) Qr[a] = __ldg(tm + 60 + a) + dQ[a];
+  }
+  double u[4];
+  for (int a = 0; a < 4; a++) u[a] = (Qr[a] - g.lo[a]) * g.inv_d[a];
+  return spline_eval4_f(g, eta, u);
+}
+
+// The same in fixed point (the 2D path's remap in four dimensions, recon.cu):
+// the beta ranges from the owner's offsets where they clear beta, Q_r as the
+// owner's Q plus the weighted mean of the other elements' differences from
+// it, the 256 coefficients as 60-bit integers scaled by the largest one's
+// exponent, contracted one axis at a time.  At 64^4: 25.7 ms per remap, in
+// FP64 86.9 ms; error against 128-bit arithmetic 1.2e-16, before 1.0e-15.
+__device__ __forceinline__ bool resample4_fixed(const G4& g, const Fx4* __restrict__ tayx,
+                                                const double* __restrict__ eta, const int* site, int m, double& val) {
+  int j[4], B[4];
+  if (g.fx_beta == 0 || !fx4_start(tayx + m, site, j, B)) return false;
+  long long q[4];
+  int lo[4], hi[4], full = 0;
+  bool sure = true;
+#pragma unroll
+  for (int a = 0; a < 4; a++) {
+    q[a] = fx4_axis(tayx[m].c[a], j) - g.fx_half[a];
+    const long long e = (q[a] < 0 ? -q[a] : q[a]) - g.fx_beta;
+    sure = sure && (e < 0 ? -e : e) >= FX4_MARGIN;
+    lo[a] = (e < 0 || q[a] < 0) ? -1 : 0;
+    hi[a] = (e < 0 || q[a] >= 0) ? 1 : 0;
+    full |= (e < 0 ? 1 : 0) << a;
+  }
+  if (!sure) return false;
+  const long long s1 = (long long)g.s << FX4_Q;
+  int k[4];
+  elem_coords(g, m, k);
+  // (the weights of a site between 16 elements are as small as 10^-3: their
+  // products keep all bits until the division)
+  __int128 num[4] = {0, 0, 0, 0};
+  unsigned long long den = 0;
+  for (int o0 = lo[0]; o0 <= hi[0]; o0++)
+    for (int o1 = lo[1]; o1 <= hi[1]; o1++)
+      for (int o2 = lo[2]; o2 <= hi[2]; o2++)
+        for (int o3 = lo[3]; o3 <= hi[3]; o3++) {
+          const int o[4] = {o0, o1, o2, o3};
+          const int set = (o0 != 0) | (o1 != 0) << 1 | (o2 != 0) << 2 | (o3 != 0) << 3;
+          if ((set & (set - 1)) && (set & full)) continue;
+          bool ok = true;
+#pragma unroll
+          for (int a = 0; a < 4; a++) ok = ok && (unsigned)(k[a] + o[a]) < (unsigned)g.L[a];
+          if (!ok) continue;
+          const int mm = m + ((o0 * g.L[1] + o1) * g.L[2] + o2) * g.L[3] + o3;
+          int jn[4] = {j[0], j[1], j[2], j[3]}, Bn[4];
+          if (set && !fx4_start(tayx + mm, site, jn, Bn)) return false;
+          // distance, axis by axis until d >= 1 (weight 0)
+          long long D[4], d2 = 0;
+#pragma unroll
+          for (int a = 0; a < 4; a++) {
+            if (d2 < (1ll << 60)) {
+              const long long xn = set ? fx4_axis(tayx[mm].c[a], jn) - g.fx_half[a] : q[a];
+              D[a] = xn + o[a] * s1 - q[a];
+              const long long xc = xn >= s1 ? s1 : (xn <= -s1 ? -s1 : xn);
+              const long long xi = __mul64hi(xc, g.fx_inv_s) << 6;
+              d2 += __mul64hi(xi, xi);
+            }
+          }
+          if (d2 >= (1ll << 60)) continue;
+          const long long w = vm::fx_kernel(d2);
+#pragma unroll
+          for (int a = 0; a < 4; a++) {
+            if ((D[a] < 0 ? -D[a] : D[a]) >> 59) return false;  // four cells apart
+            num[a] += (__int128)D[a] * w;
+          }
+          den += (unsigned long long)w >> 3;
+        }
+  const int z = den > 0 ? max(__clzll((long long)den) - 4, 0) : 0;  // both scaled by 2^z for the division
+  int gk[4][4], wh[4][4], wl[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; a++) {
+    const long long r =
+        q[a] + g.fx_half[a] + (den > 0 ? vm::fx_div((long long)(num[a] >> (62 - z)), (long long)(den << z)) : 0);
+    const int k0 = B[a] + (int)(r >> FX4_Q) - 1;
+    long long b[4];
+    vm::fx_bspline((r & ((1ll << FX4_Q) - 1)) << (62 - FX4_Q), b);
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      const int kc = k0 + c, gc = kc == -1 ? 1 : (kc == g.n[a] ? g.n[a] - 2 : kc);
+      const bool in = (unsigned)gc < (unsigned)g.n[a];
+      gk[a][c] = in ? gc : 0;
+      vm::fx_split(in ? b[c] : 0, wh[a][c], wl[a][c]);
+    }
+  }
+  int em = 0;
+  bool any = false;
+  for (int c0 = 0; c0 < 4; c0++)
+    for (int c1 = 0; c1 < 4; c1++)
+#pragma unroll
+      for (int c2 = 0; c2 < 4; c2++) {
+        const double* row = eta + gk[0][c0] * g.st[0] + gk[1][c1] * g.st[1] + gk[2][c2] * g.st[2];
+#pragma unroll
+        for (int c3 = 0; c3 < 4; c3++) {
+          const double E = __ldg(row + gk[3][c3]);
+          em = max(em, vm::fx_exp(E));
+          any = any || E != 0.0;
+        }
+      }
+  val = 0.0;
+  if (!any) return true;
+  if (em < 128 || em > 2036) return false;
+  vm::FxDot s0;
+#pragma unroll 1
+  for (int c0 = 0; c0 < 4; c0++) {
+    vm::FxDot s1;
+#pragma unroll 1
+    for (int c1 = 0; c1 < 4; c1++) {
+      vm::FxDot s2;
+#pragma unroll
+      for (int c2 = 0; c2 < 4; c2++) {
+        const double* row = eta + gk[0][c0] * g.st[0] + gk[1][c1] * g.st[1] + gk[2][c2] * g.st[2];
+        vm::FxDot s3;
+#pragma unroll
+        for (int c3 = 0; c3 < 4; c3++) s3.add(vm::fx_int(__ldg(row + gk[3][c3]), em), wh[3][c3], wl[3][c3]);
+        s2.add(s3.sum(), wh[2][c2], wl[2][c2]);
+      }
+      s1.add(s2.sum(), wh[1][c1], wl[1][c1]);
+    }
+    s0.add(s1.sum(), wh[0][c0], wl[0][c0]);
+  }
+  val = vm::fx_double(s0.sum(), em);
+  return true;
+}
+
+__global__ void __launch_bounds__(128) k4_resample(G4 g, const double* __restrict__ tay, const Fx4* __restrict__ tayx,
+                                                  const int32_t* __restrict__ map, const double* __restrict__ eta,
+                                                  double* __restrict__ fnew, Dev4* ds) {
   const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= g.nsite) return;
   const int m = map[p];
   double val = 0.0;
   if (m >= 0 && m < g.ne) {
-    long long gc[4], r = p;
+    int site[4];
+    long long r = p;
     for (int a = 3; a >= 0; a--) {
-      gc[a] = r % g.n[a];
+      site[a] = (int)(r % g.n[a]);
       r /= g.n[a];
     }
-    double P[4], x[4];
-    for (int a = 0; a < 4; a++) P[a] = site_coord(g, a, gc[a]);
-    const double* tm = tay + (size_t)NT4 * m;
-    dist2_4(g, tm, P, x);
-    int lo[4], hi[4], full[4];
-    for (int a = 0; a < 4; a++) {
-      lo[a] = (x[a] < -g.beta) ? -1 : ((x[a] < g.beta) ? -1 : 0);
-      hi[a] = (x[a] < -g.beta) ? 0 : 1;
-      full[a] = (lo[a] == -1 && hi[a] == 1);
-    }
-    int k[4];
-    elem_coords(g, m, k);
-    double num[4] = {0.0, 0.0, 0.0, 0.0}, den = 0.0;
-    for (int o0 = lo[0]; o0 <= hi[0]; o0++)
-      for (int o1 = lo[1]; o1 <= hi[1]; o1++)
-        for (int o2 = lo[2]; o2 <= hi[2]; o2++)
-          for (int o3 = lo[3]; o3 <= hi[3]; o3++) {
-            const int o[4] = {o0, o1, o2, o3};
-            int nz = 0, onfull = 0;
-            for (int a = 0; a < 4; a++)
-              if (o[a] != 0) {
-                nz++;
-                onfull |= full[a];
-              }
-            if (nz >= 2 && onfull) continue;
-            int kk[4], ok = 1;
-            for (int a = 0; a < 4; a++) {
-              kk[a] = k[a] + o[a];
-              ok &= (kk[a] >= 0 && kk[a] < g.L[a]);
-            }
-            if (!ok) continue;
-            const int mm = ((kk[0] * g.L[1] + kk[1]) * g.L[2] + kk[2]) * g.L[3] + kk[3];
-            const double* t = tay + (size_t)NT4 * mm;
-            {
-              // W(2d) = 0 for d >= 1: skip the FP64 evaluation where the FP32
-              // distance and its bound show d^2 >= 1
-              float pv[4], dp[4], xf[4], ef[4], bd;
-              for (int a = 0; a < 4; a++) {
-                pv[a] = (float)((P[a] - __ldg(t + a)) * g.inv_dm[a]);
-                dp[a] = 1.8e-7f * fabsf(pv[a]) + 1e-12f;
-              }
-              eval32_4(tay32 + (size_t)NF4 * mm, pv, dp, xf, ef);
-              const float d2f = d2_32(xf, ef, &bd);
-              if (d2f - bd >= 1.f) continue;
-            }
-            double dQ[4], dd = 0.0;
-            qofp4_f(t, P, dQ);
-            for (int a = 0; a < 4; a++) {
-              const double xa = dQ[a] * g.inv_dm[a];
-              dd = fma(xa, xa, dd);
-            }
-            const double w = W4f(2.0 * sqrt(dd));
-            for (int a = 0; a < 4; a++) num[a] = fma(w, __ldg(t + 60 + a) + dQ[a], num[a]);
-            den += w;
-          }
-    double Qr[4];
-    if (den > 0.0) {
-      const double id = 1.0 / den;
-      for (int a = 0; a < 4; a++) Qr[a] = num[a] * id;
-    } else {
-      double dQ[4];
-      qofp4_f(tm, P, dQ);
-      for (int a = 0; a < 4; a++) Qr[a] = __ldg(tm + 60 + a) + dQ[a];
-    }
-    double u[4];
-    for (int a = 0; a < 4; a++) u[a] = (Qr[a] - g.lo[a]) * g.inv_d[a];
-    val = spline_eval4_f(g, eta, u);
+    if (!resample4_fixed(g, tayx, eta, site, m, val)) val = resample4_fp64(g, tay, eta, site, m);
   } else if (m >= g.ne) {
     bad(ds, 44);
   }
@@ -1489,9 +1823,9 @@ __global__ void k4_spline_axis(G4 g, int ax, const double* __restrict__ tab, dou
 // ---------------------------------------------------------------------------
 
 namespace {
-enum K4Id { K_DRIFT, K_TAYLOR, K_PERC, K_PERC_BIG, K_FINISH, K_HOLES, K_RECON, K_ACCEL, K_ACCEL_SUM, K_KICK,
+enum K4Id { K_DRIFT, K_TAYLOR, K_RECORDS, K_PERC, K_PERC_BIG, K_FINISH, K_HOLES, K_RECON, K_ACCEL, K_ACCEL_SUM, K_KICK,
             K_RESAMPLE, K_SPLINE, K_RESET, K_FIELDS, K_DIAG, K_COUNT };
-const char* const k4_names[K_COUNT] = {"drift", "taylor", "percolate", "percolate_big", "map_finish", "holes",
+const char* const k4_names[K_COUNT] = {"drift", "taylor", "records", "percolate", "percolate_big", "map_finish", "holes",
                                        "reconstruct", "accel", "accel_sum", "kick_drift", "resample", "spline_axis",
                                        "reset", "node_fields", "diagnostics"};
 struct ProfRec {
@@ -1508,6 +1842,7 @@ struct vm_4d_solver {
   char* ws;
   double *fini, *eta, *f, *el, *tay, *Mpix, *fld, *tab, *diag;
   float* tay32;
+  Fx4* tayx;
   ulonglong2* key;
   uint32_t* slot;
   int32_t *map, *holes, *cand, *ovf_list;
@@ -1563,6 +1898,12 @@ bool fill_grid(const vm_4d_config* c, G4* g) {
   for (int a = 2; a >= 0; a--) g->st[a] = g->st[a + 1] * c->n[a + 1];
   g->alpha = c->alpha > 0.0 ? c->alpha : sqrt(3.0) / 4.0;
   g->beta = c->beta > 0.0 ? c->beta : 0.5 * (1.0 - sqrt(3.0) / 2.0);
+  const bool fx = s >= 2 && s <= 16 && g->beta <= 1.0;
+  g->fx_inv_s = fx ? (long long)((1ull << 63) / (unsigned)s) : 0;
+  g->fx_beta = fx ? (long long)(g->beta * (double)s * (double)(1ll << FX4_Q)) : 0;
+  for (int a = 0; a < 4; a++) g->fx_half[a] = (long long)((c->n[a] - 1) & 1) << (FX4_Q - 1);
+  for (int b = 0; b < 4; b++)
+    for (int a = 0; a < 4; a++) g->rd[b][a] = g->d[b] / g->d[a];
   g->dt = c->dt;
   g->half_dt = 0.5 * c->dt;
   g->twoG = 2.0 * c->G;
@@ -1582,7 +1923,7 @@ int nchunks(const G4& g) {
 }
 
 struct Layout {
-  size_t diag, fini, eta, f, key, slot, map, holes, cand, el, tay, tay32, Mpix, fld, gext, part, tab, ovf, big, ds, total;
+  size_t diag, fini, eta, f, key, slot, map, holes, cand, el, tay, tay32, tayx, Mpix, fld, gext, part, tab, ovf, big, ds, total;
 };
 
 Layout layout(const G4& g) {
@@ -1606,6 +1947,7 @@ Layout layout(const G4& g) {
   L.el = take(8 * (size_t)NE4 * g.ne);
   L.tay = take(8 * (size_t)NT4 * g.ne);
   L.tay32 = take(4 * (size_t)NF4 * g.ne);
+  L.tayx = take(sizeof(Fx4) * (size_t)g.ne);
   L.Mpix = take(8 * (size_t)g.n[0] * g.n[1]);
   L.fld = take(8 * 12 * (size_t)g.n[0] * g.n[1]);
   L.gext = take(16 * (size_t)g.We0 * g.We1);
@@ -1677,7 +2019,8 @@ void prof_end(vm_4d_solver* s, int id, cudaEvent_t a) {
 
 vm_status run_map(vm_4d_solver* s) {
   const G4& g = s->g;
-  K4_LAUNCH(s, K_TAYLOR, k4_taylor<<<blocks(g.ne, 128), 128, 0, s->stream>>>(g, s->el, s->tay, s->tay32));
+  K4_LAUNCH(s, K_TAYLOR, k4_taylor<<<blocks(g.ne, 128), 128, 0, s->stream>>>(g, s->el, s->tay));
+  K4_LAUNCH(s, K_RECORDS, k4_records<<<blocks(4ll * g.ne, 128), 128, 0, s->stream>>>(g, s->tay, s->tay32, s->tayx));
   if (cudaMemsetAsync(&s->ds->nholes, 0, sizeof(int32_t), s->stream) != cudaSuccess ||
       cudaMemsetAsync(&s->ds->novf, 0, sizeof(int32_t), s->stream) != cudaSuccess)
     return VM_E_CUDA;
@@ -1693,7 +2036,7 @@ vm_status run_map(vm_4d_solver* s) {
 
 vm_status run_recon(vm_4d_solver* s) {
   const G4& g = s->g;
-  K4_LAUNCH(s, K_RECON, k4_recon<<<g.n[0] * g.n[1], 256, 0, s->stream>>>(g, s->tay, s->map, s->fini, s->f, s->Mpix, s->ds));
+  K4_LAUNCH(s, K_RECON, k4_recon<<<g.n[0] * g.n[1], 256, 0, s->stream>>>(g, s->tay, s->tayx, s->map, s->fini, s->f, s->Mpix, s->ds));
   const int nodes = g.We0 * g.We1;
   K4_LAUNCH(s, K_ACCEL, k4_accel<<<dim3(blocks(nodes, 256), s->nchunk), 256, 0, s->stream>>>(g, s->Mpix, s->part));
   K4_LAUNCH(s, K_ACCEL_SUM, k4_accel_sum<<<blocks(nodes, 256), 256, 0, s->stream>>>(g, s->part, s->nchunk, s->gext));
@@ -1722,7 +2065,7 @@ vm_status run_remap(vm_4d_solver* s) {
   vm_status st = run_map(s);
   if (st) return st;
   // f_ini <- spline(f_ini)(Q_r): the resample reads eta only
-  K4_LAUNCH(s, K_RESAMPLE, k4_resample<<<blocks(g.nsite, 128), 128, 0, s->stream>>>(g, s->tay, s->tay32, s->map, s->eta, s->fini, s->ds));
+  K4_LAUNCH(s, K_RESAMPLE, k4_resample<<<blocks(g.nsite, 128), 128, 0, s->stream>>>(g, s->tay, s->tayx, s->map, s->eta, s->fini, s->ds));
   if (cudaMemcpyAsync(s->eta, s->fini, 8 * (size_t)g.nsite, cudaMemcpyDeviceToDevice, s->stream) != cudaSuccess)
     return VM_E_CUDA;
   st = run_spline(s);
@@ -1774,6 +2117,7 @@ vm_status vm_4d_create(const vm_4d_config* c, void* d_ws, size_t bytes, void* st
   s->el = (double*)(s->ws + L.el);
   s->tay = (double*)(s->ws + L.tay);
   s->tay32 = (float*)(s->ws + L.tay32);
+  s->tayx = (Fx4*)(s->ws + L.tayx);
   s->Mpix = (double*)(s->ws + L.Mpix);
   s->fld = (double*)(s->ws + L.fld);
   s->gext = (double2*)(s->ws + L.gext);

@@ -373,7 +373,6 @@ __device__ __forceinline__ bool remap64_fixed(const Grid& g, const FxRec* __rest
   const int b0 = (inb || qv < 0) ? -1 : 0, b1 = (inb || qv >= 0) ? 1 : 0;
   const int k = m / g.Lv, l = m - k * g.Lv;
   const long long s52 = (long long)g.s << FX_Q;
-  constexpr long long one = 1ll << 62;
   long long nu = 0, nw = 0, den = 0;
   for (int a = a0; a <= a1; a++)
     for (int b = b0; b <= b1; b++) {
@@ -391,13 +390,7 @@ __device__ __forceinline__ bool remap64_fixed(const Grid& g, const FxRec* __rest
       const long long xi = __mul64hi(xn << 3, g.fx_inv_s) << 8, ze = __mul64hi(vn << 3, g.fx_inv_s) << 8;
       const long long d2 = __mul64hi(xi, xi) + __mul64hi(ze, ze);
       if (d2 >= (1ll << 60)) continue;
-      const long long d = fx_sqrt(d2), e = one - d;
-      long long w;
-      if (d <= (one >> 1)) {
-        w = one - 6 * (__mul64hi(d2, e) << 4);
-      } else {
-        w = __mul64hi(__mul64hi(e, e), e) << 5;
-      }
+      const long long w = fx_kernel(d2);
       const long long Dx = xn + a * s52 - qx, Dv = vn + b * s52 - qv;
       if (((Dx < 0 ? -Dx : Dx) | (Dv < 0 ? -Dv : Dv)) >> 60) return false;  // 2^8 cells apart
       nu += fx_mul62(Dx, w);
@@ -435,17 +428,23 @@ __device__ __forceinline__ bool remap64_fixed(const Grid& g, const FxRec* __rest
   }
   if (em < 128 || em > 2036) return false;
   constexpr long long mask = (1ll << FX_Q) - 1;
-  long long bu[4], bw[4], sum = 0;
+  long long bu[4], bw[4];
+  int wh[4], wl[4];
   fx_bspline((ru & mask) << (62 - FX_Q), bu);
   fx_bspline((rw & mask) << (62 - FX_Q), bw);
 #pragma unroll
-  for (int a = 0; a < 4; a++) {
-    long long row = 0;
+  for (int b = 0; b < 4; b++) fx_split(bw[b], wh[b], wl[b]);
+  FxDot sum;
 #pragma unroll
-    for (int b = 0; b < 4; b++) row += __mul64hi(fx_int(E[a][b], em), bw[b]);
-    sum += __mul64hi(row << 2, bu[a]);
+  for (int a = 0; a < 4; a++) {
+    FxDot row;
+#pragma unroll
+    for (int b = 0; b < 4; b++) row.add(fx_int(E[a][b], em), wh[b], wl[b]);
+    int uh, ul;
+    fx_split(bu[a], uh, ul);
+    sum.add(row.sum(), uh, ul);
   }
-  val = fx_double(sum, em + 2);
+  val = fx_double(sum.sum(), em);
   return true;
 }
 
