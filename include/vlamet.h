@@ -118,7 +118,7 @@ typedef struct {
   int32_t cycle;    /* steps since the last remap */
   int32_t holes;    /* unexplored sites repaired by the last map */
   int32_t hole_rounds;
-  int32_t overflow_elements; /* elements that needed the large flood-fill window */
+  int32_t overflow_elements; /* elements whose component leaves the 32 x 64 window */
   int32_t tier1_more;        /* elements whose small-window fill tested sites beyond
                                 the region predicted from the linear part of the map */
   int32_t last_tier_elements; /* elements filled in the whole-lattice window */

@@ -19,7 +19,7 @@ constexpr double kPi = 3.14159265358979323846;
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct Layout {
-  size_t fini, eta, f, tmp, map, slot1, rec_key, rec_site, holes_a, holes_b, ovf, gwin, seed, el, tay, tayf, tayx, M, a, da, d2a,
+  size_t fini, eta, f, tmp, map, slot1, rec_key, rec_site, holes_a, holes_b, ovf, gwin, flags, seed, el, tay, tayf, tayl, tayx, M, a, da, d2a,
       thx, thv, thxf, thvf, rect, mpart, dpart, ds, total;
 };
 
@@ -76,10 +76,12 @@ Layout layout(const vm_config* c) {
   L.ovf = take(2 * ne * 8);
   const long long pad = c->pad ? c->pad : c->elem_stride;
   L.gwin = take(vm::kGlobalBlocks * vm::global_window_words(c->nx, c->nv, pad) * 8);
+  L.flags = take(ne * 4);
   L.seed = take(std::min<size_t>(ne, vm::kSeedRecords) * 96 * 8);
   L.el = take(12 * ne * 8);
   L.tay = take(16 * ne * 8);
   L.tayf = take(32 * ne * 4);
+  L.tayl = take(vm::TL_N * ne * 4);
   L.tayx = take(sr == 8 ? ne * sizeof(vm::FxRec) : 0);
   L.M = take(c->nx * 8);
   L.a = take(c->nx * 8);
@@ -320,7 +322,7 @@ vm_status read_real(vm_solver* s, const void* src, void* out, int32_t dtype, int
 const char* const kKernelNames[vm::KID_N] = {
     "drift_taylor", "taylor", "kick_drift", "reset_elements", "scan_force", "diagnostics",
     "map_begin", "claim_small", "claim_large", "find_holes", "holes", "resolve", "read_map",
-    "reconstruct", "remap_resample", "convert", "spline_rows", "spline_cols", "claim_pair", "emap_gate"};
+    "reconstruct", "remap_resample", "convert", "spline_rows", "spline_cols", "claim_pair", "emap_gate", "map_sites"};
 
 }  // namespace
 
@@ -462,6 +464,7 @@ vm_status vm::solver_create(const vm_config* c, void* d_workspace, size_t bytes,
   g.half_dt = 0.5 * c->dt;
   g.A = 2.0 * kPi * c->G;
   g.literal_fd = c->literal_fd;
+  g.tie_v = (g.nv - 1 + g.s) % 2 == 0;
   g.max_hole_rounds = s->cfg.max_hole_rounds;
   g.fth_on = c->f_th > 0.0 ? 1 : 0;
   g.recon_tiles = (c->precision == VM_FP32_MIXED && c->recon_mode == 1) ? 1 : 0;
@@ -485,11 +488,13 @@ vm_status vm::solver_create(const vm_config* c, void* d_workspace, size_t bytes,
   s->overflow_list = (int2*)(base + L.ovf);
   s->overflow_list2 = s->overflow_list + ne_total(s);
   s->gwin = (unsigned long long*)(base + L.gwin);
+  s->flags = (uint32_t*)(base + L.flags);
   s->t1seed = (unsigned long long*)(base + L.seed);
   s->t1seed_cap = (int32_t)std::min<size_t>(ne_total(s), vm::kSeedRecords);
   s->el = (double*)(base + L.el);
   s->tay = (double*)(base + L.tay);
   s->tayf = (float*)(base + L.tayf);
+  s->tayl = (float*)(base + L.tayl);
   s->tayx = s->fp32 ? nullptr : (vm::FxRec*)(base + L.tayx);
   s->M = (double*)(base + L.M);
   s->a = (double*)(base + L.a);
@@ -786,7 +791,7 @@ vm_status vm_diagnostics(vm_solver* s, vm_diag* d) {
   d->cycle = vm::device_cycle(s) ? h.cyc : s->cyc;
   d->holes = h.holes_found;
   d->hole_rounds = h.hole_rounds;
-  d->overflow_elements = h.overflow_stat;
+  d->overflow_elements = h.overflow_stat + h.wide;
   d->tier1_more = h.t1_more;
   d->last_tier_elements = s->cfg.map_windows == 0 ? h.overflow3_stat : h.overflow_stat;
   d->exact_tests = h.n_exact;

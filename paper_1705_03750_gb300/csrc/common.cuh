@@ -46,6 +46,9 @@ struct Grid {
   // llo..lhi (the whole lattice when fth_on is 0)
   int32_t fth_on;
   int32_t klo, khi, llo, lhi;
+  // Sites lie exactly midway between lattice lines along v: in the first map
+  // after a reset, whose elements have moved along x only, all of them tie
+  int32_t tie_v;
   int32_t recon_tiles;  // FP32-mixed path: 1 = reconstruction in tiles staged by bulk copies
   // Remap decided on the device (Sec. 2.3.2): when set, every kernel of a
   // remap enqueued with this Grid returns at once while *gate is 0
@@ -77,7 +80,11 @@ struct DevState {
   int32_t noverflow_back; // tier-1 escapes of elements with all eight neighbours (listed from the end)
   int32_t nseed;          // tier-1 mask records written for the next tier
   int32_t n_pair_esc;     // tier-0 escapes listed for tier 1
-  uint32_t epoch;        // epoch of the current influence map (0..kEpochs-1)
+  int32_t n_flood;        // elements the site pass left to the flood fill
+  int32_t fresh;          // the elements were reset (isotropic, on their lattice) since the last map
+  int32_t skip_sites;     // the current map runs without the site pass (kept ties, see Grid::tie_v)
+  int32_t wide;           // elements of the site pass whose component leaves the 32 x 64 window (statistics)
+  uint32_t epoch;        // epoch of the current influence map (even, below kEpochs)
   double Mtot;           // total mass of the last reconstruction
   double sum_mass, sum_kin, sum_pot;
   unsigned long long det_min_key, det_max_key;
@@ -100,10 +107,11 @@ struct DevState {
   int32_t emap_hit;  // the current map's E_map exceeds the threshold (set by the test, cleared at map start)
 };
 
-// Owner slots of the influence map: (epoch << 24) | element index.  A slot
-// whose epoch is not the current map's is empty; every site is rewritten
-// each map (claimed or repaired), so stale values are never more than one
-// map old.  The second slot of a contested site holds (epoch << 24) while
+// Owner slots of the influence map: (epoch << 24) | element index, with the
+// map's even epoch where the site pass placed the element, and the odd one
+// after it where the flood fill claimed or repaired the site.  A slot of
+// another epoch is empty; every site is rewritten each map, so stale values
+// are never more than one map old.  The second slot of a contested site holds (epoch << 24) while
 // the site is listed for resolution, and is cleared when it is resolved.
 constexpr uint32_t SLOT_EMPTY = 0xFFFFFFFFu;
 
@@ -121,7 +129,10 @@ constexpr uint32_t SLOT_MASK = 0x00FFFFFFu;
 constexpr uint32_t SLOT_OUTSIDE = SLOT_MASK;
 // Blocks of the domain-rectangle reduction (partials kept in the workspace).
 constexpr int kRectBlocks = 256;
-constexpr int kEpochs = 255;  // epochs 0..254; 255 never current
+constexpr int kEpochs = 254;  // epochs 0..253 in pairs; 255 never current
+
+// Does owner slot t belong to the map of (even) epoch E?
+__device__ __forceinline__ bool tag_current(uint32_t t, uint32_t E) { return (t >> 25) == (E >> 1); }
 
 // Element state: 12 doubles per element, structure of arrays.
 enum { EL_X = 0, EL_V, EL_TXX, EL_TXV, EL_TVX, EL_TVV, EL_HXXX, EL_HXXV, EL_HXVV, EL_HVXX, EL_HVXV, EL_HVVV, EL_N };
@@ -137,14 +148,24 @@ enum { TY_X = 0, TY_V, TY_TI00, TY_TI01, TY_TI10, TY_TI11, TY_GX00, TY_GX01, TY_
 // |each term| of q_a bounded by C1_a |p|_inf + C2_a |p|_inf^2, C2_a from the
 // uncombined terms (the coefficients of the bound are rounded up).  UF/WF
 // and UI/WI split the element's index position u_m = (x_m - x_lo)/dx into
-// integer and fraction.
+// integer and fraction; I0/J0 are the grid site nearest to it (INT_MIN/2 where
+// it is not finite).
 // Words 20-23 repeat u_m and w_m in FP64 (a 16-byte aligned pair), so that
 // the map's first tiers read one 128-byte line per neighbour.
 enum { TF_T00 = 0, TF_T01, TF_T10, TF_T11, TF_AX, TF_BX, TF_CX, TF_AV, TF_BV, TF_CV,
-       TF_C1X, TF_C2X, TF_C1V, TF_C2V, TF_UF, TF_WF, TF_UI, TF_WI, TF_UD = 20, TF_N = 32 };
+       TF_C1X, TF_C2X, TF_C1V, TF_C2V, TF_UF, TF_WF, TF_UI, TF_WI, TF_I0, TF_J0, TF_UD = 20, TF_N = 32 };
 // the reconstruction reads words 0-15 of the FP32 record as four float4
 static_assert(TF_T00 == 0 && TF_AX == 4 && TF_BV == 8 && TF_C1V == 12 && TF_WF == 15, "FP32 record layout");
-static_assert(TF_UD % 4 == 0 && TF_UD >= TF_WI + 1 && TF_UD + 4 <= TF_N, "FP64 index positions in the FP32 record");
+static_assert(TF_UD % 4 == 0 && TF_UD >= TF_J0 + 1 && TF_UD + 4 <= TF_N, "FP64 index positions in the FP32 record");
+
+// The part of the FP32 record that the map's site pass reads, 64 bytes: the
+// map's coefficients, the index position as its start site and the FP32 offset
+// from it, and bounds on the FP32 offset over |p|_inf and on d^2 over |p|_inf^2
+// that hold for |p|_inf <= TL_P (ED negative: the element's start site is off
+// the padded lattice, or not finite, and it claims nothing).
+enum { TL_T00 = 0, TL_AX = 4, TL_BV = 8, TL_CV, TL_F0, TL_G0, TL_I0, TL_J0, TL_EQ, TL_ED, TL_N };
+static_assert(TL_N == 16, "site record layout");
+constexpr float TL_P = 2.0f;
 
 constexpr unsigned long long KEY_EMPTY = ~0ull;
 
@@ -153,7 +174,7 @@ enum KernelId {
   KID_DRIFT = 0, KID_TAYLOR, KID_KICK_DRIFT, KID_RESET, KID_SCAN_FORCE, KID_DIAG,
   KID_MAP_CLEAR, KID_CLAIM_SMALL, KID_CLAIM_LARGE, KID_FINALIZE, KID_HOLES,
   KID_RESOLVE, KID_READ_MAP,
-  KID_RECON, KID_REMAP, KID_CONVERT, KID_SPLINE_ROWS, KID_SPLINE_COLS, KID_CLAIM_PAIR, KID_EMAP, KID_N
+  KID_RECON, KID_REMAP, KID_CONVERT, KID_SPLINE_ROWS, KID_SPLINE_COLS, KID_CLAIM_PAIR, KID_EMAP, KID_MAP_SITES, KID_N
 };
 constexpr int PROF_CAP = 1024;
 
@@ -181,11 +202,13 @@ struct vm_solver {
   int2* overflow_list;      // (element, window mode) for the second tier
   int2* overflow_list2;     // for the last-resort tier
   unsigned long long* gwin; // bit masks of the whole-lattice windows (kGlobalBlocks of them), kept zeroed
+  uint32_t* flags;          // per element: flags of the map's site pass (EF_* in map.cu)
   unsigned long long* t1seed; // tier-1 masks of escaped elements: t1seed_cap records of 3 x 32 words
   int32_t t1seed_cap;
   double* el;               // 12 x ne
   double* tay;              // ne x 16
   float* tayf;              // ne x 32 (FP32 record, element units)
+  float* tayl;              // ne x 16 (the site pass's part of it)
   vm::FxRec* tayx;          // ne fixed-point records (FP64 solves; else NULL)
   double* M;                // pixel masses of the last step
   double* a;
@@ -241,6 +264,29 @@ vm_status solver_create(const vm_config* c, void* d_workspace, size_t bytes, cud
 // ---- one step, enqueue only (api.cu) ----
 void step_transport(vm_solver* s);
 cudaError_t step_remap(vm_solver* s);
+
+// Which maps take the site pass (the others are flooded as a whole): lattices
+// whose positions fit a tile word, and grids that fill the chip's blocks with
+// tiles; below about 250 x 250 sites both kernels last as long as their chains
+// and the pass is a launch more (20 steps at stride 8: 147 x 136 sites 1.70 ms
+// with it, 1.59 ms without; 301 x 217 2.03 and 1.93; 256 x 256 1.86 and 1.91;
+// 400 x 400 2.03 and 2.21; 1024 x 1024 2.87 and 3.53).  The solves of a group
+// are flooded: their smaller elements' maps agree less, and a group of 48 took
+// 1.3 ms more for the pass than the fill became shorter.
+inline bool site_pass_on(const Grid& g) {
+  return g.Lx < 4096 && g.Lv < 4096 && (long long)g.nx * g.nv >= 1 << 17;
+}
+
+// What the Taylor kernels write besides the elements: the inverse map's
+// records, the map's per-element flags, and (by one thread) the map's start.
+struct TaylorOut {
+  double* tay;
+  float* tayf;
+  float* tayl;  // NULL: no site pass
+  FxRec* tayx;  // NULL: FP32 solve
+  uint32_t* flags;
+  DevState* ds;
+};
 
 // ---- launchers (each in the translation unit of its kernels) ----
 // elements.cu
@@ -306,6 +352,7 @@ struct SolveDesc {
   int2* ovf2;
   unsigned long long* gwin;
   size_t gwin_words;
+  uint32_t* flags;
   unsigned long long* t1seed;
   int32_t t1seed_cap;
   double* el;
@@ -361,7 +408,7 @@ struct GroupPlan {
   cudaStream_t stream;
   // host-known offsets (device arrays of ns + 1 ints) and totals
   const int* off_elem64; int tot_elem64;   // 64-element chunks
-  const int* off_pair; int tot_pair;       // tier-0 blocks (2 * TP elements)
+  const int* off_pair; int tot_pair;       // blocks of tier 0 (8 elements)
   const int* off_rows; int tot_rows;       // x rows
   const int* off_diff; int tot_diff;       // 128 x-node chunks
   const int* off_sites; int tot_sites;     // 1024-site chunks (4 per thread)
@@ -379,7 +426,7 @@ struct GroupPlan {
 };
 
 enum GroupPhase : int {
-  GP_DRIFT = 0, GP_TAYLOR, GP_MAP_BEGIN, GP_PAIR, GP_SMALL, GP_BIG1, GP_BIG2, GP_BIG3, GP_RESOLVE,
+  GP_DRIFT = 0, GP_TAYLOR, GP_PAIR, GP_SMALL, GP_BIG1, GP_BIG2, GP_BIG3, GP_RESOLVE,
   GP_FIND_HOLES, GP_HOLES, GP_RECON, GP_SCAN, GP_DIFF, GP_KICK, GP_REMAP, GP_COPY, GP_ROWS, GP_COLS,
   GP_RESET, GP_UNITS, GP_EMAP, GP_N
 };
@@ -440,6 +487,7 @@ void group_remap_resample(const GroupPlan& G);   // into each solve's tmp
 void group_copy_tmp_to_fini(const GroupPlan& G);
 void group_remap_gate(const GroupPlan& G);        // E_map + decision of each solve (gated plans)
 void group_spline(const GroupPlan& G);           // fini -> eta
+int pair_units(const Grid& g);                   // work units of the map's tier 0
 size_t group_big_smem(const Grid& g);            // the large windows' shared memory for grid g
 bool group_map_prepare();
 
@@ -502,6 +550,27 @@ __device__ __forceinline__ double site_v(const Grid& g, long long j) {
 
 __device__ __forceinline__ unsigned long long dkey(double d) {
   return (unsigned long long)__double_as_longlong(d);
+}
+
+// Start of a map: next epoch, counters cleared (by the Taylor kernels, which
+// precede every map).
+__device__ __forceinline__ void map_begin(const Grid& g, DevState* ds) {
+  ds->skip_sites = ds->fresh && g.tie_v;
+  ds->fresh = 0;
+  ds->epoch = (ds->epoch + 2) % kEpochs;
+  ds->nholes = ds->holes_found = ds->hole_rounds = 0;
+  ds->noverflow = ds->overflow_stat = ds->noverflow2 = ds->overflow2_stat = 0;
+  ds->noverflow3 = ds->overflow3_stat = 0;
+  ds->nrec = 0;
+  ds->t1_more = 0;
+  ds->n_exact = 0;
+  ds->take[0] = ds->take[1] = ds->take[2] = 0;
+  ds->noverflow_back = 0;
+  ds->nseed = 0;
+  ds->n_pair_esc = 0;
+  ds->n_flood = ds->wide = 0;
+  ds->emap2_bits = 0ull;  // E_map describes the current map only
+  ds->emap_hit = 0;
 }
 
 }  // namespace vm

@@ -31,7 +31,8 @@ __device__ __forceinline__ float f32_of(double d) {
 // certified decisions' bound constants; the bound coefficients are rounded
 // upwards at every operation, with a slack of 1e-5 over the FP32 values
 // that also covers their distance to the FP64 ones.
-__device__ __forceinline__ void taylor_f32(const Grid& g, const double (&t)[TY_N], float (&F)[TF_N]) {
+__device__ __forceinline__ void taylor_f32(const Grid& g, const double (&t)[TY_N], double su, double sw,
+                                           float (&F)[TF_N]) {
   const float dxm = g.dxm_f, dvm = g.dvm_f;
   const float ti00 = f32_of(t[TY_TI00]), ti01 = f32_of(t[TY_TI01]), ti10 = f32_of(t[TY_TI10]), ti11 = f32_of(t[TY_TI11]);
   const float T00 = ti00, T01 = ti01 * g.r_vx_f, T10 = ti10 * g.r_xv_f, T11 = ti11;
@@ -68,7 +69,8 @@ __device__ __forceinline__ void taylor_f32(const Grid& g, const double (&t)[TY_N
   F[TF_WF] = ok ? f32_of(w - wi) : 0.f;
   F[TF_UI] = __int_as_float(ok ? (int)ui : INT_MIN / 2);
   F[TF_WI] = __int_as_float(ok ? (int)wi : INT_MIN / 2);
-  F[TF_WI + 1] = F[TF_WI + 2] = 0.f;  // (unused words)
+  F[TF_I0] = __int_as_float(ok ? (int)su : INT_MIN / 2);
+  F[TF_J0] = __int_as_float(ok ? (int)sw : INT_MIN / 2);
   F[TF_UD] = __int_as_float(__double2loint(u));
   F[TF_UD + 1] = __int_as_float(__double2hiint(u));
   F[TF_UD + 2] = __int_as_float(__double2loint(w));
@@ -120,13 +122,19 @@ __device__ __forceinline__ void taylor_fixed(const Grid& g, const double (&t)[TY
   X->lim = lim;
 }
 
+inline TaylorOut taylor_out(const vm_solver& s) {
+  return TaylorOut{s.tay, s.tayf, site_pass_on(s.g) ? s.tayl : nullptr, s.tayx, s.flags, s.ds};
+}
+__device__ __forceinline__ TaylorOut taylor_out(const SolveDesc& d) {
+  return TaylorOut{d.tay, d.tayf, nullptr, d.tayx, d.flags, d.ds};
+}
+
 __device__ __forceinline__ void load_element(const Grid& g, const double* __restrict__ el, int m, double (&e)[EL_N]) {
 #pragma unroll
   for (int q = 0; q < EL_N; q++) e[q] = el[(size_t)q * g.ne + m];
 }
 
-__device__ __forceinline__ void taylor_one(const Grid& g, const double (&e)[EL_N], int m, double* __restrict__ tay,
-                                           float* __restrict__ tayf, FxRec* __restrict__ tayx) {
+__device__ __forceinline__ void taylor_one(const Grid& g, const double (&e)[EL_N], int m, const TaylorOut& O) {
   const double x = e[EL_X], v = e[EL_V];
   const double Txx = e[EL_TXX], Txv = e[EL_TXV], Tvx = e[EL_TVX], Tvv = e[EL_TVV];
   // T^-1 = adj(T) (1/det T): one division (FP64 division is slow here)
@@ -161,20 +169,37 @@ __device__ __forceinline__ void taylor_one(const Grid& g, const double (&e)[EL_N
   // index position of P_m, as the start site of the percolation uses it
   t[TY_U] = dmul(dsub(x, g.x_lo), g.inv_dx);
   t[TY_W] = dmul(dsub(v, g.v_lo), g.inv_dv);
-  taylor_f32(g, t, F);
-  if (tayx) taylor_fixed(g, t, floor(t[TY_U] + 0.5), floor(t[TY_W] + 0.5), k, l, F, tayx + m);
-  double2* to = reinterpret_cast<double2*>(tay + (size_t)m * TY_N);
+  // the grid site nearest to P_m, in the fixed order
+  const double su = floor(dadd(t[TY_U], 0.5)), sw = floor(dadd(t[TY_W], 0.5));
+  taylor_f32(g, t, su, sw, F);
+  O.flags[m] = 0u;
+  if (m == 0) map_begin(g, O.ds);
+  if (O.tayl) {
+    // the site pass's record; for |p| <= TL_P the terms C1 |p| + C2 |p|^2 that
+    // bound the percolation's FP32 tests are at most (C1 + C2 TL_P) |p|
+    const float ax = F[TF_C1X] + F[TF_C2X] * TL_P, av = F[TF_C1V] + F[TF_C2V] * TL_P;
+    const int i0 = __float_as_int(F[TF_I0]), j0 = __float_as_int(F[TF_J0]);
+    const bool on = i0 >= -g.pad && i0 < g.nx + g.pad && j0 >= -g.pad && j0 < g.nv + g.pad;
+    const float ed = 4.02e-6f * (ax * ax + av * av) + 1.0e-12f;
+    float4* lo = reinterpret_cast<float4*>(O.tayl + (size_t)m * TL_N);
+    lo[0] = make_float4(F[TF_T00], F[TF_T01], F[TF_T10], F[TF_T11]);
+    lo[1] = make_float4(F[TF_AX], F[TF_BX], F[TF_CX], F[TF_AV]);
+    lo[2] = make_float4(F[TF_BV], F[TF_CV], f32_of(t[TY_U] - su), f32_of(t[TY_W] - sw));
+    lo[3] = make_float4(F[TF_I0], F[TF_J0], 2.01e-6f * (ax + av), on ? ed : -ed);
+  }
+  if (O.tayx) taylor_fixed(g, t, su, sw, k, l, F, O.tayx + m);
+  double2* to = reinterpret_cast<double2*>(O.tay + (size_t)m * TY_N);
 #pragma unroll
   for (int c = 0; c < TY_N / 2; c++) to[c] = make_double2(t[2 * c], t[2 * c + 1]);
-  float4* Fo = reinterpret_cast<float4*>(tayf + (size_t)m * TF_N);
+  float4* Fo = reinterpret_cast<float4*>(O.tayf + (size_t)m * TF_N);
 #pragma unroll
   for (int c = 0; c < (TF_UD + 4) / 4; c++) Fo[c] = make_float4(F[4 * c], F[4 * c + 1], F[4 * c + 2], F[4 * c + 3]);
 }
 
 // Half drift (predictor or corrector of Sec. 2.4): x, T_x. and H_x.. move
 // with v, T_v. and H_v..; optionally followed by the Taylor terms.
-__device__ __forceinline__ void drift_body(const Grid& g, double* __restrict__ el, double* __restrict__ tay,
-                                           float* __restrict__ tayf, FxRec* __restrict__ tayx, int taylor, int vb) {
+__device__ __forceinline__ void drift_body(const Grid& g, double* __restrict__ el, const TaylorOut& O, int taylor,
+                                           int vb) {
   int m = vb * blockDim.x + threadIdx.x;
   if (m >= g.ne) return;
   const int ne = g.ne;
@@ -191,22 +216,20 @@ __device__ __forceinline__ void drift_body(const Grid& g, double* __restrict__ e
   el[EL_TXV * ne + m] = e[EL_TXV];
 #pragma unroll
   for (int q = 0; q < 3; q++) el[(EL_HXXX + q) * ne + m] = e[EL_HXXX + q];
-  if (taylor) taylor_one(g, e, m, tay, tayf, tayx);
+  if (taylor) taylor_one(g, e, m, O);
 }
 
-__global__ void k_drift(Grid g, double* __restrict__ el, double* __restrict__ tay, float* __restrict__ tayf,
-                        FxRec* __restrict__ tayx, int taylor) {
-  drift_body(g, el, tay, tayf, tayx, taylor, blockIdx.x);
+__global__ void k_drift(Grid g, double* __restrict__ el, TaylorOut O, int taylor) {
+  drift_body(g, el, O, taylor, blockIdx.x);
 }
 
-__global__ void k_taylor(Grid g, const double* __restrict__ el, double* __restrict__ tay, float* __restrict__ tayf,
-                         FxRec* __restrict__ tayx) {
+__global__ void k_taylor(Grid g, const double* __restrict__ el, TaylorOut O) {
   if (gate_shut(g)) return;
   int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= g.ne) return;
   double e[EL_N];
   load_element(g, el, m, e);
-  taylor_one(g, e, m, tay, tayf, tayx);
+  taylor_one(g, e, m, O);
 }
 
 // Dual TSC interpolation (Sec. 2.5) at index coordinate u; beyond the grid
@@ -271,9 +294,10 @@ __global__ void k_kick_drift(Grid g, double* __restrict__ el, const double* __re
 }
 
 // Isotropic elements on the lattice (remap, Sec. 1): P_m = Q_m, T = I, H = 0.
-__device__ __forceinline__ void reset_body(const Grid& g, double* __restrict__ el, int vb) {
+__device__ __forceinline__ void reset_body(const Grid& g, double* __restrict__ el, DevState* ds, int vb) {
   int m = vb * blockDim.x + threadIdx.x;
   if (m >= g.ne) return;
+  if (m == 0) ds->fresh = 1;
   const int ne = g.ne;
   int k = m / g.Lv, l = m - k * g.Lv;
   el[EL_X * ne + m] = dadd(g.cx, dmul((double)(k - g.Kx - 1), g.dxm));
@@ -286,9 +310,9 @@ __device__ __forceinline__ void reset_body(const Grid& g, double* __restrict__ e
   for (int q = EL_HXXX; q < EL_N; q++) el[q * ne + m] = 0.0;
 }
 
-__global__ void k_reset(Grid g, double* __restrict__ el) {
+__global__ void k_reset(Grid g, double* __restrict__ el, DevState* ds) {
   if (gate_shut(g)) return;
-  reset_body(g, el, blockIdx.x);
+  reset_body(g, el, ds, blockIdx.x);
 }
 
 constexpr int SCAN_T = 512;
@@ -483,7 +507,7 @@ __global__ void k_force_diff(Grid g, const double* __restrict__ a, double* __res
 __global__ void k_drift_group(const SolveDesc* __restrict__ D, const int* __restrict__ off, int ns, int total,
                               int taylor) {
   GROUP_LOOP(off, ns, total)
-  drift_body(gsh, d.el, d.tay, d.tayf, d.tayx, taylor, vb);
+  drift_body(gsh, d.el, taylor_out(d), taylor, vb);
   GROUP_END
 }
 
@@ -493,7 +517,7 @@ __global__ void k_taylor_group(const SolveDesc* __restrict__ D, const int* __res
   if (m < gsh.ne) {
     double e[EL_N];
     load_element(gsh, d.el, m, e);
-    taylor_one(gsh, e, m, d.tay, d.tayf, d.tayx);
+    taylor_one(gsh, e, m, taylor_out(d));
   }
   GROUP_END
 }
@@ -506,7 +530,7 @@ __global__ void k_kick_group(const SolveDesc* __restrict__ D, const int* __restr
 
 __global__ void k_reset_group(const SolveDesc* __restrict__ D, const int* __restrict__ off, int ns, int total) {
   GROUP_LOOP(off, ns, total)
-  reset_body(gsh, d.el, vb);
+  reset_body(gsh, d.el, d.ds, vb);
   GROUP_END
 }
 
@@ -751,12 +775,12 @@ inline int elem_threads(int ne) { return ne <= 152 * 2 * ET ? 32 : ET; }
 }  // namespace
 
 void launch_drift(vm_solver* s, bool taylor) {
-  { const int ps_ = prof_begin(s, KID_DRIFT); k_drift<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el, s->tay, s->tayf, s->tayx, taylor ? 1 : 0); prof_end(s, ps_); }
+  { const int ps_ = prof_begin(s, KID_DRIFT); k_drift<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el, taylor_out(*s), taylor ? 1 : 0); prof_end(s, ps_); }
   s->launches++;
 }
 
 void launch_taylor(vm_solver* s) {
-  { const int ps_ = prof_begin(s, KID_TAYLOR); k_taylor<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el, s->tay, s->tayf, s->tayx); prof_end(s, ps_); }
+  { const int ps_ = prof_begin(s, KID_TAYLOR); k_taylor<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el, taylor_out(*s)); prof_end(s, ps_); }
   s->launches++;
 }
 
@@ -766,7 +790,7 @@ void launch_kick_drift(vm_solver* s) {
 }
 
 void launch_reset_elements(vm_solver* s) {
-  { const int ps_ = prof_begin(s, KID_RESET); k_reset<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el); prof_end(s, ps_); }
+  { const int ps_ = prof_begin(s, KID_RESET); k_reset<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el, s->ds); prof_end(s, ps_); }
   s->launches++;
 }
 

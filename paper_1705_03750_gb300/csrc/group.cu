@@ -48,6 +48,7 @@ SolveDesc desc_of(const vm_solver* s, bool gated) {
   d.ovf2 = s->overflow_list2;
   d.gwin = s->gwin;
   d.gwin_words = global_window_words(s->g.nx, s->g.nv, s->g.pad);
+  d.flags = s->flags;
   d.t1seed = s->t1seed;
   d.t1seed_cap = s->t1seed_cap;
   d.el = s->el;
@@ -75,7 +76,7 @@ enum { U_ELEM64 = 0, U_PAIR, U_ROWS, U_DIFF, U_SITES, U_COPY, U_ROWS4, U_COLS, U
 void units_of(const vm_solver* s, int (&u)[U_N]) {
   const long long n = (long long)s->g.nx * s->g.nv;
   u[U_ELEM64] = cdiv(s->g.ne, 64);
-  u[U_PAIR] = cdiv(s->g.ne, 8);
+  u[U_PAIR] = pair_units(s->g);
   u[U_ROWS] = s->g.nx;
   u[U_DIFF] = cdiv(s->g.nx, 128);
   u[U_SITES] = std::max(1, cdiv(n / 4, 256));

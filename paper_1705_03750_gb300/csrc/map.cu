@@ -1,5 +1,8 @@
 // Influence map of the elements of metric (Sec. 2.3.1).
 //
+// A pass over the sites settles nearly every element (the site pass below);
+// the flood fill runs for those it leaves.
+//
 // Element-parallel percolation: the claimed set of element m is the
 // 4-connected component, containing the grid site nearest to P_m, of the
 // sites that pass m's test (no investigated neighbour proposes a strictly
@@ -227,6 +230,12 @@ __device__ __forceinline__ void key_min(unsigned long long* key2, unsigned long 
   }
 }
 
+// Per-element flags of the site pass (vm_solver::flags): (a), (b) or (c) does
+// not hold somewhere; counted as wide; its start site is its own.  The site
+// pass's proposals stand for the elements with the last and not the first.
+constexpr uint32_t EF_BAD = 1u, EF_WIDE = 2u, EF_START = 4u;
+__device__ __forceinline__ bool elem_settled(uint32_t w) { return (w & ~EF_WIDE) == EF_START; }
+
 struct Slots {
   uint32_t* slot0;
   uint32_t* slot1;
@@ -236,6 +245,7 @@ struct Slots {
   const double* tay;
   DevState* ds;
   uint32_t epoch;  // filled in on the device from ds->epoch
+  const uint32_t* flags;  // per element: EF_* of the site pass
   // tier 1's masks of escaped elements (32 rows x {component, tested,
   // passing}), handed to tier 2's first window; seed_cap records at most
   unsigned long long* seed;
@@ -247,29 +257,6 @@ struct Slots {
 __device__ __forceinline__ Slots with_epoch(Slots S) {
   S.epoch = *(volatile uint32_t*)&S.ds->epoch;
   return S;
-}
-
-// Start of a map: next epoch, counters cleared.
-__device__ __forceinline__ void map_begin_body(DevState* ds) {
-  {
-    ds->epoch = (ds->epoch + 1) % kEpochs;
-    ds->nholes = ds->holes_found = ds->hole_rounds = 0;
-    ds->noverflow = ds->overflow_stat = ds->noverflow2 = ds->overflow2_stat = 0;
-    ds->noverflow3 = ds->overflow3_stat = 0;
-    ds->nrec = 0;
-    ds->t1_more = 0;
-    ds->n_exact = 0;
-    ds->take[0] = ds->take[1] = ds->take[2] = 0;
-    ds->noverflow_back = 0;
-    ds->nseed = 0;
-    ds->n_pair_esc = 0;
-    ds->emap2_bits = 0ull;  // E_map describes the current map only
-    ds->emap_hit = 0;
-  }
-}
-
-__global__ void k_map_begin(DevState* ds, const int32_t* gate) {
-  if (threadIdx.x == 0 && blockIdx.x == 0 && !(gate != nullptr && __ldcg(gate) == 0)) map_begin_body(ds);
 }
 
 __device__ __noinline__ void contest(const Slots& S, const Grid& g, long long i, long long j, size_t p, int m,
@@ -302,14 +289,17 @@ __device__ __noinline__ void contest(const Slots& S, const Grid& g, long long i,
 // all N exchanges issued before any result is looked at.
 template <int N>
 __device__ __forceinline__ void claim_sites(const Slots& S, const Grid& g, const size_t (&pos)[N], int m) {
-  const uint32_t tag = (S.epoch << 24) | (uint32_t)m;
+  const uint32_t tag = ((S.epoch + 1u) << 24) | (uint32_t)m;
   uint32_t old[N];
 #pragma unroll
   for (int u = 0; u < N; u++) old[u] = (pos[u] != ~(size_t)0) ? atomicExch(&S.slot0[pos[u]], tag) : tag;
 #pragma unroll
   for (int u = 0; u < N; u++) {
     // first claimant this map, or the same element again: nothing to resolve
-    if ((old[u] >> 24) != S.epoch || old[u] == tag) continue;
+    // (nor against the site pass's guess for an element left to this fill)
+    if (!tag_current(old[u], S.epoch) || old[u] == tag) continue;
+    if ((old[u] >> 24) == S.epoch && (int)(old[u] & SLOT_MASK) < g.ne && !elem_settled(S.flags[old[u] & SLOT_MASK]))
+      continue;
     const long long i = (long long)(pos[u] / (size_t)g.nv), j = (long long)(pos[u] - (size_t)i * g.nv);
     contest(S, g, i, j, pos[u], m, old[u]);
   }
@@ -424,11 +414,43 @@ __device__ __forceinline__ bool test_site(const Grid& g, const Elem9& E, const C
 }
 
 // ---------------------------------------------------------------------------
-// tier 1: 32 x 64 window held in registers, one warp per element
+// the site pass: owners proposed and proved site by site
 // ---------------------------------------------------------------------------
-
-constexpr int TR = 32, TCAP = 256, TE = 4;  // rows (one per lane), list capacity, elements per block
-constexpr unsigned FULL = 0xffffffffu;
+//
+// Where the elements' maps agree with one another, which is nearly everywhere,
+// the percolation need not be run.  Every site p of the padded lattice takes
+// the element O(p) that is closest among the ones its test would compare, from
+// a guess of where Q(p) lies on the element lattice (one Newton iteration per
+// block of sites, affine inside it).  Let R(m) be the sites with O = m.  If
+//   (a) m's test passes at every site of R(m),
+//   (b) m's test fails at every site outside R(m) next to one of R(m), and
+//   (c) every site of R(m) but the start site (the one nearest to P_m) has a
+//       neighbour in R(m) one step nearer to the start along x or along v,
+// then R(m), if not empty, is m's component: it is connected to the start by
+// (c), passes by (a), and nothing else is reached by (b).  Each condition
+// concerns a site and its four neighbours, so a tile of sites and one ring
+// around it decides its share; the tests are the certified FP32 ones, and the
+// exact FP64 ones where those stay open, so R(m) is the component of the
+// all-FP64 order.  An element with a site where one of the conditions does not
+// hold, or whose start site went to another element, is left to the flood fill
+// below, which then claims for it (with the odd epoch); the sites proposed for
+// it count as unclaimed.  The other elements need no claim resolution among
+// themselves, since the R(m) are disjoint.
+//
+// O(p) is a function of p and the records alone, so neighbouring tiles agree
+// on their rings.  The work is in dense phases, since a warp of 32 sites holds
+// some of every kind: every site's own evaluation; the sites outside the alpha
+// box of their guess (a quarter), listed and compared with one or three
+// neighbours; every site's (c) and the other owners next to it; and those
+// pairs (about one for every two sites), listed and tested.
+//
+// Bound by instruction issue (65 to 72 % of the slots; about 12 warp
+// instructions a site) and by the barriers between the phases.  4096 x 4096,
+// stride 8: 302 us, and 15 us for the elements left to the fill, where the fill
+// of all of them took 396 + 90 us; 8192 x 8192, step and map together: 76 ms a
+// cycle against 163.  Tiles of 16 x 64 with 128 threads do as well; longer
+// columns per thread (64 x 64 with 128 threads, 32 x 64 with 64) are 10 to 25 %
+// slower.
 
 // The exact test of site (i, j) for element (k, l), FP64 records read from
 // global memory (the rare fallback of the FP32 test).
@@ -449,6 +471,530 @@ __device__ __noinline__ bool pass_exact_g(const Grid& g, const double* __restric
     }
   return true;
 }
+
+constexpr unsigned FULL = 0xffffffffu;
+constexpr int TR = 32;  // rows of the flood fill's first register window (below)
+constexpr int SITE_T = 256, SITE_BPS = 4;   // threads of a block, blocks per SM
+constexpr int SITE_R = 32, SITE_C = 64;     // tile of padded-lattice sites
+constexpr int SITE_RR = SITE_R + 2, SITE_CC = SITE_C + 2;
+constexpr int HINT_S = 8;                // side of the blocks of sites that share one affine guess
+constexpr int HINT_R = SITE_R / HINT_S + 2, HINT_C = SITE_C / HINT_S + 2;
+constexpr int SITE_HB = SITE_R * SITE_C / (SITE_T * HINT_S);  // blocks of guesses a thread walks down
+constexpr int SITE_LIST = SITE_HB * HINT_S * 32 + 64;  // entries of a warp's lists (it has 64 fewer sites)
+constexpr int SITE_HARD = SITE_RR * SITE_CC;  // entries of the block's list
+// A tile word holds the owner's lattice position, k << 12 | l, the directions
+// (-x, -v, +x, +v) that lead nearer to its start site, and flags.
+constexpr int SO_DIR = 24;
+constexpr uint32_t SO_ELEM = 0xFFFFFFu;
+constexpr uint32_t SO_NONE = SO_ELEM;     // no owner proposed (outside the padded lattice)
+constexpr uint32_t SO_UNSURE = 1u << 28;  // (a) does not hold
+constexpr uint32_t SO_FAR = 1u << 29;     // the site lies outside a 32 x 64 window around the owner
+constexpr uint32_t SO_OUT = 1u << 30;     // the owner starts outside the padded lattice: it claims nothing
+static_assert(SITE_RR * SITE_CC < 4096 && SITE_R % HINT_S == 0 && SITE_C % HINT_S == 0, "tile index in 12 bits");
+static_assert(HINT_R * HINT_C <= SITE_T, "one thread per guess");
+static_assert(SITE_HB * SITE_T * HINT_S == SITE_R * SITE_C && SITE_T % SITE_C == 0 && HINT_S == 8, "a thread's column");
+
+struct SiteQ {
+  float qx, qv, d2;  // offset in element units, its square
+  float e, ed;       // bounds of the offsets' and of d2's distance to the FP64 values
+  int di, dj;        // the site's offset from the element's start site
+  bool out;          // the element claims nothing
+};
+
+// The certified evaluation of pass_f32 at grid site (i, j) from the element's
+// 64-byte record (TL_*), whose bounds (times |p| and |p|^2) hold up to |p| = TL_P; beyond it they
+// are formed from the FP32 record's coefficients.
+__device__ __forceinline__ SiteQ site_q(const float* __restrict__ tayl, const float* __restrict__ tayf, int m, int i,
+                                        int j, float inv_s) {
+  static_assert(TL_T00 == 0 && TL_AX == 4 && TL_BV == 8 && TL_F0 == 10 && TL_I0 == 12 && TL_EQ == 14, "record words");
+  const float4* F = reinterpret_cast<const float4*>(tayl + (size_t)m * TL_N);
+  const float4 a = __ldg(F), b = __ldg(F + 1), c = __ldg(F + 2), d = __ldg(F + 3);
+  SiteQ q;
+  q.di = i - __float_as_int(d.x);
+  q.dj = j - __float_as_int(d.y);
+  const float px = ((float)q.di - c.z) * inv_s, pv = ((float)q.dj - c.w) * inv_s;
+  const float tx = fmaf(b.x, px, fmaf(b.y, pv, a.x)), ux = fmaf(b.z, pv, a.y);
+  const float tv = fmaf(b.w, px, fmaf(c.x, pv, a.z)), uv = fmaf(c.y, pv, a.w);
+  q.qx = fmaf(px, tx, pv * ux);
+  q.qv = fmaf(px, tv, pv * uv);
+  q.d2 = fmaf(q.qx, q.qx, q.qv * q.qv);
+  q.out = d.w < 0.f;
+  const float Pm = fmaxf(fabsf(px), fabsf(pv));
+  q.e = fmaf(d.z, Pm, kAbs);
+  q.ed = fmaf(fabsf(d.w), Pm * Pm, kAbs);
+  if (!(Pm <= TL_P)) {
+    const float4 f2 = __ldg(reinterpret_cast<const float4*>(tayf + (size_t)m * TF_N) + 2);
+    const float4 f3 = __ldg(reinterpret_cast<const float4*>(tayf + (size_t)m * TF_N) + 3);
+    const float ax = Pm * fmaf(f2.w, Pm, f2.z), av = Pm * fmaf(f3.y, Pm, f3.x);
+    q.e = fmaf(1.001f * kRelQ, ax + av, kAbs);
+    q.ed = fmaf(1.001f * kRelD, fmaf(ax, ax, av * av), kAbs);
+  }
+  return q;
+}
+
+// Side of the alpha box on one axis: -1, 0 or 1, or 2 where the bound does not
+// tell (range_f's 1, 2, 3 and 0).
+__device__ __forceinline__ int side_f(float q, float e, float alo, float ahi) {
+  const float a = fabsf(q);
+  return a + e < alo ? 0 : (a - e > ahi ? (q < 0.f ? -1 : 1) : 2);
+}
+
+__device__ __forceinline__ int clampi(int x, int lo, int hi) { return min(max(x, lo), hi); }
+
+struct SiteHint {  // lattice position of Q at a block's centre and its change per site
+  float k, l, kj, kl, lj, ll;
+};
+
+// Newton steps from element to element, starting from the undeformed lattice;
+// far from an element only the linear part of its map is used.
+__device__ __forceinline__ SiteHint site_hint(const Grid& g, const float* __restrict__ tayl, float ci, float cj,
+                                              float inv_s) {
+  int k = clampi(__float2int_rn((ci - 0.5f * (float)(g.nx - 1)) * inv_s) + g.Kx + 1, g.klo, g.khi);
+  int l = clampi(__float2int_rn((cj - 0.5f * (float)(g.nv - 1)) * inv_s) + g.Kv + 1, g.llo, g.lhi);
+  SiteHint h;
+  for (int it = 0; it < 8; it++) {
+    const float4* R = reinterpret_cast<const float4*>(tayl + (size_t)(k * g.Lv + l) * TL_N);
+    const float4 a = __ldg(R), b = __ldg(R + 1), c = __ldg(R + 2);
+    const int2 ui = __ldg(reinterpret_cast<const int2*>(R + 3));
+    const float px = ((ci - (float)ui.x) - c.z) * inv_s, pv = ((cj - (float)ui.y) - c.w) * inv_s;
+    const float near = fmaxf(fabsf(px), fabsf(pv)) < 4.f ? 1.f : 0.f;
+    const float A = near * b.x, B = near * b.y, C = near * b.z, D = near * b.w, E = near * c.x, F = near * c.y;
+    h.k = (float)k + (px * (a.x + A * px + B * pv) + pv * (a.y + C * pv));
+    h.l = (float)l + (px * (a.z + D * px + E * pv) + pv * (a.w + F * pv));
+    h.kj = (a.x + 2.f * A * px + B * pv) * inv_s;
+    h.kl = (a.y + B * px + 2.f * C * pv) * inv_s;
+    h.lj = (a.z + 2.f * D * px + E * pv) * inv_s;
+    h.ll = (a.w + E * px + 2.f * F * pv) * inv_s;
+    const int k2 = clampi(__float2int_rn(h.k), g.klo, g.khi), l2 = clampi(__float2int_rn(h.l), g.llo, g.lhi);
+    if (k2 == k && l2 == l) break;
+    k = k2;
+    l = l2;
+  }
+  return h;
+}
+
+__device__ __forceinline__ uint32_t site_word(int k, int l, int di, int dj, bool sure, bool out, bool far) {
+  const uint32_t to = (di > 0 ? 1u : 0u) | (dj > 0 ? 2u : 0u) | (di < 0 ? 4u : 0u) | (dj < 0 ? 8u : 0u);
+  return (uint32_t)(k << 12 | l) | to << SO_DIR | (sure ? 0u : SO_UNSURE) | (out ? SO_OUT : 0u) | (far ? SO_FAR : 0u);
+}
+
+// The owner of site (i, j) from the exact FP64 distances, starting from
+// element (k, l): the closest of it and the neighbours its test compares,
+// until an element's own test passes (its neighbours are none closer).
+__device__ __noinline__ uint32_t site_owner_exact(const Grid& g, const double* __restrict__ tay,
+                                                  const float* __restrict__ tayl, int k, int l, int i, int j,
+                                                  float& dup) {
+  const double Px = site_x(g, i), Pv = site_v(g, j);
+  bool sure = false;
+  double d2 = 0.0;
+  for (int it = 0; it < 4 && !sure; it++) {
+    double xi, ze;
+    d2 = dist2_exact(tay + (size_t)(k * g.Lv + l) * TY_N, g, Px, Pv, xi, ze);
+    int a0, a1, b0, b1, ba = 0, bb = 0;
+    alpha_range(xi, g.alpha, a0, a1);
+    alpha_range(ze, g.alpha, b0, b1);
+    double bd = d2;
+    for (int a = a0; a <= a1; a++)
+      for (int b = b0; b <= b1; b++) {
+        if ((a == 0 && b == 0) || !elem_exists(g, k + a, l + b)) continue;
+        double x2, z2;
+        const double dn = dist2_exact(tay + (size_t)((k + a) * g.Lv + l + b) * TY_N, g, Px, Pv, x2, z2);
+        if (dn < bd) {
+          bd = dn;
+          ba = a;
+          bb = b;
+        }
+      }
+    sure = ba == 0 && bb == 0 && d2 >= 0.0;
+    k += ba;
+    l += bb;
+  }
+  dup = __double2float_ru(d2);
+  const float* R = tayl + (size_t)(k * g.Lv + l) * TL_N;
+  const int2 st = __ldg(reinterpret_cast<const int2*>(R + TL_I0));
+  return site_word(k, l, i - st.x, j - st.y, sure && dup < 1e30f, __ldg(R + TL_ED) < 0.f, false);
+}
+
+// Does the test of element (k, l) fail at site (i, j)?  The neighbours it
+// compares in FP32, then the exact test.
+__device__ __noinline__ bool site_fails_slow(const Grid& g, const double* __restrict__ tay,
+                                             const float* __restrict__ tayl, const float* __restrict__ tayf, int k,
+                                             int l, int i, int j, float inv_s, float alo, float ahi) {
+  const SiteQ q = site_q(tayl, tayf, k * g.Lv + l, i, j, inv_s);
+  const int A = side_f(q.qx, q.e, alo, ahi), B = side_f(q.qv, q.e, alo, ahi);
+  const float low = q.d2 - q.ed;
+  if (A != 2 && B != 2)
+    for (int t = 0; t < 3; t++) {
+      const int a = t == 1 ? 0 : A, b = t == 0 ? 0 : B;
+      if ((a == 0 && b == 0) || !elem_exists(g, k + a, l + b)) continue;
+      const SiteQ c = site_q(tayl, tayf, (k + a) * g.Lv + l + b, i, j, inv_s);
+      if (c.d2 + c.ed < low) return true;
+    }
+  return !pass_exact_g(g, tay, k, l, site_x(g, i), site_v(g, j));
+}
+
+__device__ __forceinline__ void leave_to_flood(uint32_t* flags, int m) {
+  if (!(__ldcg(flags + m) & EF_BAD)) atomicOr(flags + m, EF_BAD);
+}
+
+// Exclusive prefix over the warp's lanes of n <= 31, and its total.
+__device__ __forceinline__ int warp_offsets(int n, int& total) {
+  const unsigned below = (1u << (threadIdx.x & 31)) - 1u;
+  int off = 0;
+  total = 0;
+#pragma unroll
+  for (int b = 0; b < 5; b++) {
+    const unsigned v = __ballot_sync(FULL, (n >> b) & 1);
+    off += __popc(v & below) << b;
+    total += __popc(v) << b;
+  }
+  return off;
+}
+
+struct SiteShared {
+  uint32_t so[SITE_RR * SITE_CC];
+  float sd[SITE_RR * SITE_CC];  // an upper bound of the owner's d^2
+  SiteHint hint[HINT_R * HINT_C];
+  // each warp's list: sites outside the alpha box on one axis (tile index |
+  // axis << 12 | side << 13), then pairs (tile index | direction << 12)
+  unsigned short list[SITE_T / 32][SITE_LIST];
+  unsigned short hard[SITE_HARD];  // the block's: other sites outside it, then pairs that need more
+  int nhard[2];
+};
+
+struct SiteArgs {
+  const double* tay;
+  const float* tayf;
+  const float* tayl;
+  uint32_t* slot0;
+  uint32_t* flags;
+  DevState* ds;
+  float alo, ahi;
+};
+
+// The owner of a site outside the alpha box of its guess, in general: the
+// closest of the guess and the neighbours its test compares, proved where the
+// bounds settle it.
+__device__ __noinline__ void site_edge(const Grid& g, const SiteArgs& X, SiteShared& S, int idx, int i, int j,
+                                       float inv_s) {
+  const uint32_t w0 = S.so[idx];
+  int k = (int)(w0 >> 12) & 4095, l = (int)w0 & 4095;
+  SiteQ q = site_q(X.tayl, X.tayf, k * g.Lv + l, i, j, inv_s);
+  if (fmaxf(fabsf(q.qx), fabsf(q.qv)) > 0.75f) {  // a poor guess, or beyond the lattice's edge
+    const int k2 = clampi(__float2int_rn((float)k + q.qx), g.klo, g.khi);
+    const int l2 = clampi(__float2int_rn((float)l + q.qv), g.llo, g.lhi);
+    if (k2 != k || l2 != l) {
+      k = k2;
+      l = l2;
+      q = site_q(X.tayl, X.tayf, k * g.Lv + l, i, j, inv_s);
+    }
+  }
+  const int A = side_f(q.qx, q.e, X.alo, X.ahi), B = side_f(q.qv, q.e, X.alo, X.ahi);
+  bool sure = A != 2 && B != 2;
+  int ba = 0, bb = 0;
+  if (sure && (A != 0 || B != 0)) {
+    float others = 1e38f;  // the smallest lower bound of the others' d^2
+    for (int t = 0; t < 3; t++) {
+      const int a = t == 1 ? 0 : A, b = t == 0 ? 0 : B;
+      if ((a == 0 && b == 0) || (t == 2 && (A == 0 || B == 0)) || !elem_exists(g, k + a, l + b)) continue;
+      const SiteQ n = site_q(X.tayl, X.tayf, (k + a) * g.Lv + l + b, i, j, inv_s);
+      sure = sure && n.d2 < 1e30f;  // (not a number: left to the exact test)
+      if (n.d2 < q.d2) {
+        others = fminf(others, q.d2 - q.ed);
+        q = n;
+        ba = a;
+        bb = b;
+      } else {
+        others = fminf(others, n.d2 - n.ed);
+      }
+    }
+    sure = sure && q.d2 + q.ed <= others;
+    if (ba != 0 || bb != 0) {
+      // the chosen neighbour's own test may compare with elements seen here only
+      const int A2 = side_f(q.qx, q.e, X.alo, X.ahi), B2 = side_f(q.qv, q.e, X.alo, X.ahi);
+      sure = sure && A2 != 2 && B2 != 2 && (A2 == 0 || (A != 0 && (ba + A2 == 0 || ba + A2 == A))) &&
+             (B2 == 0 || (B != 0 && (bb + B2 == 0 || bb + B2 == B)));
+    }
+  }
+  float dup = q.d2 + q.ed;
+  uint32_t w;
+  if (sure && dup < 1e30f)
+    w = site_word(k + ba, l + bb, q.di, q.dj, true, q.out, abs(q.di) > TR / 2 || abs(q.dj) > 32);
+  else
+    w = site_owner_exact(g, X.tay, X.tayl, k + ba, l + bb, i, j, dup);
+  S.so[idx] = w;
+  S.sd[idx] = dup;
+}
+
+__device__ __forceinline__ void map_sites_body(const Grid& g, const SiteArgs& X, int vb) {
+  __shared__ SiteShared S;
+  if (g.khi < g.klo || g.lhi < g.llo) return;  // no element exists
+  const float inv_s = 1.0f / (float)g.s;
+  const int PX = g.nx + 2 * g.pad, PV = g.nv + 2 * g.pad;
+  const int tc = (PV + SITE_C - 1) / SITE_C;
+  const int ti = (vb / tc) * SITE_R, tj = (vb % tc) * SITE_C;  // tile origin on the padded lattice
+  const int i00 = ti - 1 - g.pad, j00 = tj - 1 - g.pad;        // grid coordinates of the ring's corner
+  const int tid = threadIdx.x, lane = tid & 31;
+  unsigned short* list = S.list[tid >> 5];
+  const uint32_t E = __ldcg(&X.ds->epoch) << 24;
+  if (tid < HINT_R * HINT_C) {
+    const int hr = tid / HINT_C, hc = tid - hr * HINT_C;
+    const float ci = (float)(i00 + 1 + (hr - 1) * HINT_S) + 0.5f * (HINT_S - 1);
+    const float cj = (float)(j00 + 1 + (hc - 1) * HINT_S) + 0.5f * (HINT_S - 1);
+    S.hint[tid] = site_hint(g, X.tayl, ci, cj, inv_s);
+  }
+  if (tid < 2) S.nhard[tid] = 0;
+  __syncthreads();
+  // Every site of the tile: the guess and its own evaluation.  A thread walks
+  // down one column of one block of guesses; it mostly stays in one element,
+  // whose map along the column is two quadratics in px.
+  const int c0 = tid % SITE_C + 1, g0 = tid / SITE_C * SITE_HB;
+  const int j0 = j00 + c0;
+  const bool col_in = (unsigned)(j0 + g.pad) < (unsigned)PV;
+  int n1 = 0;  // entries of the warp's list
+  for (int hb = 0; hb < SITE_HB; hb++) {
+    const int at0 = ((g0 + hb) * HINT_S + 1) * SITE_CC + c0;  // the first site of the block
+    const int i0 = i00 + (g0 + hb) * HINT_S + 1;
+    uint32_t e1 = 0u, eax = 0u, esg = 0u, e2 = 0u;  // per row: on the warp's list, its axis and side; on the block's
+    const SiteHint h = S.hint[(g0 + hb + 1) * HINT_C + (c0 + HINT_S - 1) / HINT_S];
+    const float dj = (float)((c0 - 1) % HINT_S) - 0.5f * (HINT_S - 1);
+    float kf = fmaf(h.kl, dj, fmaf(h.kj, -0.5f * (HINT_S - 1), h.k));
+    float lf = fmaf(h.ll, dj, fmaf(h.lj, -0.5f * (HINT_S - 1), h.l));
+    uint32_t cur = SO_NONE, base = SO_NONE;
+    float ax = 0.f, bx = 0.f, cx = 0.f, av = 0.f, bv = 0.f, cv = 0.f, f0 = 0.f, pa = 0.f, eq = 0.f, eD = 0.f;
+    int is = 0;
+    for (int t = 0; t < HINT_S; t++) {
+      const int i = i0 + t, idx = at0 + t * SITE_CC;
+      const int k = clampi(__float2int_rn(kf), g.klo, g.khi), l = clampi(__float2int_rn(lf), g.llo, g.lhi);
+      kf += h.kj;
+      lf += h.lj;
+      const uint32_t kl = (uint32_t)(k << 12 | l);
+      if (kl != cur) {
+        const float4* F = reinterpret_cast<const float4*>(X.tayl + (size_t)(k * g.Lv + l) * TL_N);
+        const float4 ra = __ldg(F), rb = __ldg(F + 1), rc = __ldg(F + 2), rd = __ldg(F + 3);
+        const int js = j0 - __float_as_int(rd.y);
+        const float pv = ((float)js - rc.w) * inv_s;
+        is = __float_as_int(rd.x);
+        f0 = -rc.z * inv_s;
+        ax = rb.x;
+        bx = fmaf(rb.y, pv, ra.x);
+        cx = pv * fmaf(rb.z, pv, ra.y);
+        av = rb.w;
+        bv = fmaf(rc.x, pv, ra.z);
+        cv = pv * fmaf(rc.y, pv, ra.w);
+        pa = fabsf(pv);
+        eq = rd.z;
+        eD = fabsf(rd.w);
+        base = site_word(k, l, 0, js, true, rd.w < 0.f, false);
+        cur = kl;
+      }
+      const int di = i - is;
+      const float px = fmaf((float)di, inv_s, f0);
+      const float qx = fmaf(px, fmaf(ax, px, bx), cx), qv = fmaf(px, fmaf(av, px, bv), cv);
+      const float Pm = fmaxf(fabsf(px), pa), e = fmaf(eq, Pm, kAbs), ed = fmaf(eD, Pm * Pm, kAbs);
+      const float mx = fabsf(qx), mv = fabsf(qv), lo = X.alo - e, hi = X.ahi + e;
+      const bool on = col_in && (unsigned)(i + g.pad) < (unsigned)PX;
+      S.so[idx] = on ? base | ((di > 0 ? 1u : 0u) | (di < 0 ? 4u : 0u)) << SO_DIR : SO_NONE;
+      S.sd[idx] = fmaf(qx, qx, qv * qv) + ed;
+      // inside the alpha box no neighbour is compared; outside it on one axis,
+      // one; the rest (both axes, an open side, a poor guess, beyond the
+      // record's bounds) are the block's list
+      const bool good = Pm <= TL_P, ix = mx < lo, iv = mv < lo;
+      const bool in = good && ix && iv;
+      const bool one = good && ((ix && mv > hi && mv <= 0.75f) || (iv && mx > hi && mx <= 0.75f));
+      const uint32_t bit = 1u << t;
+      if (on && one) e1 |= bit;
+      if (on && !one && !in) e2 |= bit;
+      if (ix) eax |= bit;
+      if ((ix ? qv : qx) > 0.f) esg |= bit;
+    }
+    int k1, k2;
+    int o1 = n1 + warp_offsets(__popc(e1), k1), o2 = warp_offsets(__popc(e2), k2);
+    n1 += k1;
+    for (; e1; e1 &= e1 - 1u) {
+      const int t = __ffs(e1) - 1;
+      list[o1++] = (unsigned short)((at0 + t * SITE_CC) | ((eax >> t) & 1u) << 12 | ((esg >> t) & 1u) << 13);
+    }
+    if (k2) {
+      int p = 0;
+      if (lane == 0) p = atomicAdd(&S.nhard[0], k2);
+      o2 += __shfl_sync(FULL, p, 0);
+      for (; e2; e2 &= e2 - 1u) S.hard[o2++] = (unsigned short)(at0 + (__ffs(e2) - 1) * SITE_CC);
+    }
+  }
+  // the ring around the tile: the rows above and below, then the side columns
+  constexpr int RING = 2 * SITE_CC + 2 * SITE_R;
+  for (int qb = tid & ~31; qb < RING; qb += SITE_T) {
+    const int q0 = qb + lane, s2 = q0 - 2 * SITE_CC;
+    const int r = s2 < 0 ? (q0 < SITE_CC ? 0 : SITE_RR - 1) : 1 + (s2 >> 1);
+    const int c = s2 < 0 ? (q0 < SITE_CC ? q0 : q0 - SITE_CC) : (s2 & 1) * (SITE_CC - 1);
+    const int idx = r * SITE_CC + c, i = i00 + r, j = j00 + c;
+    bool one = false, hard = false, ix = false, pos = false;
+    if (q0 < RING) {
+      uint32_t w = SO_NONE;
+      float dup = 0.f;
+      if ((unsigned)(i + g.pad) < (unsigned)PX && (unsigned)(j + g.pad) < (unsigned)PV) {
+        const int hr = (r + HINT_S - 1) / HINT_S, hc = (c + HINT_S - 1) / HINT_S;
+        const SiteHint& h = S.hint[hr * HINT_C + hc];
+        const float dj = (float)(c + HINT_S - 1 - hc * HINT_S) - 0.5f * (HINT_S - 1);
+        float kf = fmaf(h.kl, dj, fmaf(h.kj, -0.5f * (HINT_S - 1), h.k));
+        float lf = fmaf(h.ll, dj, fmaf(h.lj, -0.5f * (HINT_S - 1), h.l));
+        for (int t = r + HINT_S - 1 - hr * HINT_S; t > 0; t--) {  // (as the column walk of the tile that holds it)
+          kf += h.kj;
+          lf += h.lj;
+        }
+        const int k = clampi(__float2int_rn(kf), g.klo, g.khi), l = clampi(__float2int_rn(lf), g.llo, g.lhi);
+        const SiteQ q = site_q(X.tayl, X.tayf, k * g.Lv + l, i, j, inv_s);
+        const float mx = fabsf(q.qx), mv = fabsf(q.qv), lo = X.alo - q.e, hi = X.ahi + q.e;
+        const bool iv = mv < lo;
+        ix = mx < lo;
+        one = (ix && mv > hi && mv <= 0.75f) || (iv && mx > hi && mx <= 0.75f);
+        hard = !one && !(ix && iv);
+        pos = (ix ? q.qv : q.qx) > 0.f;
+        dup = q.d2 + q.ed;
+        w = site_word(k, l, q.di, q.dj, true, q.out, false);
+      }
+      S.so[idx] = w;
+      S.sd[idx] = dup;
+    }
+    if (hard) S.hard[atomicAdd(&S.nhard[0], 1)] = (unsigned short)idx;
+    const unsigned b = __ballot_sync(FULL, one);
+    if (one)
+      list[n1 + __popc(b & ((1u << lane) - 1u))] = (unsigned short)(idx | (ix ? 1 << 12 : 0) | (pos ? 1 << 13 : 0));
+    n1 += __popc(b);
+  }
+  __syncwarp();
+  // the sites outside the box on one axis: the guess m or its neighbour there
+  for (int e = lane; e < n1; e += 32) {
+    const int ent = list[e], idx = ent & 4095, r = idx / SITE_CC, i = i00 + r, j = j00 + idx - r * SITE_CC;
+    const uint32_t w0 = S.so[idx];
+    const int k = (int)(w0 >> 12) & 4095, l = (int)w0 & 4095;
+    const int sg = ((ent >> 13) & 1) * 2 - 1, B = (ent >> 12) & 1 ? sg : 0, A = (ent >> 12) & 1 ? 0 : sg;
+    if (!elem_exists(g, k + A, l + B)) continue;  // none to compare with: m's
+    // d2 of m is at most hi, and at least hi less twice its bound (|p| is at
+    // most half a site more than the offset from the start site)
+    const float4 rd = __ldg(reinterpret_cast<const float4*>(X.tayl + (size_t)(k * g.Lv + l) * TL_N) + 3);
+    const float Pm = ((float)max(abs(i - __float_as_int(rd.x)), abs(j - __float_as_int(rd.y))) + 0.51f) * inv_s;
+    const float hi = S.sd[idx], low = hi - 2.f * fmaf(fabsf(rd.w), Pm * Pm, kAbs);
+    const SiteQ n = site_q(X.tayl, X.tayf, (k + A) * g.Lv + l + B, i, j, inv_s);
+    if (n.d2 - n.ed >= hi) continue;  // certainly m's
+    uint32_t w;
+    float dup = n.d2 + n.ed;
+    // certainly the neighbour's, whose own test then compares with m only
+    const int A2 = side_f(n.qx, n.e, X.alo, X.ahi), B2 = side_f(n.qv, n.e, X.alo, X.ahi);
+    if (dup < low && (A2 == 0 || (A2 == -A && A != 0)) && (B2 == 0 || (B2 == -B && B != 0)))
+      w = site_word(k + A, l + B, n.di, n.dj, true, n.out, false);
+    else
+      w = site_owner_exact(g, X.tay, X.tayl, k, l, i, j, dup);
+    S.so[idx] = w;
+    S.sd[idx] = dup;
+  }
+  __syncthreads();
+  const int nh = S.nhard[0];
+  for (int e = SITE_T - 1 - tid; e < nh; e += SITE_T) {
+    const int idx = S.hard[e], r = idx / SITE_CC;
+    site_edge(g, X, S, idx, i00 + r, j00 + idx - r * SITE_CC, inv_s);
+  }
+  __syncthreads();
+  // every site of the tile: owner slot, (c), and the other owners around it
+  int np = 0;
+  for (int hb = 0; hb < SITE_HB; hb++) {
+    const int at0 = ((g0 + hb) * HINT_S + 1) * SITE_CC + c0, i0 = i00 + (g0 + hb) * HINT_S + 1;
+    uint32_t foreign = 0u;  // per row, directions -x, -v, +x, +v whose owner tests the site (each owner once)
+    uint32_t up = S.so[at0 - SITE_CC] & SO_ELEM, mid = S.so[at0];
+    uint32_t* slot = X.slot0 + (ptrdiff_t)i0 * g.nv + j0;
+    const bool jin = (unsigned)j0 < (unsigned)g.nv;
+    for (int t = 0; t < HINT_S; t++, slot += g.nv) {
+      const int at = at0 + t * SITE_CC;
+      const uint32_t next = S.so[at + SITE_CC];
+      const uint32_t w = mid, kl = w & SO_ELEM, n0 = up, n2_ = next & SO_ELEM;
+      const uint32_t n1_ = S.so[at - 1] & SO_ELEM, n3 = S.so[at + 1] & SO_ELEM;
+      up = kl;
+      mid = next;
+      if (kl == SO_NONE) continue;
+      const bool s0 = n0 == kl, s1 = n1_ == kl, s2 = n2_ == kl, s3 = n3 == kl;
+      const uint32_t same = (s0 ? 1u : 0u) | (s1 ? 2u : 0u) | (s2 ? 4u : 0u) | (s3 ? 8u : 0u);
+      foreign |= ((s0 ? 0u : 1u) | (s1 || n1_ == n0 ? 0u : 2u) | (s2 || n2_ == n0 || n2_ == n1_ ? 0u : 4u) |
+                  (s3 || n3 == n0 || n3 == n1_ || n3 == n2_ ? 0u : 8u))
+                 << (4 * t);
+      const int m = (int)(kl >> 12) * g.Lv + (int)(kl & 4095u);
+      const bool in = jin && (unsigned)(i0 + t) < (unsigned)g.nx;
+      if (in) *slot = E | (uint32_t)m;
+      if (!((w >> SO_DIR) & same) || (w & (SO_UNSURE | SO_FAR | SO_OUT))) {  // rare, but for start sites
+        const bool start = ((w >> SO_DIR) & 15u) == 0u;
+        if (w & SO_OUT) {
+          if (in) leave_to_flood(X.flags, m);
+        } else {
+          if (start) atomicOr(X.flags + m, EF_START);
+          if ((!start && !((w >> SO_DIR) & same)) || (w & SO_UNSURE)) leave_to_flood(X.flags, m);
+          // statistics: components no small window would have held
+          if ((w & SO_FAR) && !(__ldcg(X.flags + m) & EF_WIDE) && !(atomicOr(X.flags + m, EF_WIDE) & EF_WIDE))
+            atomicAdd(&X.ds->wide, 1);
+        }
+      }
+    }
+    // (up to 32 entries a lane: the two halves of the rows apart)
+    int na, nb;
+    int oa = np + warp_offsets(__popc(foreign & 0xFFFFu), na), ob = warp_offsets(__popc(foreign >> 16), nb);
+    ob += np + na;
+    np += na + nb;
+    for (; foreign; foreign &= foreign - 1u) {
+      const int b = __ffs(foreign) - 1, o = b < 16 ? oa++ : ob++;
+      if (o < SITE_LIST) {
+        list[o] = (unsigned short)((at0 + (b >> 2) * SITE_CC) | (b & 3) << 12);
+      } else {
+        // (more of them than the list holds: their elements are left to the fill)
+        const int t = b & 3;
+        const uint32_t kl = S.so[at0 + (b >> 2) * SITE_CC + ((t & 1) ? t - 2 : (t - 1) * SITE_CC)] & SO_ELEM;
+        if (kl != SO_NONE) leave_to_flood(X.flags, (int)(kl >> 12) * g.Lv + (int)(kl & 4095u));
+      }
+    }
+  }
+  np = min(np, SITE_LIST);
+  __syncwarp();
+  // (b): the listed foreign owners fail at the site.  The site's owner being in
+  // the ranges of their test and certainly closer settles nearly all of them.
+  for (int e = lane; e < np; e += 32) {
+    const int ent = list[e], at = ent & 4095, t = ent >> 12;
+    const uint32_t wn = S.so[at + ((t & 1) ? t - 2 : (t - 1) * SITE_CC)];
+    if ((wn & SO_OUT) || (wn & SO_ELEM) == SO_NONE) continue;  // claims nothing; off the padded lattice
+    const int r = at / SITE_CC, i = i00 + r, j = j00 + at - r * SITE_CC;
+    const uint32_t kl = S.so[at];
+    const int kn = (int)(wn >> 12) & 4095, ln = (int)wn & 4095;
+    const int a = ((int)(kl >> 12) & 4095) - kn, b = ((int)kl & 4095) - ln;
+    const SiteQ q = site_q(X.tayl, X.tayf, kn * g.Lv + ln, i, j, inv_s);
+    const float hi = X.ahi + q.e;
+    const bool fails = S.sd[at] < q.d2 - q.ed && (a == 0 || (abs(a) == 1 && (float)a * q.qx > hi)) &&
+                       (b == 0 || (abs(b) == 1 && (float)b * q.qv > hi));
+    if (!fails) {
+      const int o = atomicAdd(&S.nhard[1], 1);
+      if (o < SITE_HARD)
+        S.hard[o] = (unsigned short)ent;
+      else
+        leave_to_flood(X.flags, kn * g.Lv + ln);
+    }
+  }
+  __syncthreads();
+  const int nq = min(S.nhard[1], SITE_HARD);
+  for (int e = tid; e < nq; e += SITE_T) {
+    const int ent = S.hard[e], at = ent & 4095, t = ent >> 12;
+    const uint32_t wn = S.so[at + ((t & 1) ? t - 2 : (t - 1) * SITE_CC)];
+    const int r = at / SITE_CC, kn = (int)(wn >> 12) & 4095, ln = (int)wn & 4095;
+    if (!site_fails_slow(g, X.tay, X.tayl, X.tayf, kn, ln, i00 + r, j00 + at - r * SITE_CC, inv_s, X.alo, X.ahi))
+      leave_to_flood(X.flags, kn * g.Lv + ln);
+  }
+}
+
+__global__ void __launch_bounds__(SITE_T, SITE_BPS) k_map_sites(Grid g, SiteArgs X) {
+  if (gate_shut(g) || __ldcg(&X.ds->skip_sites)) return;
+  map_sites_body(g, X, blockIdx.x);
+}
+
+// ---------------------------------------------------------------------------
+// tier 1: 32 x 64 window held in registers, one warp per element
+// ---------------------------------------------------------------------------
+
+constexpr int TCAP = 256, TE = 4;  // list capacity, elements per block
 
 struct __align__(16) WarpShared {
   float F9[9][TF_M];
@@ -905,18 +1451,13 @@ __device__ __forceinline__ int nth_bit32(unsigned w, int n) {
   return pos;
 }
 
-__device__ __forceinline__ void claim_pair_body(const Grid& g, const double* __restrict__ tay,
-                                                         const float* __restrict__ tayf, Slots Sin, float alo,
-                                                         float ahi, int32_t* __restrict__ esc_list,
-                                                         int2* __restrict__ ovf_list, int vb) {
-  __shared__ HalfShared shp[2 * TP];
-  const Slots S = with_epoch(Sin);
-  const int lane = threadIdx.x & 31, h = lane >> 4, hl = lane & 15;
-  const int wq = threadIdx.x >> 5;
-  HalfShared& sh = shp[2 * wq + h];
-  const int m = (vb * TP + wq) * 2 + h;
-  if (__all_sync(FULL, m >= g.ne)) return;
-  bool live = m < g.ne;
+// The elements m (one per half; negative: none) of one warp.
+__device__ __forceinline__ void claim_two(const Grid& g, const double* __restrict__ tay,
+                                          const float* __restrict__ tayf, const Slots& S, float alo, float ahi,
+                                          int32_t* __restrict__ esc_list, int2* __restrict__ ovf_list, HalfShared& sh,
+                                          int lane, int m) {
+  const int h = lane >> 4, hl = lane & 15;
+  bool live = m >= 0;
   const int k = live ? m / g.Lv : 0, l = live ? m - k * g.Lv : 0;
   live = live && elem_exists(g, k, l);  // elements off the computing domain claim nothing
   // set-up: the 3x3 neighbourhood's index positions as integer part and
@@ -1194,12 +1735,63 @@ __device__ __forceinline__ void claim_pair_body(const Grid& g, const double* __r
   }
 }
 
+// The elements the site pass left over: those it marked, and those whose
+// condition (c) does not hold though their start site is on the padded lattice
+// (every element with all set, when the site pass did not run).  A warp looks
+// at up to 32 elements' flags and fills their windows two at a time.
+__device__ __forceinline__ void claim_pair_body(const Grid& g, const double* __restrict__ tay,
+                                                const float* __restrict__ tayf, Slots Sin, float alo, float ahi,
+                                                int all, int32_t* __restrict__ esc_list,
+                                                int2* __restrict__ ovf_list, int vb,
+                                                int vg) {
+  __shared__ HalfShared shp[2 * TP];
+  const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
+  const Slots S = with_epoch(Sin);
+  if (all || __ldcg(&S.ds->skip_sites)) {
+    // all of them: two per warp and turn, over as many warps as there are
+    if (vb == 0 && threadIdx.x == 0) atomicAdd(&S.ds->n_flood, g.ne);
+    for (int w = vb * TP + wq; 2 * w < g.ne; w += vg * TP) {
+      const int m = 2 * w + (lane >> 4);
+      claim_two(g, tay, tayf, S, alo, ahi, esc_list, ovf_list, shp[2 * wq + (lane >> 4)], lane, m < g.ne ? m : -1);
+      __syncwarp();
+    }
+    return;
+  }
+  // elements a warp looks at in one turn: few enough to use every warp
+  const int nw = vg * TP, per = min(32, max(2, (g.ne + nw - 1) / nw));
+  for (int base = (vb * TP + wq) * per; base < g.ne; base += nw * per) {
+    const int m = base + lane;
+    bool left = false;
+    if (lane < per && m < g.ne) {
+      const uint32_t w = S.flags[m];
+      left = w & EF_BAD;
+      if (!left && !elem_settled(w)) {
+        const int2 st = __ldg(reinterpret_cast<const int2*>(tayf + (size_t)m * TF_N + TF_I0));
+        const int k = m / g.Lv;
+        left = elem_exists(g, k, m - k * g.Lv) && st.x >= -g.pad && st.x < g.nx + g.pad && st.y >= -g.pad &&
+               st.y < g.nv + g.pad;
+      }
+    }
+    unsigned todo = __ballot_sync(FULL, left);
+    if (todo && lane == 0) atomicAdd(&S.ds->n_flood, __popc(todo));
+    while (todo) {
+      const int b0 = __ffs(todo) - 1;
+      todo &= todo - 1u;
+      const int b1 = todo ? __ffs(todo) - 1 : -1;
+      todo &= todo - 1u;
+      const int b = lane < 16 ? b0 : b1;
+      claim_two(g, tay, tayf, S, alo, ahi, esc_list, ovf_list, shp[2 * wq + (lane >> 4)], lane, b < 0 ? -1 : base + b);
+      __syncwarp();
+    }
+  }
+}
+
 __global__ void __launch_bounds__(32 * TP, 8) k_claim_pair(Grid g, const double* __restrict__ tay,
                                                          const float* __restrict__ tayf, Slots Sin, float alo,
-                                                         float ahi, int32_t* __restrict__ esc_list,
+                                                         float ahi, int all, int32_t* __restrict__ esc_list,
                                                          int2* __restrict__ ovf_list) {
   if (gate_shut(g)) return;
-  claim_pair_body(g, tay, tayf, Sin, alo, ahi, esc_list, ovf_list, blockIdx.x);
+  claim_pair_body(g, tay, tayf, Sin, alo, ahi, all, esc_list, ovf_list, blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -1766,7 +2358,7 @@ __device__ __forceinline__ void resolve_body(const Grid& g, const Slots& Sin, in
       continue;
     }
     const unsigned long long win = S.rec_key[2 * p];
-    S.slot0[p] = (S.epoch << 24) | (uint32_t)win;
+    S.slot0[p] = ((S.epoch + 1u) << 24) | (uint32_t)win;
     S.rec_key[2 * p] = KEY_EMPTY;
     S.rec_key[2 * p + 1] = KEY_EMPTY;
     S.slot1[p] = SLOT_EMPTY;
@@ -1780,28 +2372,37 @@ __global__ void k_resolve(Grid g, Slots Sin) {
 
 // Sites no element claimed, four owner slots per 16-byte load (the slot
 // array is 256-byte aligned); the list's order does not matter (the hole
-// rounds are Jacobi rounds).
-__device__ __forceinline__ void find_holes_body(const Grid& g, const uint32_t* __restrict__ slot0,
-                                                int32_t* __restrict__ holes, DevState* ds, int vb, int vg) {
+// rounds are Jacobi rounds).  Without elements left to the flood fill every
+// site is owned by the site pass, and there is nothing to look for.
+__device__ __forceinline__ void find_holes_body(const Grid& g, uint32_t* __restrict__ slot0,
+                                                const uint32_t* __restrict__ flags, int32_t* __restrict__ holes,
+                                                DevState* ds, int vb, int vg) {
+  if (*(volatile int32_t*)&ds->n_flood == 0) return;
   const uint32_t epoch = *(volatile uint32_t*)&ds->epoch;
   const size_t n = (size_t)g.nx * g.nv, n4 = n / 4;
   const size_t t0 = vb * (size_t)blockDim.x + threadIdx.x, stride = (size_t)vg * blockDim.x;
   const uint4* s4 = reinterpret_cast<const uint4*>(slot0);
+  auto look = [&](uint32_t t, size_t p) {
+    if ((t >> 24) == epoch + 1u) return;
+    if ((t >> 24) == epoch && (int)(t & SLOT_MASK) < g.ne && elem_settled(__ldg(flags + (t & SLOT_MASK)))) return;
+    slot0[p] = SLOT_EMPTY;  // (no guess of the site pass stays)
+    holes[atomicAdd(&ds->nholes, 1)] = (int32_t)p;
+  };
 #pragma unroll 4
   for (size_t q = t0; q < n4; q += stride) {
     const uint4 t = __ldcs(s4 + q);  // read once: streamed past the caches
-    const uint32_t e[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-    for (int u = 0; u < 4; u++)
-      if ((e[u] >> 24) != epoch) holes[atomicAdd(&ds->nholes, 1)] = (int32_t)(4 * q + u);
+    look(t.x, 4 * q);
+    look(t.y, 4 * q + 1);
+    look(t.z, 4 * q + 2);
+    look(t.w, 4 * q + 3);
   }
-  for (size_t p = 4 * n4 + t0; p < n; p += stride)
-    if ((slot0[p] >> 24) != epoch) holes[atomicAdd(&ds->nholes, 1)] = (int32_t)p;
+  for (size_t p = 4 * n4 + t0; p < n; p += stride) look(slot0[p], p);
 }
 
-__global__ void k_find_holes(Grid g, const uint32_t* __restrict__ slot0, int32_t* __restrict__ holes, DevState* ds) {
+__global__ void k_find_holes(Grid g, uint32_t* __restrict__ slot0, const uint32_t* __restrict__ flags,
+                             int32_t* __restrict__ holes, DevState* ds) {
   if (gate_shut(g)) return;
-  find_holes_body(g, slot0, holes, ds, blockIdx.x, gridDim.x);
+  find_holes_body(g, slot0, flags, holes, ds, blockIdx.x, gridDim.x);
 }
 
 constexpr int HT = 1024;
@@ -1842,7 +2443,7 @@ __device__ __forceinline__ void holes_body(const Grid& g, const double* __restri
         const int ii = i + di[q], jj = j + dj[q];
         if (ii < 0 || ii >= g.nx || jj < 0 || jj >= g.nv) continue;
         const uint32_t t = slot0[(size_t)ii * g.nv + jj];
-        if ((t >> 24) != epoch || (int)(t & SLOT_MASK) >= g.ne) continue;
+        if (!tag_current(t, epoch) || (int)(t & SLOT_MASK) >= g.ne) continue;
         const int cand = (int)(t & SLOT_MASK);
         const unsigned long long key = exact_key(g, tay, cand, Px, Pv);
         if (best < 0 || key < bestk || (key == bestk && cand < best)) {
@@ -1857,7 +2458,7 @@ __device__ __forceinline__ void holes_body(const Grid& g, const double* __restri
     for (int idx = threadIdx.x; idx < n; idx += HT) {
       const int ch = cho[idx];
       if (ch >= 0)
-        slot0[la[idx]] = (epoch << 24) | (uint32_t)ch;
+        slot0[la[idx]] = ((epoch + 1u) << 24) | (uint32_t)ch;
       else if (ch == -1)
         lb[atomicAdd(&next_s, 1)] = la[idx];
     }
@@ -1895,7 +2496,7 @@ __device__ __forceinline__ void emap_body(const Grid& g, const uint32_t* __restr
   double worst = 0.0;
   for (size_t p = (size_t)vb * blockDim.x + threadIdx.x; p < n; p += (size_t)vg * blockDim.x) {
     const uint32_t t = slot0[p];
-    if ((t >> 24) != epoch) continue;
+    if (!tag_current(t, epoch)) continue;
     const int m = (int)(t & SLOT_MASK);
     if (m >= g.ne) continue;
     const int i = (int)(p / (size_t)g.nv), j = (int)(p - (size_t)i * g.nv);
@@ -2000,7 +2601,7 @@ __device__ __forceinline__ void emap_test_body(const Grid& g, const uint32_t* __
     const uint32_t* row = slot0 + (size_t)i * g.nv;
     for (int j = threadIdx.x; j < g.nv; j += blockDim.x) {
       const uint32_t t = row[j];
-      if ((t >> 24) != epoch) continue;
+      if (!tag_current(t, epoch)) continue;
       const int m = (int)(t & SLOT_MASK);
       if (m >= g.ne) continue;
       float exm, evm;
@@ -2070,7 +2671,7 @@ __global__ void k_read_map(const uint32_t* __restrict__ slot0, const DevState* d
   const uint32_t epoch = *(const volatile uint32_t*)&ds->epoch;
   for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < n; p += (size_t)gridDim.x * blockDim.x) {
     const uint32_t t = slot0[p];
-    out[p] = ((t >> 24) == epoch && (int)(t & SLOT_MASK) < ne) ? (int32_t)(t & SLOT_MASK) : -1;
+    out[p] = (tag_current(t, epoch) && (int)(t & SLOT_MASK) < ne) ? (int32_t)(t & SLOT_MASK) : -1;
   }
 }
 
@@ -2080,7 +2681,7 @@ __global__ void k_read_map(const uint32_t* __restrict__ slot0, const DevState* d
 __global__ void k_clear_outside(Grid g, uint32_t* __restrict__ slot0, const DevState* ds) {
   const uint32_t epoch = *(const volatile uint32_t*)&ds->epoch;
   const int i0 = ds->rect[0], i1 = ds->rect[1], j0 = ds->rect[2], j1 = ds->rect[3];
-  const uint32_t tag = (epoch << 24) | SLOT_OUTSIDE;
+  const uint32_t tag = ((epoch + 1u) << 24) | SLOT_OUTSIDE;
   for (int i = blockIdx.x; i < g.nx; i += gridDim.x) {
     uint32_t* row = slot0 + (size_t)i * g.nv;
     if (i < i0 || i > i1 || j0 > j1) {
@@ -2094,6 +2695,7 @@ __global__ void k_clear_outside(Grid g, uint32_t* __restrict__ slot0, const DevS
 
 // ---- group launches: the influence maps of every solve of a group ----
 
+
 __device__ __forceinline__ Slots slots_of(const SolveDesc& d) {
   Slots S;
   S.slot0 = d.map;
@@ -2104,14 +2706,10 @@ __device__ __forceinline__ Slots slots_of(const SolveDesc& d) {
   S.tay = d.tay;
   S.ds = d.ds;
   S.epoch = 0u;
+  S.flags = d.flags;
   S.seed = d.t1seed;
   S.seed_cap = d.t1seed_cap;
   return S;
-}
-
-__global__ void k_map_begin_group(const SolveDesc* __restrict__ D, int ns) {
-  for (int sv = blockIdx.x * blockDim.x + threadIdx.x; sv < ns; sv += gridDim.x * blockDim.x)
-    if (!gate_shut(D[sv].g)) map_begin_body(D[sv].ds);
 }
 
 // Units of a dynamic phase, per solve, from the solve's counters (read after
@@ -2191,7 +2789,8 @@ __global__ void __launch_bounds__(1024) k_units(const SolveDesc* __restrict__ D,
 __global__ void __launch_bounds__(32 * TP, 8) k_claim_pair_group(const SolveDesc* __restrict__ D,
                                                                const int* __restrict__ off, int ns, int total) {
   GROUP_LOOP(off, ns, total)
-  claim_pair_body(gsh, d.tay, d.tayf, slots_of(d), d.alo, d.ahi, d.holes_a, d.ovf1, vb);
+  const int vg = __ldg(off + sv + 1) - __ldg(off + sv);
+  claim_pair_body(gsh, d.tay, d.tayf, slots_of(d), d.alo, d.ahi, 1, d.holes_a, d.ovf1, vb, vg);
   GROUP_END
 }
 
@@ -2233,7 +2832,7 @@ __global__ void k_resolve_group(const SolveDesc* __restrict__ D, const int* __re
 __global__ void k_find_holes_group(const SolveDesc* __restrict__ D, const int* __restrict__ off, int ns, int total) {
   GROUP_LOOP(off, ns, total)
   const int vg = __ldg(off + sv + 1) - __ldg(off + sv);
-  find_holes_body(gsh, d.map, d.holes_a, d.ds, vb, vg);
+  find_holes_body(gsh, d.map, d.flags, d.holes_a, d.ds, vb, vg);
   GROUP_END
 }
 
@@ -2329,20 +2928,31 @@ bool map_prepare(const Grid& g) {
          cudaSuccess;
 }
 
+static int site_tiles(const Grid& g) {
+  const int PX = g.nx + 2 * g.pad, PV = g.nv + 2 * g.pad;
+  return ((PX + SITE_R - 1) / SITE_R) * ((PV + SITE_C - 1) / SITE_C);
+}
+int pair_units(const Grid& g) { return (g.ne + 2 * TP - 1) / (2 * TP); }
+
 void launch_map(vm_solver* s) {
-  Slots S{s->map, s->slot1, s->rec_key, s->rec_site, s->rec_cap, s->tay, s->ds, 0u, s->t1seed, s->t1seed_cap};
+  Slots S{s->map, s->slot1, s->rec_key, s->rec_site, s->rec_cap, s->tay, s->ds, 0u, s->flags, s->t1seed, s->t1seed_cap};
   float alo, ahi;
   alpha_bounds(s->g.alpha, alo, ahi);
-  int ps = prof_begin(s, KID_MAP_CLEAR);
+  int ps = -1;
   if (s->g.fth_on) launch_domain_rect(s);
-  k_map_begin<<<1, 32, 0, s->stream>>>(s->ds, s->g.gate);
-  prof_end(s, ps);
+  const int all = s->cfg.map_windows != 0 || !site_pass_on(s->g);
+  if (!all) {
+    ps = prof_begin(s, KID_MAP_SITES);
+    k_map_sites<<<(unsigned)site_tiles(s->g), SITE_T, 0, s->stream>>>(
+        s->g, SiteArgs{s->tay, s->tayf, s->tayl, s->map, s->flags, s->ds, alo, ahi});
+    prof_end(s, ps);
+  }
   // tier 0 (two elements per warp), its escapes to tier 1 through the first
   // hole list (free until the holes are looked for)
   ps = prof_begin(s, KID_CLAIM_PAIR);
-  k_claim_pair<<<(unsigned)((s->g.ne + 2 * TP - 1) / (2 * TP)), 32 * TP, 0, s->stream>>>(s->g, s->tay, s->tayf, S,
-                                                                                        alo, ahi, s->holes_a,
-                                                                                        s->overflow_list);
+  const unsigned t0 = (unsigned)std::min<long long>(152 * 16, pair_units(s->g));
+  k_claim_pair<<<t0, 32 * TP, 0, s->stream>>>(s->g, s->tay, s->tayf, S, alo, ahi, all, s->holes_a,
+                                              s->overflow_list);
   prof_end(s, ps);
   ps = prof_begin(s, KID_CLAIM_SMALL);
   const unsigned t1 = (unsigned)std::min<long long>(152 * 8, (s->g.ne + TE - 1) / TE);
@@ -2382,12 +2992,12 @@ void launch_map(vm_solver* s) {
   if (nb > 152 * 16) nb = 152 * 16;
   if (nb == 0) nb = 1;
   ps = prof_begin(s, KID_FINALIZE);
-  k_find_holes<<<nb, 256, 0, s->stream>>>(s->g, s->map, s->holes_a, s->ds);
+  k_find_holes<<<nb, 256, 0, s->stream>>>(s->g, s->map, s->flags, s->holes_a, s->ds);
   prof_end(s, ps);
   ps = prof_begin(s, KID_HOLES);
   k_holes<<<1, HT, 0, s->stream>>>(s->g, s->tay, s->map, s->holes_a, s->holes_b, s->holes_b + s->n, s->ds);
   prof_end(s, ps);
-  s->launches += s->cfg.map_windows == 0 ? 10 : 8;
+  s->launches += s->cfg.map_windows == 0 ? 9 : 6;
 }
 
 void launch_read_map(vm_solver* s, int32_t* dst) {
@@ -2407,9 +3017,7 @@ void group_map(const GroupPlan& G) {
   cudaStream_t st = G.stream;
   const int ns = G.ns;
   const int persist = 152 * 8;
-  k_map_begin_group<<<(unsigned)((ns + 255) / 256), 256, 0, st>>>(G.D, ns);
-  if (G.tot_pair > 0)
-    k_claim_pair_group<<<group_grid(G, GP_PAIR, G.tot_pair), 32 * TP, 0, st>>>(G.D, G.off_pair, ns, G.tot_pair);
+  k_claim_pair_group<<<group_grid(G, GP_PAIR, G.tot_pair), 32 * TP, 0, st>>>(G.D, G.off_pair, ns, G.tot_pair);
   k_units<<<1, 1024, 0, st>>>(G.D, ns, GC_PAIR_ESC, persist, G.off_dyn);
   k_claim_small_group<<<group_grid(G, GP_SMALL, persist), 32 * TE, 0, st>>>(G.D, G.off_dyn, ns);
   const int capb = G.big_blocks_cap > 0 ? G.big_blocks_cap : BLOCKS_PER_SM * 152;

@@ -62,7 +62,7 @@ __device__ __forceinline__ uint32_t ds_epoch(const DevState* ds) { return *(cons
 __device__ __forceinline__ int owner(const uint32_t* __restrict__ map, size_t p, uint32_t epoch, int ne) {
   const uint32_t t = map[p];
   const int m = (int)(t & SLOT_MASK);
-  return ((t >> 24) == epoch && m < ne) ? m : -1;
+  return (tag_current(t, epoch) && m < ne) ? m : -1;
 }
 
 // The columns [j0, j1] of row i inside the map's computing domain (the whole
