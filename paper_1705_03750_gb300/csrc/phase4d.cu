@@ -1823,11 +1823,11 @@ __global__ void k4_spline_axis(G4 g, int ax, const double* __restrict__ tab, dou
 // ---------------------------------------------------------------------------
 
 namespace {
-enum K4Id { K_DRIFT, K_TAYLOR, K_RECORDS, K_PERC, K_PERC_BIG, K_FINISH, K_HOLES, K_RECON, K_ACCEL, K_ACCEL_SUM, K_KICK,
-            K_RESAMPLE, K_SPLINE, K_RESET, K_FIELDS, K_DIAG, K_COUNT };
-const char* const k4_names[K_COUNT] = {"drift", "taylor", "records", "percolate", "percolate_big", "map_finish", "holes",
+enum K4Id { K_DRIFT, K_TAYLOR, K_PERC, K_PERC_BIG, K_FINISH, K_HOLES, K_RECON, K_ACCEL, K_ACCEL_SUM, K_KICK,
+            K_RESAMPLE, K_SPLINE, K_RESET, K_FIELDS, K_DIAG, K_RECORDS, K_COUNT };
+const char* const k4_names[K_COUNT] = {"drift", "taylor", "percolate", "percolate_big", "map_finish", "holes",
                                        "reconstruct", "accel", "accel_sum", "kick_drift", "resample", "spline_axis",
-                                       "reset", "node_fields", "diagnostics"};
+                                       "reset", "node_fields", "diagnostics", "records"};
 struct ProfRec {
   int id;
   cudaEvent_t a, b;
