@@ -83,6 +83,7 @@ struct DevState {
   int32_t n_flood;        // elements the site pass left to the flood fill
   int32_t fresh;          // the elements were reset (isotropic, on their lattice) since the last map
   int32_t skip_sites;     // the current map runs without the site pass (kept ties, see Grid::tie_v)
+  uint32_t barrier;       // arrivals at the flood fill's grid barriers
   int32_t wide;           // elements of the site pass whose component leaves the 32 x 64 window (statistics)
   uint32_t epoch;        // epoch of the current influence map (even, below kEpochs)
   double Mtot;           // total mass of the last reconstruction
@@ -172,8 +173,7 @@ constexpr unsigned long long KEY_EMPTY = ~0ull;
 // Kernel identities for the optional per-launch timing (vm_profile).
 enum KernelId {
   KID_DRIFT = 0, KID_TAYLOR, KID_KICK_DRIFT, KID_RESET, KID_SCAN_FORCE, KID_DIAG,
-  KID_MAP_CLEAR, KID_CLAIM_SMALL, KID_CLAIM_LARGE, KID_FINALIZE, KID_HOLES,
-  KID_RESOLVE, KID_READ_MAP,
+  KID_FLOOD, KID_READ_MAP,
   KID_RECON, KID_REMAP, KID_CONVERT, KID_SPLINE_ROWS, KID_SPLINE_COLS, KID_CLAIM_PAIR, KID_EMAP, KID_MAP_SITES, KID_N
 };
 constexpr int PROF_CAP = 1024;
@@ -265,17 +265,13 @@ vm_status solver_create(const vm_config* c, void* d_workspace, size_t bytes, cud
 void step_transport(vm_solver* s);
 cudaError_t step_remap(vm_solver* s);
 
-// Which maps take the site pass (the others are flooded as a whole): lattices
-// whose positions fit a tile word, and grids that fill the chip's blocks with
-// tiles; below about 250 x 250 sites both kernels last as long as their chains
-// and the pass is a launch more (20 steps at stride 8: 147 x 136 sites 1.70 ms
-// with it, 1.59 ms without; 301 x 217 2.03 and 1.93; 256 x 256 1.86 and 1.91;
-// 400 x 400 2.03 and 2.21; 1024 x 1024 2.87 and 3.53).  The solves of a group
-// are flooded: their smaller elements' maps agree less, and a group of 48 took
-// 1.3 ms more for the pass than the fill became shorter.
-inline bool site_pass_on(const Grid& g) {
-  return g.Lx < 4096 && g.Lv < 4096 && (long long)g.nx * g.nv >= 1 << 17;
-}
+// Which solves take the map's site pass: lattices whose positions fit a tile
+// word.  20 steps at stride 8, with it and flooded as a whole: 100 x 100 sites
+// 1.27 and 1.34 ms, 301 x 217 1.56 and 1.74, 512 x 512 1.55 and 2.34, 1024 x
+// 1024 2.17 and 3.29.  The solves of a group are flooded: a group's map lasts
+// as long as its large windows, and 48 solves took 1.3 ms more for the pass
+// than the fill became shorter.
+inline bool site_pass_on(const Grid& g) { return g.Lx < 4096 && g.Lv < 4096; }
 
 // What the Taylor kernels write besides the elements: the inverse map's
 // records, the map's per-element flags, and (by one thread) the map's start.
@@ -498,8 +494,6 @@ void launch_fth_box(vm_solver* s);
 void launch_fth_cut(vm_solver* s);
 // the map's site rectangle from the existing elements' positions into ds->rect
 void launch_domain_rect(vm_solver* s);
-// map.cu: owner slots outside ds->rect tagged SLOT_OUTSIDE
-void launch_clear_outside(vm_solver* s);
 
 // Does element (kk, ll) exist (inside the lattice and the part of it that
 // covers the computing domain)?
@@ -569,6 +563,7 @@ __device__ __forceinline__ void map_begin(const Grid& g, DevState* ds) {
   ds->nseed = 0;
   ds->n_pair_esc = 0;
   ds->n_flood = ds->wide = 0;
+  ds->barrier = 0;
   ds->emap2_bits = 0ull;  // E_map describes the current map only
   ds->emap_hit = 0;
 }

@@ -1085,17 +1085,17 @@ __device__ __forceinline__ void claim_element(const Grid& g, const double* __res
 // window (list of n_in entries).  (A warp-strided loop that prefetched the
 // next element's records cut the set-up latency but cost more in register
 // spills than it saved.)
+template <int NW>
 __device__ __forceinline__ void claim_small_body(const Grid& g, const double* __restrict__ tay,
                                                          const float* __restrict__ tayf, Slots Sin, float alo,
                                                          float ahi, int2* __restrict__ ovf_list,
                                                          const int32_t* __restrict__ list_in,
-                                                         const int* __restrict__ n_in, int vb, int vg) {
-  __shared__ WarpShared shw[TE];
+                                                         const int* __restrict__ n_in, WarpShared* shw, int vb, int vg) {
   const Slots S = with_epoch(Sin);
   const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
-  const int n = *n_in;
-  for (int idx = vb * TE + wq; idx < n; idx += vg * TE) {
-    const int m = list_in[idx];
+  const int n = __ldcg(n_in);
+  for (int idx = vb * NW + wq; idx < n; idx += vg * NW) {
+    const int m = __ldcg(list_in + idx);
     if (m < 0 || m >= g.ne) {  // (never expected; keeps every index in bounds)
       if (lane == 0) VM_BAD(S.ds, 6);
       continue;
@@ -1103,15 +1103,6 @@ __device__ __forceinline__ void claim_small_body(const Grid& g, const double* __
     claim_element(g, tay, tayf, S, alo, ahi, ovf_list, shw[wq], lane, m);
     __syncwarp();
   }
-}
-
-__global__ void __launch_bounds__(32 * TE, 8) k_claim_small(Grid g, const double* __restrict__ tay,
-                                                         const float* __restrict__ tayf, Slots Sin, float alo,
-                                                         float ahi, int2* __restrict__ ovf_list,
-                                                         const int32_t* __restrict__ list_in,
-                                                         const int* __restrict__ n_in) {
-  if (gate_shut(g)) return;
-  claim_small_body(g, tay, tayf, Sin, alo, ahi, ovf_list, list_in, n_in, blockIdx.x, gridDim.x);
 }
 
 __device__ __forceinline__ void claim_element(const Grid& g, const double* __restrict__ tay,
@@ -1871,20 +1862,6 @@ __device__ __forceinline__ int find_entry_from(const int* incl, int s0, int n, i
   return lo;
 }
 
-// Entry holding item e of a compacted list (first s with incl[s] > e; e is
-// below incl[n - 1]).
-__device__ __forceinline__ int find_entry(const int* incl, int n, int e) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (incl[mid] > e)
-      hi = mid;
-    else
-      lo = mid + 1;
-  }
-  return lo;
-}
-
 // Window modes of the attempts after tier 1, by the sides its component
 // escaped from (1: rows, 2: columns, 3: both); the last attempt covers the
 // whole padded lattice, its bit masks in global memory.
@@ -2020,7 +1997,7 @@ __device__ __forceinline__ void claim_big_body(const Grid& g, const double* __re
   const int tid = threadIdx.x;
   const int pad = g.pad;
   // n_in items from the front of the list, n_back (if given) from its end
-  const int nf = *n_in, n = nf + (n_back ? *n_back : 0);
+  const int nf = __ldcg(n_in), n = nf + (n_back ? __ldcg(n_back) : 0);
   // items are taken one at a time from a shared counter, so that blocks that
   // drew short components take more of them
   for (;;) {
@@ -2028,7 +2005,7 @@ __device__ __forceinline__ void claim_big_body(const Grid& g, const double* __re
     __syncthreads();
     const int item = H.item;
     if (item >= n) break;
-    const int2 it2 = list_in[item < nf ? item : g.ne - 1 - (item - nf)];
+    const int2 it2 = __ldcg(list_in + (item < nf ? item : g.ne - 1 - (item - nf)));
     const int m = it2.x;
     if (m < 0 || m >= g.ne) {  // (never expected; keeps every index in bounds)
       if (tid == 0) VM_BAD(S.ds, 4);
@@ -2074,7 +2051,7 @@ __device__ __forceinline__ void claim_big_body(const Grid& g, const double* __re
     if (!kGlobal && seed >= 0 && seed < S.seed_cap && !W.trans && H.ok) {
       if (tid < TR) {
         const unsigned long long* rec = S.seed + (size_t)seed * (3 * TR);
-        const unsigned long long mc = rec[tid], mt = rec[TR + tid], mp = rec[2 * TR + tid];
+        const unsigned long long mc = __ldcg(rec + tid), mt = __ldcg(rec + TR + tid), mp = __ldcg(rec + 2 * TR + tid);
         const long long r = (i0 - TR / 2 + tid) - W.r0;
         const long long off = (j0 - 32) - W.c0;  // window bit of tier 1's column 0
         const long long w0 = (off >= 0) ? off / 64 : -((-off + 63) / 64);
@@ -2322,19 +2299,6 @@ __device__ __forceinline__ void claim_big_body(const Grid& g, const double* __re
   if (vb == 0 && tid == 0) *stat = n;
 }
 
-template <bool kGlobal>
-__global__ void __launch_bounds__(BT, BLOCKS_PER_SM) k_claim_big(Grid g, const double* __restrict__ tay,
-                                                  const float* __restrict__ tayf, Slots Sin, float alo, float ahi,
-                                                  const int2* __restrict__ list_in, const int* __restrict__ n_in,
-                                                  const int* __restrict__ n_back,
-                                                  int* __restrict__ stat, int2* __restrict__ list_out,
-                                                  int* __restrict__ n_out, int* __restrict__ take,
-                                                  unsigned long long* __restrict__ gwin, size_t gwin_words) {
-  if (gate_shut(g)) return;
-  claim_big_body<kGlobal>(g, tay, tayf, Sin, alo, ahi, list_in, n_in, n_back, stat, list_out, n_out, take, gwin,
-                          gwin_words, blockIdx.x);
-}
-
 // ---------------------------------------------------------------------------
 // conflicts, extra claimants, holes
 // ---------------------------------------------------------------------------
@@ -2349,25 +2313,20 @@ __device__ __forceinline__ unsigned long long exact_key(const Grid& g, const dou
 // flag are emptied for the next map.
 __device__ __forceinline__ void resolve_body(const Grid& g, const Slots& Sin, int vb, int vg) {
   const Slots S = with_epoch(Sin);
-  const int n = min(S.ds->nrec, S.rec_cap);
+  const int n = min(__ldcg(&S.ds->nrec), S.rec_cap);
   const size_t nsites = (size_t)g.nx * g.nv;
   for (int r = vb * blockDim.x + threadIdx.x; r < n; r += vg * blockDim.x) {
-    const size_t p = (size_t)(uint32_t)S.rec_site[r];
+    const size_t p = (size_t)(uint32_t)__ldcg(S.rec_site + r);
     if (p >= nsites) {
       VM_BAD(S.ds, 2);
       continue;
     }
-    const unsigned long long win = S.rec_key[2 * p];
+    const unsigned long long win = __ldcg(S.rec_key + 2 * p);
     S.slot0[p] = ((S.epoch + 1u) << 24) | (uint32_t)win;
     S.rec_key[2 * p] = KEY_EMPTY;
     S.rec_key[2 * p + 1] = KEY_EMPTY;
     S.slot1[p] = SLOT_EMPTY;
   }
-}
-
-__global__ void k_resolve(Grid g, Slots Sin) {
-  if (gate_shut(g)) return;
-  resolve_body(g, Sin, blockIdx.x, gridDim.x);
 }
 
 // Sites no element claimed, four owner slots per 16-byte load (the slot
@@ -2399,24 +2358,19 @@ __device__ __forceinline__ void find_holes_body(const Grid& g, uint32_t* __restr
   for (size_t p = 4 * n4 + t0; p < n; p += stride) look(slot0[p], p);
 }
 
-__global__ void k_find_holes(Grid g, uint32_t* __restrict__ slot0, const uint32_t* __restrict__ flags,
-                             int32_t* __restrict__ holes, DevState* ds) {
-  if (gate_shut(g)) return;
-  find_holes_body(g, slot0, flags, holes, ds, blockIdx.x, gridDim.x);
-}
-
 constexpr int HT = 1024;
 
 // Unexplored sites (Sec. 2.3.1, end): Jacobi rounds; in each round every
 // hole takes, among the elements its in-grid 4-neighbours held at the end of
 // the previous round, the one with the smallest d at the hole, then the
 // smaller index.
+template <int NT>
 __device__ __forceinline__ void holes_body(const Grid& g, const double* __restrict__ tay, uint32_t* __restrict__ slot0,
                                            int32_t* la, int32_t* lb, int32_t* cho, DevState* ds) {
   const uint32_t epoch = *(volatile uint32_t*)&ds->epoch;
   __shared__ int n_s, next_s;
   if (threadIdx.x == 0) {
-    n_s = ds->nholes;
+    n_s = __ldcg(&ds->nholes);
     ds->holes_found = n_s;
   }
   __syncthreads();
@@ -2427,8 +2381,8 @@ __device__ __forceinline__ void holes_body(const Grid& g, const double* __restri
       break;
     }
     const int n = n_s;
-    for (int idx = threadIdx.x; idx < n; idx += HT) {
-      const int p = la[idx];
+    for (int idx = threadIdx.x; idx < n; idx += NT) {
+      const int p = __ldcg(la + idx);
       if (p < 0 || (size_t)p >= (size_t)g.nx * g.nv) {
         VM_BAD(ds, 3);
         cho[idx] = -2;  // dropped
@@ -2442,7 +2396,7 @@ __device__ __forceinline__ void holes_body(const Grid& g, const double* __restri
       for (int q = 0; q < 4; q++) {
         const int ii = i + di[q], jj = j + dj[q];
         if (ii < 0 || ii >= g.nx || jj < 0 || jj >= g.nv) continue;
-        const uint32_t t = slot0[(size_t)ii * g.nv + jj];
+        const uint32_t t = __ldcg(slot0 + (size_t)ii * g.nv + jj);
         if (!tag_current(t, epoch) || (int)(t & SLOT_MASK) >= g.ne) continue;
         const int cand = (int)(t & SLOT_MASK);
         const unsigned long long key = exact_key(g, tay, cand, Px, Pv);
@@ -2455,12 +2409,12 @@ __device__ __forceinline__ void holes_body(const Grid& g, const double* __restri
     }
     if (threadIdx.x == 0) next_s = 0;
     __syncthreads();
-    for (int idx = threadIdx.x; idx < n; idx += HT) {
-      const int ch = cho[idx];
+    for (int idx = threadIdx.x; idx < n; idx += NT) {
+      const int ch = __ldcg(cho + idx);
       if (ch >= 0)
-        slot0[la[idx]] = ((epoch + 1u) << 24) | (uint32_t)ch;
+        slot0[__ldcg(la + idx)] = ((epoch + 1u) << 24) | (uint32_t)ch;
       else if (ch == -1)
-        lb[atomicAdd(&next_s, 1)] = la[idx];
+        lb[atomicAdd(&next_s, 1)] = __ldcg(la + idx);
     }
     __syncthreads();
     int32_t* t = la;
@@ -2474,12 +2428,6 @@ __device__ __forceinline__ void holes_body(const Grid& g, const double* __restri
     ds->hole_rounds = rounds;
     ds->nholes = 0;
   }
-}
-
-__global__ void __launch_bounds__(HT) k_holes(Grid g, const double* __restrict__ tay, uint32_t* __restrict__ slot0,
-                                              int32_t* la, int32_t* lb, int32_t* cho, DevState* ds) {
-  if (gate_shut(g)) return;
-  holes_body(g, tay, slot0, la, lb, cho, ds);
 }
 
 // E_map (Sec. 2.3.2) of the current influence map: for every grid site with
@@ -2678,7 +2626,7 @@ __global__ void k_read_map(const uint32_t* __restrict__ slot0, const DevState* d
 // Adaptive computing domain: sites outside the map's rectangle ds->rect get
 // the current epoch with no element (SLOT_OUTSIDE), so that they are
 // neither holes to repair nor candidates of a repair, and read as unowned.
-__global__ void k_clear_outside(Grid g, uint32_t* __restrict__ slot0, const DevState* ds) {
+__device__ __forceinline__ void clear_outside_body(const Grid& g, uint32_t* __restrict__ slot0, const DevState* ds) {
   const uint32_t epoch = *(const volatile uint32_t*)&ds->epoch;
   const int i0 = ds->rect[0], i1 = ds->rect[1], j0 = ds->rect[2], j1 = ds->rect[3];
   const uint32_t tag = ((epoch + 1u) << 24) | SLOT_OUTSIDE;
@@ -2691,6 +2639,89 @@ __global__ void k_clear_outside(Grid g, uint32_t* __restrict__ slot0, const DevS
       for (int j = j1 + 1 + threadIdx.x; j < g.nv; j += blockDim.x) row[j] = tag;
     }
   }
+}
+
+// ---- the flood fill's later stages of one solve in one launch ----
+//
+// Tier 1, the large windows, the whole lattice, the contested sites, the holes:
+// each needs all of the one before, so the launch is cooperative (its blocks
+// are resident together) and a barrier over the grid stands between them.  As
+// seven launches they took 10 to 25 us a map with little or nothing to do; a
+// map whose every element the site pass settled now leaves at the first line
+// (a step at 147 x 136 sites 79 -> 60 us, at 512 x 512 104 -> 73 us).
+// What other blocks wrote in this launch is read past L1 (__ldcg).
+struct FloodArgs {
+  Slots S;
+  const double* tay;
+  const float* tayf;
+  float alo, ahi;
+  int2* ovf1;
+  int2* ovf2;
+  int32_t* holes_a;
+  int32_t* holes_b;
+  unsigned long long* gwin;
+  size_t gwin_words;
+  int map_windows;
+};
+
+// Barrier over the grid: the counter rises by the grid's blocks each time (it
+// is cleared with the map's other counters).  The wait is bounded (a minute); a
+// wait that runs out is reported, and its block leaves.
+__device__ __forceinline__ bool grid_barrier(DevState* ds, unsigned& round) {
+  __shared__ int ok;
+  __syncthreads();
+  round += gridDim.x;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(&ds->barrier, 1u);
+    ok = 0;
+    for (int it = 0; it < (1 << 28) && !ok; it++) {
+      ok = *(volatile unsigned*)&ds->barrier >= round;
+      if (!ok) __nanosleep(it < 64 ? 64 : 256);
+    }
+    if (!ok) VM_BAD(ds, 8);
+    __threadfence();
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
+__global__ void __launch_bounds__(BT, BLOCKS_PER_SM) k_flood(Grid g, FloodArgs A) {
+  if (gate_shut(g)) return;
+  DevState* ds = A.S.ds;
+  const bool any = __ldcg(&ds->n_flood) != 0;
+  if (!any && !g.fth_on) return;
+  unsigned round = 0;
+  if (any) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];  // (also the large windows')
+    claim_small_body<BT / 32>(g, A.tay, A.tayf, A.S, A.alo, A.ahi, A.ovf1, A.holes_a, &ds->n_pair_esc,
+                              reinterpret_cast<WarpShared*>(smem_raw), blockIdx.x, gridDim.x);
+    if (!grid_barrier(ds, round)) return;
+    const bool windows = A.map_windows == 0;  // else tier 1's escapes go straight to the last tier
+    if (windows)
+      for (int t = 0; t < 2; t++) {
+        claim_big_body<false>(g, A.tay, A.tayf, A.S, A.alo, A.ahi, t ? A.ovf2 : A.ovf1,
+                              t ? &ds->noverflow2 : &ds->noverflow, t ? nullptr : &ds->noverflow_back,
+                              t ? &ds->overflow2_stat : &ds->overflow_stat, t ? A.ovf1 : A.ovf2,
+                              t ? &ds->noverflow3 : &ds->noverflow2, &ds->take[t], nullptr, 0, blockIdx.x);
+        if (!grid_barrier(ds, round)) return;
+      }
+    if (blockIdx.x < kGlobalBlocks)
+      claim_big_body<true>(g, A.tay, A.tayf, A.S, A.alo, A.ahi, A.ovf1, windows ? &ds->noverflow3 : &ds->noverflow,
+                           windows ? nullptr : &ds->noverflow_back, windows ? &ds->overflow3_stat : &ds->overflow_stat,
+                           nullptr, nullptr, &ds->take[2], A.gwin, A.gwin_words, blockIdx.x);
+    if (!grid_barrier(ds, round)) return;
+    resolve_body(g, A.S, blockIdx.x, gridDim.x);
+    if (!grid_barrier(ds, round)) return;
+  }
+  if (g.fth_on) {
+    clear_outside_body(g, A.S.slot0, ds);
+    if (!any || !grid_barrier(ds, round)) return;
+  }
+  find_holes_body(g, A.S.slot0, A.S.flags, A.holes_a, ds, blockIdx.x, gridDim.x);
+  if (!grid_barrier(ds, round)) return;
+  if (blockIdx.x == 0)
+    holes_body<BT>(g, A.tay, A.S.slot0, A.holes_a, A.holes_b, A.holes_b + (size_t)g.nx * g.nv, ds);
 }
 
 // ---- group launches: the influence maps of every solve of a group ----
@@ -2797,7 +2828,9 @@ __global__ void __launch_bounds__(32 * TP, 8) k_claim_pair_group(const SolveDesc
 __global__ void __launch_bounds__(32 * TE, 8) k_claim_small_group(const SolveDesc* __restrict__ D,
                                                                 const int* __restrict__ off, int ns) {
   GROUP_DYN_LOOP(off, ns)
-  claim_small_body(gsh, d.tay, d.tayf, slots_of(d), d.alo, d.ahi, d.ovf1, d.holes_a, &d.ds->n_pair_esc, vb, vg);
+  __shared__ WarpShared shw[TE];
+  claim_small_body<TE>(gsh, d.tay, d.tayf, slots_of(d), d.alo, d.ahi, d.ovf1, d.holes_a, &d.ds->n_pair_esc, shw, vb,
+                       vg);
   GROUP_END
 }
 
@@ -2853,17 +2886,11 @@ __global__ void __launch_bounds__(HT) k_holes_group(const SolveDesc* __restrict_
                                                   int ns) {
   GROUP_DYN_LOOP(off, ns)
   (void)vb;
-  holes_body(gsh, d.tay, d.map, d.holes_a, d.holes_b, d.holes_b + (size_t)gsh.nx * gsh.nv, d.ds);
+  holes_body<HT>(gsh, d.tay, d.map, d.holes_a, d.holes_b, d.holes_b + (size_t)gsh.nx * gsh.nv, d.ds);
   GROUP_END
 }
 
 }  // namespace
-
-void launch_clear_outside(vm_solver* s) {
-  const unsigned nb = (unsigned)std::min(s->g.nx, 152 * 8);
-  k_clear_outside<<<nb, 256, 0, s->stream>>>(s->g, s->map, s->ds);
-  s->launches++;
-}
 
 void launch_emap(vm_solver* s) {
   unsigned nb = (unsigned)((s->n + 255) / 256);
@@ -2910,6 +2937,9 @@ size_t big_smem_bytes(const Grid& g) {
   return sizeof(BigHeader) + 3 * (size_t)nw * sizeof(unsigned long long);
 }
 
+// Dynamic shared memory of the flood fill: a large window, or tier 1's warps.
+size_t flood_smem(const Grid& g) { return std::max(big_smem_bytes(g), (BT / 32) * sizeof(WarpShared)); }
+
 // alpha rounded down and up to FP32
 void alpha_bounds(double alpha, float& lo, float& hi) {
   const float f = (float)alpha;
@@ -2919,13 +2949,23 @@ void alpha_bounds(double alpha, float& lo, float& hi) {
 
 }  // namespace
 
-// Opt the large-window kernel in to shared memory.  The limit is a property
+// Opt a kernel in to shared memory, up to the per-block limit less its static
+// part.
+template <typename K>
+static cudaError_t opt_in(K kernel) {
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(SMEM_MAX - fa.sharedSizeBytes));
+}
+
+// Opt the flood fill in to shared memory.  The limit is a property
 // of the kernel, shared by every solver of the process, so it is set to the
 // largest size any grid can ask for rather than to this grid's need.
 bool map_prepare(const Grid& g) {
-  if (big_smem_bytes(g) > SMEM_MAX || BLOCKS_PER_SM * (big_smem_bytes(g) + 1024) > SMEM_SM) return false;
-  return cudaFuncSetAttribute(k_claim_big<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX) ==
-         cudaSuccess;
+  if (flood_smem(g) > SMEM_MAX || BLOCKS_PER_SM * (flood_smem(g) + 1024) > SMEM_SM) return false;
+  return opt_in(k_flood) == cudaSuccess;
 }
 
 static int site_tiles(const Grid& g) {
@@ -2933,6 +2973,15 @@ static int site_tiles(const Grid& g) {
   return ((PX + SITE_R - 1) / SITE_R) * ((PV + SITE_C - 1) / SITE_C);
 }
 int pair_units(const Grid& g) { return (g.ne + 2 * TP - 1) / (2 * TP); }
+
+// Blocks of the flood fill's launch: those resident together.
+static int flood_blocks(size_t smem) {
+  int dev = 0, sms = 0, per = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_flood, BT, smem) != cudaSuccess) per = 1;
+  return sms * std::max(1, std::min(per, BLOCKS_PER_SM));
+}
 
 void launch_map(vm_solver* s) {
   Slots S{s->map, s->slot1, s->rec_key, s->rec_site, s->rec_cap, s->tay, s->ds, 0u, s->flags, s->t1seed, s->t1seed_cap};
@@ -2954,50 +3003,18 @@ void launch_map(vm_solver* s) {
   k_claim_pair<<<t0, 32 * TP, 0, s->stream>>>(s->g, s->tay, s->tayf, S, alo, ahi, all, s->holes_a,
                                               s->overflow_list);
   prof_end(s, ps);
-  ps = prof_begin(s, KID_CLAIM_SMALL);
-  const unsigned t1 = (unsigned)std::min<long long>(152 * 8, (s->g.ne + TE - 1) / TE);
-  k_claim_small<<<t1, 32 * TE, 0, s->stream>>>(s->g, s->tay, s->tayf, S, alo, ahi, s->overflow_list, s->holes_a,
-                                              &s->ds->n_pair_esc);
+  // the rest of the flood fill; the elements that can escape tier 1 are few on
+  // a small lattice, and an idle block still takes a whole SM
+  ps = prof_begin(s, KID_FLOOD);
+  const size_t smem = flood_smem(s->g);
+  Grid g = s->g;
+  FloodArgs A{S, s->tay, s->tayf, alo, ahi, s->overflow_list, s->overflow_list2, s->holes_a, s->holes_b, s->gwin,
+              global_window_words(s->g.nx, s->g.nv, s->g.pad), s->cfg.map_windows};
+  void* args[2] = {&g, &A};
+  const long long blocks = std::min<long long>(flood_blocks(smem), std::max<long long>(kGlobalBlocks, s->g.ne / 16));
+  cudaLaunchCooperativeKernel((const void*)k_flood, dim3((unsigned)blocks), dim3(BT), args, smem, s->stream);
   prof_end(s, ps);
-  const size_t smem = big_smem_bytes(s->g);
-  DevState* d = s->ds;
-  // Blocks of the large windows: the elements that can escape tier 1 are
-  // few on a small lattice, and an idle block still takes a whole SM.
-  const unsigned big1 = (unsigned)std::min<long long>(BLOCKS_PER_SM * 152, std::max<long long>(16, s->g.ne / 16));
-  const unsigned big2 = big1;
-  const unsigned bigG = (unsigned)std::min<long long>(kGlobalBlocks, big1);
-  ps = prof_begin(s, KID_CLAIM_LARGE);
-  if (s->cfg.map_windows == 0) {
-    k_claim_big<false><<<big1, BT, smem, s->stream>>>(s->g, s->tay, s->tayf, S, alo, ahi, s->overflow_list,
-                                                         &d->noverflow, &d->noverflow_back, &d->overflow_stat,
-                                                         s->overflow_list2,
-                                                         &d->noverflow2, &d->take[0], nullptr, 0);
-    k_claim_big<false><<<big2, BT, smem, s->stream>>>(s->g, s->tay, s->tayf, S, alo, ahi, s->overflow_list2,
-                                                     &d->noverflow2, nullptr, &d->overflow2_stat, s->overflow_list,
-                                                     &d->noverflow3, &d->take[1], nullptr, 0);
-  }
-  // tier-1 escapes go straight here when the shared-memory windows are off
-  int* n_last = s->cfg.map_windows == 0 ? &d->noverflow3 : &d->noverflow;
-  int* stat_last = s->cfg.map_windows == 0 ? &d->overflow3_stat : &d->overflow_stat;
-  k_claim_big<true><<<bigG, BT, sizeof(BigHeader), s->stream>>>(
-      s->g, s->tay, s->tayf, S, alo, ahi, s->overflow_list, n_last,
-      s->cfg.map_windows == 0 ? nullptr : &d->noverflow_back, stat_last, nullptr, nullptr, &d->take[2],
-      s->gwin, global_window_words(s->g.nx, s->g.nv, s->g.pad));
-  prof_end(s, ps);
-  ps = prof_begin(s, KID_RESOLVE);
-  k_resolve<<<(unsigned)std::min<size_t>(152, (s->n + 1023) / 1024), 256, 0, s->stream>>>(s->g, S);
-  if (s->g.fth_on) launch_clear_outside(s);
-  prof_end(s, ps);
-  unsigned nb = (unsigned)((s->n / 4 + 255) / 256);
-  if (nb > 152 * 16) nb = 152 * 16;
-  if (nb == 0) nb = 1;
-  ps = prof_begin(s, KID_FINALIZE);
-  k_find_holes<<<nb, 256, 0, s->stream>>>(s->g, s->map, s->flags, s->holes_a, s->ds);
-  prof_end(s, ps);
-  ps = prof_begin(s, KID_HOLES);
-  k_holes<<<1, HT, 0, s->stream>>>(s->g, s->tay, s->map, s->holes_a, s->holes_b, s->holes_b + s->n, s->ds);
-  prof_end(s, ps);
-  s->launches += s->cfg.map_windows == 0 ? 9 : 6;
+  s->launches += all ? 2 : 3;
 }
 
 void launch_read_map(vm_solver* s, int32_t* dst) {
@@ -3036,16 +3053,7 @@ void group_map(const GroupPlan& G) {
 }
 
 // Opt the group's large-window kernels in to shared memory (as map_prepare
-// does), up to the per-block limit less their static shared memory.
-template <typename K>
-static cudaError_t opt_in(K kernel) {
-  cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(SMEM_MAX - fa.sharedSizeBytes));
-}
-
+// does).
 bool group_map_prepare() {
   cudaError_t e = opt_in(k_claim_big_group<0>);
   if (e == cudaSuccess) e = opt_in(k_claim_big_group<1>);
