@@ -30,7 +30,7 @@
 //   3. the whole padded lattice, its masks in global memory.
 //      Outer-layer elements whose neighbours moved away claim long thin
 //      bands; to cross them in few rounds, any 64-site word near the
-//      component is tested whole (three rows ahead, one word ahead) and the
+//      component is tested whole (six rows ahead, one word ahead) and the
 //      component is extended through runs of passing sites inside a word
 //      with one carry-propagating addition.
 //
@@ -1789,13 +1789,18 @@ __global__ void __launch_bounds__(32 * TP, 8) k_claim_pair(Grid g, const double*
 // tier 2: larger windows, cooperative block, word-granular tests
 // ---------------------------------------------------------------------------
 
-constexpr int BT = 256;       // threads
-constexpr int BLOCKS_PER_SM = 3;
+// A component takes tens of rounds, one after the other, and there are fewer of
+// them than the chip has room for: a round's tests are spread over many threads
+// and reach further ahead (8192 x 8192 78.2 -> 72.5 ms, 576 x 2048 with the
+// E_map criterion 8.2 -> 7.6 ms, a group of 48 53.4 -> 50.8 ms, against 3
+// blocks of 256 threads and 3 rows; 1024 threads: 71.4, 7.4, 51.8).
+constexpr int BT = 512;       // threads
+constexpr int BLOCKS_PER_SM = 2;
 constexpr int BAND_R = 128, BAND_W = 20;  // band window: 128 rows across, up to 1280 sites along
 constexpr int FAT_R = 160, FAT_W = 12;    // 160 x 768 sites
 constexpr int LIST_CAP = 512;
 constexpr int UNS_CAP = 512;  // sites per round whose FP32 test is left open, tested exactly together
-constexpr int AHEAD = 3;      // rows tested ahead of the component per round
+constexpr int AHEAD = 6;      // rows tested ahead of the component per round
 constexpr size_t SMEM_MAX = 227 * 1024;   // opt-in limit per block
 constexpr size_t SMEM_SM = 228 * 1024;    // shared memory per SM
 
@@ -1958,10 +1963,10 @@ __device__ __forceinline__ unsigned long long dilate(const unsigned long long* c
 
 // Sites worth testing ahead of the component in word q: the word's column
 // within AHEAD rows of it, the whole word if the word or a neighbouring word
-// of its row holds some.  (Deeper speculation, 4 to 12 rows and two words,
-// tested more sites than it saved rounds; growing inside a word one site per
-// round, as the column rule alone does, made a component that starts from one
-// site and runs along the bits take one round per site.)
+// of its row holds some.  (Growing inside a word one site per round, as the
+// column rule alone does, made a component that starts from one site and runs
+// along the bits take one round per site; sites predicted from the element's
+// own map saved no rounds: a large component is where the maps disagree.)
 __device__ __forceinline__ unsigned long long ahead(const unsigned long long* comp, const Win& W, int q) {
   const int r = q / W.W, w = q - r * W.W;
   unsigned long long d = dilate(comp, W, q);
