@@ -57,6 +57,37 @@ struct Grid {
 
 // True when the remap this Grid was enqueued for is not to run (read by
 // every thread of a kernel before any barrier, so all return together).
+// The kernels of a step follow one another closely (launch_next below): a
+// kernel's blocks are placed while the one before drains, and wait here, before
+// their first access, for it to have completed.  Each lets the next one's
+// blocks in as soon as its own are all placed.
+// The result is always true; returning on it keeps every load of the kernel,
+// also those marked read-only, behind the wait.
+__device__ __forceinline__ bool after_prior() {
+  unsigned nt;
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;\n\tmov.u32 %0, %%ntid.x;" : "=r"(nt)::"memory");
+  return nt != 0u;
+}
+
+// Launch on the stream behind the kernel before it; only for kernels that call
+// after_prior first.  A step at 128 x 128 FP64 68 -> 54 us, at 512 x 512 FP32 73
+// -> 68 us; 4096 x 4096 1 %.  Not the spline's sweeps: the waiting column blocks'
+// shared memory is the row sweep's L1 (4096 x 4096 FP64 1.55 -> 1.96 ms).
+template <typename... P, typename... A>
+inline void launch_next(void (*k)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+
 __device__ __forceinline__ bool gate_shut(const Grid& g) { return g.gate != nullptr && __ldcg(g.gate) == 0; }
 
 // Small device-resident control block.

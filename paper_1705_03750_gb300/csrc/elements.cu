@@ -220,10 +220,12 @@ __device__ __forceinline__ void drift_body(const Grid& g, double* __restrict__ e
 }
 
 __global__ void k_drift(Grid g, double* __restrict__ el, TaylorOut O, int taylor) {
+  if (!after_prior()) return;
   drift_body(g, el, O, taylor, blockIdx.x);
 }
 
 __global__ void k_taylor(Grid g, const double* __restrict__ el, TaylorOut O) {
+  if (!after_prior()) return;
   if (gate_shut(g)) return;
   int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= g.ne) return;
@@ -290,6 +292,7 @@ __device__ __forceinline__ void kick_body(const Grid& g, double* __restrict__ el
 __global__ void k_kick_drift(Grid g, double* __restrict__ el, const double* __restrict__ a,
                              const double* __restrict__ da, const double* __restrict__ d2a,
                              const DevState* __restrict__ ds) {
+  if (!after_prior()) return;
   kick_body(g, el, a, da, d2a, ds, blockIdx.x);
 }
 
@@ -311,6 +314,7 @@ __device__ __forceinline__ void reset_body(const Grid& g, double* __restrict__ e
 }
 
 __global__ void k_reset(Grid g, double* __restrict__ el, DevState* ds) {
+  if (!after_prior()) return;
   if (gate_shut(g)) return;
   reset_body(g, el, ds, blockIdx.x);
 }
@@ -478,6 +482,7 @@ __device__ __forceinline__ void scan_body(const Grid& g, const double* __restric
 
 __global__ void __launch_bounds__(SCAN_T) k_scan_force(Grid g, const double* __restrict__ M,
                                                        double* __restrict__ a, DevState* ds) {
+  if (!after_prior()) return;
   scan_body(g, M, a, ds);
 }
 
@@ -499,6 +504,7 @@ __device__ __forceinline__ void diff_body(const Grid& g, const double* __restric
 
 __global__ void k_force_diff(Grid g, const double* __restrict__ a, double* __restrict__ da,
                              double* __restrict__ d2a, const DevState* __restrict__ ds) {
+  if (!after_prior()) return;
   diff_body(g, a, da, d2a, ds, blockIdx.x);
 }
 
@@ -775,22 +781,22 @@ inline int elem_threads(int ne) { return ne <= 152 * 2 * ET ? 32 : ET; }
 }  // namespace
 
 void launch_drift(vm_solver* s, bool taylor) {
-  { const int ps_ = prof_begin(s, KID_DRIFT); k_drift<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el, taylor_out(*s), taylor ? 1 : 0); prof_end(s, ps_); }
+  { const int ps_ = prof_begin(s, KID_DRIFT); launch_next(k_drift, blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream, s->g, s->el, taylor_out(*s), taylor ? 1 : 0); prof_end(s, ps_); }
   s->launches++;
 }
 
 void launch_taylor(vm_solver* s) {
-  { const int ps_ = prof_begin(s, KID_TAYLOR); k_taylor<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el, taylor_out(*s)); prof_end(s, ps_); }
+  { const int ps_ = prof_begin(s, KID_TAYLOR); launch_next(k_taylor, blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream, s->g, s->el, taylor_out(*s)); prof_end(s, ps_); }
   s->launches++;
 }
 
 void launch_kick_drift(vm_solver* s) {
-  { const int ps_ = prof_begin(s, KID_KICK_DRIFT); k_kick_drift<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el, s->a, s->da, s->d2a, s->ds); prof_end(s, ps_); }
+  { const int ps_ = prof_begin(s, KID_KICK_DRIFT); launch_next(k_kick_drift, blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream, s->g, s->el, s->a, s->da, s->d2a, s->ds); prof_end(s, ps_); }
   s->launches++;
 }
 
 void launch_reset_elements(vm_solver* s) {
-  { const int ps_ = prof_begin(s, KID_RESET); k_reset<<<blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream>>>(s->g, s->el, s->ds); prof_end(s, ps_); }
+  { const int ps_ = prof_begin(s, KID_RESET); launch_next(k_reset, blocks_for(s->g.ne, elem_threads(s->g.ne)), elem_threads(s->g.ne), 0, s->stream, s->g, s->el, s->ds); prof_end(s, ps_); }
   s->launches++;
 }
 
@@ -836,8 +842,8 @@ void launch_scan_force(vm_solver* s) {
 // allocation-free entry point.
 void launch_scan_force_raw(const Grid& g, const double* M, double* a, double* da, double* d2a, DevState* ds,
                            cudaStream_t stream) {
-  k_scan_force<<<1, SCAN_T, 0, stream>>>(g, M, a, ds);
-  k_force_diff<<<blocks_for(g.nx, 128), 128, 0, stream>>>(g, a, da, d2a, ds);
+  launch_next(k_scan_force, 1, SCAN_T, 0, stream, g, M, a, ds);
+  launch_next(k_force_diff, blocks_for(g.nx, 128), 128, 0, stream, g, a, da, d2a, ds);
 }
 
 void launch_fth_box(vm_solver* s) {

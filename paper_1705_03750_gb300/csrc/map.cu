@@ -986,6 +986,7 @@ __device__ __forceinline__ void map_sites_body(const Grid& g, const SiteArgs& X,
 }
 
 __global__ void __launch_bounds__(SITE_T, SITE_BPS) k_map_sites(Grid g, SiteArgs X) {
+  if (!after_prior()) return;
   if (gate_shut(g) || __ldcg(&X.ds->skip_sites)) return;
   map_sites_body(g, X, blockIdx.x);
 }
@@ -1781,6 +1782,7 @@ __global__ void __launch_bounds__(32 * TP, 8) k_claim_pair(Grid g, const double*
                                                          const float* __restrict__ tayf, Slots Sin, float alo,
                                                          float ahi, int all, int32_t* __restrict__ esc_list,
                                                          int2* __restrict__ ovf_list) {
+  if (!after_prior()) return;
   if (gate_shut(g)) return;
   claim_pair_body(g, tay, tayf, Sin, alo, ahi, all, esc_list, ovf_list, blockIdx.x, gridDim.x);
 }
@@ -2597,6 +2599,7 @@ __device__ __forceinline__ void emap_test_body(const Grid& g, const uint32_t* __
 
 __global__ void k_emap_test(Grid g, const uint32_t* __restrict__ slot0, const double* __restrict__ tay,
                             const float* __restrict__ tayf, DevState* ds, double thr, int n_s, float alo, float ahi) {
+  if (!after_prior()) return;
   emap_test_body(g, slot0, tay, tayf, ds, thr, n_s, alo, ahi, blockIdx.x, gridDim.x);
 }
 
@@ -2616,6 +2619,7 @@ __device__ __forceinline__ void remap_decide(DevState* ds, int n_s, double thr) 
 }
 
 __global__ void k_remap_gate(DevState* ds, int n_s, double thr) {
+  if (!after_prior()) return;
   if (threadIdx.x == 0 && blockIdx.x == 0) remap_decide(ds, n_s, thr);
 }
 
@@ -2692,6 +2696,7 @@ __device__ __forceinline__ bool grid_barrier(DevState* ds, unsigned& round) {
 }
 
 __global__ void __launch_bounds__(BT, BLOCKS_PER_SM) k_flood(Grid g, FloodArgs A) {
+  if (!after_prior()) return;
   if (gate_shut(g)) return;
   DevState* ds = A.S.ds;
   const bool any = __ldcg(&ds->n_flood) != 0;
@@ -2914,9 +2919,9 @@ void launch_remap_gate(vm_solver* s) {
   alpha_bounds(s->g.alpha, alo, ahi);
   unsigned nb = (unsigned)((s->n + 255) / 256);
   if (nb > 152 * 8) nb = 152 * 8;
-  k_emap_test<<<nb, 256, 0, s->stream>>>(s->g, s->map, s->tay, s->tayf, s->ds, s->cfg.emap_remap, s->cfg.n_s, alo,
-                                         ahi);
-  k_remap_gate<<<1, 32, 0, s->stream>>>(s->ds, s->cfg.n_s, s->cfg.emap_remap);
+  launch_next(k_emap_test, nb, 256, 0, s->stream, s->g, s->map, s->tay, s->tayf, s->ds, s->cfg.emap_remap, s->cfg.n_s,
+              alo, ahi);
+  launch_next(k_remap_gate, 1, 32, 0, s->stream, s->ds, s->cfg.n_s, s->cfg.emap_remap);
   prof_end(s, ps);
   s->launches++;
 }
@@ -2997,16 +3002,16 @@ void launch_map(vm_solver* s) {
   const int all = s->cfg.map_windows != 0 || !site_pass_on(s->g);
   if (!all) {
     ps = prof_begin(s, KID_MAP_SITES);
-    k_map_sites<<<(unsigned)site_tiles(s->g), SITE_T, 0, s->stream>>>(
-        s->g, SiteArgs{s->tay, s->tayf, s->tayl, s->map, s->flags, s->ds, alo, ahi});
+    launch_next(k_map_sites, (unsigned)site_tiles(s->g), SITE_T, 0, s->stream, s->g, SiteArgs{s->tay, s->tayf,
+                s->tayl, s->map, s->flags, s->ds, alo, ahi});
     prof_end(s, ps);
   }
   // tier 0 (two elements per warp), its escapes to tier 1 through the first
   // hole list (free until the holes are looked for)
   ps = prof_begin(s, KID_CLAIM_PAIR);
   const unsigned t0 = (unsigned)std::min<long long>(152 * 16, pair_units(s->g));
-  k_claim_pair<<<t0, 32 * TP, 0, s->stream>>>(s->g, s->tay, s->tayf, S, alo, ahi, all, s->holes_a,
-                                              s->overflow_list);
+  launch_next(k_claim_pair, t0, 32 * TP, 0, s->stream, s->g, s->tay, s->tayf, S, alo, ahi, all, s->holes_a,
+              s->overflow_list);
   prof_end(s, ps);
   // the rest of the flood fill; the elements that can escape tier 1 are few on
   // a small lattice, and an idle block still takes a whole SM

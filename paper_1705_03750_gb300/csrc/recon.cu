@@ -186,6 +186,7 @@ __global__ void __launch_bounds__(256) k_recon64(Grid g, const uint32_t* __restr
                                                  const double* __restrict__ tay, const FxRec* __restrict__ tayx,
                                                  const double* __restrict__ fini, double* __restrict__ f,
                                                  double* __restrict__ M) {
+  if (!after_prior()) return;
   k_recon64_body(g, map, ds, tay, tayx, fini, f, M, blockIdx.x);
 }
 
@@ -474,6 +475,7 @@ __device__ __forceinline__ void k_remap64_body(const Grid& g, const uint32_t* __
 __global__ void __launch_bounds__(256) k_remap64(Grid g, const uint32_t* __restrict__ map, const DevState* ds,
                                                  const double* __restrict__ tay, const FxRec* __restrict__ tayx,
                                                  const double* __restrict__ eta, double* __restrict__ out) {
+  if (!after_prior()) return;
   if (gate_shut(g)) return;
   k_remap64_body(g, map, ds, tay, tayx, eta, out, blockIdx.x);
 }
@@ -763,6 +765,7 @@ __global__ void __launch_bounds__(256, 6) k_recon32(Grid g, const uint32_t* __re
                                                  const double* __restrict__ tay, const float* __restrict__ tayf,
                                                  const float* __restrict__ fini, float* __restrict__ f,
                                                  double* __restrict__ M) {
+  if (!after_prior()) return;
   k_recon32_body(g, map, ds, tay, tayf, fini, f, M, blockIdx.x);
 }
 
@@ -1144,6 +1147,7 @@ __global__ void __launch_bounds__(256) k_remap32(Grid g, const uint32_t* __restr
                                                  const double* __restrict__ tay, const float* __restrict__ tayf,
                                                  const float* __restrict__ eta, float* __restrict__ out, float blo,
                                                  float bhi) {
+  if (!after_prior()) return;
   if (gate_shut(g)) return;
   k_remap32_body(g, map, ds, tay, tayf, eta, out, blo, bhi, blockIdx.x);
 }
@@ -1208,6 +1212,7 @@ __global__ void __launch_bounds__(256) k_copy_group(const SolveDesc* __restrict_
 // on the device may skip; element by element, any site count).
 template <typename R>
 __global__ void __launch_bounds__(256) k_copy_gated(Grid g, const R* __restrict__ src, R* __restrict__ dst) {
+  if (!after_prior()) return;
   if (gate_shut(g)) return;
   const size_t n = (size_t)g.nx * g.nv;
   for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < n; p += (size_t)gridDim.x * blockDim.x)
@@ -1255,9 +1260,9 @@ void group_remap_resample(const GroupPlan& G) {
 void launch_copy_gated(vm_solver* s) {
   const unsigned nb = grid_for(s->n);
   if (s->fp32)
-    k_copy_gated<float><<<nb, 256, 0, s->stream>>>(s->g, (const float*)s->tmp, (float*)s->fini);
+    launch_next(k_copy_gated<float>, nb, 256, 0, s->stream, s->g, (const float*)s->tmp, (float*)s->fini);
   else
-    k_copy_gated<double><<<nb, 256, 0, s->stream>>>(s->g, (const double*)s->tmp, (double*)s->fini);
+    launch_next(k_copy_gated<double>, nb, 256, 0, s->stream, s->g, (const double*)s->tmp, (double*)s->fini);
   s->launches++;
 }
 
@@ -1296,11 +1301,11 @@ void launch_reconstruct(vm_solver* s) {
     k_row_mass<<<(s->g.nx + 127) / 128, 128, 0, s->stream>>>(s->g, s->Mpart, s->M);
     s->launches++;
   } else if (s->fp32)
-    k_recon32<<<s->g.nx, nt, 0, s->stream>>>(s->g, s->map, s->ds, s->tay, s->tayf, (const float*)s->fini,
-                                              (float*)s->f, s->M);
+    launch_next(k_recon32, s->g.nx, nt, 0, s->stream, s->g, s->map, s->ds, s->tay, s->tayf, (const float*)s->fini,
+                (float*)s->f, s->M);
   else
-    k_recon64<<<s->g.nx, nt, 0, s->stream>>>(s->g, s->map, s->ds, s->tay, s->tayx, (const double*)s->fini,
-                                              (double*)s->f, s->M);
+    launch_next(k_recon64, s->g.nx, nt, 0, s->stream, s->g, s->map, s->ds, s->tay, s->tayx, (const double*)s->fini,
+                (double*)s->f, s->M);
   prof_end(s, ps_);
   s->launches++;
 }
@@ -1312,11 +1317,11 @@ void launch_remap_resample(vm_solver* s, void* out) {
     const float fb = (float)s->g.beta;
     const float blo = ((double)fb <= s->g.beta) ? fb : nextafterf(fb, -INFINITY);
     const float bhi = ((double)fb >= s->g.beta) ? fb : nextafterf(fb, INFINITY);
-    k_remap32<<<s->g.nx, nt, 0, s->stream>>>(s->g, s->map, s->ds, s->tay, s->tayf, (const float*)s->eta,
-                                              (float*)out, blo, bhi);
+    launch_next(k_remap32, s->g.nx, nt, 0, s->stream, s->g, s->map, s->ds, s->tay, s->tayf, (const float*)s->eta,
+                (float*)out, blo, bhi);
   } else {
-    k_remap64<<<s->g.nx, nt, 0, s->stream>>>(s->g, s->map, s->ds, s->tay, s->tayx, (const double*)s->eta,
-                                              (double*)out);
+    launch_next(k_remap64, s->g.nx, nt, 0, s->stream, s->g, s->map, s->ds, s->tay, s->tayx, (const double*)s->eta,
+                (double*)out);
   }
   prof_end(s, ps_);
   s->launches++;
