@@ -42,6 +42,7 @@
 // element trajectories agree to rounding.
 
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
@@ -84,6 +85,8 @@ struct Dev4 {
   int32_t nholes;
   int32_t bad_where;
   int32_t novf;  // elements whose component left the shared-memory window (this map)
+  int32_t nflood;  // elements left to the flood fill (this map)
+  int32_t wide;  // other elements whose component reaches beyond the window (this map)
   int32_t rounds;  // hole-repair rounds of the last map
   unsigned long long d2_evals;  // distance evaluations of the percolation kernels (cumulative)
 };
@@ -270,6 +273,8 @@ __device__ void inverse4(const double* A, double* B) {
 // K_a = (1/2) sum_l |T^-1_al| max_bc |G_l,bc| dm_b dm_c / dm_a (bounds the
 // absolute terms of that FP64 evaluation), nA_a = sum_b |A_ab|,
 // nB_a = sum_bc |B_a,bc|.  Layout: A[16], B[40], K[4], nA[4], nB[4], pad.
+// FP32 record of an element's inverse map in element units: A (16), B (4 x 10),
+// K (4), the row norms of A and B (4 + 4), the start site's offset from P_m (4)
 constexpr int NF4 = 72;
 
 __global__ void __launch_bounds__(128) k4_taylor(G4 g, const double* __restrict__ el, double* __restrict__ tay) {
@@ -320,7 +325,8 @@ constexpr long long FX4_MARGIN = 1ll << (FX4_Q - 26);
 // values (fixed point), four threads per element, one per axis of Q: the
 // second-order coefficients sum_l T^-1_al G_l,bc serve both.
 __global__ void __launch_bounds__(128) k4_records(G4 g, const double* __restrict__ tay, float* __restrict__ tay32,
-                                                  Fx4* __restrict__ tayx) {
+                                                  Fx4* __restrict__ tayx, int* __restrict__ start,
+                                                  uint32_t* __restrict__ flags) {
   const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const int m = (int)(tid >> 2), a = (int)(tid & 3);
   const unsigned quad = 0xFu << (threadIdx.x & 28);  // this element's lanes
@@ -368,7 +374,6 @@ __global__ void __launch_bounds__(128) k4_records(G4 g, const double* __restrict
   nb *= 1.000001f;
   r[60 + a] = na;
   r[64 + a] = nb;
-  r[68 + a] = 0.f;
   // the largest offset up to which the terms on every axis together stay
   // below FX4_MAX cells (the FP64 evaluation's uncombined ones, bounded by
   // 16 K p^2, below 10^5: its error then stays far inside FX4_MARGIN)
@@ -387,9 +392,12 @@ __global__ void __launch_bounds__(128) k4_records(G4 g, const double* __restrict
     if (lim == 0 && 0.51f + sf * (n1 * p + n2 * (p * p)) < (float)FX4_MAX && sf * n3 * (p * p) < 6e3f) lim = Lm;
   }
   // start site along this axis and its distance from P_m
-  const double u = (t[a] - g.lo[a]) * g.inv_d[a];
+  const double u = M_(S_(t[a], g.lo[a]), g.inv_d[a]);
   const bool near = u > -1e6 && u < 1e6;
-  const double i0 = near ? floor(u + 0.5) : 0.0;
+  const double i0 = near ? floor(A_(u, 0.5)) : 0.0;
+  start[4 * m + a] = near ? (int)i0 : INT_MIN / 2;
+  r[68 + a] = near ? (float)((site_coord(g, a, (long long)i0) - t[a]) * g.inv_dm[a]) : 0.f;
+  if (a == 0) flags[m] = 0u;
   if (__any_sync(quad, !near || !fin)) lim = 0;
   const long long de = near ? vm::fx_of(vm::cells_from(t[a], g.lo[a], g.d[a], g.inv_d[a], i0), 62) : 0;
   long long E[4];
@@ -539,6 +547,421 @@ __device__ __forceinline__ void claim4(ulonglong2* key, unsigned long long dbits
   }
 }
 
+// ---- the site pass: owners proposed and proved site by site ----
+//
+// The 2D path's certificate (map.cu) in four dimensions.  Every site p of the
+// padded lattice takes the element O(p) that is closest among those its test
+// would compare; R(m) is the set of sites with O = m.  If m's test passes on
+// R(m), fails at every site next to R(m), R(m) holds m's start site, and every
+// other site of R(m) has a neighbour in R(m) one step nearer to the start along
+// one axis, then R(m) is m's component and its sites need no claims.  The tests
+// are FP32 with bounds only: an element with a site that they do not settle is
+// left to the flood fill, and the sites proposed for it count as unclaimed.
+//
+// k4_site_hints prepares each tile's guess, k4_sites proposes the owners and
+// tests them, k4_sites_check looks at each site's eight neighbours.  A site
+// costs about one evaluation of its own, 0.7 of neighbours beyond the alpha box
+// and 2 of owners next to it, where the flood fill tested three sites for each
+// of a component's and formed its shell: 64^4 sites 1.3 + 1.7 ms and 0.4 ms for
+// the elements left to the fill, where the fill of all took 8.8 ms.  Bound by
+// the records' reads (288 bytes an evaluation through L1) and by occupancy: with
+// whole records held in registers (2 blocks an SM) and the guess formed inside
+// each tile the two kernels took 4.8 ms.
+constexpr uint32_t EF4_BAD = 1u, EF4_START = 2u, EF4_WIDE = 4u;
+
+struct Sites4 {
+  const int* start;     // 4 per element: start site (INT_MIN/2 where not finite)
+  uint32_t* flags;      // per element: EF4_*
+  uint32_t* cand;       // per site of the padded lattice: O(p)'s lattice position, a byte per axis
+  float* up;            // per site: an upper bound of O(p)'s d^2, negative if its test is not settled
+  int32_t* list;        // elements for the flood fill; NULL: no site pass, all of them
+  float* hints;         // 20 per tile: lattice position at its middle site, change per site
+};
+
+// Lattices whose positions fit the owners' words (others are flooded).
+bool sites_fit(const G4& g) { return g.L[0] < 256 && g.L[1] < 256 && g.L[2] < 256 && g.L[3] < 256; }
+
+__device__ __forceinline__ int elem_of(const G4& g, uint32_t w) {
+  return ((int)((w >> 24) * g.L[1] + ((w >> 16) & 255u)) * g.L[2] + (int)((w >> 8) & 255u)) * g.L[3] + (int)(w & 255u);
+}
+
+__device__ __forceinline__ bool starts_inside(const G4& g, const int4 s) {
+  return s.x >= -g.pad && s.x < g.n[0] + g.pad && s.y >= -g.pad && s.y < g.n[1] + g.pad && s.z >= -g.pad &&
+         s.z < g.n[2] + g.pad && s.w >= -g.pad && s.w < g.n[3] + g.pad;
+}
+
+// The settled element that owns grid site gs, or -1.
+__device__ __forceinline__ int settled_owner(const G4& g, const Sites4& S, const long long* gs) {
+  if (!S.list) return -1;
+  long long pi = 0;
+  for (int a = 0; a < 4; a++) pi = pi * (g.n[a] + 2 * g.pad) + (gs[a] + g.pad);
+  const int m = elem_of(g, S.cand[pi]);
+  if ((S.flags[m] & (EF4_BAD | EF4_START)) != EF4_START) return -1;
+  return m;  // (an element that starts off the padded lattice has no start flag)
+}
+
+// Offsets of element m at a site, their bounds, d^2 and its bound (eval32_4's
+// operations, the record's rows used as they are read).
+__device__ __forceinline__ float site_eval(const G4& g, const float* __restrict__ tay32, const int4 st, int m,
+                                           const int (&c)[4], const float (&h)[4], float (&x)[4], float (&e)[4],
+                                           float* bd) {
+  const float* R = tay32 + (size_t)NF4 * m;
+  const float4* R4 = reinterpret_cast<const float4*>(R);
+  const float2* R2 = reinterpret_cast<const float2*>(R);
+  const float4 ro = __ldg(R4 + 17), nA4 = __ldg(R4 + 15), nB4 = __ldg(R4 + 16), K4 = __ldg(R4 + 14);
+  const float r[4] = {ro.x, ro.y, ro.z, ro.w}, nA[4] = {nA4.x, nA4.y, nA4.z, nA4.w},
+              nB[4] = {nB4.x, nB4.y, nB4.z, nB4.w}, K[4] = {K4.x, K4.y, K4.z, K4.w};
+  const float jh[4] = {(float)(c[0] - st.x) * h[0], (float)(c[1] - st.y) * h[1], (float)(c[2] - st.z) * h[2],
+                       (float)(c[3] - st.w) * h[3]};
+  float p[4], dp[4];
+  p_of(jh, r, p, dp);
+  const float pm = fmaxf(fmaxf(fabsf(p[0]), fabsf(p[1])), fmaxf(fabsf(p[2]), fabsf(p[3])));
+  const float dm = fmaxf(fmaxf(dp[0], dp[1]), fmaxf(dp[2], dp[3]));
+  const float dpp = fmaf(2.f * pm, dm, dm * dm), S = 4.f * pm;
+  const float p00 = p[0] * p[0], p01 = p[0] * p[1], p02 = p[0] * p[2], p03 = p[0] * p[3], p11 = p[1] * p[1],
+              p12 = p[1] * p[2], p13 = p[1] * p[3], p22 = p[2] * p[2], p23 = p[2] * p[3], p33 = p[3] * p[3];
+#pragma unroll
+  for (int a = 0; a < 4; a++) {
+    const float4 A = __ldg(R4 + a);
+    const float2 b0 = __ldg(R2 + 8 + 5 * a), b1 = __ldg(R2 + 9 + 5 * a), b2 = __ldg(R2 + 10 + 5 * a),
+                 b3 = __ldg(R2 + 11 + 5 * a), b4 = __ldg(R2 + 12 + 5 * a);
+    float v = A.x * p[0];
+    v = fmaf(A.y, p[1], v);
+    v = fmaf(A.z, p[2], v);
+    v = fmaf(A.w, p[3], v);
+    v = fmaf(b0.x, p00, v);
+    v = fmaf(b0.y, p01, v);
+    v = fmaf(b1.x, p02, v);
+    v = fmaf(b1.y, p03, v);
+    v = fmaf(b2.x, p11, v);
+    v = fmaf(b2.y, p12, v);
+    v = fmaf(b3.x, p13, v);
+    v = fmaf(b3.y, p22, v);
+    v = fmaf(b4.x, p23, v);
+    x[a] = fmaf(b4.y, p33, v);
+    const float E = fmaf(nB[a], pm * pm, nA[a] * pm), Ep = fmaf(nB[a], dpp, nA[a] * dm);
+    e[a] = kRel4 * E + kAbs4 * (1.f + E) + 1.00001f * Ep + 1e-13f * K[a] * (S * S) * 16.f;
+  }
+  return d2_32(x, e, bd);
+}
+
+constexpr int T4_0 = 2, T4_1 = 4, T4_2 = 4, T4_3 = 8;  // tile of sites, one per thread
+constexpr int T4 = T4_0 * T4_1 * T4_2 * T4_3;
+constexpr int P4CAP = 1536;  // listed pairs of a tile
+
+// The thread's site (grid coordinates), whether it lies on the padded lattice,
+// and its index there.
+__device__ __forceinline__ bool tile_site(const G4& g, int b, int t, int (&c)[4], long long& pi) {
+  const int pw1 = g.n[1] + 2 * g.pad, pw2 = g.n[2] + 2 * g.pad, pw3 = g.n[3] + 2 * g.pad;
+  const int nt3 = (pw3 + T4_3 - 1) / T4_3, nt2 = (pw2 + T4_2 - 1) / T4_2, nt1 = (pw1 + T4_1 - 1) / T4_1;
+  const int b3 = b % nt3;
+  b /= nt3;
+  const int b2 = b % nt2;
+  b /= nt2;
+  const int b1 = b % nt1, b0 = b / nt1;
+  c[3] = b3 * T4_3 + t % T4_3;
+  c[2] = b2 * T4_2 + t / T4_3 % T4_2;
+  c[1] = b1 * T4_1 + t / (T4_3 * T4_2) % T4_1;
+  c[0] = b0 * T4_0 + t / (T4_3 * T4_2 * T4_1);
+  const bool on = c[0] < g.n[0] + 2 * g.pad && c[1] < pw1 && c[2] < pw2 && c[3] < pw3;
+  pi = (((long long)c[0] * pw1 + c[1]) * pw2 + c[2]) * pw3 + c[3];
+  for (int a = 0; a < 4; a++) c[a] -= g.pad;
+  return on;
+}
+
+// Tiles of the padded lattice.
+size_t site_tiles4(const G4& g) {
+  const int T[4] = {T4_0, T4_1, T4_2, T4_3};
+  size_t n = 1;
+  for (int a = 0; a < 4; a++) n *= (size_t)(g.n[a] + 2 * g.pad + T[a] - 1) / T[a];
+  return n;
+}
+
+__device__ __forceinline__ int nearest_elem(float k, int L) { return min(max(__float2int_rn(k), 0), L - 1); }
+
+// Per tile: the lattice position of Q at its middle site, by Newton steps from
+// element to element starting from the undeformed lattice, and its change per
+// site.  One thread per tile: in the tile's own block the others would wait.
+__global__ void __launch_bounds__(128) k4_site_hints(G4 g, const float* __restrict__ tay32, Sites4 S, int tiles) {
+  const int tile = blockIdx.x * 128 + threadIdx.x;
+  if (tile >= tiles) return;
+  const int4* start = reinterpret_cast<const int4*>(S.start);
+  const float h[4] = {(float)(g.d[0] * g.inv_dm[0]), (float)(g.d[1] * g.inv_dm[1]), (float)(g.d[2] * g.inv_dm[2]),
+                      (float)(g.d[3] * g.inv_dm[3])};
+  const float inv_s = 1.f / (float)g.s;
+  int c[4], k[4], m = 0;
+  long long pi;
+  tile_site(g, tile, 0, c, pi);
+  const int T[4] = {T4_0, T4_1, T4_2, T4_3};
+  for (int a = 0; a < 4; a++) {
+    c[a] += T[a] / 2;
+    k[a] = nearest_elem(((float)c[a] - 0.5f * (float)(g.n[a] - 1)) * inv_s + (float)(g.K[a] + 1), g.L[a]);
+  }
+  float x[4], e[4], bd;
+  int k0[4];
+  for (int it = 0; it < 6; it++) {
+    m = ((k[0] * g.L[1] + k[1]) * g.L[2] + k[2]) * g.L[3] + k[3];
+    site_eval(g, tay32, __ldg(start + m), m, c, h, x, e, &bd);
+    bool same = true;
+    for (int a = 0; a < 4; a++) {
+      k0[a] = k[a];
+      k[a] = nearest_elem((float)k[a] + x[a], g.L[a]);
+      same = same && k[a] == k0[a];
+    }
+    if (same) break;
+  }
+  const int4 st = __ldg(start + m);
+  const float* R = tay32 + (size_t)NF4 * m;
+  const float p[4] = {(float)(c[0] - st.x) * h[0] + R[68], (float)(c[1] - st.y) * h[1] + R[69],
+                      (float)(c[2] - st.z) * h[2] + R[70], (float)(c[3] - st.w) * h[3] + R[71]};
+  float* o = S.hints + 20 * (size_t)tile;
+  for (int a = 0; a < 4; a++) {
+    o[a] = (float)k0[a] + x[a];
+    for (int b = 0; b < 4; b++) {
+      float v = R[4 * a + b];
+      for (int q = 0; q < 4; q++) v = fmaf(R[16 + 10 * a + sym4(b, q)] * (b == q ? 2.f : 1.f), p[q], v);
+      o[4 + 4 * a + b] = v * h[b];
+    }
+  }
+}
+
+__global__ void __launch_bounds__(T4, 3) k4_sites(G4 g, const float* __restrict__ tay32, Sites4 S, float alpha) {
+  __shared__ int sh_k[T4][4];  // the sites' proposed owners
+  __shared__ float sh_d[T4], sh_b[T4];
+  __shared__ unsigned long long sh_best[T4];  // closest neighbour that is certainly closer (d^2 bits, offset code)
+  __shared__ unsigned char sh_open[T4];
+  __shared__ unsigned short pairs[P4CAP];  // site of the tile | offset code << 8
+  __shared__ int npairs;
+  const int4* start = reinterpret_cast<const int4*>(S.start);
+  const int tid = threadIdx.x;
+  int c[4];
+  long long pi;
+  const bool on = tile_site(g, blockIdx.x, tid, c, pi);
+  const float h[4] = {(float)(g.d[0] * g.inv_dm[0]), (float)(g.d[1] * g.inv_dm[1]), (float)(g.d[2] * g.inv_dm[2]),
+                      (float)(g.d[3] * g.inv_dm[3])};
+  const float aerr = 1e-7f * (1.f + alpha);
+  float x[4], e[4], bd;
+  int k[4];
+  {
+    const float4* H = reinterpret_cast<const float4*>(S.hints + 20 * (size_t)blockIdx.x);
+    const float4 x0 = __ldg(H);
+    const float xc[4] = {x0.x, x0.y, x0.z, x0.w};
+    // offsets from the tile's middle site
+    const float j3 = (float)(tid % T4_3 - T4_3 / 2), j2 = (float)(tid / T4_3 % T4_2 - T4_2 / 2),
+                j1 = (float)(tid / (T4_3 * T4_2) % T4_1 - T4_1 / 2), j0 = (float)(tid / (T4_3 * T4_2 * T4_1) - T4_0 / 2);
+#pragma unroll
+    for (int a = 0; a < 4; a++) {
+      const float4 J = __ldg(H + 1 + a);
+      k[a] = nearest_elem(fmaf(J.x, j0, fmaf(J.y, j1, fmaf(J.z, j2, fmaf(J.w, j3, xc[a])))), g.L[a]);
+    }
+  }
+  bool todo = on, sure = false;
+  float d2 = 0.f;
+  int4 st = make_int4(0, 0, 0, 0);
+  int m = 0;
+  for (int round = 0; round < 4; round++) {
+    if (tid == 0) npairs = 0;
+    __syncthreads();
+    if (todo) {
+      m = ((k[0] * g.L[1] + k[1]) * g.L[2] + k[2]) * g.L[3] + k[3];
+      st = __ldg(start + m);
+      d2 = site_eval(g, tay32, st, m, c, h, x, e, &bd);
+      if (round == 0) {
+        // a guess from too far away: once more from the element it led to
+        bool off = false;
+        for (int a = 0; a < 4; a++) {
+          const int k2 = nearest_elem((float)k[a] + x[a], g.L[a]);
+          off = off || (k2 != k[a] && fabsf(x[a]) > 0.75f);
+        }
+        if (off) {
+          for (int a = 0; a < 4; a++) k[a] = nearest_elem((float)k[a] + x[a], g.L[a]);
+          m = ((k[0] * g.L[1] + k[1]) * g.L[2] + k[2]) * g.L[3] + k[3];
+          st = __ldg(start + m);
+          d2 = site_eval(g, tay32, st, m, c, h, x, e, &bd);
+        }
+      }
+      sure = d2 < 1e30f && bd < 1e30f;
+      // the ranges, widened where the bound does not settle them (a neighbour
+      // more to compare does no harm: the test then passes against all)
+      int side[4], cnt = 0, ns = 0;
+      for (int a = 0; a < 4; a++) {
+        const float E = e[a] + aerr;
+        const bool lo = !(x[a] - E > -alpha), hi = !(x[a] + E < alpha);
+        side[a] = lo ? -1 : (hi ? 1 : 0);
+        sure = sure && !(lo && hi);
+        ns += side[a] != 0;
+      }
+      sh_d[tid] = d2;
+      sh_b[tid] = bd;
+      sh_open[tid] = 0;
+      sh_best[tid] = ~0ull;
+      for (int a = 0; a < 4; a++) sh_k[tid][a] = k[a];
+      if (sure && ns) {
+        // the nonempty subsets of the sides, in the lattice
+        unsigned short codes[15];
+        for (int u = 1; u < 16; u++) {
+          bool ok = true;
+          int code = 0;
+          for (int a = 0; a < 4; a++) {
+            const bool in = u >> a & 1;
+            ok = ok && (!in || (side[a] != 0 && (unsigned)(k[a] + side[a]) < (unsigned)g.L[a]));
+            code = code * 3 + (in ? side[a] + 1 : 1);
+          }
+          if (ok) codes[cnt++] = (unsigned short)code;
+        }
+        if (cnt) {
+          const int at = atomicAdd(&npairs, cnt);
+          if (at + cnt <= P4CAP) {
+            for (int q = 0; q < cnt; q++) pairs[at + q] = (unsigned short)(tid | codes[q] << 8);
+          } else {
+            sure = false;
+            for (int q = at; q < min(at + cnt, P4CAP); q++) pairs[q] = (unsigned short)(tid | 40 << 8);
+          }
+        }
+      }
+    }
+    __syncthreads();
+    for (int j = tid; j < min(npairs, P4CAP); j += T4) {
+      const int t = pairs[j] & 255, code = pairs[j] >> 8;
+      if (code == 40) continue;
+      int cs[4];
+      long long ps;
+      tile_site(g, blockIdx.x, t, cs, ps);
+      const int o0 = code / 27 - 1, o1 = code / 9 % 3 - 1, o2 = code / 3 % 3 - 1, o3 = code % 3 - 1;
+      const int mm = (((sh_k[t][0] + o0) * g.L[1] + sh_k[t][1] + o1) * g.L[2] + sh_k[t][2] + o2) * g.L[3] + sh_k[t][3] + o3;
+      float xn[4], en[4], bn;
+      const float dn = site_eval(g, tay32, __ldg(start + mm), mm, cs, h, xn, en, &bn);
+      if (!(dn - bn > sh_d[t] + sh_b[t])) {
+        if (dn + bn < sh_d[t] - sh_b[t])
+          atomicMin(&sh_best[t], (unsigned long long)__float_as_uint(dn) << 8 | (unsigned)code);
+        else
+          sh_open[t] = 1;
+      }
+    }
+    __syncthreads();
+    bool again = false;
+    if (todo) {
+      todo = false;
+      if (sh_best[tid] != ~0ull) {
+        // a neighbour is closer: propose that one
+        const int code = (int)(sh_best[tid] & 255u);
+        k[0] += code / 27 - 1, k[1] += code / 9 % 3 - 1, k[2] += code / 3 % 3 - 1, k[3] += code % 3 - 1;
+        again = todo = round < 3;
+        sure = false;
+      } else if (sh_open[tid]) {
+        sure = false;
+      }
+    }
+    if (!__syncthreads_or(again)) break;
+  }
+  if (!on) return;
+  S.cand[pi] = (uint32_t)k[0] << 24 | (uint32_t)k[1] << 16 | (uint32_t)k[2] << 8 | (uint32_t)k[3];
+  S.up[pi] = sure ? d2 + bd : -1.f;
+  if (!sure) m = ((k[0] * g.L[1] + k[1]) * g.L[2] + k[2]) * g.L[3] + k[3];
+  if (!sure) {
+    if (!(__ldcg(S.flags + m) & EF4_BAD)) atomicOr(S.flags + m, EF4_BAD);
+    return;
+  }
+  const int j0 = c[0] - st.x, j1 = c[1] - st.y, j2 = c[2] - st.z, j3 = c[3] - st.w;
+  if ((j0 | j1 | j2 | j3) == 0) atomicOr(S.flags + m, EF4_START);
+  if (max(max(abs(j0), abs(j1)), max(abs(j2), abs(j3))) > g.R && !(__ldcg(S.flags + m) & EF4_WIDE))
+    atomicOr(S.flags + m, EF4_WIDE);
+}
+
+// Each site against its eight neighbours: one of its owner's nearer to the
+// start site, and the tests of other owners next to it, which must fail here.
+__global__ void __launch_bounds__(T4, 4) k4_sites_check(G4 g, const float* __restrict__ tay32, Sites4 S, float alpha) {
+  __shared__ uint32_t sh_w[T4];
+  __shared__ float sh_up[T4];
+  __shared__ unsigned short pairs[T4 * 8];  // site of the tile | direction << 8
+  __shared__ uint32_t nbr[T4 * 8];          // and the owner there
+  __shared__ int npairs;
+  const int4* start = reinterpret_cast<const int4*>(S.start);
+  const int tid = threadIdx.x;
+  int c[4];
+  long long pi;
+  const bool on = tile_site(g, blockIdx.x, tid, c, pi);
+  if (tid == 0) npairs = 0;
+  __syncthreads();
+  if (on) {
+    const uint32_t w = S.cand[pi];
+    const float up = S.up[pi];
+    sh_w[tid] = w;
+    sh_up[tid] = up;
+    const int m = elem_of(g, w);
+    const int4 st = __ldg(start + m);
+    const int j[4] = {c[0] - st.x, c[1] - st.y, c[2] - st.z, c[3] - st.w};
+    long long stride[4] = {0, 0, 0, 1};
+    for (int a = 2; a >= 0; a--) stride[a] = stride[a + 1] * (g.n[a + 1] + 2 * g.pad);
+    bool linked = (j[0] | j[1] | j[2] | j[3]) == 0;
+    unsigned other = 0;
+    uint32_t wn[8];
+#pragma unroll
+    for (int dir = 0; dir < 8; dir++) {
+      const int a = dir >> 1, sg = dir & 1 ? 1 : -1;
+      wn[dir] = w;
+      if ((unsigned)(c[a] + sg + g.pad) < (unsigned)(g.n[a] + 2 * g.pad)) {
+        wn[dir] = S.cand[pi + sg * stride[a]];
+        if (wn[dir] != w)
+          other |= 1u << dir;
+        else
+          linked = linked || (sg < 0 ? j[a] > 0 : j[a] < 0);
+      }
+    }
+    if (!linked && starts_inside(g, st) && !(__ldcg(S.flags + m) & EF4_BAD)) atomicOr(S.flags + m, EF4_BAD);
+    if (other) {
+      int at = atomicAdd(&npairs, __popc(other));
+#pragma unroll
+      for (int dir = 0; dir < 8; dir++)
+        if (other >> dir & 1u) {
+          pairs[at] = (unsigned short)tid;
+          nbr[at++] = wn[dir];
+        }
+    }
+  }
+  __syncthreads();
+  const float h[4] = {(float)(g.d[0] * g.inv_dm[0]), (float)(g.d[1] * g.inv_dm[1]), (float)(g.d[2] * g.inv_dm[2]),
+                      (float)(g.d[3] * g.inv_dm[3])};
+  const float aerr = 1e-7f * (1.f + alpha);
+  for (int q = tid; q < npairs; q += T4) {
+    const int t = pairs[q];
+    const uint32_t wn = nbr[q], w = sh_w[t];
+    const int n = elem_of(g, wn);
+    const int4 st = __ldg(start + n);
+    if (!starts_inside(g, st) || (__ldcg(S.flags + n) & EF4_BAD)) continue;  // claims nothing; flooded anyway
+    int cs[4];
+    long long ps;
+    tile_site(g, blockIdx.x, t, cs, ps);
+    float x[4], e[4], bd;
+    const float d2 = site_eval(g, tay32, st, n, cs, h, x, e, &bd);
+    const float up = sh_up[t];
+    bool fails = up >= 0.f && up < d2 - bd;
+#pragma unroll
+    for (int a = 0; a < 4; a++) {
+      const int b = 24 - 8 * a, da = (int)((w >> b) & 255u) - (int)((wn >> b) & 255u);
+      fails = fails && (da == 0 || ((da == 1 || da == -1) && (float)da * x[a] > alpha + e[a] + aerr));
+    }
+    if (!fails) atomicOr(S.flags + n, EF4_BAD);
+  }
+}
+
+// The elements that the site pass did not settle, for the flood fill.
+__global__ void __launch_bounds__(256) k4_flood_list(G4 g, Sites4 S, Dev4* ds) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t f = m < g.ne ? S.flags[m] : 0u;
+  const bool settled = (f & (EF4_BAD | EF4_START)) == EF4_START;
+  const bool left = m < g.ne && !settled && starts_inside(g, __ldg(reinterpret_cast<const int4*>(S.start) + m));
+  const unsigned bl = __ballot_sync(0xffffffffu, left), bw = __ballot_sync(0xffffffffu, settled && (f & EF4_WIDE));
+  const int lane = threadIdx.x & 31;
+  int at = 0;
+  if (lane == 0) {
+    if (bl) at = atomicAdd(&ds->nflood, __popc(bl));
+    if (bw) atomicAdd(&ds->wide, __popc(bw));
+  }
+  at = __shfl_sync(0xffffffffu, at, 0);
+  if (left) S.list[at + __popc(bl & ((1u << lane) - 1u))] = m;
+}
+
 // Claim of in-grid site p by element m (Sec. 2.3.1: smaller d, then smaller
 // index).  The site's slot takes m + 1 by an exchange; a first claimant needs
 // nothing more.  A claim that displaces an owner folds the exact FP64 keys of
@@ -548,8 +971,10 @@ __device__ __forceinline__ void claim4(ulonglong2* key, unsigned long long dbits
 // contested sites only.
 __device__ __forceinline__ void claim_site(const G4& g, uint32_t* __restrict__ slot, ulonglong2* __restrict__ key,
                                            long long p, int m, const double* tm, const double* __restrict__ tay,
-                                           const long long* gs, bool have_d2, double d2, unsigned& nev, Dev4* ds) {
-  const uint32_t old = atomicExch(slot + p, (uint32_t)m + 1u);
+                                           const long long* gs, bool have_d2, double d2, unsigned& nev, Dev4* ds,
+                                           const Sites4& S) {
+  uint32_t old = atomicExch(slot + p, (uint32_t)m + 1u);
+  if (old == 0u) old = (uint32_t)(settled_owner(g, S, gs) + 1);
   if (old == 0u) return;
   double P[4];
   for (int a = 0; a < 4; a++) P[a] = site_coord(g, a, gs[a]);
@@ -641,11 +1066,10 @@ __device__ __forceinline__ void decode_w(int lw, int /*W*/, int* l) {
 }
 __device__ __forceinline__ int pack_w(const int* l) { return l[0] | (l[1] << 8) | (l[2] << 16) | (l[3] << 24); }
 
-__global__ void __launch_bounds__(PERC_THREADS, 8) k4_percolate(G4 g, const double* __restrict__ el,
-                                                    const double* __restrict__ tay,
-                                                    const float* __restrict__ tay32, ulonglong2* __restrict__ key,
-                                                    uint32_t* __restrict__ slot, int32_t* __restrict__ ovf_list,
-                                                    Dev4* ds) {
+__device__ __forceinline__ void percolate_one(const G4& g, const double* __restrict__ el, const double* __restrict__ tay,
+                                              const float* __restrict__ tay32, ulonglong2* __restrict__ key,
+                                              uint32_t* __restrict__ slot, int32_t* __restrict__ ovf_list,
+                                              const Sites4& S, Dev4* ds, int m) {
   extern __shared__ uint32_t sm4[];
   const int W = g.W;
   const int nwin = W * W * W * W;
@@ -664,7 +1088,6 @@ __global__ void __launch_bounds__(PERC_THREADS, 8) k4_percolate(G4 g, const doub
   __shared__ double pst[4];      // the start site's coordinates
   __shared__ int org[4], kk[4];
   __shared__ int go, ncur, ntest, npairs, ovf;
-  const int m = blockIdx.x;
   const int tid = threadIdx.x;
   unsigned nev = 0;
   if (tid < NT4) tself[tid] = tay[(size_t)NT4 * m + tid];
@@ -866,7 +1289,7 @@ __global__ void __launch_bounds__(PERC_THREADS, 8) k4_percolate(G4 g, const doub
         in = in && gs[a] >= 0 && gs[a] < g.n[a];
         p += gs[a] * g.st[a];
       }
-      if (in) claim_site(g, slot, key, p, m, tself, tay, gs, st == ST_OPEN, d2, nev, ds);
+      if (in) claim_site(g, slot, key, p, m, tself, tay, gs, st == ST_OPEN, d2, nev, ds, S);
       const int idx = atomicAdd(&ncur, 1);
       if (idx < FCAP)
         front[idx] = tlist[i];
@@ -884,14 +1307,68 @@ __global__ void __launch_bounds__(PERC_THREADS, 8) k4_percolate(G4 g, const doub
   if ((tid & 31) == 0 && nev) atomicAdd(&ds->d2_evals, (unsigned long long)nev);
 }
 
+__global__ void __launch_bounds__(PERC_THREADS, 8) k4_percolate(G4 g, const double* __restrict__ el,
+                                                    const double* __restrict__ tay,
+                                                    const float* __restrict__ tay32, ulonglong2* __restrict__ key,
+                                                    uint32_t* __restrict__ slot, int32_t* __restrict__ ovf_list,
+                                                    Sites4 S, Dev4* ds) {
+  const int n = S.list ? ds->nflood : g.ne;
+  for (int q = blockIdx.x; q < n; q += gridDim.x) {
+    percolate_one(g, el, tay, tay32, key, slot, ovf_list, S, ds, S.list ? S.list[q] : q);
+    __syncthreads();
+  }
+}
+
+// The test of element m (lattice position k) at a site in FP32 with bounds: 1
+// passes, 0 fails, -1 left to the exact test.
+__device__ __forceinline__ int passes4_f32(const G4& g, const int* k, int m, const float* __restrict__ tay32,
+                                           const Sites4& S, const int (&c)[4], float alpha) {
+  const int4* start = reinterpret_cast<const int4*>(S.start);
+  const float h[4] = {(float)(g.d[0] * g.inv_dm[0]), (float)(g.d[1] * g.inv_dm[1]), (float)(g.d[2] * g.inv_dm[2]),
+                      (float)(g.d[3] * g.inv_dm[3])};
+  const float aerr = 1e-7f * (1.f + alpha);
+  float x[4], e[4], bd;
+  const float d2 = site_eval(g, tay32, __ldg(start + m), m, c, h, x, e, &bd);
+  int side[4];
+  for (int a = 0; a < 4; a++) {
+    const float E = e[a] + aerr;
+    if (x[a] + E < -alpha)
+      side[a] = -1;
+    else if (x[a] - E > -alpha && x[a] + E < alpha)
+      side[a] = 0;
+    else if (x[a] - E > alpha)
+      side[a] = 1;
+    else
+      return -1;
+  }
+  int res = 1;
+  for (int u = 1; u < 16; u++) {
+    bool ok = true;
+    int mm = 0;
+    for (int a = 0; a < 4; a++) {
+      const int o = u >> a & 1 ? side[a] : 0;
+      ok = ok && (!(u >> a & 1) || side[a] != 0) && (unsigned)(k[a] + o) < (unsigned)g.L[a];
+      mm = mm * g.L[a] + k[a] + o;
+    }
+    if (!ok) continue;
+    float bn;
+    const float dn = site_eval(g, tay32, __ldg(start + mm), mm, c, h, x, e, &bn);
+    if (dn + bn < d2 - bd) return 0;
+    if (!(dn - bn > d2 + bd)) res = -1;
+  }
+  return res;
+}
+
 // Whole-lattice flood fill of the listed elements: the same breadth-first
 // search over the padded lattice [-pad, n-1+pad]^4, with its visited bits and
-// frontiers in global memory (one slot per block).
+// frontiers in global memory (one slot per block), the tests in FP32 with
+// bounds first (27 ms of a 20 x 24 x 22 x 18 solve's 39 went into FP64 ones).
 __global__ void __launch_bounds__(256) k4_percolate_big(G4 g, const double* __restrict__ el,
-                                                        const double* __restrict__ tay, ulonglong2* __restrict__ key,
+                                                        const double* __restrict__ tay,
+                                                        const float* __restrict__ tay32, ulonglong2* __restrict__ key,
                                                         uint32_t* __restrict__ slot,
                                                         const int32_t* __restrict__ ovf_list, uint32_t* __restrict__ big,
-                                                        Dev4* ds) {
+                                                        Sites4 S, Dev4* ds) {
   __shared__ double tself[NT4];
   __shared__ int kk[4];
   __shared__ int go, ncur, nnext, bad_wave;
@@ -963,20 +1440,27 @@ __global__ void __launch_bounds__(256) k4_percolate_big(G4 g, const double* __re
         const long long np = ((gl[0] * pw[1] + gl[1]) * pw[2] + gl[2]) * pw[3] + gl[3];
         const uint32_t bit = 1u << (np & 31);
         if (atomicOr(&stamp[np >> 5], bit) & bit) continue;
-        double P[4], d2;
+        double d2 = 0.0;
         long long gs[4];
+        int ci[4];
         for (int a = 0; a < 4; a++) {
           gs[a] = gl[a] - g.pad;
-          P[a] = site_coord(g, a, gs[a]);
+          ci[a] = (int)gs[a];
         }
-        if (!passes4(g, kl, tself, tay, P, &d2, nev)) continue;
+        const int res = passes4_f32(g, kl, m, tay32, S, ci, (float)g.alpha);
+        if (res == 0) continue;
+        if (res < 0) {
+          double P[4];
+          for (int a = 0; a < 4; a++) P[a] = site_coord(g, a, gs[a]);
+          if (!passes4(g, kl, tself, tay, P, &d2, nev)) continue;
+        }
         bool in = true;
         long long p = 0;
         for (int a = 0; a < 4; a++) {
           in = in && gs[a] >= 0 && gs[a] < g.n[a];
           p += gs[a] * g.st[a];
         }
-        if (in) claim_site(g, slot, key, p, m, tself, tay, gs, true, d2, nev, ds);
+        if (in) claim_site(g, slot, key, p, m, tself, tay, gs, res < 0, d2, nev, ds, S);
         const int idx = atomicAdd(&nnext, 1);
         if (idx < BIG_FCAP)
           fn[idx] = (int32_t)np;
@@ -999,7 +1483,7 @@ __global__ void __launch_bounds__(256) k4_percolate_big(G4 g, const double* __re
 // owner of every site from its key (the key is emptied for the next map);
 // sites nobody claimed go to the hole list
 __global__ void k4_map_finish(G4 g, ulonglong2* __restrict__ key, uint32_t* __restrict__ slot,
-                              int32_t* __restrict__ map, int32_t* __restrict__ holes, Dev4* ds) {
+                              int32_t* __restrict__ map, int32_t* __restrict__ holes, Sites4 S, Dev4* ds) {
   const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= g.nsite) return;
   const ulonglong2 k = key[p];
@@ -1016,6 +1500,15 @@ __global__ void k4_map_finish(G4 g, ulonglong2* __restrict__ key, uint32_t* __re
       owner = (int)sl - 1;
     else
       bad(ds, 46);
+  } else if (S.list) {  // the site pass's
+    long long gs[4], r = p;
+    for (int a = 3; a > 0; a--) {
+      const long long u = (uint32_t)r / (uint32_t)g.n[a];
+      gs[a] = r - u * g.n[a];
+      r = u;
+    }
+    gs[0] = r;
+    owner = settled_owner(g, S, gs);
   }
   if (sl != 0u) slot[p] = 0u;
   map[p] = owner;
@@ -1824,10 +2317,11 @@ __global__ void k4_spline_axis(G4 g, int ax, const double* __restrict__ tab, dou
 
 namespace {
 enum K4Id { K_DRIFT, K_TAYLOR, K_PERC, K_PERC_BIG, K_FINISH, K_HOLES, K_RECON, K_ACCEL, K_ACCEL_SUM, K_KICK,
-            K_RESAMPLE, K_SPLINE, K_RESET, K_FIELDS, K_DIAG, K_RECORDS, K_COUNT };
+            K_RESAMPLE, K_SPLINE, K_RESET, K_FIELDS, K_DIAG, K_RECORDS, K_SITES,
+            K_SITES_CHECK, K_COUNT };
 const char* const k4_names[K_COUNT] = {"drift", "taylor", "percolate", "percolate_big", "map_finish", "holes",
                                        "reconstruct", "accel", "accel_sum", "kick_drift", "resample", "spline_axis",
-                                       "reset", "node_fields", "diagnostics", "records"};
+                                       "reset", "node_fields", "diagnostics", "records", "sites", "sites_check"};
 struct ProfRec {
   int id;
   cudaEvent_t a, b;
@@ -1846,6 +2340,7 @@ struct vm_4d_solver {
   ulonglong2* key;
   uint32_t* slot;
   int32_t *map, *holes, *cand, *ovf_list;
+  Sites4 sites;  // the site pass's arrays
   uint32_t* big;
   double2 *gext, *part;
   Dev4* ds;
@@ -1923,7 +2418,8 @@ int nchunks(const G4& g) {
 }
 
 struct Layout {
-  size_t diag, fini, eta, f, key, slot, map, holes, cand, el, tay, tay32, tayx, Mpix, fld, gext, part, tab, ovf, big, ds, total;
+  size_t diag, fini, eta, f, key, slot, map, holes, cand, el, tay, tay32, tayx, Mpix, fld, gext, part, tab, ovf, big, ds, start, flags,
+      site_cand, site_up, flood, hints, total;
 };
 
 Layout layout(const G4& g) {
@@ -1961,6 +2457,12 @@ Layout layout(const G4& g) {
   const size_t nwords = (size_t)((npad + 31) >> 5);
   L.big = take(4 * (size_t)BIG_SLOTS * (((nwords + 63) & ~(size_t)63) + 2 * (size_t)BIG_FCAP));
   L.ds = take(sizeof(Dev4));
+  L.start = take(16 * (size_t)g.ne);
+  L.flags = take(4 * (size_t)g.ne);
+  L.flood = take(4 * (size_t)g.ne);
+  L.site_cand = take(sites_fit(g) ? 4 * (size_t)npad : 0);
+  L.site_up = take(sites_fit(g) ? 4 * (size_t)npad : 0);
+  L.hints = take(sites_fit(g) ? 80 * site_tiles4(g) : 0);
   L.total = o;
   return L;
 }
@@ -2020,16 +2522,32 @@ void prof_end(vm_4d_solver* s, int id, cudaEvent_t a) {
 vm_status run_map(vm_4d_solver* s) {
   const G4& g = s->g;
   K4_LAUNCH(s, K_TAYLOR, k4_taylor<<<blocks(g.ne, 128), 128, 0, s->stream>>>(g, s->el, s->tay));
-  K4_LAUNCH(s, K_RECORDS, k4_records<<<blocks(4ll * g.ne, 128), 128, 0, s->stream>>>(g, s->tay, s->tay32, s->tayx));
+  K4_LAUNCH(s, K_RECORDS, k4_records<<<blocks(4ll * g.ne, 128), 128, 0, s->stream>>>(g, s->tay, s->tay32, s->tayx,
+                                                                                   (int*)s->sites.start, s->sites.flags));
   if (cudaMemsetAsync(&s->ds->nholes, 0, sizeof(int32_t), s->stream) != cudaSuccess ||
-      cudaMemsetAsync(&s->ds->novf, 0, sizeof(int32_t), s->stream) != cudaSuccess)
+      cudaMemsetAsync(&s->ds->novf, 0, 3 * sizeof(int32_t), s->stream) != cudaSuccess)
     return VM_E_CUDA;
-  K4_LAUNCH(s, K_PERC, k4_percolate<<<g.ne, PERC_THREADS, s->smem, s->stream>>>(g, s->el, s->tay, s->tay32, s->key, s->slot,
-                                                                      s->ovf_list, s->ds));
+  Sites4 S = s->sites;
+  // Where sites lie midway between elements along a velocity axis, a map whose
+  // elements have moved along x only since a reset ties at all of them.
+  const bool ties = s->cyc == 0 && ((g.n[2] - 1 + g.s) % 2 == 0 || (g.n[3] - 1 + g.s) % 2 == 0);
+  if (ties || !sites_fit(g)) {
+    S.list = nullptr;
+  } else {
+    const size_t tiles = site_tiles4(g);
+    K4_LAUNCH(s, K_SITES, k4_site_hints<<<blocks(tiles, 128), 128, 0, s->stream>>>(g, s->tay32, S, (int)tiles));
+    K4_LAUNCH(s, K_SITES, k4_sites<<<(unsigned)tiles, T4, 0, s->stream>>>(g, s->tay32, S, (float)g.alpha));
+    K4_LAUNCH(s, K_SITES_CHECK, k4_sites_check<<<(unsigned)tiles, T4, 0, s->stream>>>(g, s->tay32, S, (float)g.alpha));
+    K4_LAUNCH(s, K_SITES_CHECK, k4_flood_list<<<blocks(g.ne, 256), 256, 0, s->stream>>>(g, S, s->ds));
+  }
+  K4_LAUNCH(s, K_PERC, k4_percolate<<<S.list ? std::min(g.ne, 152 * 16) : g.ne, PERC_THREADS, s->smem, s->stream>>>(
+                           g, s->el, s->tay, s->tay32, s->key, s->slot, s->ovf_list, S, s->ds));
   // returns at once when no element left its window
   K4_LAUNCH(s, K_PERC_BIG,
-            k4_percolate_big<<<BIG_SLOTS, 256, 0, s->stream>>>(g, s->el, s->tay, s->key, s->slot, s->ovf_list, s->big, s->ds));
-  K4_LAUNCH(s, K_FINISH, k4_map_finish<<<blocks(g.nsite, 256), 256, 0, s->stream>>>(g, s->key, s->slot, s->map, s->holes, s->ds));
+            k4_percolate_big<<<BIG_SLOTS, 256, 0, s->stream>>>(g, s->el, s->tay, s->tay32, s->key, s->slot, s->ovf_list,
+                                                               s->big, S, s->ds));
+  K4_LAUNCH(s, K_FINISH, k4_map_finish<<<blocks(g.nsite, 256), 256, 0, s->stream>>>(g, s->key, s->slot, s->map, s->holes,
+                                                                                       S, s->ds));
   K4_LAUNCH(s, K_HOLES, k4_holes<<<1, 1024, 0, s->stream>>>(g, s->tay, s->map, s->holes, s->cand, s->ds));
   return VM_OK;
 }
@@ -2126,6 +2644,8 @@ vm_status vm_4d_create(const vm_4d_config* c, void* d_ws, size_t bytes, void* st
   s->ovf_list = (int32_t*)(s->ws + L.ovf);
   s->big = (uint32_t*)(s->ws + L.big);
   s->ds = (Dev4*)(s->ws + L.ds);
+  s->sites = Sites4{(int*)(s->ws + L.start), (uint32_t*)(s->ws + L.flags), (uint32_t*)(s->ws + L.site_cand),
+                    (float*)(s->ws + L.site_up), (int32_t*)(s->ws + L.flood), (float*)(s->ws + L.hints)};
   s->nchunk = nchunks(g);
   const int nwin = g.W * g.W * g.W * g.W;
   const int nwords = (nwin + 31) / 32;
@@ -2280,7 +2800,7 @@ vm_status vm_4d_map_stats(vm_4d_solver* s, int32_t* out3, int64_t* d2_evals) {
   if (cudaStreamSynchronize(s->stream) != cudaSuccess) return VM_E_CUDA;
   Dev4 h;
   if (cudaMemcpy(&h, s->ds, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess) return VM_E_CUDA;
-  out3[0] = h.novf;
+  out3[0] = h.novf + h.wide;
   out3[1] = h.nholes;
   out3[2] = h.rounds;
   if (d2_evals) *d2_evals = (int64_t)h.d2_evals;
