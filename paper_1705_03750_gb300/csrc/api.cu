@@ -495,7 +495,7 @@ vm_status vm::solver_create(const vm_config* c, void* d_workspace, size_t bytes,
   s->tay = (double*)(base + L.tay);
   s->tayf = (float*)(base + L.tayf);
   s->tayl = (float*)(base + L.tayl);
-  s->tayx = s->fp32 ? nullptr : (vm::FxRec*)(base + L.tayx);
+  s->tayx = s->fp32 || !vm::fixed_on(s->g) ? nullptr : (vm::FxRec*)(base + L.tayx);
   s->M = (double*)(base + L.M);
   s->a = (double*)(base + L.a);
   s->da = (double*)(base + L.da);

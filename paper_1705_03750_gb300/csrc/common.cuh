@@ -240,7 +240,7 @@ struct vm_solver {
   double* tay;              // ne x 16
   float* tayf;              // ne x 32 (FP32 record, element units)
   float* tayl;              // ne x 16 (the site pass's part of it)
-  vm::FxRec* tayx;          // ne fixed-point records (FP64 solves; else NULL)
+  vm::FxRec* tayx;          // ne fixed-point records (FP64 solves with fixed_on; else NULL)
   double* M;                // pixel masses of the last step
   double* a;
   double* da;
@@ -295,6 +295,13 @@ vm_status solver_create(const vm_config* c, void* d_workspace, size_t bytes, cud
 // ---- one step, enqueue only (api.cu) ----
 void step_transport(vm_solver* s);
 cudaError_t step_remap(vm_solver* s);
+
+// Which FP64 solves have fixed-point records (the others' values are formed in
+// FP64).  The records are worth writing from some 30000 sites on: 20 steps and a
+// remap at 128 x 128 sites 1.18 ms with them and 1.11 without, 160 x 160 1.20
+// and 1.17, 200 x 170 1.20 and 1.21, 256 x 256 1.33 and 1.40, 400 x 350 1.60 and
+// 1.94.
+inline bool fixed_on(const Grid& g) { return (long long)g.nx * g.nv >= 1 << 15; }
 
 // Which solves take the map's site pass: lattices whose positions fit a tile
 // word.  20 steps at stride 8, with it and flooded as a whole: 100 x 100 sites

@@ -8,7 +8,8 @@
 //
 // FP64 path: offsets and sums in 64-bit fixed point (fixed.cuh), the node and
 // beta decisions those of the FP64 evaluation in a fixed operation order, which
-// also serves the sites the fixed-point records do not reach.  FP32-mixed path: Q from the element's FP32
+// also serves the sites the fixed-point records do not reach; small grids in
+// FP64 throughout.  FP32-mixed path: Q from the element's FP32
 // record in element units, anchored on the exact lattice position of Q_m, so
 // that only the small offset carries FP32 rounding; the integer decisions
 // (nearest node, containing square, beta ranges) are taken from the FP32
@@ -144,8 +145,35 @@ __device__ __forceinline__ bool recon64_fixed(const Grid& g, const FxRec* __rest
   return true;
 }
 
+// The same value in FP64, for the solves without fixed-point records
+// (fixed_on).  The integer decisions (nearest node, containing cell) come from
+// the FP32 record's certified evaluation, which is the fixed-order FP64
+// evaluation's whenever its bound clears every decision boundary (as on the
+// FP32-mixed path); the offset Q - Q_m is then evaluated in FP64 with fused
+// operations, anchored on the exact lattice position of Q_m, and the
+// six-point value with fused operations.  A site whose decision the bound
+// leaves open (the step after a remap puts every Q on a node) is evaluated
+// entirely in the fixed order.
+__device__ __forceinline__ bool recon64_fast(const Grid& g, const double* __restrict__ t, const float* __restrict__ F,
+                                             int m, int i, int j, double Px, double Pv,
+                                             const double* __restrict__ fini, float inv_Lv, double& val);
+
+__device__ __forceinline__ double qinterp64_fused(const double* __restrict__ F, const Grid& g, long long in,
+                                                  long long jn, long long ic, long long jc, double x, double y) {
+  const double hx = 0.5 * x, hy = 0.5 * y;
+  double f = F_at(F, g, in, jn) * fma(-y, y, fma(-x, x, 1.0));
+  f = fma(F_at(F, g, in + 1, jn), fma(hx, x, hx), f);
+  f = fma(F_at(F, g, in - 1, jn), fma(hx, x, -hx), f);
+  f = fma(F_at(F, g, in, jn + 1), fma(hy, y, hy), f);
+  f = fma(F_at(F, g, in, jn - 1), fma(hy, y, -hy), f);
+  const double cross = (F_at(F, g, ic + 1, jc + 1) + F_at(F, g, ic, jc)) - (F_at(F, g, ic + 1, jc) + F_at(F, g, ic, jc + 1));
+  return fma(cross, x * y, f);
+}
+
+template <bool kFixed>
 __device__ __forceinline__ void k_recon64_body(const Grid& g, const uint32_t* __restrict__ map, const DevState* ds,
-                                                 const double* __restrict__ tay, const FxRec* __restrict__ tayx,
+                                                 const double* __restrict__ tay, const float* __restrict__ tayf,
+                                                 const FxRec* __restrict__ tayx,
                                                  const double* __restrict__ fini, double* __restrict__ f,
                                                  double* __restrict__ M, int vb) {
   using R = double;
@@ -155,6 +183,7 @@ __device__ __forceinline__ void k_recon64_body(const Grid& g, const uint32_t* __
   row_span(g, ds, i, js, je);
   zero_outside(g, f + (size_t)i * g.nv, js, je);
   const uint32_t epoch = ds_epoch(ds);
+  const float inv_Lv = 1.0f / (float)g.Lv;
   double acc = 0.0;
   // the owner of the thread's next site is loaded one iteration ahead
   int m = (js + (int)threadIdx.x <= je) ? owner(map, (size_t)i * g.nv + js + threadIdx.x, epoch, g.ne) : -1;
@@ -163,9 +192,13 @@ __device__ __forceinline__ void k_recon64_body(const Grid& g, const uint32_t* __
     const int mn = (j + (int)blockDim.x <= je) ? owner(map, p + blockDim.x, epoch, g.ne) : -1;
     double val = 0.0;
     if (m >= 0) {
-      if (!recon64_fixed(g, tayx + m, i, j, fini, val)) {
-        // outside the fixed-point record's reach: the fixed order in FP64
-        const double* t = tay + (size_t)m * TY_N;
+      const double* t = tay + (size_t)m * TY_N;
+      const bool done = kFixed ? recon64_fixed(g, tayx + m, i, j, fini, val)
+                               : recon64_fast(g, t, tayf + (size_t)m * TF_N, m, i, j, site_x(g, i), site_v(g, j), fini,
+                                              inv_Lv, val);
+      if (!done) {
+        // outside the fixed-point record's reach, or a decision the FP32 bound
+        // cannot settle: the fixed order in FP64
         double dqx, dqv;
         qofp_exact(t, site_x(g, i), site_v(g, j), dqx, dqv);
         const double u = dmul(dsub(dadd(t[TY_QX], dqx), g.x_lo), g.inv_dx);
@@ -182,12 +215,13 @@ __device__ __forceinline__ void k_recon64_body(const Grid& g, const uint32_t* __
   if (threadIdx.x == 0) M[i] = dmul(rowsum, g.dxdv);
 }
 
+template <bool kFixed>
 __global__ void __launch_bounds__(256) k_recon64(Grid g, const uint32_t* __restrict__ map, const DevState* ds,
-                                                 const double* __restrict__ tay, const FxRec* __restrict__ tayx,
-                                                 const double* __restrict__ fini, double* __restrict__ f,
-                                                 double* __restrict__ M) {
+                                                 const double* __restrict__ tay, const float* __restrict__ tayf,
+                                                 const FxRec* __restrict__ tayx, const double* __restrict__ fini,
+                                                 double* __restrict__ f, double* __restrict__ M) {
   if (!after_prior()) return;
-  k_recon64_body(g, map, ds, tay, tayx, fini, f, M, blockIdx.x);
+  k_recon64_body<kFixed>(g, map, ds, tay, tayf, tayx, fini, f, M, blockIdx.x);
 }
 
 // Monaghan M4 kernel, unnormalised (Sec. 2.3.2).
@@ -461,7 +495,7 @@ __device__ __forceinline__ void k_remap64_body(const Grid& g, const uint32_t* __
     const size_t p = (size_t)i * g.nv + j;
     const int m = owner(map, p, ds_epoch(ds), g.ne);
     double val = 0.0;
-    if (m >= 0 && !remap64_fixed(g, tayx, m, i, j, eta, val)) {
+    if (m >= 0 && !(tayx && remap64_fixed(g, tayx, m, i, j, eta, val))) {
       double Qx, Qv;
       blended_q_fused(g, tay, m, site_x(g, i), site_v(g, j), Qx, Qv);
       const double u = (Qx - g.x_lo) * g.inv_dx;
@@ -759,6 +793,41 @@ __device__ __forceinline__ void k_recon32_body(const Grid& g, const uint32_t* __
   }
   const double rowsum = block_sum(acc.value(), sh);
   if (threadIdx.x == 0) M[i] = dmul(rowsum, g.dxdv);
+}
+
+__device__ __forceinline__ bool recon64_fast(const Grid& g, const double* __restrict__ t, const float* __restrict__ F,
+                                             int m, int i, int j, double Px, double Pv,
+                                             const double* __restrict__ fini, float inv_Lv, double& val) {
+  const float inv_s = 1.0f / (float)g.s, fs = (float)g.s;
+  float px, pv;
+  p_of(F, i, j, inv_s, px, pv);
+  const QF q = qeval(F, px, pv);
+  int Bu, Bw;
+  float bu, bw;
+  anchor_r(g, m, inv_Lv, Bu, bu, Bw, bw);
+  const float ru = bu + fs * q.qx, rw = bw + fs * q.qv;
+  const float eu = fs * q.ex + 1e-6f * (1.f + fabsf(ru)), ew = fs * q.ev + 1e-6f * (1.f + fabsf(rw));
+  if (!(fabsf(ru) < 1e6f && fabsf(rw) < 1e6f)) return false;
+  const float tu = 2.f * ru, tw = 2.f * rw;
+  const float fu = floorf(tu), fw = floorf(tw);
+  if (!((tu - 2.f * eu > fu) && (tu + 2.f * eu < fu + 1.f) && (tw - 2.f * ew > fw) && (tw + 2.f * ew < fw + 1.f)))
+    return false;
+  const int iu = (int)fu, iw = (int)fw;
+  const long long in = Bu + ((iu + 1) >> 1), jn = Bw + ((iw + 1) >> 1);
+  const long long ic = Bu + (iu >> 1), jc = Bw + (iw >> 1);
+  // FP64 offset, fused, on the exact lattice index of Q_m
+  const double dPx = Px - t[TY_X], dPv = Pv - t[TY_V];
+  const double yx = fma(t[TY_TI00], dPx, t[TY_TI01] * dPv), yv = fma(t[TY_TI10], dPx, t[TY_TI11] * dPv);
+  double g0 = fma(t[TY_GX00], dPx, t[TY_GX01] * dPv), g1 = fma(t[TY_GX01], dPx, t[TY_GX11] * dPv);
+  const double sx = fma(dPx, g0, dPv * g1);
+  g0 = fma(t[TY_GV00], dPx, t[TY_GV01] * dPv);
+  g1 = fma(t[TY_GV01], dPx, t[TY_GV11] * dPv);
+  const double sv = fma(dPx, g0, dPv * g1);
+  const double dqx = fma(-0.5, fma(t[TY_TI00], sx, t[TY_TI01] * sv), yx);
+  const double dqv = fma(-0.5, fma(t[TY_TI10], sx, t[TY_TI11] * sv), yv);
+  const double u = fma(dqx, g.inv_dx, (double)Bu + (double)bu), w = fma(dqv, g.inv_dv, (double)Bw + (double)bw);
+  val = qinterp64_fused(fini, g, in, jn, ic, jc, u - (double)in, w - (double)jn);
+  return true;
 }
 
 __global__ void __launch_bounds__(256, 6) k_recon32(Grid g, const uint32_t* __restrict__ map, const DevState* ds,
@@ -1164,7 +1233,10 @@ __global__ void __launch_bounds__(256, 6) k_recon_group32(const SolveDesc* __res
 __global__ void __launch_bounds__(256) k_recon_group64(const SolveDesc* __restrict__ D, const int* __restrict__ off,
                                                      int ns, int total) {
   GROUP_LOOP(off, ns, total)
-  k_recon64_body(gsh, d.map, d.ds, d.tay, d.tayx, (const double*)d.fini, (double*)d.f, d.M, vb);
+  if (d.tayx)
+    k_recon64_body<true>(gsh, d.map, d.ds, d.tay, d.tayf, d.tayx, (const double*)d.fini, (double*)d.f, d.M, vb);
+  else
+    k_recon64_body<false>(gsh, d.map, d.ds, d.tay, d.tayf, d.tayx, (const double*)d.fini, (double*)d.f, d.M, vb);
   GROUP_END
 }
 
@@ -1304,8 +1376,8 @@ void launch_reconstruct(vm_solver* s) {
     launch_next(k_recon32, s->g.nx, nt, 0, s->stream, s->g, s->map, s->ds, s->tay, s->tayf, (const float*)s->fini,
                 (float*)s->f, s->M);
   else
-    launch_next(k_recon64, s->g.nx, nt, 0, s->stream, s->g, s->map, s->ds, s->tay, s->tayx, (const double*)s->fini,
-                (double*)s->f, s->M);
+    launch_next(s->tayx ? k_recon64<true> : k_recon64<false>, s->g.nx, nt, 0, s->stream, s->g, s->map, s->ds, s->tay,
+                s->tayf, s->tayx, (const double*)s->fini, (double*)s->f, s->M);
   prof_end(s, ps_);
   s->launches++;
 }

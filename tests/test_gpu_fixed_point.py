@@ -31,7 +31,10 @@ from paper_1705_03750_gb300 import vlamet as V  # noqa: E402
 @pytest.mark.parametrize("nx,nv,s,shear,curve", [
     (64, 64, 4, 0.0, 0.0), (65, 47, 4, 0.1, 0.0), (48, 51, 1, 0.05, 0.0), (50, 49, 2, 0.1, 0.02),
     (131, 96, 3, 0.2, 0.05), (200, 150, 8, 0.3, 0.02), (260, 200, 64, 0.1, 0.01), (300, 280, 65, 0.1, 0.0),
-    (90, 300, 8, 1.5, 0.0), (96, 96, 8, 0.1, 0.4)])
+    (90, 300, 8, 1.5, 0.0), (96, 96, 8, 0.1, 0.4),
+    # from 2^15 sites on the values are formed in fixed point, below in FP64
+    (181, 181, 4, 0.1, 0.0), (182, 181, 4, 0.1, 0.02), (210, 190, 1, 0.05, 0.0), (255, 180, 2, 0.2, 0.02),
+    (190, 260, 8, 1.5, 0.0), (200, 200, 8, 0.1, 0.4)])
 @pytest.mark.parametrize("scale", [1.0, 1e-290, 1e300])
 def test_values_match_the_oracle(nx, nv, s, shear, curve, scale):
     rc = I.SPITZER_128.with_(nx=nx, nv=nv, s=s, G=0.0)
