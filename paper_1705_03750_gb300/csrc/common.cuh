@@ -301,7 +301,8 @@ cudaError_t step_remap(vm_solver* s);
 // remap at 128 x 128 sites 1.18 ms with them and 1.11 without, 160 x 160 1.20
 // and 1.17, 200 x 170 1.20 and 1.21, 256 x 256 1.33 and 1.40, 400 x 350 1.60 and
 // 1.94.
-inline bool fixed_on(const Grid& g) { return (long long)g.nx * g.nv >= 1 << 15; }
+constexpr long long kFixedSites = 1 << 15;
+inline bool fixed_on(const Grid& g) { return (long long)g.nx * g.nv >= kFixedSites; }
 
 // Which solves take the map's site pass: lattices whose positions fit a tile
 // word.  20 steps at stride 8, with it and flooded as a whole: 100 x 100 sites
@@ -353,6 +354,8 @@ void launch_convert(vm_solver* s, const void* src, void* dst, int32_t dst_dtype,
 void launch_store_real(vm_solver* s, const double* src, void* dst, size_t count);
 // spline.cu
 void launch_spline_solve(vm_solver* s, const void* src, void* dst);
+bool spline_prepare();
+void group_spline_smem(const Grid& g, bool fp32, size_t& rows, size_t& cols);
 
 // ---- many solves in one launch per phase (group.cu drives them) ----
 //
@@ -456,6 +459,7 @@ struct GroupPlan {
   int* off_dyn;                            // scratch for one dynamic phase at a time
   int big_blocks_cap;                      // virtual blocks per solve of the large windows
   size_t big_smem;                         // dynamic shared memory of the large windows
+  size_t row_smem, col_smem;               // and of the spline's sweeps
   GroupShape shape[32];                    // per phase (GroupPhase)
 };
 

@@ -124,7 +124,7 @@ void group_plan(GroupPlan& P, vm_solver* const* solvers, int n, void* d_table, v
   SolveDesc* hd = (SolveDesc*)hb;
   int* hoff = (int*)(hb + dbytes);
   int tot[U_N] = {0};
-  size_t big = 0;
+  size_t big = 0, row_smem = 0, col_smem = 0;
   for (int i = 0; i < n; i++) {
     hd[i] = desc_of(solvers[i], gated);
     int u[U_N];
@@ -134,6 +134,10 @@ void group_plan(GroupPlan& P, vm_solver* const* solvers, int n, void* d_table, v
       tot[k] += u[k];
     }
     big = std::max(big, group_big_smem(solvers[i]->g));
+    size_t rs, cs;
+    group_spline_smem(solvers[i]->g, solvers[i]->fp32, rs, cs);
+    row_smem = std::max(row_smem, rs);
+    col_smem = std::max(col_smem, cs);
   }
   for (int k = 0; k < U_N; k++) hoff[k * (n + 1) + n] = tot[k];
   const int* doff = (const int*)(db + dbytes);
@@ -163,6 +167,8 @@ void group_plan(GroupPlan& P, vm_solver* const* solvers, int n, void* d_table, v
   P.recon_tiles = solvers[0]->g.recon_tiles;
   P.off_dyn = (int*)(db + dbytes) + U_N * (n + 1);
   P.big_smem = big;
+  P.row_smem = row_smem;
+  P.col_smem = col_smem;
   P.big_blocks_cap = 0;
   cudaMemcpyAsync(d_table, host, dbytes + (size_t)U_N * (n + 1) * sizeof(int), cudaMemcpyHostToDevice, stream);
 }
