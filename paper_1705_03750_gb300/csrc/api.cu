@@ -508,7 +508,7 @@ vm_status vm::solver_create(const vm_config* c, void* d_workspace, size_t bytes,
   s->Mpart = (double*)(base + L.mpart);
   s->diag_part = (double*)(base + L.dpart);
   s->ds = (vm::DevState*)(base + L.ds);
-  if (!vm::map_prepare(g) || !vm::spline_prepare() || !vm::recon_prepare()) {
+  if (!vm::map_prepare(g) || !vm::spline_prepare(s) || !vm::recon_prepare()) {
     free(s);
     return VM_E_INVALID_ARG;
   }

@@ -156,7 +156,7 @@ extern "C" vm_status vm_batch_create(vm_solver* const* solvers, int32_t n, int32
   const int32_t n_s = hosts.empty() ? 0 : hosts[0]->cfg.n_s, cyc = hosts.empty() ? 0 : hosts[0]->cyc;
   for (vm_solver* s : hosts)
     if (s->cfg.n_s != n_s || s->cyc != cyc) return VM_E_STATE;  // one remap phase for the host-cycle solves
-  if (!vm::group_map_prepare()) return VM_E_CUDA;
+  if (!vm::group_map_prepare() || !vm::group_spline_prepare()) return VM_E_CUDA;
   vm_batch* b = new vm_batch();
   b->solvers.assign(solvers, solvers + n);
   b->hosts = hosts;

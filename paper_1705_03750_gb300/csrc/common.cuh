@@ -354,7 +354,8 @@ void launch_convert(vm_solver* s, const void* src, void* dst, int32_t dst_dtype,
 void launch_store_real(vm_solver* s, const double* src, void* dst, size_t count);
 // spline.cu
 void launch_spline_solve(vm_solver* s, const void* src, void* dst);
-bool spline_prepare();
+bool spline_prepare(const vm_solver* s);
+bool group_spline_prepare();
 void group_spline_smem(const Grid& g, bool fp32, size_t& rows, size_t& cols);
 
 // ---- many solves in one launch per phase (group.cu drives them) ----

@@ -341,7 +341,7 @@ vm_status vm_server_create(const vm_server_config* c, void* d_pool, size_t pool_
   *out = nullptr;
   const size_t reserve = vm_server_pool_bytes(c);
   if (pool_bytes <= reserve) return VM_E_OOM;
-  if (!vm::group_map_prepare()) return VM_E_CUDA;
+  if (!vm::group_map_prepare() || !vm::group_spline_prepare()) return VM_E_CUDA;
   vm_server* S = new vm_server();
   S->c = *c;
   S->pool = (char*)d_pool;

@@ -502,11 +502,15 @@ void launch_spline_solve(vm_solver* s, const void* src, void* dst) {
   s->launches += 2;
 }
 
-// Opt the filters in to shared memory (up to the largest they ask for).
-bool spline_prepare() {
-  return cols_prepare(k_cols_filter<double, COL_W>, 8) && cols_prepare(k_cols_filter<double, COL_W_FEW>, 8) &&
-         cols_prepare(k_cols_filter<float, COL_W>, 4) && cols_prepare(k_cols_filter<float, COL_W_FEW>, 4) &&
-         cols_prepare(k_cols_group<double>, 8) && cols_prepare(k_cols_group<float>, 4) &&
+// Opt the filters in to shared memory (up to the largest they ask for): a
+// solver's, and a group's.
+bool spline_prepare(const vm_solver* s) {
+  if (!filters_on(s->g)) return true;
+  return s->fp32 ? cols_prepare(k_cols_filter<float, COL_W>, 4) && cols_prepare(k_cols_filter<float, COL_W_FEW>, 4)
+                 : cols_prepare(k_cols_filter<double, COL_W>, 8) && cols_prepare(k_cols_filter<double, COL_W_FEW>, 8);
+}
+bool group_spline_prepare() {
+  return cols_prepare(k_cols_group<double>, 8) && cols_prepare(k_cols_group<float>, 4) &&
          rows_prepare(k_rows_group<double>, 8) && rows_prepare(k_rows_group<float>, 4);
 }
 
