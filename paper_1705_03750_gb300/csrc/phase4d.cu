@@ -560,10 +560,11 @@ __device__ __forceinline__ void claim4(ulonglong2* key, unsigned long long dbits
 //
 // k4_site_hints prepares each tile's guess, k4_sites proposes the owners and
 // tests them, k4_sites_check looks at each site's eight neighbours.  A site
-// costs about one evaluation of its own, 0.7 of neighbours beyond the alpha box
-// and 2 of owners next to it, where the flood fill tested three sites for each
-// of a component's and formed its shell: 64^4 sites 1.3 + 1.7 ms and 0.4 ms for
-// the elements left to the fill, where the fill of all took 8.8 ms.  Bound by
+// costs about one evaluation of its own, up to 0.7 of neighbours beyond the alpha
+// box and up to 2 of owners next to it, where the flood fill tested three sites for each
+// of a component's and formed its shell: 64^4 sites 2.5 ms and 0.4 ms for
+// the elements left to the fill, where the fill of all took 8.8 ms; without
+// k4_gaps, which settles most neighbours without an evaluation, 3.1 ms.  Bound by
 // the records' reads (288 bytes an evaluation through L1) and by occupancy: with
 // whole records held in registers (2 blocks an SM) and the guess formed inside
 // each tile the two kernels took 4.8 ms.
@@ -573,9 +574,11 @@ struct Sites4 {
   const int* start;     // 4 per element: start site (INT_MIN/2 where not finite)
   uint32_t* flags;      // per element: EF4_*
   uint32_t* cand;       // per site of the padded lattice: O(p)'s lattice position, a byte per axis
-  float* up;            // per site: an upper bound of O(p)'s d^2, negative if its test is not settled
+  float* up;            // per site: an upper bound of O(p)'s d^2, negative if its test is not settled; its low
+                        // byte holds, per axis and side, that the neighbour there certainly fails at the site
   int32_t* list;        // elements for the flood fill; NULL: no site pass, all of them
   float* hints;         // 20 per tile: lattice position at its middle site, change per site
+  float* gap;           // 8 per element: how far its map and a neighbour's differ (k4_gaps)
 };
 
 // Lattices whose positions fit the owners' words (others are flooded).
@@ -679,6 +682,91 @@ size_t site_tiles4(const G4& g) {
 
 __device__ __forceinline__ int nearest_elem(float k, int L) { return min(max(__float2int_rn(k), 0), L - 1); }
 
+// Largest |x_n - (x_m - o)| over the sites with |p| <= GAP_P of m, for its
+// neighbours n one step o along each axis (gap[2 a], towards -a; gap[2 a + 1],
+// towards +a), from the difference of the two polynomials.  Where it is small, n
+// is certainly farther than m at m's sites short of the middle, and m lies in the
+// ranges of n's test: no evaluation of n is needed there.  The roundings
+// here (2e-6 of the absolute terms) and of the FP64 evaluations (K's) are added.
+constexpr float GAP_P = 1.5f;
+
+__global__ void __launch_bounds__(128) k4_gaps(G4 g, const float* __restrict__ tay32, Sites4 S) {
+  const int q = blockIdx.x * 128 + threadIdx.x;
+  const int m = q >> 2, ax = q & 3;  // the pair (m, m + e_ax)
+  if (m >= g.ne) return;
+  int k[4], stride = 1;
+  elem_coords(g, m, k);
+  for (int a = 3; a > ax; a--) stride *= g.L[a];
+  bool last = false;
+  for (int a = 0; a < 4; a++) last = last || (a == ax && k[a] + 1 >= g.L[a]);
+  bool first = false;
+  for (int a = 0; a < 4; a++) first = first || (a == ax && k[a] == 0);
+  if (first) S.gap[8 * (size_t)m + 2 * ax] = 1e30f;
+  if (last) {
+    S.gap[8 * (size_t)m + 2 * ax + 1] = 1e30f;
+    return;
+  }
+  const int n = m + stride;
+  const float4* R = reinterpret_cast<const float4*>(tay32 + (size_t)NF4 * m);
+  const float4* T = reinterpret_cast<const float4*>(tay32 + (size_t)NF4 * n);
+  const int4 sm = __ldg(reinterpret_cast<const int4*>(S.start) + m), sn = __ldg(reinterpret_cast<const int4*>(S.start) + n);
+  const float4 rm = __ldg(R + 17), rn = __ldg(T + 17), Km = __ldg(R + 14), Kn = __ldg(T + 14);
+  // n's p minus m's
+  const float t[4] = {(float)(sm.x - sn.x) * (float)(g.d[0] * g.inv_dm[0]) + (rn.x - rm.x),
+                      (float)(sm.y - sn.y) * (float)(g.d[1] * g.inv_dm[1]) + (rn.y - rm.y),
+                      (float)(sm.z - sn.z) * (float)(g.d[2] * g.inv_dm[2]) + (rn.z - rm.z),
+                      (float)(sm.w - sn.w) * (float)(g.d[3] * g.inv_dm[3]) + (rn.w - rm.w)};
+  const float K[4] = {Km.x + Kn.x, Km.y + Kn.y, Km.z + Kn.z, Km.w + Kn.w};
+  float worst[2] = {0.f, 0.f};  // about m and about n
+#pragma unroll
+  for (int a = 0; a < 4; a++) {
+    const float4 Am = __ldg(R + a), An = __ldg(T + a);
+    const float am[4] = {Am.x, Am.y, Am.z, Am.w}, an[4] = {An.x, An.y, An.z, An.w};
+    float bm[10], bn[10];
+#pragma unroll
+    for (int c = 0; c < 5; c++) {
+      const float2 u = __ldg(reinterpret_cast<const float2*>(R) + 8 + 5 * a + c);
+      const float2 v = __ldg(reinterpret_cast<const float2*>(T) + 8 + 5 * a + c);
+      bm[2 * c] = u.x, bm[2 * c + 1] = u.y, bn[2 * c] = v.x, bn[2 * c + 1] = v.y;
+    }
+    float quad = 0.f, mag = 1.f;
+#pragma unroll
+    for (int b = 0; b < 4; b++) {
+      mag += (fabsf(am[b]) + fabsf(an[b])) * (fabsf(t[b]) + GAP_P);
+#pragma unroll
+      for (int c = b; c < 4; c++) {
+        quad += fabsf(bn[sym4(b, c)] - bm[sym4(b, c)]);
+        mag += 2.f * (fabsf(bn[sym4(b, c)]) + fabsf(bm[sym4(b, c)])) * (fabsf(t[b]) + GAP_P) * (fabsf(t[c]) + GAP_P);
+      }
+    }
+#pragma unroll
+    for (int side = 0; side < 2; side++) {
+      // the other's polynomial about this element, minus its own, plus o
+      const float sg = side ? -1.f : 1.f;
+      float c0 = a == ax ? sg : 0.f, lin = 0.f;
+#pragma unroll
+      for (int b = 0; b < 4; b++) {
+        float d = sg * (an[b] - am[b]), half = 0.f;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          const float B = side ? bm[sym4(b, c)] : bn[sym4(b, c)], tc = sg * t[c];
+          d = fmaf(b == c ? 2.f * B : B, tc, d);
+          half = fmaf(b == c ? B : 0.5f * B, tc, half);
+        }
+        lin += fabsf(d);
+        c0 = fmaf((side ? am[b] : an[b]) + half, sg * t[b], c0);
+      }
+      const float e = fabsf(c0) + GAP_P * (lin + GAP_P * quad) + 2e-6f * mag + 1e-8f * K[a];
+      worst[side] = e > worst[side] || !(e == e) ? e : worst[side];
+    }
+  }
+#pragma unroll
+  for (int side = 0; side < 2; side++) {
+    const float w = worst[side] * 1.001f + 1e-5f;
+    S.gap[8 * (size_t)(side ? n : m) + 2 * ax + (side ? 0 : 1)] = w < 1e30f ? w : 1e30f;
+  }
+}
+
 // Per tile: the lattice position of Q at its middle site, by Newton steps from
 // element to element starting from the undeformed lattice, and its change per
 // site.  One thread per tile: in the tile's own block the others would wait.
@@ -725,6 +813,27 @@ __global__ void __launch_bounds__(128) k4_site_hints(G4 g, const float* __restri
   }
 }
 
+// Per axis and side (bits 2 a, towards -a, and 2 a + 1): the neighbour n there is
+// certainly farther than m at the site, and m's side of n's alpha box certainly
+// left (alo; -1e30: not asked).  With x_n = x_m - o + delta, |delta| <= gap per
+// component: d_n^2 - d_m^2 >= 1 - 2 y - 2 gap (sum |x| + 1), y = o . x_m.
+__device__ __forceinline__ unsigned neighbours_fail(const Sites4& S, int m, const float (&x)[4], const float (&e)[4],
+                                                    bool near, float alo) {
+  if (!near) return 0u;
+  const float4* G = reinterpret_cast<const float4*>(S.gap + 8 * (size_t)m);
+  const float4 g0 = __ldg(G), g1 = __ldg(G + 1);
+  const float gap[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+  const float E = fmaxf(fmaxf(e[0], e[1]), fmaxf(e[2], e[3]));
+  const float sum = fabsf(x[0]) + fabsf(x[1]) + fabsf(x[2]) + fabsf(x[3]) + 1.f + 4.f * E;
+  unsigned bits = 0u;
+#pragma unroll
+  for (int q = 0; q < 8; q++) {
+    const float y = (q & 1 ? x[q >> 1] : -x[q >> 1]) + E;
+    if (1.f - 2.f * y - 2.f * gap[q] * sum > 1e-5f && y - 1.f + gap[q] < -alo) bits |= 1u << q;
+  }
+  return bits;
+}
+
 __global__ void __launch_bounds__(T4, 3) k4_sites(G4 g, const float* __restrict__ tay32, Sites4 S, float alpha) {
   __shared__ int sh_k[T4][4];  // the sites' proposed owners
   __shared__ float sh_d[T4], sh_b[T4];
@@ -755,7 +864,7 @@ __global__ void __launch_bounds__(T4, 3) k4_sites(G4 g, const float* __restrict_
       k[a] = nearest_elem(fmaf(J.x, j0, fmaf(J.y, j1, fmaf(J.z, j2, fmaf(J.w, j3, xc[a])))), g.L[a]);
     }
   }
-  bool todo = on, sure = false;
+  bool todo = on, sure = false, near = false;  // near: |p| <= GAP_P
   float d2 = 0.f;
   int4 st = make_int4(0, 0, 0, 0);
   int m = 0;
@@ -781,6 +890,8 @@ __global__ void __launch_bounds__(T4, 3) k4_sites(G4 g, const float* __restrict_
         }
       }
       sure = d2 < 1e30f && bd < 1e30f;
+      near = fmaxf(fmaxf(fabsf((float)(c[0] - st.x) * h[0]), fabsf((float)(c[1] - st.y) * h[1])),
+                   fmaxf(fabsf((float)(c[2] - st.z) * h[2]), fabsf((float)(c[3] - st.w) * h[3]))) <= GAP_P - 0.51f;
       // the ranges, widened where the bound does not settle them (a neighbour
       // more to compare does no harm: the test then passes against all)
       int side[4], cnt = 0, ns = 0;
@@ -796,6 +907,12 @@ __global__ void __launch_bounds__(T4, 3) k4_sites(G4 g, const float* __restrict_
       sh_open[tid] = 0;
       sh_best[tid] = ~0ull;
       for (int a = 0; a < 4; a++) sh_k[tid][a] = k[a];
+      if (sure && ns == 1 && near) {
+        // one neighbour, certainly farther: nothing to compare
+        const unsigned far = neighbours_fail(S, m, x, e, true, -1e30f);
+        for (int a = 0; a < 4; a++)
+          if (side[a] != 0 && (far >> (2 * a + (side[a] > 0)) & 1u)) ns = 0;
+      }
       if (sure && ns) {
         // the nonempty subsets of the sides, in the lattice
         unsigned short codes[15];
@@ -855,8 +972,11 @@ __global__ void __launch_bounds__(T4, 3) k4_sites(G4 g, const float* __restrict_
     if (!__syncthreads_or(again)) break;
   }
   if (!on) return;
+  unsigned fails = 0;
+  if (sure) fails = neighbours_fail(S, m, x, e, near, alpha + aerr);
   S.cand[pi] = (uint32_t)k[0] << 24 | (uint32_t)k[1] << 16 | (uint32_t)k[2] << 8 | (uint32_t)k[3];
-  S.up[pi] = sure ? d2 + bd : -1.f;
+  // (an upper bound still with the low byte set; a negative number has it clear)
+  S.up[pi] = sure ? __uint_as_float((__float_as_uint(d2 + bd) | 255u) & (~255u | fails)) : -1.f;
   if (!sure) m = ((k[0] * g.L[1] + k[1]) * g.L[2] + k[2]) * g.L[3] + k[3];
   if (!sure) {
     if (!(__ldcg(S.flags + m) & EF4_BAD)) atomicOr(S.flags + m, EF4_BAD);
@@ -909,6 +1029,18 @@ __global__ void __launch_bounds__(T4, 4) k4_sites_check(G4 g, const float* __res
       }
     }
     if (!linked && starts_inside(g, st) && !(__ldcg(S.flags + m) & EF4_BAD)) atomicOr(S.flags + m, EF4_BAD);
+    // neighbours one step along one axis that the site's own evaluation settled
+    if (up >= 0.f)
+#pragma unroll
+      for (int dir = 0; dir < 8; dir++) {
+        const uint32_t diff = wn[dir] - w;  // (the positions differ by at least one; a borrow makes no single step)
+#pragma unroll
+        for (int a = 0; a < 4; a++) {
+          const unsigned b = __float_as_uint(up) >> (2 * a);
+          if ((diff == 1u << (24 - 8 * a) && (b >> 1 & 1u)) || (diff == 0u - (1u << (24 - 8 * a)) && (b & 1u)))
+            other &= ~(1u << dir);
+        }
+      }
     if (other) {
       int at = atomicAdd(&npairs, __popc(other));
 #pragma unroll
@@ -934,7 +1066,7 @@ __global__ void __launch_bounds__(T4, 4) k4_sites_check(G4 g, const float* __res
     tile_site(g, blockIdx.x, t, cs, ps);
     float x[4], e[4], bd;
     const float d2 = site_eval(g, tay32, st, n, cs, h, x, e, &bd);
-    const float up = sh_up[t];
+    const float up = __uint_as_float(__float_as_uint(sh_up[t]) | 255u);  // (the bits' place in the bound)
     bool fails = up >= 0.f && up < d2 - bd;
 #pragma unroll
     for (int a = 0; a < 4; a++) {
@@ -2487,7 +2619,7 @@ int nchunks(const G4& g) { return (g.n[0] * g.n[1] + accel_run(g) - 1) / accel_r
 
 struct Layout {
   size_t diag, fini, eta, f, key, slot, map, holes, cand, el, tay, tay32, tayx, Mpix, fld, gext, part, tab, ovf, big, ds, start, flags,
-      site_cand, site_up, flood, hints, green, fields, total;
+      site_cand, site_up, flood, hints, gaps, green, fields, total;
 };
 
 Layout layout(const G4& g) {
@@ -2533,6 +2665,7 @@ Layout layout(const G4& g) {
   L.site_cand = take(sites_fit(g) ? 4 * (size_t)npad : 0);
   L.site_up = take(sites_fit(g) ? 4 * (size_t)npad : 0);
   L.hints = take(sites_fit(g) ? 80 * site_tiles4(g) : 0);
+  L.gaps = take(sites_fit(g) ? 32 * (size_t)g.ne : 0);
   L.total = o;
   return L;
 }
@@ -2605,6 +2738,7 @@ vm_status run_map(vm_4d_solver* s) {
     S.list = nullptr;
   } else {
     const size_t tiles = site_tiles4(g);
+    K4_LAUNCH(s, K_SITES, k4_gaps<<<blocks(4ll * g.ne, 128), 128, 0, s->stream>>>(g, s->tay32, S));
     K4_LAUNCH(s, K_SITES, k4_site_hints<<<blocks(tiles, 128), 128, 0, s->stream>>>(g, s->tay32, S, (int)tiles));
     K4_LAUNCH(s, K_SITES, k4_sites<<<(unsigned)tiles, T4, 0, s->stream>>>(g, s->tay32, S, (float)g.alpha));
     K4_LAUNCH(s, K_SITES_CHECK, k4_sites_check<<<(unsigned)tiles, T4, 0, s->stream>>>(g, s->tay32, S, (float)g.alpha));
@@ -2719,7 +2853,8 @@ vm_status vm_4d_create(const vm_4d_config* c, void* d_ws, size_t bytes, void* st
   s->big = (uint32_t*)(s->ws + L.big);
   s->ds = (Dev4*)(s->ws + L.ds);
   s->sites = Sites4{(int*)(s->ws + L.start), (uint32_t*)(s->ws + L.flags), (uint32_t*)(s->ws + L.site_cand),
-                    (float*)(s->ws + L.site_up), (int32_t*)(s->ws + L.flood), (float*)(s->ws + L.hints)};
+                    (float*)(s->ws + L.site_up), (int32_t*)(s->ws + L.flood), (float*)(s->ws + L.hints),
+                    (float*)(s->ws + L.gaps)};
   s->nchunk = nchunks(g);
   const int nwin = g.W * g.W * g.W * g.W;
   const int nwords = (nwin + 31) / 32;
