@@ -88,12 +88,15 @@ struct Dev4 {
   int32_t nflood;  // elements left to the flood fill (this map)
   int32_t wide;  // other elements whose component reaches beyond the window (this map)
   int32_t rounds;  // hole-repair rounds of the last map
+  unsigned long long nclaims;  // sites of the whole-lattice fills, claimed after them (0 between maps)
   unsigned long long d2_evals;  // distance evaluations of the percolation kernels (cumulative)
 };
 
 // whole-lattice flood fill of the elements that left their window: per slot,
 // a bit per site of the padded lattice and two frontier buffers
-constexpr int BIG_SLOTS = 8;
+constexpr int BIG_SLOTS = 16;
+constexpr int BIG_T = 512;      // threads of a block
+constexpr int BIG_LIST = 4096;  // newly reached sites tested together
 constexpr int BIG_FCAP = 1 << 18;
 
 __device__ __forceinline__ double M_(double a, double b) { return __dmul_rn(a, b); }
@@ -1494,16 +1497,21 @@ __device__ __forceinline__ int passes4_f32(const G4& g, const int* k, int m, con
 // Whole-lattice flood fill of the listed elements: the same breadth-first
 // search over the padded lattice [-pad, n-1+pad]^4, with its visited bits and
 // frontiers in global memory (one slot per block), the tests in FP32 with
-// bounds first (27 ms of a 20 x 24 x 22 x 18 solve's 39 went into FP64 ones).
-__global__ void __launch_bounds__(256) k4_percolate_big(G4 g, const double* __restrict__ el,
+// bounds first (27 ms of a 20 x 24 x 22 x 18 solve's 39 went into FP64 ones), the
+// claims listed for k4_late_claims.  Bound by the arithmetic of one SM: a
+// component of most of the lattice 2.2 ms there, 3.6 with its claims and a warp's
+// tests left where the frontier's order put them.
+__global__ void __launch_bounds__(BIG_T) k4_percolate_big(G4 g, const double* __restrict__ el,
                                                         const double* __restrict__ tay,
                                                         const float* __restrict__ tay32, ulonglong2* __restrict__ key,
                                                         uint32_t* __restrict__ slot,
                                                         const int32_t* __restrict__ ovf_list, uint32_t* __restrict__ big,
+                                                        int32_t* __restrict__ claim_p, int32_t* __restrict__ claim_m,
                                                         Sites4 S, Dev4* ds) {
   __shared__ double tself[NT4];
   __shared__ int kk[4];
-  __shared__ int go, ncur, nnext, bad_wave;
+  __shared__ int go, ncur, nnext, bad_wave, nnew;
+  __shared__ int32_t fresh[BIG_LIST];  // newly reached sites of the wave, not tested yet
   const int nlist = ds->novf;
   long long pw[4], npad = 1;
   for (int a = 0; a < 4; a++) {
@@ -1559,45 +1567,73 @@ __global__ void __launch_bounds__(256) k4_percolate_big(G4 g, const double* __re
       const int32_t* fc = cur ? front1 : front0;
       int32_t* fn = cur ? front0 : front1;
       const long long ntask = (long long)ncur * 8;
-      for (long long t = tid; t < ntask; t += blockDim.x) {
-        const long long e = t >> 3;
-        const int dir = (int)(t & 7), ax = dir >> 1, sg = (dir & 1) ? 1 : -1;
-        long long r = fc[e], gl[4];
-        for (int a = 3; a >= 0; a--) {
-          gl[a] = r % pw[a];
-          r /= pw[a];
+      // the frontier's neighbours are stamped a block's worth at a time; the new
+      // ones, about one in five, are collected and tested by full warps
+      for (long long t0 = 0; t0 < ntask;) {
+        if (tid == 0) nnew = 0;
+        __syncthreads();
+        for (int held = 0; t0 < ntask && held <= BIG_LIST - BIG_T; t0 += BIG_T) {
+          const long long t = t0 + tid;
+          if (t < ntask) {
+            const int dir = (int)(t & 7), ax = dir >> 1, sg = (dir & 1) ? 1 : -1;
+            long long r = __ldcg(fc + (t >> 3)), gl[4];
+            for (int a = 3; a >= 0; a--) {
+              const uint32_t u = (uint32_t)r / (uint32_t)pw[a];
+              gl[a] = r - (long long)u * pw[a];
+              r = u;
+            }
+            gl[ax] += sg;
+            if (gl[ax] >= 0 && gl[ax] < pw[ax]) {
+              const long long np = ((gl[0] * pw[1] + gl[1]) * pw[2] + gl[2]) * pw[3] + gl[3];
+              const uint32_t bit = 1u << (np & 31);
+              if (!(atomicOr(&stamp[np >> 5], bit) & bit)) fresh[atomicAdd(&nnew, 1)] = (int32_t)np;
+            }
+          }
+          __syncthreads();
+          held = nnew;
+          __syncthreads();
         }
-        gl[ax] += sg;
-        if (gl[ax] < 0 || gl[ax] >= pw[ax]) continue;
-        const long long np = ((gl[0] * pw[1] + gl[1]) * pw[2] + gl[2]) * pw[3] + gl[3];
-        const uint32_t bit = 1u << (np & 31);
-        if (atomicOr(&stamp[np >> 5], bit) & bit) continue;
-        double d2 = 0.0;
-        long long gs[4];
-        int ci[4];
-        for (int a = 0; a < 4; a++) {
-          gs[a] = gl[a] - g.pad;
-          ci[a] = (int)gs[a];
+        const int nn = nnew;
+        for (int q = tid; q < nn; q += BIG_T) {
+          const int32_t np = fresh[q];
+          long long gs[4], p = 0;
+          int ci[4];
+          uint32_t r = (uint32_t)np;
+          for (int a = 3; a >= 0; a--) {
+            const uint32_t u = r / (uint32_t)pw[a];
+            gs[a] = (long long)(r - u * (uint32_t)pw[a]) - g.pad;
+            ci[a] = (int)gs[a];
+            r = u;
+          }
+          double d2 = 0.0;
+          const int res = passes4_f32(g, kl, m, tay32, S, ci, (float)g.alpha);
+          if (res == 0) continue;
+          if (res < 0) {
+            double P[4];
+            for (int a = 0; a < 4; a++) P[a] = site_coord(g, a, gs[a]);
+            if (!passes4(g, kl, tself, tay, P, &d2, nev)) continue;
+          }
+          bool in = true;
+          for (int a = 0; a < 4; a++) {
+            in = in && gs[a] >= 0 && gs[a] < g.n[a];
+            p += gs[a] * g.st[a];
+          }
+          if (in) {
+            const unsigned long long at = atomicAdd(&ds->nclaims, 1ull);
+            if (at < (unsigned long long)g.nsite) {
+              claim_p[at] = (int32_t)p;
+              claim_m[at] = m;
+            } else {
+              claim_site(g, slot, key, p, m, tself, tay, gs, res < 0, d2, nev, ds, S);
+            }
+          }
+          const int idx = atomicAdd(&nnext, 1);
+          if (idx < BIG_FCAP)
+            fn[idx] = np;
+          else
+            bad_wave = 1;
         }
-        const int res = passes4_f32(g, kl, m, tay32, S, ci, (float)g.alpha);
-        if (res == 0) continue;
-        if (res < 0) {
-          double P[4];
-          for (int a = 0; a < 4; a++) P[a] = site_coord(g, a, gs[a]);
-          if (!passes4(g, kl, tself, tay, P, &d2, nev)) continue;
-        }
-        bool in = true;
-        long long p = 0;
-        for (int a = 0; a < 4; a++) {
-          in = in && gs[a] >= 0 && gs[a] < g.n[a];
-          p += gs[a] * g.st[a];
-        }
-        if (in) claim_site(g, slot, key, p, m, tself, tay, gs, res < 0, d2, nev, ds, S);
-        const int idx = atomicAdd(&nnext, 1);
-        if (idx < BIG_FCAP)
-          fn[idx] = (int32_t)np;
-        else
-          bad_wave = 1;
+        __syncthreads();
       }
       __syncthreads();
       if (tid == 0) {
@@ -1612,12 +1648,36 @@ __global__ void __launch_bounds__(256) k4_percolate_big(G4 g, const double* __re
   if ((tid & 31) == 0 && nev) atomicAdd(&ds->d2_evals, (unsigned long long)nev);
 }
 
+// Claims of the whole-lattice fills.  Nearly all of their sites are contested,
+// with two FP64 distances each: on the fill's own SM those took most of its time.
+__global__ void __launch_bounds__(128) k4_late_claims(G4 g, const double* __restrict__ tay,
+                                                      ulonglong2* __restrict__ key, uint32_t* __restrict__ slot,
+                                                      const int32_t* __restrict__ claim_p,
+                                                      const int32_t* __restrict__ claim_m, Sites4 S, Dev4* ds) {
+  const int n = (int)min(ds->nclaims, (unsigned long long)g.nsite);
+  unsigned nev = 0;
+  for (int q = blockIdx.x * 128 + threadIdx.x; q < n; q += gridDim.x * 128) {
+    const long long p = claim_p[q];
+    const int m = claim_m[q];
+    long long gs[4], r = p;
+    for (int a = 3; a >= 0; a--) {
+      const uint32_t u = (uint32_t)r / (uint32_t)g.n[a];
+      gs[a] = r - (long long)u * g.n[a];
+      r = u;
+    }
+    claim_site(g, slot, key, p, m, tay + (size_t)NT4 * m, tay, gs, false, 0.0, nev, ds, S);
+  }
+  for (int o = 16; o > 0; o >>= 1) nev += __shfl_down_sync(0xffffffffu, nev, o);
+  if ((threadIdx.x & 31) == 0 && nev) atomicAdd(&ds->d2_evals, (unsigned long long)nev);
+}
+
 // owner of every site from its key (the key is emptied for the next map);
 // sites nobody claimed go to the hole list
 __global__ void k4_map_finish(G4 g, ulonglong2* __restrict__ key, uint32_t* __restrict__ slot,
                               int32_t* __restrict__ map, int32_t* __restrict__ holes, Sites4 S, Dev4* ds) {
   const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= g.nsite) return;
+  if (p == 0) ds->nclaims = 0;
   const ulonglong2 k = key[p];
   const uint32_t sl = slot[p];
   int owner = -1;
@@ -2748,8 +2808,10 @@ vm_status run_map(vm_4d_solver* s) {
                            g, s->el, s->tay, s->tay32, s->key, s->slot, s->ovf_list, S, s->ds));
   // returns at once when no element left its window
   K4_LAUNCH(s, K_PERC_BIG,
-            k4_percolate_big<<<BIG_SLOTS, 256, 0, s->stream>>>(g, s->el, s->tay, s->tay32, s->key, s->slot, s->ovf_list,
-                                                               s->big, S, s->ds));
+            k4_percolate_big<<<BIG_SLOTS, BIG_T, 0, s->stream>>>(g, s->el, s->tay, s->tay32, s->key, s->slot, s->ovf_list,
+                                                                 s->big, s->holes, s->cand, S, s->ds));
+  K4_LAUNCH(s, K_PERC_BIG, k4_late_claims<<<152 * 4, 128, 0, s->stream>>>(g, s->tay, s->key, s->slot, s->holes, s->cand,
+                                                                          S, s->ds));
   K4_LAUNCH(s, K_FINISH, k4_map_finish<<<blocks(g.nsite, 256), 256, 0, s->stream>>>(g, s->key, s->slot, s->map, s->holes,
                                                                                        S, s->ds));
   K4_LAUNCH(s, K_HOLES, k4_holes<<<1, 1024, 0, s->stream>>>(g, s->tay, s->map, s->holes, s->cand, s->ds));
