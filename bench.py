@@ -167,23 +167,14 @@ def algorithmic(kernel: str, rc, fp32: bool, ne: int):
     return None
 
 
-# FP64 floating-point operations per site of the FP64 path's reconstruction
-# on its certified branch (a fused multiply-add counts 2): site position 2,
-# P - P_m 2, the second-order offset Q - Q_m 36, the anchored index
-# coordinates 4, the offsets from the nodes 2, the six-point value 29.
-FP64_FLOPS_PER_SITE = 75
-
-
-def fp64_roofline(sites: int, avg_s: float) -> dict:
-    """The FP64 reconstruction against the FP64 arithmetic peak measured on
-    this device in the same run (vm_measure_fp64_peak: FMA chains, 2 FLOP per
-    FMA)."""
-    from paper_1705_03750_gb300 import vlamet as V
-    peak = V.measure_fp64_peak(20000)
-    ach = FP64_FLOPS_PER_SITE * sites / avg_s
-    return {"kernel": "reconstruct", "bound": "alu", "achieved": ach / 1e12, "peak": peak / 1e12,
-            "unit": "TFLOP/s (FP64)", "frac": ach / peak, "per_unit": f"{FP64_FLOPS_PER_SITE} FP64 FLOP/site",
-            "units": sites, "avg_ms": avg_s * 1e3, "peak_kind": "measured in this run (FMA chains)"}
+def fp64_roofline(rc, ne: int, avg_s: float, hbm_gbs: float, peak_kind: str) -> dict:
+    """The FP64 path's reconstruction, whose values are formed in 64-bit fixed
+    point on the integer pipes: its algorithmic bytes against the HBM copy
+    peak."""
+    b, units, per = algorithmic("reconstruct", rc, False, ne)
+    ach = b / avg_s / 1e9
+    return {"kernel": "reconstruct", "bound": "hbm", "achieved": ach, "peak": hbm_gbs, "unit": "GB/s",
+            "frac": ach / hbm_gbs, "per_unit": per, "units": units, "avg_ms": avg_s * 1e3, "peak_kind": peak_kind}
 
 
 def step_bytes_per_update(rc, fp32: bool) -> float:
@@ -215,14 +206,11 @@ NCU_INSTR = {
 }
 SCHEDULERS = 4 * 152
 
-# The same figures for the 4D phase-space path's dominant kernel, captured on
-# its 64^4 workload (profiles/percolate4d_halos4d64_fp64.md).  The key hashes
-# the source up to the start of its reconstruction section: the percolation
-# kernels and everything they use come before it in the translation unit, so
-# changes further down cannot change their code.
+# The same figures for the 4D phase-space path, keyed over the source before
+# its reconstruction section (the map and what it uses): none of the present one.
 PHASE4D_PREFIX_END = "// Sec. 2.2.1: 15-point quadratic interpolation; transport reconstruction"
-NCU4_TRAFFIC = {"percolate": (236_288_768, "phase4d.cu", "908be1a679b46900")}
-NCU4_INSTR = {"percolate": (4_068_047_765, "phase4d.cu", "908be1a679b46900")}
+NCU4_TRAFFIC = {}
+NCU4_INSTR = {}
 
 
 def issue_roofline(kernel: str, avg_s: float, sm_mhz):
@@ -544,7 +532,7 @@ def run_native(args, rank: int, world: int, dist):
                              "top_kernels": {k: round(v[1], 3) for k, v in sorted(f64["stats"].items(), key=lambda kv: -kv[1][1])[:4]}}
         rl = f64["stats"].get("reconstruct")
         if rl and rl[0] > 0:
-            line["fp64_path"]["roofline"] = fp64_roofline(cells, rl[1] / rl[0] / 1e3)
+            line["fp64_path"]["roofline"] = fp64_roofline(rc, f64["ne"], rl[1] / rl[0] / 1e3, peaks["hbm_gbs"], peak_kind)
     if world == 1 and not args.no_ab:
         line["recon_tiles"] = recon_tiles_ab(V, rc, f0_dev, args, stats)
     if world == 1 and not args.no_cpu_baseline:
@@ -616,15 +604,22 @@ def run_reference(args, rank: int):
 # other workloads (their own JSON lines; not the headline)
 # ---------------------------------------------------------------------------
 
-# FP64 operations per unit of work of the 4D kernels, counted from the code:
-# one inverse-map evaluation Q(P) is 208 (dP 4, s_l 4 x 35, y 28, T^-1 s 28,
-# dQ 8); a distance d^2 adds 11; the 15-point interpolation with its
-# coordinates adds 97 per reconstructed site
-FLOP4_D2 = 219
-FLOP4_SITE = 305
+def algorithmic4(kernel: str, sites: int, padded: int, ne: int):
+    """(bytes, per-unit description) of one launch of a 4D kernel: what the
+    method must move at minimum."""
+    if kernel in ("reconstruct", "resample"):
+        # map, one read and one write of 8 bytes a site, a fixed-point record per element
+        return 20 * sites + 512 * ne, "20 B/site + 512 B/element"
+    if kernel == "sites":
+        # the proposed owner and its distance per padded site, the FP32 record per element
+        # (the three kernels of the pass: per launch a third of it)
+        return (8 * padded + 288 * ne) / 3, "8 B/padded site + 288 B/element over three launches"
+    if kernel == "sites_check":
+        return (8 * padded + 288 * ne) / 2, "8 B/padded site + 288 B/element over two launches"
+    return None
 
 
-def phase4d_run(args, dev, peaks, fp64_peak=None, clock_mhz=None) -> dict:
+def phase4d_run(args, dev, peaks, clock_mhz=None) -> dict:
     """The 4D phase-space path (2D space) on its 64^4 halo workload: K steps
     device-timed after the warm-up (remaps at their cadence inside), a
     profiled pass over the same step indices for the kernel shares and the
@@ -669,8 +664,6 @@ def phase4d_run(args, dev, peaks, fp64_peak=None, clock_mhz=None) -> dict:
     ev1 = s.map_stats()["d2_evals"]
     s.sync()
     del s
-    if fp64_peak is None:
-        fp64_peak = V.measure_fp64_peak()
     total = sum(v[1] for v in stats.values())
     dom = max(stats, key=lambda k: stats[k][1])
     nl, tms = stats[dom]
@@ -678,6 +671,16 @@ def phase4d_run(args, dev, peaks, fp64_peak=None, clock_mhz=None) -> dict:
     L4 = 1
     for a in range(4):
         L4 *= 2 * ((rc.n[a] - 1 + 2 * rc.s - 1) // (2 * rc.s)) + 3
+    padded = 1
+    for a in range(4):
+        padded *= rc.n[a] + 2 * rc.s
+
+    def hbm4(kernel: str, avg_ms: float) -> dict:
+        b, per = algorithmic4(kernel, sites, padded, L4)
+        ach = b / (avg_ms / 1e3) / 1e9
+        return {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
+                "frac": ach / peaks["hbm_gbs"], "per_unit": per, "units": sites}
+
     if dom == "percolate":
         # bound by instruction issue (FP32 tests, integer bookkeeping, atomics;
         # FP64 only at open decisions and contested claims): the capture's
@@ -695,12 +698,8 @@ def phase4d_run(args, dev, peaks, fp64_peak=None, clock_mhz=None) -> dict:
                      "peak_kind": "4 schedulers x 152 SMs x the SM clock",
                      "algorithmic_bytes": 4 * sites + (8 * 64 + 4 * 72) * L4,
                      "fp64_exact_distances_per_launch": (ev1 - ev0) / nl})
-    elif dom == "reconstruct":
-        flop = FLOP4_SITE * sites
-        ach = flop / (tms / nl / 1e3) / 1e12
-        roof.update({"bound": "alu", "achieved": ach, "peak": fp64_peak / 1e12, "unit": "TFLOP/s (FP64)",
-                     "frac": ach / (fp64_peak / 1e12), "per_unit": f"{FLOP4_SITE} FP64 FLOP per site",
-                     "units": sites, "peak_kind": "measured in this run (FP64 FMA chains)"})
+    elif algorithmic4(dom, sites, 1, L4) is not None:
+        roof.update(hbm4(dom, tms / nl))
     # end to end through the C ABI with host buffers over the same step
     # indices: upload of f0 from pinned host memory, then every timed step
     # reads the pixel masses back to the host
@@ -732,11 +731,7 @@ def phase4d_run(args, dev, peaks, fp64_peak=None, clock_mhz=None) -> dict:
     out["elements"] = L4
     rl = stats.get("reconstruct")
     if rl and rl[0] > 0:
-        # the FP64 reconstruction against the FP64 peak measured in this run
-        a_r = FLOP4_SITE * sites / (rl[1] / rl[0] / 1e3) / 1e12
-        out["reconstruct_roofline"] = {"bound": "alu", "achieved": a_r, "peak": fp64_peak / 1e12,
-                                       "unit": "TFLOP/s (FP64)", "frac": a_r / (fp64_peak / 1e12),
-                                       "per_unit": f"{FLOP4_SITE} FP64 FLOP per site", "avg_ms": rl[1] / rl[0]}
+        out["reconstruct_roofline"] = dict(hbm4("reconstruct", rl[1] / rl[0]), avg_ms=rl[1] / rl[0])
     if not args.no_cpu_baseline:
         out["cpu_baseline"] = cpu_baseline_4d(rc, f0)
     return out
