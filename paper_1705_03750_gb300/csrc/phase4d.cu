@@ -1182,9 +1182,9 @@ __device__ bool passes4(const G4& g, const int* k, const double* tself, const do
 //      pairs they name are listed;
 //   3. pair distances: one lane per pair, FP32 with bounds: a neighbour
 //      certainly closer fails the site, one whose comparison the bound
-//      leaves open sends the site to the exact test;
-//   4. exact work: the sites left open run the FP64 test in the oracle's
-//      order; every passing site's claim key takes its FP64 d^2.
+//      leaves open is compared in FP64, with the others left open;
+//   4. exact work: the sites whose ranges were left open run the FP64 test in
+//      the oracle's order; the passing sites are claimed.
 // The outcome is the all-FP64 percolation's.  Passing sites are claimed and
 // form the next frontier.  An element whose component would leave the window,
 // or whose lists outgrow their buffers, is listed for k4_percolate_big.
@@ -1222,7 +1222,7 @@ __device__ __forceinline__ void percolate_one(const G4& g, const double* __restr
   __shared__ float jht[4][32];   // (float)(l - R) * h_a for window coordinate l
   __shared__ double pst[4];      // the start site's coordinates
   __shared__ int org[4], kk[4];
-  __shared__ int go, ncur, ntest, npairs, ovf;
+  __shared__ int go, ncur, ntest, npairs, nopen, ovf;
   const int tid = threadIdx.x;
   unsigned nev = 0;
   if (tid < NT4) tself[tid] = tay[(size_t)NT4 * m + tid];
@@ -1316,7 +1316,7 @@ __device__ __forceinline__ void percolate_one(const G4& g, const double* __restr
       }
     }
     first = false;
-    if (tid == 0) npairs = 0;
+    if (tid == 0) npairs = nopen = 0;
     __syncthreads();
     const int nt = ovf ? 0 : min(ntest, TCAP);
     if (nt == 0) break;
@@ -1397,12 +1397,35 @@ __device__ __forceinline__ void percolate_one(const G4& g, const double* __restr
       eval32_4(tay32 + (size_t)NF4 * mm, pv, dp, x, e);
       const float dn = d2_32(x, e, &bn);
       const float dm = d2f[i], bm = bdf[i];
-      if (dn + bn < dm - bm)
+      if (dn + bn < dm - bm) {
         status[i] = ST_FAIL;
-      else if (!(dn - bn > dm + bm))
-        atomicMax(&status[i], ST_OPEN);
+      } else if (!(dn - bn > dm + bm)) {
+        const int at = atomicAdd(&nopen, 1);
+        if (at < FCAP)
+          front[at] = pr;  // (the frontier has been expanded)
+        else
+          atomicMax(&status[i], ST_OPEN);
+      }
     }
     if (tid == 0) ncur = 0;
+    __syncthreads();
+    // the pairs that the bounds left open, in FP64 (the other neighbours of the
+    // site's ranges are certainly farther or have failed it)
+    for (int j = tid; j < min(nopen, FCAP); j += blockDim.x) {
+      const int pr = front[j], i = pr >> 7;
+      if (status[i] != ST_PASS) continue;
+      int code = pr & 127, o[4], l[4], mm = 0;
+      for (int a = 3; a >= 0; a--) {
+        o[a] = code % 3 - 1;
+        code /= 3;
+      }
+      for (int a = 0; a < 4; a++) mm = mm * g.L[a] + kl[a] + o[a];
+      decode_w(tlist[i], W, l);
+      double P[4];
+      for (int a = 0; a < 4; a++) P[a] = site_coord(g, a, (long long)org[a] + l[a]);
+      nev += 2;
+      if (dist2_4(g, tay + (size_t)NT4 * mm, P, nullptr) < dist2_4(g, tself, P, nullptr)) status[i] = ST_FAIL;
+    }
     __syncthreads();
     // 4. exact tests where the bounds left them open; claims
     for (int i = tid; i < nt; i += blockDim.x) {
