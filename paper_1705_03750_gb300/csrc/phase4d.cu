@@ -9,20 +9,27 @@
 //   k4_drift        half drift of every element (one thread per element)
 //   k4_taylor       T^-1 = adj(T)/det T and G_l = [T^-1]^T H_l T^-1
 //   k4_records      the inverse map's FP32 and fixed-point records
-//   k4_percolate    one block per element: breadth-first flood fill of its
+//   k4_sites, k4_sites_check   the site pass: the closest element of every
+//                   site and the local conditions under which these sites are
+//                   its component (k4_gaps and k4_site_hints prepare it,
+//                   k4_flood_list lists the elements it leaves)
+//   k4_percolate    one block per element left: breadth-first flood fill of its
 //                   component in a shared-memory bit window around its start
 //                   site, frontier waves in shared memory, claims by a 128-bit
 //                   compare-and-swap minimum of (d^2 bits, element index);
 //                   k4_percolate_big fills the elements that left their window
-//                   again over the whole padded lattice (global-memory bits)
-//   k4_map_finish   owner of every site from its slot or record; hole list
+//                   again over the whole padded lattice (global-memory bits),
+//                   k4_late_claims makes its claims
+//   k4_map_finish   owner of every site from its slot, record or the site
+//                   pass; hole list
 //   k4_holes        Jacobi rounds of the unexplored-site repair (one block)
 //   k4_recon        one block per (x, y) pixel: f at its vx-vy plane by the
 //                   15-point interpolation of f_ini at Q(P); pixel mass by a
 //                   block reduction (the v-integration fused in)
-//   k4_accel        direct sum of the 2D Green function over the pixel masses
-//                   for the nodes of the grid and a halo, sources split over
-//                   blocks; k4_accel_sum adds the partial sums in order
+//   k4_accel        direct sum of the 2D Green function (k4_green's table) over
+//                   the pixel masses for the nodes of the grid and a halo,
+//                   sources split over blocks; k4_accel_sum adds the partial
+//                   sums in order, k4_cache_fields forms the nodes' differences
 //   k4_kick_drift   2D TSC of the field, its gradient and Hessian (centred
 //                   differences) at the element; kick; second half drift
 //   remap           k4_resample (Q_r blend of the beta set, 4^4-term cubic
@@ -37,9 +44,9 @@
 // outcome; the map is therefore exactly the one that restatement gives for
 // the same elements.  Values that feed no such decision (the interpolated f,
 // the Q_r blend, the spline sums) use 64-bit fixed point (fixed.cuh) or fused
-// FP64 arithmetic and agree with it to rounding; the spline solve divides by the same pivots in the same order;
-// the pixel masses are block sums and the field is summed over blocks, so
-// element trajectories agree to rounding.
+// FP64 arithmetic and agree with it to rounding; the spline solve divides by the
+// same pivots in the same order; the pixel masses are block sums and the field
+// is summed over blocks, so element trajectories agree to rounding.
 
 #include <cuda_runtime.h>
 #include <limits.h>
@@ -564,9 +571,9 @@ __device__ __forceinline__ void claim4(ulonglong2* key, unsigned long long dbits
 // k4_site_hints prepares each tile's guess, k4_sites proposes the owners and
 // tests them, k4_sites_check looks at each site's eight neighbours.  A site
 // costs about one evaluation of its own, up to 0.7 of neighbours beyond the alpha
-// box and up to 2 of owners next to it, where the flood fill tested three sites for each
-// of a component's and formed its shell: 64^4 sites 2.5 ms and 0.4 ms for
-// the elements left to the fill, where the fill of all took 8.8 ms; without
+// box and up to 2 of owners next to it, where the flood fill tested three sites
+// for each of a component's and formed its shell: 64^4 sites 2.5 ms and 0.4 ms
+// for the elements left to the fill, where the fill of all took 8.8 ms; without
 // k4_gaps, which settles most neighbours without an evaluation, 3.1 ms.  Bound by
 // the records' reads (288 bytes an evaluation through L1) and by occupancy: with
 // whole records held in registers (2 blocks an SM) and the guess formed inside
