@@ -506,8 +506,10 @@ void launch_spline_solve(vm_solver* s, const void* src, void* dst) {
 // solver's, and a group's.
 bool spline_prepare(const vm_solver* s) {
   if (!filters_on(s->g)) return true;
-  return s->fp32 ? cols_prepare(k_cols_filter<float, COL_W>, 4) && cols_prepare(k_cols_filter<float, COL_W_FEW>, 4)
-                 : cols_prepare(k_cols_filter<double, COL_W>, 8) && cols_prepare(k_cols_filter<double, COL_W_FEW>, 8);
+  const bool few = col_warps(s->g) == COL_W_FEW;
+  if (s->fp32)
+    return few ? cols_prepare(k_cols_filter<float, COL_W_FEW>, 4) : cols_prepare(k_cols_filter<float, COL_W>, 4);
+  return few ? cols_prepare(k_cols_filter<double, COL_W_FEW>, 8) : cols_prepare(k_cols_filter<double, COL_W>, 8);
 }
 bool group_spline_prepare() {
   return cols_prepare(k_cols_group<double>, 8) && cols_prepare(k_cols_group<float>, 4) &&
