@@ -1375,15 +1375,18 @@ __device__ __forceinline__ void percolate_one(const G4& g, const double* __restr
             }
       if (cnt) {
         const int at = atomicAdd(&npairs, cnt);
-        if (at + cnt <= PCAP) {
+        if (at + cnt <= PCAP)
           for (int q = 0; q < cnt; q++) pairs[at + q] = (i << 7) | codes[q];
-        } else {
-          ovf = 1;
-        }
       }
     }
     __syncthreads();
-    if (ovf) break;
+    // (the count itself tells that the list is full: ovf, which decides the exit
+    // above, is not written while a warp may still read it there, so that every
+    // exit is taken by the whole block, whose next element reuses all of this)
+    if (npairs > PCAP) {
+      if (tid == 0) ovf = 1;
+      break;
+    }
     // 3. the neighbours' distances at the listed sites, FP32 with bounds
     const int np = npairs;
     for (int j = tid; j < np; j += blockDim.x) {
