@@ -92,7 +92,7 @@ __device__ __forceinline__ void taylor_fixed(const Grid& g, const double (&t)[TY
 #pragma unroll
   for (int L = FX_LIM; L >= 2; L >>= 1) {
     const float p = ((float)L + 0.51f) / sf;
-    if (lim == 0 && 0.51f + sf * (C1 * p + C2 * (p * p)) < (float)FX_MAX) lim = L;
+    if (lim == 0 && 0.51f + sf * (C1 * p + C2 * (p * p)) < (float)FX_MAX) lim = L + 1;
   }
   if (!(fabs(iu) < 1e6 && fabs(iw) < 1e6)) lim = 0;
   if (lim == 0) {

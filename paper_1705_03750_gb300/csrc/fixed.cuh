@@ -29,7 +29,7 @@ constexpr long long FX_MARGIN = 1ll << (FX_Q - 26);
 struct __align__(16) FxRec {
   long long c[12];
   int i0, l0, Bu, Bw;
-  int lim;  // largest |j|, |l| the record serves (0: none)
+  int lim;  // the record serves sites with |j|, |l| < lim (0: none, not the start site either)
   int pad[3];
 };
 static_assert(sizeof(FxRec) == 128, "one cache line per element");
@@ -128,7 +128,7 @@ __device__ __forceinline__ bool fx_offset(const FxRec* __restrict__ X, int i, in
   const int dj = i - o.x, dl = j - o.y;
   ru = fx_poly(x0, x1, x2, dj, dl);
   rw = fx_poly(v0, v1, v2, dj, dl);
-  return max(abs(dj), abs(dl)) <= lim;
+  return max(abs(dj), abs(dl)) < lim;
 }
 
 // Square root of d2 (2^-60 units, 0 <= d2 < 2^60) in 2^-62 units: an FP32

@@ -317,8 +317,8 @@ __global__ void __launch_bounds__(128) k4_taylor(G4 g, const double* __restrict_
 // axis the 15 coefficients of the index position of Q at a site, relative to
 // the integer anchor B, as a polynomial of the site's offset j from the
 // element's start site i0: c0 + sum_b j_b (c_b + sum_{c>=b} j_c c_bc); the
-// sixteenth word packs i0 (low half) and B << 8 | lim, lim the largest |j|
-// served (0: none).
+// sixteenth word packs i0 (low half) and B << 8 | lim, the sites with every |j|
+// below lim being served (0: none, not the start site either).
 struct Fx4 {
   long long c[4][16];
 };
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(128) k4_records(G4 g, const double* __restrict
   for (int Lm = FX4_LIM; Lm >= 2; Lm -= 2) {
     const float p = ((float)Lm + 0.51f) / (float)g.s;
     const float sf = (float)g.s;
-    if (lim == 0 && 0.51f + sf * (n1 * p + n2 * (p * p)) < (float)FX4_MAX && sf * n3 * (p * p) < 6e3f) lim = Lm;
+    if (lim == 0 && 0.51f + sf * (n1 * p + n2 * (p * p)) < (float)FX4_MAX && sf * n3 * (p * p) < 6e3f) lim = Lm + 1;
   }
   // start site along this axis and its distance from P_m
   const double u = M_(S_(t[a], g.lo[a]), g.inv_d[a]);
@@ -467,7 +467,7 @@ __device__ __forceinline__ bool fx4_start(const Fx4* __restrict__ X, const int* 
     lim = hi & 255;
     far = max(far, abs(j[a]));
   }
-  return far <= lim;
+  return far < lim;
 }
 
 // FP32 offsets xi of an element at a site with rigorous bounds e_a >=
