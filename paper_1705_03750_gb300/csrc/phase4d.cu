@@ -378,7 +378,9 @@ __global__ void __launch_bounds__(128) k4_records(G4 g, const double* __restrict
       const float Bf = (float)B;
       r[16 + 10 * a + sym4(b, c)] = Bf;
       nb += fabsf(Bf);
-      Q[sym4(b, c)] = fabs(B) < FX4_MAX ? vm::fx_of(B * inv_s, FX4_Q) : 0;
+      // (cells per site^2: B itself may be up to s times the format's range where
+      // the record still serves a few sites)
+      Q[sym4(b, c)] = fabs(B * inv_s) < FX4_MAX ? vm::fx_of(B * inv_s, FX4_Q) : 0;
     }
   na *= 1.000001f;
   nb *= 1.000001f;

@@ -105,3 +105,40 @@ def test_4d_values_beside_an_element_without_a_record(n, s, change):
     g.remap()
     g.sync()
     assert np.abs(g.read_fini() - fr).max() <= 1e-12 * np.abs(fr).max()
+
+
+# a second-order term that a served offset multiplies by little: 65 element
+# spacings per spacing squared, 6 at two sites from the start at stride 8
+@pytest.mark.parametrize("b", [40.0, 65.0])
+def test_4d_values_of_an_element_with_a_strong_second_order_term(b):
+    n, s = (17, 11, 19, 12), 8
+    rc = I4.HALOS4D_16.with_(n=n, s=s, n_s=50)
+    f0 = I4.initial_f4(rc)
+    g = V4.Solver4D(V4.config(rc))
+    o = Q.Oracle4D.from_run(rc)
+    g.set_f(f0)
+    o.set_f(f0)
+    g.step(1)
+    o.step(1)
+    el = o.elements()
+    m = 0
+    for a in range(4):
+        m = m * o.Ldims[a] + o.Ldims[a] // 2
+    dm = s * np.array(rc.d)
+    j = round((el[m, 2] - rc.lo[2]) / rc.d[2])
+    el[m, 2] = rc.lo[2] + (j - 0.3) * rc.d[2]
+    el[m, 4:20] = np.eye(4).ravel()
+    el[m, 20:60] = 0.0
+    el[m, 20 + 7] = -2.0 * b * dm[0] / dm[2] ** 2       # H_x,vx vx
+    o.set_elements(el)
+    g.set_elements(el)
+    fo = o.reconstruct()
+    owners = o.last_map()
+    g.reconstruct()
+    g.sync()
+    assert (g.read_map() == owners).all() and (owners == m).any()
+    assert np.abs(g.read_f() - fo).max() <= 1e-12 * np.abs(fo).max()
+    fr, _ = o.remap_resample()
+    g.remap()
+    g.sync()
+    assert np.abs(g.read_fini() - fr).max() <= 1e-12 * np.abs(fr).max()
