@@ -651,6 +651,65 @@ __device__ __forceinline__ int warp_offsets(int n, int& total) {
   return off;
 }
 
+// An element's map along the column j of sites, two quadratics in px.
+struct SiteColumn {
+  float ax, bx, cx, av, bv, cv, f0, pa, eq, eD;
+  int is;         // row of the element's start site
+  uint32_t base;  // its tile word at that row
+};
+
+__device__ __forceinline__ SiteColumn site_column(const Grid& g, const float* __restrict__ tayl, int k, int l, int j,
+                                                  float inv_s) {
+  const float4* F = reinterpret_cast<const float4*>(tayl + (size_t)(k * g.Lv + l) * TL_N);
+  const float4 ra = __ldg(F), rb = __ldg(F + 1), rc = __ldg(F + 2), rd = __ldg(F + 3);
+  const int js = j - __float_as_int(rd.y);
+  const float pv = ((float)js - rc.w) * inv_s;
+  SiteColumn c;
+  c.is = __float_as_int(rd.x);
+  c.f0 = -rc.z * inv_s;
+  c.ax = rb.x;
+  c.bx = fmaf(rb.y, pv, ra.x);
+  c.cx = pv * fmaf(rb.z, pv, ra.y);
+  c.av = rb.w;
+  c.bv = fmaf(rc.x, pv, ra.z);
+  c.cv = pv * fmaf(rc.y, pv, ra.w);
+  c.pa = fabsf(pv);
+  c.eq = rd.z;
+  c.eD = fabsf(rd.w);
+  c.base = site_word(k, l, 0, js, true, rd.w < 0.f, false);
+  return c;
+}
+
+// The guess at row i of the column: its tile word, an upper bound of its d^2, and
+// whether it needs no comparison (inside the alpha box), one (outside it on one
+// axis: beyond v where ix, else beyond x; towards + where pos) or more (both axes,
+// an open side, a poor guess, beyond the bounds' |p|).  The tile and the ring of
+// its neighbours both take a site's class from here, by the same operations: the
+// lists choose differently among elements that are equally close, so a site on
+// two different ones could have two owners.
+struct SiteGuess {
+  uint32_t w;
+  float up;
+  bool in, one, ix, pos;
+};
+
+__device__ __forceinline__ SiteGuess site_guess(const SiteColumn& c, int i, float inv_s, float alo, float ahi) {
+  const int di = i - c.is;
+  const float px = fmaf((float)di, inv_s, c.f0);
+  const float qx = fmaf(px, fmaf(c.ax, px, c.bx), c.cx), qv = fmaf(px, fmaf(c.av, px, c.bv), c.cv);
+  const float Pm = fmaxf(fabsf(px), c.pa), e = fmaf(c.eq, Pm, kAbs), ed = fmaf(c.eD, Pm * Pm, kAbs);
+  const float mx = fabsf(qx), mv = fabsf(qv), lo = alo - e, hi = ahi + e;
+  const bool good = Pm <= TL_P, iv = mv < lo;
+  SiteGuess s;
+  s.w = c.base | ((di > 0 ? 1u : 0u) | (di < 0 ? 4u : 0u)) << SO_DIR;
+  s.up = fmaf(qx, qx, qv * qv) + ed;
+  s.ix = mx < lo;
+  s.in = good && s.ix && iv;
+  s.one = good && ((s.ix && mv > hi && mv <= 0.75f) || (iv && mx > hi && mx <= 0.75f));
+  s.pos = (s.ix ? qv : qx) > 0.f;
+  return s;
+}
+
 struct SiteShared {
   uint32_t so[SITE_RR * SITE_CC];
   float sd[SITE_RR * SITE_CC];  // an upper bound of the owner's d^2
@@ -760,9 +819,8 @@ __device__ __forceinline__ void map_sites_body(const Grid& g, const SiteArgs& X,
     const float dj = (float)((c0 - 1) % HINT_S) - 0.5f * (HINT_S - 1);
     float kf = fmaf(h.kl, dj, fmaf(h.kj, -0.5f * (HINT_S - 1), h.k));
     float lf = fmaf(h.ll, dj, fmaf(h.lj, -0.5f * (HINT_S - 1), h.l));
-    uint32_t cur = SO_NONE, base = SO_NONE;
-    float ax = 0.f, bx = 0.f, cx = 0.f, av = 0.f, bv = 0.f, cv = 0.f, f0 = 0.f, pa = 0.f, eq = 0.f, eD = 0.f;
-    int is = 0;
+    uint32_t cur = SO_NONE;
+    SiteColumn col = {};
     for (int t = 0; t < HINT_S; t++) {
       const int i = i0 + t, idx = at0 + t * SITE_CC;
       const int k = clampi(__float2int_rn(kf), g.klo, g.khi), l = clampi(__float2int_rn(lf), g.llo, g.lhi);
@@ -770,43 +828,18 @@ __device__ __forceinline__ void map_sites_body(const Grid& g, const SiteArgs& X,
       lf += h.lj;
       const uint32_t kl = (uint32_t)(k << 12 | l);
       if (kl != cur) {
-        const float4* F = reinterpret_cast<const float4*>(X.tayl + (size_t)(k * g.Lv + l) * TL_N);
-        const float4 ra = __ldg(F), rb = __ldg(F + 1), rc = __ldg(F + 2), rd = __ldg(F + 3);
-        const int js = j0 - __float_as_int(rd.y);
-        const float pv = ((float)js - rc.w) * inv_s;
-        is = __float_as_int(rd.x);
-        f0 = -rc.z * inv_s;
-        ax = rb.x;
-        bx = fmaf(rb.y, pv, ra.x);
-        cx = pv * fmaf(rb.z, pv, ra.y);
-        av = rb.w;
-        bv = fmaf(rc.x, pv, ra.z);
-        cv = pv * fmaf(rc.y, pv, ra.w);
-        pa = fabsf(pv);
-        eq = rd.z;
-        eD = fabsf(rd.w);
-        base = site_word(k, l, 0, js, true, rd.w < 0.f, false);
+        col = site_column(g, X.tayl, k, l, j0, inv_s);
         cur = kl;
       }
-      const int di = i - is;
-      const float px = fmaf((float)di, inv_s, f0);
-      const float qx = fmaf(px, fmaf(ax, px, bx), cx), qv = fmaf(px, fmaf(av, px, bv), cv);
-      const float Pm = fmaxf(fabsf(px), pa), e = fmaf(eq, Pm, kAbs), ed = fmaf(eD, Pm * Pm, kAbs);
-      const float mx = fabsf(qx), mv = fabsf(qv), lo = X.alo - e, hi = X.ahi + e;
+      const SiteGuess q = site_guess(col, i, inv_s, X.alo, X.ahi);
       const bool on = col_in && (unsigned)(i + g.pad) < (unsigned)PX;
-      S.so[idx] = on ? base | ((di > 0 ? 1u : 0u) | (di < 0 ? 4u : 0u)) << SO_DIR : SO_NONE;
-      S.sd[idx] = fmaf(qx, qx, qv * qv) + ed;
-      // inside the alpha box no neighbour is compared; outside it on one axis,
-      // one; the rest (both axes, an open side, a poor guess, beyond the
-      // record's bounds) are the block's list
-      const bool good = Pm <= TL_P, ix = mx < lo, iv = mv < lo;
-      const bool in = good && ix && iv;
-      const bool one = good && ((ix && mv > hi && mv <= 0.75f) || (iv && mx > hi && mx <= 0.75f));
+      S.so[idx] = on ? q.w : SO_NONE;
+      S.sd[idx] = q.up;
       const uint32_t bit = 1u << t;
-      if (on && one) e1 |= bit;
-      if (on && !one && !in) e2 |= bit;
-      if (ix) eax |= bit;
-      if ((ix ? qv : qx) > 0.f) esg |= bit;
+      if (on && q.one) e1 |= bit;
+      if (on && !q.one && !q.in) e2 |= bit;
+      if (q.ix) eax |= bit;
+      if (q.pos) esg |= bit;
     }
     int k1, k2;
     int o1 = n1 + warp_offsets(__popc(e1), k1), o2 = warp_offsets(__popc(e2), k2);
@@ -844,15 +877,13 @@ __device__ __forceinline__ void map_sites_body(const Grid& g, const SiteArgs& X,
           lf += h.lj;
         }
         const int k = clampi(__float2int_rn(kf), g.klo, g.khi), l = clampi(__float2int_rn(lf), g.llo, g.lhi);
-        const SiteQ q = site_q(X.tayl, X.tayf, k * g.Lv + l, i, j, inv_s);
-        const float mx = fabsf(q.qx), mv = fabsf(q.qv), lo = X.alo - q.e, hi = X.ahi + q.e;
-        const bool iv = mv < lo;
-        ix = mx < lo;
-        one = (ix && mv > hi && mv <= 0.75f) || (iv && mx > hi && mx <= 0.75f);
-        hard = !one && !(ix && iv);
-        pos = (ix ? q.qv : q.qx) > 0.f;
-        dup = q.d2 + q.ed;
-        w = site_word(k, l, q.di, q.dj, true, q.out, false);
+        const SiteGuess q = site_guess(site_column(g, X.tayl, k, l, j, inv_s), i, inv_s, X.alo, X.ahi);
+        ix = q.ix;
+        one = q.one;
+        hard = !q.one && !q.in;
+        pos = q.pos;
+        dup = q.up;
+        w = q.w;
       }
       S.so[idx] = w;
       S.sd[idx] = dup;
