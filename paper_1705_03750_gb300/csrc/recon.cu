@@ -409,6 +409,7 @@ __device__ __forceinline__ bool remap64_fixed(const Grid& g, const FxRec* __rest
   const int k = m / g.Lv, l = m - k * g.Lv;
   const long long s52 = (long long)g.s << FX_Q;
   long long nu = 0, nw = 0, den = 0;
+  bool others = false;  // elements besides the owner have a weight
   for (int a = a0; a <= a1; a++)
     for (int b = b0; b <= b1; b++) {
       if ((ina || inb) && a != 0 && b != 0) continue;
@@ -431,7 +432,12 @@ __device__ __forceinline__ bool remap64_fixed(const Grid& g, const FxRec* __rest
       nu += fx_mul62(Dx, w);
       nw += fx_mul62(Dv, w);
       den += w >> 3;
+      others = others || a != 0 || b != 0;
     }
+  // the products' last bit, 2^-52 cells, and the weights', 2^-59, over a sum of 2^-7:
+  // 1e-13 to 4e-13 cells, where FP64 positions carry as much; smaller sums (an undeformed
+  // lattice has 0.2 at least) go to FP64, whose weights 2 (1 - d)^3 keep their digits
+  if (others && den < 1ll << (59 - 7)) return false;
   if (den > 0) {
     ru += fx_div(nu, den);
     rw += fx_div(nw, den);
