@@ -2383,6 +2383,7 @@ __device__ __forceinline__ bool resample4_fixed(const G4& g, const Fx4* __restri
   // products keep all bits until the division)
   __int128 num[4] = {0, 0, 0, 0};
   unsigned long long den = 0;
+  bool others = false;  // elements besides the owner have a weight
   // The elements of the blend: every subset of the axes that are not full, each
   // towards its side, and one step either way along a full axis alone; at most
   // 16, counted off by each lane for itself (nested loops over the ranges made a
@@ -2429,7 +2430,11 @@ __device__ __forceinline__ bool resample4_fixed(const G4& g, const Fx4* __restri
       num[a] += (__int128)D[a] * w;
     }
     den += (unsigned long long)w >> 3;
+    others = others || set != 0;
   }
+  // a weight's last bits, some 2^-60, over a sum of 2^-10: 2^-48 of the differences,
+  // as much as of an FP64 blend's; smaller sums take that one
+  if (others && den < 1ull << (59 - 10)) return false;
   const int z = den > 0 ? max(__clzll((long long)den) - 4, 0) : 0;  // both scaled by 2^z for the division
   int gk[4][4], wh[4][4], wl[4][4];
 #pragma unroll
