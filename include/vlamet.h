@@ -118,7 +118,9 @@ typedef struct {
   int32_t cycle;    /* steps since the last remap */
   int32_t holes;    /* unexplored sites repaired by the last map */
   int32_t hole_rounds;
-  int32_t overflow_elements; /* elements whose component leaves the 32 x 64 window */
+  int32_t overflow_elements; /* elements whose component leaves the small windows: 32 x 64 sites around the
+                                start site, 16 x 32 for an element on the rim of the lattice (its flood
+                                fill takes a large window; the site pass settles many without one) */
   int32_t tier1_more;        /* elements whose small-window fill tested sites beyond
                                 the region predicted from the linear part of the map */
   int32_t last_tier_elements; /* elements filled in the whole-lattice window */

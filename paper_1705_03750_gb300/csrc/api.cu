@@ -774,6 +774,7 @@ vm_status vm_diagnostics(vm_solver* s, vm_diag* d) {
   VM_CUDA_TRY(cudaMemcpyAsync((char*)s->ds + off, (char*)&h + off, end - off, cudaMemcpyHostToDevice, s->stream));
   vm::launch_diagnostics(s);
   vm::launch_emap(s);
+  vm::launch_count_wide(s);
   VM_CUDA_TRY(cudaMemcpyAsync(&h, s->ds, sizeof h, cudaMemcpyDeviceToHost, s->stream));
   vm_status st = vm_sync(s);
   if (st != VM_OK) return st;

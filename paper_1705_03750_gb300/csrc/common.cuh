@@ -115,7 +115,7 @@ struct DevState {
   int32_t fresh;          // the elements were reset (isotropic, on their lattice) since the last map
   int32_t skip_sites;     // the current map runs without the site pass (kept ties, see Grid::tie_v)
   uint32_t barrier;       // arrivals at the flood fill's grid barriers
-  int32_t wide;           // elements of the site pass whose component leaves the 32 x 64 window (statistics)
+  int32_t wide;           // settled elements whose component leaves the small windows (launch_count_wide)
   uint32_t epoch;        // epoch of the current influence map (even, below kEpochs)
   double Mtot;           // total mass of the last reconstruction
   double sum_mass, sum_kin, sum_pot;
@@ -214,6 +214,7 @@ constexpr int PROF_CAP = 1024;
 struct vm_solver {
   vm_config cfg;
   vm::Grid g;
+  vm::Grid gmap;            // of the last single-solve map (its computing domain); ne 0: none yet
   cudaStream_t stream;
   int32_t fp32;            // 1: f_ini, eta, f stored as float
   size_t sreal;            // bytes per stored real
@@ -344,6 +345,7 @@ void launch_rho_max(vm_solver* s);
 // map.cu
 bool map_prepare(const Grid& g);
 void launch_map(vm_solver* s);
+void launch_count_wide(vm_solver* s);
 void launch_read_map(vm_solver* s, int32_t* dst);
 // recon.cu
 void launch_reconstruct(vm_solver* s);
@@ -614,7 +616,7 @@ __device__ __forceinline__ void map_begin(const Grid& g, DevState* ds) {
   ds->noverflow_back = 0;
   ds->nseed = 0;
   ds->n_pair_esc = 0;
-  ds->n_flood = ds->wide = 0;
+  ds->n_flood = ds->wide = 0;  // (wide stays 0 until it is asked for)
   ds->barrier = 0;
   ds->emap2_bits = 0ull;  // E_map describes the current map only
   ds->emap_hit = 0;

@@ -231,7 +231,8 @@ __device__ __forceinline__ void key_min(unsigned long long* key2, unsigned long 
 }
 
 // Per-element flags of the site pass (vm_solver::flags): (a), (b) or (c) does
-// not hold somewhere; counted as wide; its start site is its own.  The site
+// not hold somewhere; its component leaves the small windows (set when asked for,
+// k_map_wide); its start site is its own.  The site
 // pass's proposals stand for the elements with the last and not the first.
 constexpr uint32_t EF_BAD = 1u, EF_WIDE = 2u, EF_START = 4u;
 __device__ __forceinline__ bool elem_settled(uint32_t w) { return (w & ~EF_WIDE) == EF_START; }
@@ -488,8 +489,7 @@ constexpr int SO_DIR = 24;
 constexpr uint32_t SO_ELEM = 0xFFFFFFu;
 constexpr uint32_t SO_NONE = SO_ELEM;     // no owner proposed (outside the padded lattice)
 constexpr uint32_t SO_UNSURE = 1u << 28;  // (a) does not hold
-constexpr uint32_t SO_FAR = 1u << 29;     // the site lies outside a 32 x 64 window around the owner
-constexpr uint32_t SO_OUT = 1u << 30;     // the owner starts outside the padded lattice: it claims nothing
+constexpr uint32_t SO_OUT = 1u << 29;     // the owner starts outside the padded lattice: it claims nothing
 static_assert(SITE_RR * SITE_CC < 4096 && SITE_R % HINT_S == 0 && SITE_C % HINT_S == 0, "tile index in 12 bits");
 static_assert(HINT_R * HINT_C <= SITE_T, "one thread per guess");
 static_assert(SITE_HB * SITE_T * HINT_S == SITE_R * SITE_C && SITE_T % SITE_C == 0 && HINT_S == 8, "a thread's column");
@@ -559,12 +559,13 @@ __device__ __forceinline__ SiteHint site_hint(const Grid& g, const float* __rest
     const float px = ((ci - (float)ui.x) - c.z) * inv_s, pv = ((cj - (float)ui.y) - c.w) * inv_s;
     const float near = fmaxf(fabsf(px), fabsf(pv)) < 4.f ? 1.f : 0.f;
     const float A = near * b.x, B = near * b.y, C = near * b.z, D = near * b.w, E = near * c.x, F = near * c.y;
-    h.k = (float)k + (px * (a.x + A * px + B * pv) + pv * (a.y + C * pv));
-    h.l = (float)l + (px * (a.z + D * px + E * pv) + pv * (a.w + F * pv));
-    h.kj = (a.x + 2.f * A * px + B * pv) * inv_s;
-    h.kl = (a.y + B * px + 2.f * C * pv) * inv_s;
-    h.lj = (a.z + 2.f * D * px + E * pv) * inv_s;
-    h.ll = (a.w + E * px + 2.f * F * pv) * inv_s;
+    // (fused where written: every kernel forms the same guesses)
+    h.k = fmaf(px, fmaf(A, px, fmaf(B, pv, a.x)), fmaf(pv, fmaf(C, pv, a.y), (float)k));
+    h.l = fmaf(px, fmaf(D, px, fmaf(E, pv, a.z)), fmaf(pv, fmaf(F, pv, a.w), (float)l));
+    h.kj = fmaf(2.f * A, px, fmaf(B, pv, a.x)) * inv_s;
+    h.kl = fmaf(B, px, fmaf(2.f * C, pv, a.y)) * inv_s;
+    h.lj = fmaf(2.f * D, px, fmaf(E, pv, a.z)) * inv_s;
+    h.ll = fmaf(E, px, fmaf(2.f * F, pv, a.w)) * inv_s;
     const int k2 = clampi(__float2int_rn(h.k), g.klo, g.khi), l2 = clampi(__float2int_rn(h.l), g.llo, g.lhi);
     if (k2 == k && l2 == l) break;
     k = k2;
@@ -573,9 +574,20 @@ __device__ __forceinline__ SiteHint site_hint(const Grid& g, const float* __rest
   return h;
 }
 
-__device__ __forceinline__ uint32_t site_word(int k, int l, int di, int dj, bool sure, bool out, bool far) {
+__device__ __forceinline__ uint32_t site_word(int k, int l, int di, int dj, bool sure, bool out) {
   const uint32_t to = (di > 0 ? 1u : 0u) | (dj > 0 ? 2u : 0u) | (di < 0 ? 4u : 0u) | (dj < 0 ? 8u : 0u);
-  return (uint32_t)(k << 12 | l) | to << SO_DIR | (sure ? 0u : SO_UNSURE) | (out ? SO_OUT : 0u) | (far ? SO_FAR : 0u);
+  return (uint32_t)(k << 12 | l) | to << SO_DIR | (sure ? 0u : SO_UNSURE) | (out ? SO_OUT : 0u);
+}
+
+// Does the component of element (k, l) leave the flood fill's last small window at
+// site (i, j) of it, by being on its edge or beyond where the padded lattice goes
+// on?  32 x 64 sites about the start site; 16 x 32 for an element with a neighbour
+// missing, which goes from tier 0 straight to the large windows.
+__device__ __forceinline__ bool leaves_window(const Grid& g, const float* __restrict__ tayl, int k, int l, int i, int j) {
+  const int2 st = __ldg(reinterpret_cast<const int2*>(tayl + (size_t)(k * g.Lv + l) * TL_N + TL_I0));
+  const int h = k <= g.klo || k >= g.khi || l <= g.llo || l >= g.lhi ? 8 : TR / 2, di = i - st.x, dj = j - st.y;
+  return (di <= -h && st.x - h - 1 >= -g.pad) || (di >= h - 1 && st.x + h < g.nx + g.pad) ||
+         (dj <= -2 * h && st.y - 2 * h - 1 >= -g.pad) || (dj >= 2 * h - 1 && st.y + 2 * h < g.nv + g.pad);
 }
 
 // The owner of site (i, j) from the exact FP64 distances, starting from
@@ -612,7 +624,7 @@ __device__ __noinline__ uint32_t site_owner_exact(const Grid& g, const double* _
   dup = __double2float_ru(d2);
   const float* R = tayl + (size_t)(k * g.Lv + l) * TL_N;
   const int2 st = __ldg(reinterpret_cast<const int2*>(R + TL_I0));
-  return site_word(k, l, i - st.x, j - st.y, sure && dup < 1e30f, __ldg(R + TL_ED) < 0.f, false);
+  return site_word(k, l, i - st.x, j - st.y, sure && dup < 1e30f, __ldg(R + TL_ED) < 0.f);
 }
 
 // Does the test of element (k, l) fail at site (i, j)?  The neighbours it
@@ -676,7 +688,7 @@ __device__ __forceinline__ SiteColumn site_column(const Grid& g, const float* __
   c.pa = fabsf(pv);
   c.eq = rd.z;
   c.eD = fabsf(rd.w);
-  c.base = site_word(k, l, 0, js, true, rd.w < 0.f, false);
+  c.base = site_word(k, l, 0, js, true, rd.w < 0.f);
   return c;
 }
 
@@ -778,13 +790,17 @@ __device__ __noinline__ void site_edge(const Grid& g, const SiteArgs& X, SiteSha
   float dup = q.d2 + q.ed;
   uint32_t w;
   if (sure && dup < 1e30f)
-    w = site_word(k + ba, l + bb, q.di, q.dj, true, q.out, abs(q.di) > TR / 2 || abs(q.dj) > 32);
+    w = site_word(k + ba, l + bb, q.di, q.dj, true, q.out);
   else
     w = site_owner_exact(g, X.tay, X.tayl, k + ba, l + bb, i, j, dup);
   S.so[idx] = w;
   S.sd[idx] = dup;
 }
 
+// kWide: instead of the owner slots and the proof, mark the settled elements whose
+// component leaves the small windows (a statistic, formed when it is asked for: in
+// the map's own pass it took 18 us of 300 at 4096 x 4096).
+template <bool kWide>
 __device__ __forceinline__ void map_sites_body(const Grid& g, const SiteArgs& X, int vb) {
   __shared__ SiteShared S;
   if (g.khi < g.klo || g.lhi < g.llo) return;  // no element exists
@@ -914,7 +930,7 @@ __device__ __forceinline__ void map_sites_body(const Grid& g, const SiteArgs& X,
     // certainly the neighbour's, whose own test then compares with m only
     const int A2 = side_f(n.qx, n.e, X.alo, X.ahi), B2 = side_f(n.qv, n.e, X.alo, X.ahi);
     if (dup < low && (A2 == 0 || (A2 == -A && A != 0)) && (B2 == 0 || (B2 == -B && B != 0)))
-      w = site_word(k + A, l + B, n.di, n.dj, true, n.out, false);
+      w = site_word(k + A, l + B, n.di, n.dj, true, n.out);
     else
       w = site_owner_exact(g, X.tay, X.tayl, k, l, i, j, dup);
     S.so[idx] = w;
@@ -927,6 +943,18 @@ __device__ __forceinline__ void map_sites_body(const Grid& g, const SiteArgs& X,
     site_edge(g, X, S, idx, i00 + r, j00 + idx - r * SITE_CC, inv_s);
   }
   __syncthreads();
+  if constexpr (kWide) {
+    for (int at = tid; at < SITE_R * SITE_C; at += SITE_T) {
+      const int r = at / SITE_C + 1, c = at % SITE_C + 1;
+      const uint32_t kl = S.so[r * SITE_CC + c] & SO_ELEM;
+      if (kl == SO_NONE) continue;
+      const int k = (int)(kl >> 12), l = (int)(kl & 4095u), m = k * g.Lv + l;
+      const uint32_t w = __ldcg(X.flags + m);
+      if (elem_settled(w) && !(w & EF_WIDE) && leaves_window(g, X.tayl, k, l, i00 + r, j00 + c))
+        atomicOr(X.flags + m, EF_WIDE);
+    }
+    return;
+  }
   // every site of the tile: owner slot, (c), and the other owners around it
   int np = 0;
   for (int hb = 0; hb < SITE_HB; hb++) {
@@ -951,16 +979,13 @@ __device__ __forceinline__ void map_sites_body(const Grid& g, const SiteArgs& X,
       const int m = (int)(kl >> 12) * g.Lv + (int)(kl & 4095u);
       const bool in = jin && (unsigned)(i0 + t) < (unsigned)g.nx;
       if (in) *slot = E | (uint32_t)m;
-      if (!((w >> SO_DIR) & same) || (w & (SO_UNSURE | SO_FAR | SO_OUT))) {  // rare, but for start sites
+      if (!((w >> SO_DIR) & same) || (w & (SO_UNSURE | SO_OUT))) {  // rare, but for start sites
         const bool start = ((w >> SO_DIR) & 15u) == 0u;
         if (w & SO_OUT) {
           if (in) leave_to_flood(X.flags, m);
         } else {
           if (start) atomicOr(X.flags + m, EF_START);
           if ((!start && !((w >> SO_DIR) & same)) || (w & SO_UNSURE)) leave_to_flood(X.flags, m);
-          // statistics: components no small window would have held
-          if ((w & SO_FAR) && !(__ldcg(X.flags + m) & EF_WIDE) && !(atomicOr(X.flags + m, EF_WIDE) & EF_WIDE))
-            atomicAdd(&X.ds->wide, 1);
         }
       }
     }
@@ -1019,7 +1044,15 @@ __device__ __forceinline__ void map_sites_body(const Grid& g, const SiteArgs& X,
 __global__ void __launch_bounds__(SITE_T, SITE_BPS) k_map_sites(Grid g, SiteArgs X) {
   if (!after_prior()) return;
   if (gate_shut(g) || __ldcg(&X.ds->skip_sites)) return;
-  map_sites_body(g, X, blockIdx.x);
+  map_sites_body<false>(g, X, blockIdx.x);
+}
+
+__global__ void __launch_bounds__(SITE_T) k_map_wide(Grid g, SiteArgs X) { map_sites_body<true>(g, X, blockIdx.x); }
+
+__global__ void __launch_bounds__(256) k_count_wide(const uint32_t* __restrict__ flags, int ne, DevState* ds) {
+  const int m = blockIdx.x * 256 + threadIdx.x;
+  const int n = __syncthreads_count(m < ne && (flags[m] & EF_WIDE));
+  if (threadIdx.x == 0 && n) atomicAdd(&ds->wide, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -3032,6 +3065,8 @@ void launch_map(vm_solver* s) {
   int ps = -1;
   if (s->g.fth_on) launch_domain_rect(s);
   const int all = s->cfg.map_windows != 0 || !site_pass_on(s->g);
+  s->gmap = s->g;
+  s->gmap.gate = nullptr;
   if (!all) {
     ps = prof_begin(s, KID_MAP_SITES);
     launch_next(k_map_sites, (unsigned)site_tiles(s->g), SITE_T, 0, s->stream, s->g, SiteArgs{s->tay, s->tayf,
@@ -3057,6 +3092,20 @@ void launch_map(vm_solver* s) {
   cudaLaunchCooperativeKernel((const void*)k_flood, dim3((unsigned)blocks), dim3(BT), args, smem, s->stream);
   prof_end(s, ps);
   s->launches += all ? 2 : 3;
+}
+
+// Count into ds->wide the elements that the last map's site pass settled and whose
+// component leaves the small windows (none where there was no site pass: no flag
+// of the map says settled).
+void launch_count_wide(vm_solver* s) {
+  if (s->cfg.map_windows != 0 || !site_pass_on(s->g) || s->gmap.ne == 0) return;
+  float alo, ahi;
+  alpha_bounds(s->g.alpha, alo, ahi);
+  cudaMemsetAsync(&s->ds->wide, 0, sizeof s->ds->wide, s->stream);
+  k_map_wide<<<(unsigned)site_tiles(s->g), SITE_T, 0, s->stream>>>(
+      s->gmap, SiteArgs{s->tay, s->tayf, s->tayl, s->map, s->flags, s->ds, alo, ahi});
+  k_count_wide<<<(unsigned)((s->g.ne + 255) / 256), 256, 0, s->stream>>>(s->flags, s->g.ne, s->ds);
+  s->launches += 2;
 }
 
 void launch_read_map(vm_solver* s, int32_t* dst) {
