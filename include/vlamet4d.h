@@ -127,8 +127,10 @@ int32_t vm_4d_num_elements(const vm_4d_solver* s, int32_t* L4);
 int64_t vm_4d_launches(const vm_4d_solver* s);
 
 /* Statistics of the last influence map (synchronises): out3[0] elements whose
- * component outgrew the shared-memory flood window of side 2*min(2s, 12)+1
- * and were filled again over the whole padded lattice, out3[1] unexplored
+ * component outgrew the flood window of side 2*min(2s, 12)+1 (reached its edge
+ * where the padded lattice goes on, or for the flood fill outgrew its lists):
+ * those left to the flood fill, which were filled again over the whole padded
+ * lattice, and those that the site pass settled without it; out3[1] unexplored
  * sites left by the percolation, out3[2] repair rounds (Sec. 2.3.1);
  * *d2_evals (may be NULL): the FP64 distance evaluations d^2 = |Q(P) - Q_m|^2
  * in the fixed order since creation (219 FP64 operations each), the ones the

@@ -93,7 +93,7 @@ struct Dev4 {
   int32_t bad_where;
   int32_t novf;  // elements whose component left the shared-memory window (this map)
   int32_t nflood;  // elements left to the flood fill (this map)
-  int32_t wide;  // other elements whose component reaches beyond the window (this map)
+  int32_t wide;  // other elements whose component reaches the window's edge (this map)
   int32_t rounds;  // hole-repair rounds of the last map
   unsigned long long nclaims;  // sites of the whole-lattice fills, claimed after them (0 between maps)
   unsigned long long d2_evals;  // distance evaluations of the percolation kernels (cumulative)
@@ -996,8 +996,15 @@ __global__ void __launch_bounds__(T4, 3) k4_sites(G4 g, const float* __restrict_
   }
   const int j0 = c[0] - st.x, j1 = c[1] - st.y, j2 = c[2] - st.z, j3 = c[3] - st.w;
   if ((j0 | j1 | j2 | j3) == 0) atomicOr(S.flags + m, EF4_START);
-  if (max(max(abs(j0), abs(j1)), max(abs(j2), abs(j3))) > g.R && !(__ldcg(S.flags + m) & EF4_WIDE))
-    atomicOr(S.flags + m, EF4_WIDE);
+  // on or beyond the edge of the flood fill's window, where the padded lattice goes on
+  if (max(max(abs(j0), abs(j1)), max(abs(j2), abs(j3))) >= g.R && !(__ldcg(S.flags + m) & EF4_WIDE)) {
+    const int j[4] = {j0, j1, j2, j3}, s0[4] = {st.x, st.y, st.z, st.w};
+    bool wide = false;
+#pragma unroll
+    for (int a = 0; a < 4; a++)
+      wide = wide || (j[a] <= -g.R && s0[a] - g.R - 1 >= -g.pad) || (j[a] >= g.R && s0[a] + g.R + 1 < g.n[a] + g.pad);
+    if (wide) atomicOr(S.flags + m, EF4_WIDE);
+  }
 }
 
 // Each site against its eight neighbours: one of its owner's nearer to the
