@@ -2366,7 +2366,7 @@ __device__ __noinline__ double resample4_fp64(const G4& g, const double* __restr
 // the beta ranges from the owner's offsets where they clear beta, Q_r as the
 // owner's Q plus the weighted mean of the other elements' differences from
 // it, the 256 coefficients as 60-bit integers scaled by the largest one's
-// exponent, contracted one axis at a time.  At 64^4: 25.7 ms per remap, in
+// exponent, contracted one axis at a time.  At 64^4: 24.4 ms per remap, in
 // FP64 86.9 ms; error against 128-bit arithmetic 1.2e-16, before 1.0e-15.
 __device__ __forceinline__ bool resample4_fixed(const G4& g, const Fx4* __restrict__ tayx,
                                                 const double* __restrict__ eta, const int* site, int m, double& val) {
@@ -2390,7 +2390,7 @@ __device__ __forceinline__ bool resample4_fixed(const G4& g, const Fx4* __restri
   // products keep all bits until the division)
   __int128 num[4] = {0, 0, 0, 0};
   unsigned long long den = 0;
-  bool others = false;  // elements besides the owner have a weight
+  unsigned long long apart = 0;  // bits of the elements' differences
   // The elements of the blend: every subset of the axes that are not full, each
   // towards its side, and one step either way along a full axis alone; at most
   // 16, counted off by each lane for itself (nested loops over the ranges made a
@@ -2433,15 +2433,18 @@ __device__ __forceinline__ bool resample4_fixed(const G4& g, const Fx4* __restri
     const long long w = vm::fx_kernel(d2);
 #pragma unroll
     for (int a = 0; a < 4; a++) {
-      if ((D[a] < 0 ? -D[a] : D[a]) >> 59) return false;  // four cells apart
+      const unsigned long long Da = D[a] < 0 ? -D[a] : D[a];
+      if (Da >> 59) return false;  // four cells apart
+      apart |= Da;
       num[a] += (__int128)D[a] * w;
     }
     den += (unsigned long long)w >> 3;
-    others = others || set != 0;
   }
-  // a weight's last bits, some 2^-60, over a sum of 2^-10: 2^-48 of the differences,
-  // as much as of an FP64 blend's; smaller sums take that one
-  if (others && den < 1ull << (59 - 10)) return false;
+  // the weights' last bits, together some 2^-56, over their sum and times the
+  // differences are below 2^-46 cells down to a sum of 2^-10 times these, which
+  // elements that agree never come to; others take the FP64 blend, whose weights
+  // 2 (1 - d)^3 keep their digits
+  if (den < apart >> (10 - (59 - FX4_Q))) return false;
   const int z = den > 0 ? max(__clzll((long long)den) - 4, 0) : 0;  // both scaled by 2^z for the division
   int gk[4][4], wh[4][4], wl[4][4];
 #pragma unroll
