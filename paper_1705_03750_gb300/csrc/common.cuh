@@ -55,8 +55,6 @@ struct Grid {
   const int32_t* gate;
 };
 
-// True when the remap this Grid was enqueued for is not to run (read by
-// every thread of a kernel before any barrier, so all return together).
 // The kernels of a step follow one another closely (launch_next below): a
 // kernel's blocks are placed while the one before drains, and wait here, before
 // their first access, for it to have completed.  Each lets the next one's
@@ -88,6 +86,8 @@ inline void launch_next(void (*k)(P...), unsigned grid, unsigned block, size_t s
   cudaLaunchKernelEx(&cfg, k, P(args)...);
 }
 
+// True when the remap this Grid was enqueued for is not to run (read by
+// every thread of a kernel before any barrier, so all return together).
 __device__ __forceinline__ bool gate_shut(const Grid& g) { return g.gate != nullptr && __ldcg(g.gate) == 0; }
 
 // Small device-resident control block.

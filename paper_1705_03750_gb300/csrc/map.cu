@@ -47,7 +47,7 @@
 // distance comparison clears its bound, otherwise the exact FP64 test runs.
 // The outcome is therefore identical to the all-FP64 evaluation.
 //
-// Claims.  A claimed site's owner slot takes (epoch << 24 | m) with one
+// Claims.  A claimed site's owner slot takes (epoch + 1) << 24 | m with one
 // atomic exchange.  A claim that displaces a current-epoch owner folds into
 // the site's record (a 128-bit key per site, empty between maps), by a
 // 128-bit compare-and-swap minimum, the exact FP64 keys (bits of d^2,

@@ -390,7 +390,7 @@ __device__ __forceinline__ double spline_eval(const R* __restrict__ eta, const G
 // spline's 16 coefficients are scaled to integers by the largest one's
 // exponent.  Q_r and the spline are continuous, so no other decision is
 // taken.  Returns false where a record, the margin, the grid's edge or the
-// values' range do not allow it.  At 4096^2: 2.58 ms per remap, in FP64
+// values' range do not allow it.  At 4096^2: 2.64 ms per remap, in FP64
 // 14.2 ms; error against 128-bit arithmetic 0.7 to 3.1e-16 (2-norm), before
 // 1.1 to 2.9e-15.
 __device__ __forceinline__ bool remap64_fixed(const Grid& g, const FxRec* __restrict__ tayx, int m, int i, int j,

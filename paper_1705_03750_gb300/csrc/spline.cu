@@ -202,8 +202,12 @@ __global__ void __launch_bounds__(32 * CW) k_cols(Grid g, R* __restrict__ x, con
 //   c_k = f_k + z c_{k-1},  e_k = c_k + z e_{k+1},  eta_k = -6 z e_k,
 // with the same coefficients everywhere.  A filter forgets its start by z per
 // step, so a chunk swept from WARM = 32 entries before its own (of the mirrored
-// data at an end) has the carry to 5e-19 of its size, far below a rounding of
-// it: no carries are chained and no chunk is corrected.  An entry takes two FP64
+// data at an end) has the carry to 5e-19 of the carry there: a thousandth of a
+// rounding of the largest coefficient around, though not of its own size where f
+// falls by more than that within the warm-up (behind a cut edge).  No carries are
+// chained and no chunk is corrected.  An entry that is not finite spreads to the
+// chunks whose sweep or warm-up holds it (the LU sweeps spread it over its whole
+// line).  An entry takes two FP64
 // operations, times 1 + WARM / chunk, where the scan of a row takes 28 and the
 // chained column sweeps 12 (this GPU has two FP64 lanes per SM); the factors of
 // both axes are applied at the end.  One pass over memory per axis, where the
@@ -388,7 +392,8 @@ __global__ void __launch_bounds__(32 * NW) k_cols_filter(Grid g, const R* __rest
 
 // Grids whose coefficients take the filters: the mirrored data of a warm-up lie
 // on the grid, and FP64 solves below fixed_on keep the sweeps' rounding along
-// with that of their values (5 to 15 us a solve).
+// with that of their values (5 to 15 us a solve).  FP32 solves have the same line
+// only to have one.
 __host__ __device__ __forceinline__ bool filters_on(const Grid& g) {
   return g.nx > WARM && g.nv > WARM && (long long)g.nx * g.nv >= kFixedSites;
 }
