@@ -445,7 +445,7 @@ __device__ __forceinline__ bool test_site(const Grid& g, const Elem9& E, const C
 // neighbours; every site's (c) and the other owners next to it; and those
 // pairs (about one for every two sites), listed and tested.
 //
-// Bound by instruction issue (70 % of the slots; about 13 warp
+// Bound by instruction issue (two thirds of the slots; about 13 warp
 // instructions a site) and by the barriers between the phases.  4096 x 4096,
 // stride 8: 302 us, and 15 us for the elements left to the fill, where the fill
 // of all of them took 396 + 90 us; 8192 x 8192, step and map together: 76 ms a

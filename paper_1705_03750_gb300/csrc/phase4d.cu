@@ -577,9 +577,10 @@ __device__ __forceinline__ void claim4(ulonglong2* key, unsigned long long dbits
 // for each of a component's and formed its shell: 64^4 sites 2.5 ms and 0.4 ms
 // for the elements left to the fill, where the fill of all took 8.8 ms; without
 // k4_gaps, which settles most neighbours without an evaluation, 3.1 ms.  Bound by
-// the records' reads (288 bytes an evaluation through L1) and by occupancy: with
-// whole records held in registers (2 blocks an SM) and the guess formed inside
-// each tile the two kernels took 4.8 ms.
+// latency: neither issue (50 and 57 % of the slots) nor L1 (52 and 37 %) is full,
+// with 36 and 42 % of the warps the barriers between the phases and the records'
+// reads (288 bytes an evaluation) show; with whole records held in registers (2
+// blocks an SM) and the guess formed inside each tile the two kernels took 4.8 ms.
 constexpr uint32_t EF4_BAD = 1u, EF4_START = 2u, EF4_WIDE = 4u;
 
 struct Sites4 {
@@ -1913,8 +1914,8 @@ __device__ __noinline__ double recon4_fp64(const G4& g, const double* __restrict
 // side of the node that holds Q along an axis and o the other,
 //   f = F0 + sum_a x_a [(Fs_a - Fo_a)/2 + x_a (Fs_a + Fo_a - 2 F0)/2
 //                       + sum_{b > a} x_b (F0 + Fd_ab - Fs_a - Fs_b)],  x >= 0.
-// At 64^4: 0.93 ms per step, bound by the integer pipes and the record's 512
-// bytes a site through L1; in fused FP64 7.46 ms.  Error against 128-bit
+// At 64^4: 0.93 ms per step, bound by the record's 512 bytes a site through L1
+// (81 %; issue 53 %); in fused FP64 7.46 ms.  Error against 128-bit
 // arithmetic (20 x 18 x 22 x 16 and 24^4): 1.4e-16, before 7.6e-16 (2-norm).
 __device__ __forceinline__ bool recon4_fixed(const G4& g, const Fx4* __restrict__ X, const double* __restrict__ F,
                                              const int* site, double& val) {
@@ -2366,7 +2367,8 @@ __device__ __noinline__ double resample4_fp64(const G4& g, const double* __restr
 // the beta ranges from the owner's offsets where they clear beta, Q_r as the
 // owner's Q plus the weighted mean of the other elements' differences from
 // it, the 256 coefficients as 60-bit integers scaled by the largest one's
-// exponent, contracted one axis at a time.  At 64^4: 24.4 ms per remap, in
+// exponent, contracted one axis at a time.  At 64^4: 24.4 ms per remap (bound by
+// latency: issue 47 %, L1 54 %, a quarter of the warps at 128 registers), in
 // FP64 86.9 ms; error against 128-bit arithmetic 1.2e-16, before 1.0e-15.
 __device__ __forceinline__ bool resample4_fixed(const G4& g, const Fx4* __restrict__ tayx,
                                                 const double* __restrict__ eta, const int* site, int m, double& val) {
