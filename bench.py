@@ -157,8 +157,11 @@ def algorithmic(kernel: str, rc, fp32: bool, ne: int):
         return n * (4 + 2 * sr) + ne * tay, n, f"{4 + 2 * sr} B/site + 128 B/element"
     if kernel == "remap_resample":
         return n * (4 + 2 * sr) + ne * tay, n, f"{4 + 2 * sr} B/site + 128 B/element"
-    if kernel in ("map_sites", "claim_pair", "flood"):
-        # the influence map written once (4 B/site), each element's record read once
+    if kernel == "map_sites":
+        # the influence map written once (4 B/site), each element's record of 64 bytes read once
+        return n * 4 + ne * 64, n, "4 B/site + 64 B/element"
+    if kernel in ("claim_pair", "flood"):
+        # the fill of everything (without the site pass): the map written once, each record read once
         return n * 4 + ne * tay, n, "4 B/site + 128 B/element"
     if kernel in ("spline_rows", "spline_cols"):
         return n * 4 * sr, n, f"{4 * sr} B/site (2 sweeps, read+write)"
@@ -169,11 +172,11 @@ def algorithmic(kernel: str, rc, fp32: bool, ne: int):
 
 def fp64_roofline(rc, ne: int, avg_s: float, hbm_gbs: float, peak_kind: str) -> dict:
     """The FP64 path's reconstruction, whose values are formed in 64-bit fixed
-    point on the integer pipes: its algorithmic bytes against the HBM copy
-    peak."""
+    point and which the integer pipes bound: its algorithmic bytes against the
+    HBM copy peak."""
     b, units, per = algorithmic("reconstruct", rc, False, ne)
     ach = b / avg_s / 1e9
-    return {"kernel": "reconstruct", "bound": "hbm", "achieved": ach, "peak": hbm_gbs, "unit": "GB/s",
+    return {"kernel": "reconstruct", "bound": "integer issue", "achieved": ach, "peak": hbm_gbs, "unit": "GB/s",
             "frac": ach / hbm_gbs, "per_unit": per, "units": units, "avg_ms": avg_s * 1e3, "peak_kind": peak_kind}
 
 
@@ -192,9 +195,9 @@ def step_bytes_per_update(rc, fp32: bool) -> float:
 # time of the capture: a source changed since makes the figure void (null).
 NCU_TRAFFIC = {
     # kernel: (bytes per launch, source file, sha256 prefix)
-    "map_sites": (48_985_600, "map.cu", "bf685670166ba9e5"),
-    "claim_pair": (137_759_488, "map.cu", "7ef7750fd3fe8b25"),  # of all elements, before the site pass
-    "reconstruct": (217_149_952, "recon.cu", "0c50efd2b296a2b4"),
+    "map_sites": (51_701_248, "map.cu", "28848838d971d0b3"),
+    "claim_pair": (1_717_760, "map.cu", "28848838d971d0b3"),  # the elements left to the fill
+    "reconstruct": (220_568_064, "recon.cu", "f590612fddb3b1aa"),
 }
 
 # Warp instructions per launch (smsp__inst_executed.sum) from the same
@@ -202,22 +205,44 @@ NCU_TRAFFIC = {
 # their issue roofline is these instructions over the launch time against
 # one warp instruction per scheduler per clock (4 schedulers x 152 SMs).
 NCU_INSTR = {
-    "map_sites": (218_392_780, "map.cu", "bf685670166ba9e5"),
-    "reconstruct": (126_556_082, "recon.cu", "0c50efd2b296a2b4"),
+    "map_sites": (218_548_290, "map.cu", "28848838d971d0b3"),
+    "reconstruct": (127_271_809, "recon.cu", "f590612fddb3b1aa"),
 }
+
+# What the captures show to bound a kernel that moves its bytes at a small part of
+# the HBM peak (at most a fifth of it in DRAM traffic); the others are taken by it.
+LIMITER = {"map_sites": "issue", "reconstruct": "l1"}
+LIMITER4 = {"sites": "latency", "sites_check": "latency", "reconstruct": "l1", "resample": "latency",
+            "percolate": "latency"}
 
 SCHEDULERS = 4 * 152
 
-# The same figures for the 4D phase-space path, keyed over the source before
-# its reconstruction section (the map and what it uses): none of the present one.
+# The same figures for the 4D phase-space path (its 64^4 workload).  The
+# percolation's key hashes the source before the reconstruction section (the map
+# and what it uses): changes further down cannot change its code.
 PHASE4D_PREFIX_END = "// Sec. 2.2.1: 15-point quadratic interpolation; transport reconstruction"
-NCU4_TRAFFIC = {}
-NCU4_INSTR = {}
+NCU4_TRAFFIC = {
+    "percolate": (75_195_648, "phase4d.cu", "733d3b575d352f14"),
+    "reconstruct": (352_078_336, "phase4d.cu", "eaa76f46813066bf"),
+    "resample": (386_545_152, "phase4d.cu", "eaa76f46813066bf"),
+}
+NCU4_INSTR = {
+    "percolate": (183_644_894, "phase4d.cu", "733d3b575d352f14"),
+    "reconstruct": (617_545_743, "phase4d.cu", "eaa76f46813066bf"),
+    "resample": (14_387_600_768, "phase4d.cu", "eaa76f46813066bf"),
+}
+
+
+def keyed4(table, kernel: str):
+    return _keyed(table, kernel, PHASE4D_PREFIX_END if kernel == "percolate" else None)
 
 
 def issue_roofline(kernel: str, avg_s: float, sm_mhz):
     """Issue roofline of a kernel with a captured instruction count, or None."""
-    n = _keyed(NCU_INSTR, kernel)
+    return issue_of(_keyed(NCU_INSTR, kernel), avg_s, sm_mhz)
+
+
+def issue_of(n, avg_s: float, sm_mhz):
     if n is None or not sm_mhz:
         return None
     peak = SCHEDULERS * sm_mhz * 1e6
@@ -492,7 +517,7 @@ def run_native(args, rank: int, world: int, dist):
     if alg is not None:
         b, units, per = alg
         ach = b / avg_s / 1e9
-        roof.update({"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
+        roof.update({"bound": LIMITER.get(dom, "hbm"), "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                      "frac": ach / peaks["hbm_gbs"], "traffic": ncu_traffic(dom), "per_unit": per,
                      "units": units, "peak_kind": peak_kind})
     # the limiter the counters show for the map and the reconstruction
@@ -618,6 +643,9 @@ def algorithmic4(kernel: str, sites: int, padded: int, ne: int):
         return (8 * padded + 288 * ne) / 3, "8 B/padded site + 288 B/element over three launches"
     if kernel == "sites_check":
         return (8 * padded + 288 * ne) / 2, "8 B/padded site + 288 B/element over two launches"
+    if kernel == "percolate":
+        # the fill of everything: the map, each element's FP64 and FP32 records
+        return 4 * sites + (8 * 64 + 4 * 72) * ne, "4 B/site + 800 B/element"
     return None
 
 
@@ -680,28 +708,14 @@ def phase4d_run(args, dev, peaks, clock_mhz=None) -> dict:
     def hbm4(kernel: str, avg_ms: float) -> dict:
         b, per = algorithmic4(kernel, sites, padded, L4)
         ach = b / (avg_ms / 1e3) / 1e9
-        return {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                "frac": ach / peaks["hbm_gbs"], "per_unit": per, "units": sites}
+        r = {"bound": LIMITER4.get(kernel, "hbm"), "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
+             "frac": ach / peaks["hbm_gbs"], "per_unit": per, "units": sites, "traffic": keyed4(NCU4_TRAFFIC, kernel)}
+        iss = issue_of(keyed4(NCU4_INSTR, kernel), avg_ms / 1e3, clock_mhz or 2070.0)
+        return r if iss is None else dict(r, issue=iss)
 
-    if dom == "percolate":
-        # bound by instruction issue (FP32 tests, integer bookkeeping, atomics;
-        # FP64 only at open decisions and contested claims): the capture's
-        # warp instructions over the launch time against one warp instruction
-        # per scheduler per clock
-        n_instr = _keyed(NCU4_INSTR, "percolate", PHASE4D_PREFIX_END)
-        mhz = clock_mhz or 2070.0
-        peak = SCHEDULERS * mhz * 1e6
-        ach = n_instr / (tms / nl / 1e3) if n_instr else None
-        roof.update({"bound": "alu", "achieved": ach, "peak": peak, "unit": "warp-instr/s",
-                     "frac": (ach / peak) if ach else None,
-                     "traffic": _keyed(NCU4_TRAFFIC, "percolate", PHASE4D_PREFIX_END),
-                     "per_unit": "warp instructions of one launch (ncu capture of this source)",
-                     "units": n_instr, "clock_mhz": mhz,
-                     "peak_kind": "4 schedulers x 152 SMs x the SM clock",
-                     "algorithmic_bytes": 4 * sites + (8 * 64 + 4 * 72) * L4,
-                     "fp64_exact_distances_per_launch": (ev1 - ev0) / nl})
-    elif algorithmic4(dom, sites, 1, L4) is not None:
+    if algorithmic4(dom, sites, 1, L4) is not None:
         roof.update(hbm4(dom, tms / nl))
+    roof["fp64_exact_distances_per_map"] = (ev1 - ev0) / stats["map_finish"][0]
     # end to end through the C ABI with host buffers over the same step
     # indices: upload of f0 from pinned host memory, then every timed step
     # reads the pixel masses back to the host
